@@ -585,26 +585,21 @@ __global__ void __launch_bounds__(256) k_group_adam(const IterArgs a, const Grou
     s_last = (atomicAdd(g.gdone, 1) == static_cast<int>(gridDim.x) - 1);
   }
   __syncthreads();
-  if (!s_last || tid != 0) return;
-  __threadfence();
-  *g.gdone = 0;
-  {
+  if (!s_last || tid >= 2) return;
+  // constants of the next iteration, t = step + 2 (bias corrections in double)
+  const_cast<float*>(a.adamc)[tid] = adam_constant(tid, a.lr, a.beta1, a.beta2, static_cast<int64_t>(step) + 2);
+  if (tid == 0) {
+    __threadfence();
+    *g.gdone = 0;
     *const_cast<int32_t*>(a.step) = step + 1;
-    // constants of the next iteration, t = step + 2 (bias corrections in double)
-    const double t2 = static_cast<double>(step) + 2.0;
-    float* ac = const_cast<float*>(a.adamc);
-    ac[0] = static_cast<float>(a.lr / (1.0 - pow(static_cast<double>(a.beta1), t2)));
-    ac[1] = static_cast<float>(1.0 / sqrt(1.0 - pow(static_cast<double>(a.beta2), t2)));
   }
 }
 
 // Adam constants for the coming iteration t = step + 1 (after init or a checkpoint load).
 __global__ void k_adam_constants(const IterArgs a) {
-  if (threadIdx.x != 0) return;
-  const double t1 = static_cast<double>(*a.step) + 1.0;
-  float* ac = const_cast<float*>(a.adamc);
-  ac[0] = static_cast<float>(a.lr / (1.0 - pow(static_cast<double>(a.beta1), t1)));
-  ac[1] = static_cast<float>(1.0 / sqrt(1.0 - pow(static_cast<double>(a.beta2), t1)));
+  if (threadIdx.x >= 2) return;
+  const_cast<float*>(a.adamc)[threadIdx.x] =
+      adam_constant(threadIdx.x, a.lr, a.beta1, a.beta2, static_cast<int64_t>(*a.step) + 1);
 }
 
 // Table refresh after the caller sets group parameters (exp(alpha), beta).

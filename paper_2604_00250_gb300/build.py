@@ -21,7 +21,7 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxe
          "-I", INCLUDE, "-I", CSRC]
 SOURCES = ["prism_api.cu", "prism_aux.cu", "prism_noalloc.cu", "prism_ubench.cu", "prism_k1.cu", "prism_k2.cu", "prism_k3.cu", "prism_k4.cu",
            "prism_k5.cu"]
-HEADERS = ["prism_device.cuh", "prism_kernels.cuh", "prism_kset.cuh", "prism_launch.h", "bessel_fit.h"]
+HEADERS = ["prism_device.cuh", "prism_kernels.cuh", "prism_kset.cuh", "prism_local.cuh", "prism_launch.h", "bessel_fit.h"]
 
 
 def nvcc():

@@ -22,6 +22,7 @@
 #include "prism.h"
 #include "prism_kernels.cuh"
 #include "prism_launch.h"
+#include "prism_local.cuh"
 
 using namespace prism;
 
@@ -95,7 +96,7 @@ struct prism_handle {
   int32_t *d_nbr = nullptr, *d_queue = nullptr, *d_done = nullptr, *d_step = nullptr, *d_status = nullptr;
   float* d_adamc = nullptr;
   int32_t *d_slot_of_vox = nullptr, *d_vox_of_slot = nullptr, *d_slot_of_grid = nullptr;
-  int32_t *d_split_off = nullptr, *d_counters = nullptr;
+  int32_t *d_split_off = nullptr, *d_counters = nullptr, *d_gbar = nullptr;
   uint32_t *d_vcoord = nullptr, *d_vflag = nullptr;
   int64_t* d_row_off = nullptr;
   int32_t* d_order = nullptr;          // [tab_rows] table position -> caller's measurement index
@@ -113,6 +114,9 @@ struct prism_handle {
   std::vector<ShellRun> runs;
   bool shells_even = true;             // every group's shells hold an even number of measurements
   bool shell = false;                  // the fused kernel takes the shell loop
+  bool local = false;                  // iterations run in k_iter_local, many per launch
+  int local_grid = 0;
+  size_t local_smem = 0;
   float* d_gtab = nullptr;
   ShellRun* d_runs = nullptr;
   double *d_tile_red = nullptr, *d_part2 = nullptr, *d_gred = nullptr, *d_gloss = nullptr;
@@ -309,6 +313,8 @@ void fill_args(prism_handle* h) {
   a.step_max = o.rprop_step_max;
   a.nb_priors = h->nb ? 1 : 0;
   a.pdl = 1;
+  a.n_it = 1;
+  a.gbar = h->d_gbar;
   a.n_nbr = o.connectivity;
   a.lam_orphan = o.lam_orphan;
   a.inv_s_orphan = 1.f / o.s_orphan;
@@ -363,6 +369,23 @@ int enqueue_fused_iter(prism_handle* h, cudaStream_t st) {
     CK(launch_bias_grad(a, h->ga, st));
     CK(launch_group_reduce(a, h->ga, 1 | 2, st));
     CK(launch_group_adam(a, h->ga, 1 | 2, st));
+  }
+  return PRISM_OK;
+}
+
+// Enqueues n fused iterations: up to kMaxIters per launch in the local kernel, or one by one.
+int enqueue_fused_iters(prism_handle* h, int n, cudaStream_t st) {
+  if (!h->local) {
+    for (; n > 0; --n) {
+      const int rc = enqueue_fused_iter(h, st);
+      if (rc != PRISM_OK) return rc;
+    }
+    return PRISM_OK;
+  }
+  IterArgs a = h->ia;
+  for (; n > 0; n -= a.n_it) {
+    a.n_it = std::min(n, kMaxIters);
+    CK(h->ks->local(a, h->opt.loss, h->TPV, h->local_grid, h->local_smem, st));
   }
   return PRISM_OK;
 }
@@ -723,6 +746,11 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   h->nb = (o.lam_sp > 0.f) || (o.lam_dir > 0.f);
   h->ks = &kernels_for_k(o.K);
   h->TV = h->NT / h->TPV;
+  int dev = 0, sms = 0;
+  if (o.fused) {
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  }
   // Host signals start their copy to the device before the plan is built: a copy needs only the
   // voxel count, and the DMA then runs while the host builds the plan. All copies start at once
   // when together they take at most a quarter of the free device memory; otherwise each volume
@@ -757,6 +785,15 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
     h->max_split = std::max(h->max_split, ns);
   }
   const int nce = (h->max_e + 255) / 256;
+  // The local kernel (prism_local.cuh): several lanes per voxel, no neighbour priors, no calibration;
+  // with the Rician NLL, whose CTAs exchange sums, only where all tiles are resident at once.
+  if (o.fused && !h->cal && !h->nb && h->TPV > 1) {
+    int bps = 0;
+    h->local_smem = local_smem(h->K, h->TPV, h->Nmax);
+    CK(h->ks->local_occupancy(o.loss, h->TPV, h->local_smem, &bps));
+    h->local_grid = std::min(h->ntiles, sms * bps);
+    h->local = bps > 0 && (o.loss == PRISM_LOSS_MSE || h->local_grid == h->ntiles);
+  }
   // allocations
   RC(h->alloc(&h->d_tiles, h->ntiles));
   RC(h->alloc(&h->d_tile_order, h->ntiles));
@@ -773,7 +810,8 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   CK(cudaMemsetAsync(h->d_pg, 0, sizeof(float) * pg_len, st));
   RC(h->alloc(&h->d_gU, Vp));
   RC(h->alloc(&h->d_tile_ab, h->ab_len));
-  RC(h->alloc(&h->d_tile_red, 4 * static_cast<size_t>(h->ntiles)));
+  const size_t red_len = static_cast<size_t>(h->ntiles) * (h->local ? kMaxIters * kLocalRed : 4);
+  RC(h->alloc(&h->d_tile_red, red_len));
   RC(h->alloc(&h->d_nbr, static_cast<size_t>(o.connectivity) * Vp));
   RC(h->alloc(&h->d_vcoord, Vp));
   RC(h->alloc(&h->d_vflag, Vp));
@@ -803,6 +841,8 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   RC(h->alloc(&h->d_part2, static_cast<size_t>(tot_split) * h->max_e));
   RC(h->alloc(&h->d_counters, static_cast<size_t>(G) * nce));
   RC(h->alloc(&h->d_gdone, 1));
+  RC(h->alloc(&h->d_gbar, G));
+  CK(cudaMemsetAsync(h->d_gbar, 0, sizeof(int32_t) * G, st));
   CK(cudaMemsetAsync(h->d_gdone, 0, sizeof(int32_t), st));
   if (h->cal) {
     // per group [nx][ny][8] then [nx][8][8] doubles for the separable bias-field adjoint
@@ -835,7 +875,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   CK(cudaMemsetAsync(h->d_lp, 0, sizeof(float) * Vp, st));
   CK(cudaMemsetAsync(h->d_gU, 0, sizeof(float) * Vp, st));
   CK(cudaMemsetAsync(h->d_tile_ab, 0, sizeof(float) * std::max<int64_t>(h->ab_len, 1), st));
-  CK(cudaMemsetAsync(h->d_tile_red, 0, sizeof(double) * 4 * h->ntiles, st));
+  CK(cudaMemsetAsync(h->d_tile_red, 0, sizeof(double) * red_len, st));
   CK(cudaMemsetAsync(h->d_gparams, 0, sizeof(float) * h->GP, st));
   CK(cudaMemsetAsync(h->d_gm, 0, sizeof(float) * h->GP, st));
   CK(cudaMemsetAsync(h->d_gv, 0, sizeof(float) * h->GP, st));
@@ -955,9 +995,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   }
   h->adj_smem = h->cal ? static_cast<size_t>(NW) * 2 * h->Nmax * sizeof(float) : 0;
   if (o.fused) {
-    int dev = 0, sms = 0, bps = 0;
-    CK(cudaGetDevice(&dev));
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int bps = 0;
     CK(h->ks->fused_occupancy(o.loss, h->cal ? 1 : 0, h->TPV, h->shell ? 1 : 0, h->NT, h->fused_smem, &bps));
     if (bps < 1) return fail(PRISM_E_CUDA, "fused kernel does not fit on an SM");
     h->fused_grid = std::max(1, std::min(h->ntiles, sms * bps));
@@ -974,9 +1012,12 @@ int choose_shape(const prism_options& o, int64_t V, bool shell, int* tpv, int* n
   // better (40^3: 7-19 % faster; calibrated, 14-19 %). Where the shell loop applies (`shell`:
   // it needs one thread per voxel) four lanes pay only above one wave: 40^3 (0.82 waves) 20 %
   // slower than the shell loop, 45^3 (1.17 waves) 2 % faster, 47^3 (1.33 waves) 4 % slower.
+  const bool local = o.fused && !o.calibration && !(o.lam_sp > 0.f) && !(o.lam_dir > 0.f);
   if (o.threads_per_voxel) {
     *tpv = o.threads_per_voxel;
-  } else if (V < 2048) {
+  } else if (V < (local ? 1400 : 2048)) {
+    // (without neighbour priors and calibration the local kernel runs: 10^3 voxels at N = 96 3.75 us
+    // an iteration with sixteen lanes, 3.88 with four, 12^3 4.8 and 4.2; NLL 8.7 and 8.4, 10.7 and 9.3)
     *tpv = 16;
   } else if (V < 32768) {
     *tpv = 4;
@@ -1068,7 +1109,8 @@ int create_handle(const prism_volume* vols, int n_vols, const std::vector<int64_
   h->TPV = tpv;
   h->NT = nt;
   RC(init_impl(h.get(), vols, n_vols, counts, st));
-  if (o.fused && o.use_graph) RC(build_graphs(h.get()));
+  // the local kernel needs no graph: one launch holds up to kMaxIters iterations
+  if (o.fused && o.use_graph && !h->local) RC(build_graphs(h.get()));
   *out = h.release();
   return PRISM_OK;
 }
@@ -1192,14 +1234,14 @@ void autotune_shape(const prism_volume* vols, int n_vols, const std::vector<int6
         continue;
       }
       int rc = PRISM_OK;
-      for (int i = 0; i < 2 && rc == PRISM_OK; ++i) rc = enqueue_fused_iter(hc, st);
+      rc = enqueue_fused_iters(hc, 2, st);
       // the fastest of three rounds of four iterations (one round of a small batch is a
       // fraction of a millisecond, where a single round's noise can reorder candidates 10 %
       // apart)
       float ms = 1e30f;
       for (int round = 0; round < 3 && rc == PRISM_OK; ++round) {
         cudaEventRecord(e0, st);
-        for (int i = 0; i < 4 && rc == PRISM_OK; ++i) rc = enqueue_fused_iter(hc, st);
+        if (rc == PRISM_OK) rc = enqueue_fused_iters(hc, 4, st);
         cudaEventRecord(e1, st);
         cudaEventSynchronize(e1);
         float r = 0.f;
@@ -1267,7 +1309,8 @@ extern "C" int prism_step(prism_handle* h, int32_t n_iters, void* stream) {
     }
     for (; n > 0; --n) CK(cudaGraphLaunch(h->g1, st));
   } else {
-    for (int i = 0; i < n_iters; ++i) RC(h->opt.fused ? enqueue_fused_iter(h, st) : enqueue_plain_iter(h, st));
+    if (h->opt.fused) RC(enqueue_fused_iters(h, n_iters, st));
+    for (int i = 0; i < n_iters && !h->opt.fused; ++i) RC(enqueue_plain_iter(h, st));
   }
   h->iters += n_iters;
   return PRISM_OK;

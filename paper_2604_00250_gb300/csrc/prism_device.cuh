@@ -118,7 +118,7 @@ struct IterArgs {
   const float* gparams;    // packed group parameters
   float* gU;               // [Vpad] dJ/dU(x)
   float* tile_ab;          // per-tile [2][N] alpha / beta gradient partials
-  double* tile_red;        // per-tile [4]: data loss, dJ/dsigma_log, prior loss, spare
+  double* tile_red;        // per-tile [4]: data loss, dJ/dsigma_log, prior loss, spare (k_iter_local: its own layout)
   int32_t* queue;          // persistent work-queue counter
   int32_t* done;           // CTAs finished (last one resets the queue)
   const int32_t* step;     // iterations completed
@@ -138,6 +138,8 @@ struct IterArgs {
   // programmatic dependents (each starts while its predecessor finishes and waits on the device,
   // griddepcontrol, before it reads what the predecessor writes).
   int32_t pdl;
+  int32_t n_it;            // iterations of this launch (k_iter_local; else 1)
+  int32_t* gbar;           // [G] arrivals of the current launch (k_iter_local, Rician NLL)
   float* gparams_rw;       // same array as gparams
   float* gm;               // group Adam moments (packed like gparams)
   float* gv;

@@ -2,6 +2,7 @@
 // through a KernelSet. Included by prism_k<K>.cu.
 #include "prism_kernels.cuh"
 #include "prism_launch.h"
+#include "prism_local.cuh"
 
 #ifndef PRISM_K
 #error "PRISM_K must be defined"
@@ -104,6 +105,44 @@ cudaError_t l_fused_occupancy(int loss, int cal, int tpv, int shell, int nt, siz
   }
 }
 
+template <typename F>
+cudaError_t local_fn(int loss, int tpv, F go) {
+  if (tpv == 4) return loss == kLossMSE ? go(k_iter_local<kK, 4, kLossMSE>) : go(k_iter_local<kK, 4, kLossNLL>);
+  if (tpv == 16) return loss == kLossMSE ? go(k_iter_local<kK, 16, kLossMSE>) : go(k_iter_local<kK, 16, kLossNLL>);
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t l_local(const IterArgs& a, int loss, int tpv, int grid, size_t smem, cudaStream_t st) {
+  return local_fn(loss, tpv, [&](auto fn) {
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    if (loss == kLossMSE) {
+      fn<<<grid, kFusedThreads, smem, st>>>(a);
+      return cudaGetLastError();
+    }
+    // the NLL's CTAs wait on one another: all of them resident, or the launch is refused
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kFusedThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, a);
+  });
+}
+
+cudaError_t l_local_occupancy(int loss, int tpv, size_t smem, int* blocks) {
+  return local_fn(loss, tpv, [&](auto fn) {
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, kFusedThreads, smem);
+  });
+}
+
 inline int nblocks(int64_t n, int b) { return static_cast<int>((n + b - 1) / b); }
 
 cudaError_t l_transform(const IterArgs& a, int tb, int te, cudaStream_t st) {
@@ -193,7 +232,7 @@ cudaError_t l_stitch(const IterArgs& a, const int32_t* sov, int64_t n_out, const
 #define PRISM_CAT2(a, b) a##b
 #define PRISM_CAT(a, b) PRISM_CAT2(a, b)
 const KernelSet& PRISM_CAT(kernels_k, PRISM_K)() {
-  static const KernelSet ks = {l_fused, l_fused_occupancy, l_transform, l_synth, l_adjoint, l_prior_prep, l_prior_grad, l_prior, l_fibers, l_stitch};
+  static const KernelSet ks = {l_fused, l_fused_occupancy, l_local, l_local_occupancy, l_transform, l_synth, l_adjoint, l_prior_prep, l_prior_grad, l_prior, l_fibers, l_stitch};
   return ks;
 }
 

@@ -13,6 +13,9 @@ struct KernelSet {
   cudaError_t (*fused)(const IterArgs& a, int loss, int cal, int tpv, int shell, int grid, int nt, size_t smem,
                        cudaStream_t st);
   cudaError_t (*fused_occupancy)(int loss, int cal, int tpv, int shell, int nt, size_t smem, int* blocks);
+  // iterations of a fit without neighbour priors and calibration, several lanes per voxel
+  cudaError_t (*local)(const IterArgs& a, int loss, int tpv, int grid, size_t smem, cudaStream_t st);
+  cudaError_t (*local_occupancy)(int loss, int tpv, size_t smem, int* blocks);
   cudaError_t (*transform)(const IterArgs& a, int tb, int te, cudaStream_t st);
   cudaError_t (*synth)(const IterArgs& a, const PlainArgs& p, int cal, int tpv, int nt, cudaStream_t st);
   cudaError_t (*adjoint)(const IterArgs& a, const PlainArgs& p, int cal, int tpv, int nt, size_t smem,

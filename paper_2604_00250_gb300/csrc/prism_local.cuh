@@ -1,0 +1,280 @@
+// Fits without neighbour priors and calibration, several lanes per voxel: many iterations per launch.
+//
+// Nothing couples two voxels of such a fit but the noise level of the Rician NLL, which the voxels
+// of a volume share. One launch therefore keeps a tile's signal, table, parameters and moments in
+// shared memory and runs up to kMaxIters iterations on it. An iteration of the general fused kernel
+// at these sizes is a chain of latencies (launch, queue, tile and group records, staging, three
+// transforms, block-wide FP64 sums, the last CTA's tail): 13.8 us for an 8^3 patch, of which the
+// arithmetic is under 1 us. Here a voxel's lanes sit in one warp and all of them carry out the
+// voxel's chain rule and update on the summed accumulators, so that an iteration has no block
+// barrier and no hand-over at all; the redundant arithmetic uses issue slots that a small fit leaves
+// idle. Measured per iteration (GB300), general kernel -> this one: XXTABXX.
+//
+// Rician NLL: dJ/dsigma is a sum over the volume in each iteration. The warps of a volume's tiles
+// write their FP64 partials, count themselves in on a per-volume counter and wait for the count of
+// the iteration; then every warp takes the same fixed-order sum and updates its own copy of sigma.
+// The launch is cooperative (every CTA resident, one tile each) and every wait has a limit. 16
+// volumes of 10^3 voxels: 75 -> 17 us an iteration (N = 96).
+#pragma once
+
+#include "prism_kernels.cuh"
+
+namespace prism {
+
+constexpr int kMaxIters = 32;      // iterations per launch (Adam's constants of each in shared memory)
+constexpr int kLocalRow = 7;       // float4 per measurement pair in shared memory: the six that the
+                                   // uncalibrated step reads and one of padding, so that eight lanes
+                                   // reading eight neighbouring rows hit different banks
+constexpr int kLocalRed = 2 * (kFusedThreads / 32);   // partials per tile and iteration: {J, dJ/dsigma} per warp
+
+__host__ __device__ inline size_t local_smem(int K, int tpv, int NP) {
+  const size_t tv = kFusedThreads / tpv;
+  return static_cast<size_t>(NP / 2) * kLocalRow * sizeof(float4) + static_cast<size_t>(NP) * tv * sizeof(float) +
+         3 * static_cast<size_t>(4 * K + 5) * tv * sizeof(float);
+}
+
+__device__ __forceinline__ int ld_acquire(const int32_t* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// Sum over a group's partials of one iteration (field 0: J, 1: dJ/dsigma_log), fixed order: strided
+// over the warp's lanes, then a butterfly; every lane ends with it.
+__device__ __forceinline__ double local_group_sum(const IterArgs& a, const GroupDev& gr, int it, int field) {
+  const double* red = a.tile_red + (static_cast<size_t>(it) * a.ntiles + gr.tile0) * kLocalRed + field;
+  double s = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x & 31; i < gr.ntiles * (kLocalRed / 2); i += 32) s += __ldcg(red + 2 * i);
+  return warp_sum_d(s);
+}
+
+template <int K, int TPV, int LOSS>
+__global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(const IterArgs a) {
+  constexpr int NF = K + 3, Q = 4 * K + 5, VW = 32 / TPV, TV = kFusedThreads / TPV, NW = kFusedThreads / 32;
+  static_assert(TPV > 1, "one warp holds a voxel's lanes and several voxels");
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int NPmax = a.Nmax;
+  float4* s_tab = reinterpret_cast<float4*>(smem);                      // [NPmax / 2][kLocalRow]
+  float* s_y = reinterpret_cast<float*>(s_tab + NPmax / 2 * kLocalRow);  // [NP][TV], packed as in HBM
+  float* s_st = s_y + static_cast<size_t>(NPmax) * TV;                   // [3][Q][TV]: theta, m, v
+  __shared__ uint64_t s_bar;
+  __shared__ float s_ac[2 * kMaxIters];
+  __shared__ int s_last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lv = lane % VW, js = lane / VW, vl = warp * VW + lv;
+  const int Vp = a.Vpad, step = *a.step, n_it = a.n_it;
+  if (tid == 0) {
+    mbar_init(&s_bar, 1);
+    fence_mbar_init();
+  }
+  if (tid < 2 * n_it)
+    s_ac[tid] = adam_constant(tid, a.lr, a.beta1, a.beta2, static_cast<int64_t>(step) + 1 + (tid >> 1));
+  uint32_t phase = 0;
+  int cur_group = -1;
+  bool failed = false;
+  for (int ti = blockIdx.x; ti < a.ntiles; ti += gridDim.x) {
+    const int t = a.tile_order[ti];
+    const Tile tl = a.tiles[t];
+    const GroupDev gr = a.groups[tl.group];
+    const int N = tl.n_meas, NP = (N + 3) & ~3;
+    __syncthreads();   // the previous tile's shared data are no longer read (and s_bar is set up)
+    if (tid == 0) {
+      const uint32_t bytes = static_cast<uint32_t>(NP) * TV * 4u;   // multiple of 16: NP % 4 == 0
+      fence_proxy_async_smem();
+      mbar_expect_tx(&s_bar, bytes);
+      tma_bulk_g2s(s_y, a.y + tl.y_off, bytes, &s_bar);
+    }
+    if (tl.group != cur_group) {
+      const float4* src = reinterpret_cast<const float4*>(a.table2 + gr.table2_off);
+      for (int e = tid; e < NP / 2 * 6; e += kFusedThreads) {
+        const int p = e / 6, c = e - 6 * p;
+        s_tab[p * kLocalRow + c] = src[8 * p + c];
+      }
+      cur_group = tl.group;
+    }
+    for (int e = tid; e < Q * TV; e += kFusedThreads) {
+      const size_t ix = static_cast<size_t>(e / TV) * Vp + tl.slot0 + e % TV;
+      s_st[e] = a.theta[ix];
+      s_st[Q * TV + e] = a.m[ix];
+      s_st[2 * Q * TV + e] = a.v[ix];
+    }
+    if (!failed && !mbar_wait(&s_bar, phase)) {
+      atomicOr(a.status, kStTimeout);
+      failed = true;
+    }
+    phase ^= 1;
+    failed = __syncthreads_or(failed);
+    const bool act = vl < tl.count;
+    float* st = s_st + vl;
+    float th[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) th[q] = st[q * TV];
+    Vox<K> P;
+    transform<K>(th, P);
+    float slog = 0.f, sgm = 0.f, sgv = 0.f;   // the volume's noise level and its moments (NLL)
+    if (LOSS == kLossNLL) {
+      slog = a.gparams[gr.gp_off];
+      sgm = a.gm[gr.gp_off];
+      sgv = a.gv[gr.gp_off];
+    }
+    const float2* yc2 = reinterpret_cast<const float2*>(s_y + static_cast<size_t>(warp) * NP * VW) + lv;
+    for (int it = 0; it < n_it; ++it) {
+      const float inv_s2 = (LOSS == kLossNLL) ? expf(-2.f * slog) : 0.f;
+      const float scale = (LOSS == kLossMSE) ? 2.f * gr.inv_M : inv_s2;
+      Acc<K> A;
+      acc_zero<K>(A);
+      {
+        VoxP<K> DP;
+        AccP<K> AP;
+        voxp_init<K>(P, DP, AP);
+        // lane js of the voxel takes pairs js, js + TPV, ...; the leading pairs of b = 0 without the
+        // fiber terms (MSE)
+        const int i0 = (LOSS == kLossMSE) ? gr.nb0p : 0;
+        if (i0 > js) step2_b0<K>(DP, yc2 + js * VW, TPV * VW, (i0 - js + TPV - 1) / TPV, AP);
+        int p = i0 + ((js - i0) % TPV + TPV) % TPV;
+#pragma unroll (K >= 4 || LOSS == kLossNLL ? 1 : 2)
+        for (; p < N / 2; p += TPV)
+          step2<K, false, LOSS>(DP, reinterpret_cast<const MeasPair&>(s_tab[p * kLocalRow]), yc2[p * VW],
+                                make_float2(1.f, 1.f), AP, inv_s2);
+        if (p < (N + 1) / 2)   // the last measurement of an odd count
+          step2<K, true, LOSS>(DP, reinterpret_cast<const MeasPair&>(s_tab[p * kLocalRow]), yc2[p * VW],
+                               make_float2(1.f, 0.f), AP, inv_s2);
+        accp_sums<K, LOSS, false>(AP, A);
+      }
+      acc_reduce_tpv<K, TPV, VW>(A);
+      A.gS0 = acc_gS0<K>(P, A);
+      float gS0, gf[NF], gd[K][3], gfin;
+      data_grad<K>(P, A, scale, gS0, gf, gd, gfin);
+      float dloss, dsig = 0.f;
+      if (LOSS == kLossMSE) {
+        dloss = A.l1 * gr.inv_M;
+      } else {
+        dloss = 2.f * slog * N + 0.5f * inv_s2 * A.l1 - A.l3;
+        dsig = 2.f * N - inv_s2 * (A.l1 + 2.f * A.l2);
+      }
+      const float ploss = priors<K, true>(a, P, 0, gr.inv_M, nullptr, gS0, gf, gd);
+      float g[Q];
+      chain_raw<K>(P, gS0, gf, gd, gfin, g);
+      const float stepsz = s_ac[2 * it], isbc2 = s_ac[2 * it + 1];
+      float m[Q], v[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        th[q] = st[q * TV];
+        m[q] = st[(Q + q) * TV];
+        v[q] = st[(2 * Q + q) * TV];
+      }
+      __syncwarp();   // every lane of the voxel has read its state
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        if (a.optimizer == 0) {
+          m[q] = fmaf(a.beta1, m[q], (1.f - a.beta1) * g[q]);
+          v[q] = fmaf(a.beta2, v[q], (1.f - a.beta2) * g[q] * g[q]);
+          th[q] -= stepsz * m[q] * frcp(fmaf(fsqrt(v[q]), isbc2, a.eps));
+        } else {
+          rprop_update(th[q], m[q], v[q], g[q], a.lr, a.eta_minus, a.eta_plus, a.step_min, a.step_max);
+        }
+        if (js == 0) {
+          st[q * TV] = th[q];
+          st[(Q + q) * TV] = m[q];
+          st[(2 * Q + q) * TV] = v[q];
+        }
+      }
+      __syncwarp();
+      transform<K>(th, P);
+      // the warp's partials of the objective and dJ/dsigma: lanes 0 .. VW - 1 hold its voxels
+      double J = act ? static_cast<double>(dloss) + static_cast<double>(ploss) : 0.0;
+      double dS = (LOSS == kLossNLL && act) ? static_cast<double>(dsig) : 0.0;
+#pragma unroll
+      for (int o = 1; o < VW; o <<= 1) {
+        J += __shfl_xor_sync(0xffffffffu, J, o);
+        if (LOSS == kLossNLL) dS += __shfl_xor_sync(0xffffffffu, dS, o);
+      }
+      double* red = a.tile_red + (static_cast<size_t>(it) * a.ntiles + t) * kLocalRed + 2 * warp;
+      if (lane == 0) {
+        red[0] = J;
+        if (LOSS == kLossNLL) red[1] = dS;
+      }
+      if (LOSS == kLossNLL) {
+        const bool leader = t == gr.tile0 && warp == 0;
+        int32_t* bar = a.gbar + tl.group;
+        if (lane == 0) {
+          __threadfence();
+          atomicAdd(bar, 1);
+        }
+        if (it + 1 < n_it || leader) {
+          const int want = gr.ntiles * NW * (it + 1);
+          if (!failed) {
+            bool ok = true;
+            if (lane == 0) {
+              int polls = 0;
+              while (ld_acquire(bar) < want && polls < (1 << 21)) ++polls;
+              ok = polls < (1 << 21);
+              if (!ok) atomicOr(a.status, kStTimeout);
+            }
+            failed = __any_sync(0xffffffffu, !ok);
+          }
+          const float gsig = static_cast<float>(local_group_sum(a, gr, it, 1));
+          if (a.optimizer == 0) {
+            sgm = fmaf(a.beta1, sgm, (1.f - a.beta1) * gsig);
+            sgv = fmaf(a.beta2, sgv, (1.f - a.beta2) * gsig * gsig);
+            slog -= stepsz * sgm / fmaf(sqrtf(sgv), isbc2, a.eps);
+          } else {
+            rprop_update(slog, sgm, sgv, gsig, a.lr, a.eta_minus, a.eta_plus, a.step_min, a.step_max);
+          }
+          if (leader) {
+            const double tot = local_group_sum(a, gr, it, 0);
+            if (lane == 0) {
+              if (!isfinite(tot)) atomicOr(a.status, kStNonfinite);
+              a.hist[static_cast<size_t>((step + it) % a.hist_len) * a.G + tl.group] = tot;
+              if (it == n_it - 1) {
+                a.gloss[tl.group] = tot;
+                a.gparams_rw[gr.gp_off] = slog;
+                a.gm[gr.gp_off] = sgm;
+                a.gv[gr.gp_off] = sgv;
+              }
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();
+    for (int e = tid; e < Q * TV; e += kFusedThreads) {
+      const int v = e % TV;
+      if (v >= tl.count) continue;
+      const size_t ix = static_cast<size_t>(e / TV) * Vp + tl.slot0 + v;
+      a.theta[ix] = s_st[e];
+      a.m[ix] = s_st[Q * TV + e];
+      a.v[ix] = s_st[2 * Q * TV + e];
+    }
+  }
+  // the last CTA: objective and history (MSE), step counter, the next constants, counters
+  if (tid == 0) {
+    __threadfence();
+    s_last = (atomicAdd(a.done, 1) == static_cast<int>(gridDim.x) - 1);
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (LOSS == kLossMSE) {
+    for (int i = warp; i < n_it * a.G; i += NW) {
+      const int it = i / a.G, gi = i - it * a.G;
+      const double J = local_group_sum(a, a.groups[gi], it, 0);
+      if (lane == 0) {
+        if (!isfinite(J)) atomicOr(a.status, kStNonfinite);
+        if (it == n_it - 1) a.gloss[gi] = J;
+        a.hist[static_cast<size_t>((step + it) % a.hist_len) * a.G + gi] = J;
+      }
+    }
+  } else {
+    for (int i = tid; i < a.G; i += kFusedThreads) a.gbar[i] = 0;
+  }
+  if (tid < 2)
+    const_cast<float*>(a.adamc)[tid] = adam_constant(tid, a.lr, a.beta1, a.beta2, static_cast<int64_t>(step) + n_it + 1);
+  if (tid == 0) {
+    *const_cast<int32_t*>(a.step) = step + n_it;
+    *a.done = 0;
+  }
+}
+
+}  // namespace prism

@@ -292,19 +292,6 @@ __global__ void k_default_init(const int32_t* __restrict__ slot_of_vox, const ui
   theta[static_cast<size_t>(4 * K + 4) * Vpad + slot] = 0.f;
 }
 
-__global__ void k_gather_yhat(const float* __restrict__ ypack, const IterArgs a,
-                              const int32_t* __restrict__ vox_of_slot, const int64_t* __restrict__ row_off,
-                              const int32_t* __restrict__ order, float* __restrict__ out) {
-  const Tile tl = a.tiles[blockIdx.x];
-  const int32_t* ord = order + a.groups[tl.group].table_off;
-  for (int e = threadIdx.x; e < tl.n_meas * a.TV; e += blockDim.x) {
-    const int n = e / a.TV, vl = e - n * a.TV;
-    if (vl >= tl.count) continue;
-    const int64_t v = vox_of_slot[tl.slot0 + vl];
-    out[row_off[v] + ord[n]] = ypack[ypos(tl, n, vl, a.VW)];
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Plain-path data term and voxel Adam.
 // ---------------------------------------------------------------------------
@@ -736,11 +723,6 @@ cudaError_t launch_default_init(const int32_t* sov, const uint32_t* vcoord, int 
                                 int Vpad, uint64_t seed, float* th, cudaStream_t st) {
   if (V == 0) return cudaSuccess;
   k_default_init<<<nblk(V, 128), 128, 0, st>>>(sov, vcoord, ny, nz, V, K, Vpad, seed, th);
-  return cudaGetLastError();
-}
-cudaError_t launch_gather_yhat(const float* ypack, const IterArgs& a, const int32_t* vos, const int64_t* roff,
-                               const int32_t* order, float* out, cudaStream_t st) {
-  k_gather_yhat<<<a.ntiles, 256, 0, st>>>(ypack, a, vos, roff, order, out);
   return cudaGetLastError();
 }
 cudaError_t launch_adam_constants(const IterArgs& a, cudaStream_t st) {

@@ -143,6 +143,8 @@ struct IterArgs {
   float* gparams_rw;       // same array as gparams
   float* gm;               // group Adam moments (packed like gparams)
   float* gv;
+  float* grad;             // [Q][Vpad] raw-parameter gradient (gradient form of the fused kernel)
+  double* gred;            // group gradients (packed like gparams)
   double* gloss;           // [G]
   double* hist;            // [hist_len][G]
 };

@@ -849,8 +849,10 @@ __device__ __forceinline__ void shell_begin(ShellState<K>& S, const Vox<K>& P, f
 #pragma unroll
     for (int c = 0; c < 3; ++c) S.dp[k][c] = dup2(P.d[k][c]);
   }
-  // log2 f_in and log2(1 - f_in), floored so that a saturated f_in gives no inf - inf
-  const float lfin = fmaxf(lg2f_(P.fin), -40.f), lomf = fmaxf(lg2f_(P.omf), -126.f);
+  // log2 f_in and log2(1 - f_in), floored so that a saturated f_in gives no inf - inf; the full-accuracy
+  // log2f, once per voxel: the special-function unit's error (2^-22 of the argument's scale) is the same
+  // for all of a voxel's measurements and showed in the objective (1.5e-7 instead of 2e-8 relative)
+  const float lfin = fmaxf(log2f(P.fin), -40.f), lomf = fmaxf(log2f(P.omf), -126.f);
   S.nlfin = dup2(-lfin);
   col[SR::s0 * C] = P.S0;
   col[SR::fcsf * C] = P.f[0];
@@ -952,7 +954,9 @@ __device__ __forceinline__ void load_moments(const IterArgs& a, int slot, bool w
 // and the next iteration's Adam constants. It runs alone after every other CTA, so its latency
 // adds to the iteration: with several groups a warp takes each (16 volumes of 10^3 voxels, one
 // after the other by the whole block: 75 us an iteration, 38 us by warps), with fewer groups
-// than warps the block takes them in turn; lane-strided sums, then a butterfly.
+// than warps the block takes them in turn; lane-strided sums, then a butterfly. With GRAD (the
+// kernel's gradient form) the objective and dJ/dsigma_log are stored and nothing is updated.
+template <bool GRAD>
 __device__ __forceinline__ void finalize_groups(const IterArgs& a) {
   constexpr int NW = kFusedThreads / 32;
   __shared__ double s_part[NW][3];
@@ -978,8 +982,12 @@ __device__ __forceinline__ void finalize_groups(const IterArgs& a) {
   auto finish = [&](int gi, const GroupDev& gr, double l, double sg, double pr) {
     const double J = l + pr;
     a.gloss[gi] = J;
-    a.hist[static_cast<size_t>(step % a.hist_len) * a.G + gi] = J;
     if (!isfinite(J)) bad = true;
+    if constexpr (GRAD) {
+      a.gred[gr.gp_off] = sg;
+      return;
+    }
+    a.hist[static_cast<size_t>(step % a.hist_len) * a.G + gi] = J;
     if (nll) {
       const int i = gr.gp_off;
       const float gsig = static_cast<float>(sg);
@@ -1028,6 +1036,7 @@ __device__ __forceinline__ void finalize_groups(const IterArgs& a) {
     }
   }
   if (bad) atomicOr(a.status, kStNonfinite);
+  if constexpr (GRAD) return;
   // the next iteration's constants, t = step + 2, by the last warp while the others finish
   float c = 0.f;
   if (warp == NW - 1 && lane < 2) c = adam_constant(lane, a.lr, a.beta1, a.beta2, static_cast<int64_t>(step) + 2);
@@ -1055,7 +1064,9 @@ constexpr int fused_min_blocks() {
 
 // SHELL: the shell loop (see ShellState) instead of the packed pairs; only for one thread per
 // voxel, the MSE, no calibration and K <= 3, with every group's shells of even length.
-template <int K, int TPV, int LOSS, bool CAL, bool SHELL = false>
+// GRAD: the gradient form behind prism_forward / prism_backward: the same pass over the signal, its
+// epilogue writes the raw-parameter gradient instead of updating, and no state advances.
+template <int K, int TPV, int LOSS, bool CAL, bool SHELL = false, bool GRAD = false>
 __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS, CAL>())) k_iter_fused(const IterArgs a) {
   constexpr int NF = K + 3, Q = 4 * K + 5, XF = 4 * K + 3;
   constexpr int NW = kFusedThreads / 32;
@@ -1185,6 +1196,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         for (int q = 0; q < Q; ++q) {
           const size_t o = static_cast<size_t>(q) * Vp + slot0;
           prefetch_l2(a.theta + o, rb);
+          if (GRAD) continue;
           prefetch_l2(a.m + o, rb);
           prefetch_l2(a.v + o, rb);
         }
@@ -1466,7 +1478,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
       // the epilogue's math; otherwise they are re-read before the update.
       float th[Q], mq[Q], vq[Q];
       load_theta<K>(a.theta, Vp, eslot, eact, th);
-      if constexpr (HOIST) load_moments<Q>(a, eslot, writer, mq, vq);
+      if constexpr (HOIST && !GRAD) load_moments<Q>(a, eslot, writer, mq, vq);
       transform<K>(th, P);
       if constexpr (TPV == 1) {
         if constexpr (SHELL) {
@@ -1504,13 +1516,18 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         ploss += tv_term(s_blr, cx, cy, cz, gr, fl, B, a.w_tv * gr.inv_M, a.tv_eps, gUv);
       }
       // ---- chain rule and the update
-      if constexpr (!HOIST) {
+      if constexpr (!HOIST && !GRAD) {
         load_theta<K>(a.theta, Vp, eslot, eact, th);
         load_moments<Q>(a, eslot, writer, mq, vq);
       }
       float gq[Q];
       chain_raw<K, SHELL>(P, gS0, gf, gd, gfin, gq);
-      if (a.optimizer == 0) {
+      if constexpr (GRAD) {
+        if (writer) {
+#pragma unroll
+          for (int q = 0; q < Q; ++q) a.grad[static_cast<size_t>(q) * Vp + eslot] = gq[q];
+        }
+      } else if (a.optimizer == 0) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
           mq[q] = fmaf(a.beta1, mq[q], (1.f - a.beta1) * gq[q]);
@@ -1522,7 +1539,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         for (int q = 0; q < Q; ++q)
           rprop_update(th[q], mq[q], vq[q], gq[q], a.lr, a.eta_minus, a.eta_plus, a.step_min, a.step_max);
       }
-      if (writer) {
+      if (writer && !GRAD) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
           const size_t ix = static_cast<size_t>(q) * Vp + eslot;
@@ -1531,7 +1548,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
           a.theta[ix] = th[q];
         }
       }
-      if (a.nb_priors && writer) {
+      if (!GRAD && a.nb_priors && writer) {
         Vox<K> Pn;
         transform<K>(th, Pn);
         store_xf<K>(xf_nxt, Vp, eslot, Pn);
@@ -1567,7 +1584,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
   __syncthreads();
   if (s_last) {
     __threadfence();
-    if (!CAL && a.fold_groups) finalize_groups(a);
+    if (!CAL && a.fold_groups) finalize_groups<GRAD>(a);
     if (tid == 0) {
       *a.queue = 0;
       *a.done = 0;
@@ -1758,6 +1775,64 @@ __global__ void __launch_bounds__(256) k_synth(const IterArgs a, const PlainArgs
     }
     const float S = P.S0 * T;
     pa.yhat[ypos(tl, n, vl, a.VW)] = CAL ? fmaf(R.A * B, S, R.beta) : S;
+  }
+}
+
+// y_hat of every (voxel, measurement) straight into the caller's rows (mask order, the caller's
+// measurement order): a tile per block, kYhatC measurements at a time computed by the voxels' lanes
+// into shared memory and written along the rows. Writing from the packed layout, a thread per voxel,
+// spread a warp's stores over 32 rows: 709 us of a 243,000-voxel volume at N = 288, plus 199 us for
+// the packed y_hat; this kernel 326 us, 280 MB written.
+constexpr int kYhatC = 32;
+template <int K, bool CAL>
+__global__ void __launch_bounds__(128) k_yhat(const IterArgs a, const int32_t* __restrict__ vox_of_slot,
+                                             const int64_t* __restrict__ row_off, const int32_t* __restrict__ order,
+                                             float* __restrict__ out) {
+  extern __shared__ float s_yh[];   // [TV][kYhatC + 1]
+  const Tile tl = a.tiles[blockIdx.x];
+  const GroupDev gr = a.groups[tl.group];
+  const MeasRow* tab = a.table + gr.table_off;
+  const int32_t* ord = order + gr.table_off;
+  const int TV = a.TV, lanes = static_cast<int>(blockDim.x) / TV;
+  const int vl = threadIdx.x % TV, js = threadIdx.x / TV, slot = tl.slot0 + vl;
+  const bool act = vl < tl.count;
+  float th[4 * K + 5];
+  load_theta<K>(a.theta, a.Vpad, slot, act, th);
+  Vox<K> P;
+  transform<K>(th, P);
+  float B = 1.f;
+  if (CAL) {
+    int x, y, z;
+    unpack_coord(act ? a.vcoord[slot] : 0u, x, y, z);
+    B = expf(tri_eval(a.gparams + gr.gp_off + 4 + 2 * gr.N4, tri_weights(x, y, z, gr.nx, gr.ny, gr.nz)));
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = static_cast<int>(blockDim.x) >> 5;
+  for (int n0 = 0; n0 < tl.n_meas; n0 += kYhatC) {
+    const int cnt = min(kYhatC, tl.n_meas - n0);
+#pragma unroll 2
+    for (int c = js; c < cnt; c += lanes) {
+      const MeasRow R = tab[n0 + c];
+      float T = P.f[0] * R.ecsf;
+      T = fmaf(P.f[1], R.egm, T);
+      T = fmaf(P.f[K + 2], R.eres, T);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const float cc = fmaf(P.d[k][0], R.gx, fmaf(P.d[k][1], R.gy, P.d[k][2] * R.gz));
+        const float c2 = cc * cc;
+        const float e1 = ex2f_(R.nkpar * c2);
+        const float p = ex2f_(fmaf(R.nkd, c2, R.nkperp));
+        T = fmaf(P.f[2 + k], fmaf(P.fin, e1, P.omf * p), T);
+      }
+      const float S = P.S0 * T;
+      s_yh[vl * (kYhatC + 1) + c] = CAL ? fmaf(R.A * B, S, R.beta) : S;
+    }
+    __syncthreads();
+    const int on = (lane < cnt) ? ord[n0 + lane] : 0;
+    for (int v = warp; v < tl.count; v += nw) {
+      const int64_t row = row_off[vox_of_slot[tl.slot0 + v]];
+      if (lane < cnt) out[row + on] = s_yh[v * (kYhatC + 1) + lane];
+    }
+    __syncthreads();
   }
 }
 

@@ -34,9 +34,9 @@ cudaError_t launch_dep(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cud
   return cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
-template <int TPV, int LOSS, bool CAL, bool SHELL = false>
+template <int TPV, int LOSS, bool CAL, bool SHELL = false, bool GRAD = false>
 cudaError_t fused_one(const IterArgs& a, int grid, int nt, size_t smem, cudaStream_t st) {
-  auto fn = k_iter_fused<kK, TPV, LOSS, CAL, SHELL>;
+  auto fn = k_iter_fused<kK, TPV, LOSS, CAL, SHELL, GRAD>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   // a programmatic dependent only after k_prior_grad (which lets it start once every one of
@@ -56,14 +56,14 @@ cudaError_t fused_occ(int nt, size_t smem, int* blocks) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, nt, smem);
 }
 
-template <int TPV>
+template <int TPV, bool GRAD>
 cudaError_t fused_tpv(const IterArgs& a, int loss, int cal, int grid, int nt, size_t smem, cudaStream_t st) {
   if (loss == kLossMSE) {
-    return cal ? fused_one<TPV, kLossMSE, true>(a, grid, nt, smem, st)
-               : fused_one<TPV, kLossMSE, false>(a, grid, nt, smem, st);
+    return cal ? fused_one<TPV, kLossMSE, true, false, GRAD>(a, grid, nt, smem, st)
+               : fused_one<TPV, kLossMSE, false, false, GRAD>(a, grid, nt, smem, st);
   }
-  return cal ? fused_one<TPV, kLossNLL, true>(a, grid, nt, smem, st)
-             : fused_one<TPV, kLossNLL, false>(a, grid, nt, smem, st);
+  return cal ? fused_one<TPV, kLossNLL, true, false, GRAD>(a, grid, nt, smem, st)
+             : fused_one<TPV, kLossNLL, false, false, GRAD>(a, grid, nt, smem, st);
 }
 
 template <int TPV>
@@ -74,20 +74,27 @@ cudaError_t occ_tpv(int loss, int cal, int nt, size_t smem, int* blocks) {
   return cal ? fused_occ<TPV, kLossNLL, true>(nt, smem, blocks) : fused_occ<TPV, kLossNLL, false>(nt, smem, blocks);
 }
 
-cudaError_t l_fused(const IterArgs& a, int loss, int cal, int tpv, int shell, int grid, int nt, size_t smem,
-                    cudaStream_t st) {
+template <bool GRAD>
+cudaError_t fused_any(const IterArgs& a, int loss, int cal, int tpv, int shell, int grid, int nt, size_t smem,
+                      cudaStream_t st) {
   if constexpr (kK <= 3) {
     if (shell) {
       if (tpv != 1 || loss != kLossMSE || cal) return cudaErrorInvalidValue;
-      return fused_one<1, kLossMSE, false, true>(a, grid, nt, smem, st);
+      return fused_one<1, kLossMSE, false, true, GRAD>(a, grid, nt, smem, st);
     }
   }
   switch (tpv) {
-    case 1: return fused_tpv<1>(a, loss, cal, grid, nt, smem, st);
-    case 4: return fused_tpv<4>(a, loss, cal, grid, nt, smem, st);
-    case 16: return fused_tpv<16>(a, loss, cal, grid, nt, smem, st);
+    case 1: return fused_tpv<1, GRAD>(a, loss, cal, grid, nt, smem, st);
+    case 4: return fused_tpv<4, GRAD>(a, loss, cal, grid, nt, smem, st);
+    case 16: return fused_tpv<16, GRAD>(a, loss, cal, grid, nt, smem, st);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t l_fused(const IterArgs& a, int loss, int cal, int tpv, int shell, int grad, int grid, int nt, size_t smem,
+                    cudaStream_t st) {
+  return grad ? fused_any<true>(a, loss, cal, tpv, shell, grid, nt, smem, st)
+              : fused_any<false>(a, loss, cal, tpv, shell, grid, nt, smem, st);
 }
 
 cudaError_t l_fused_occupancy(int loss, int cal, int tpv, int shell, int nt, size_t smem, int* blocks) {
@@ -170,6 +177,16 @@ cudaError_t l_synth(const IterArgs& a, const PlainArgs& p, int cal, int tpv, int
   }
 }
 
+cudaError_t l_yhat(const IterArgs& a, int cal, const int32_t* vos, const int64_t* roff, const int32_t* order,
+                   float* out, cudaStream_t st) {
+  if (a.ntiles <= 0) return cudaSuccess;
+  const int nt = max(128, a.TV);   // TV: 8, 32, 128 or, on a plain handle with 256-thread CTAs, up to 256
+  const size_t smem = static_cast<size_t>(a.TV) * (kYhatC + 1) * sizeof(float);   // at most 33 KB
+  if (cal) k_yhat<kK, true><<<a.ntiles, nt, smem, st>>>(a, vos, roff, order, out);
+  else k_yhat<kK, false><<<a.ntiles, nt, smem, st>>>(a, vos, roff, order, out);
+  return cudaGetLastError();
+}
+
 template <int TPV>
 cudaError_t adjoint_tpv(const IterArgs& a, const PlainArgs& p, int cal, int nt, size_t smem, cudaStream_t st) {
   const int g = p.tile_end - p.tile_begin;
@@ -232,7 +249,7 @@ cudaError_t l_stitch(const IterArgs& a, const int32_t* sov, int64_t n_out, const
 #define PRISM_CAT2(a, b) a##b
 #define PRISM_CAT(a, b) PRISM_CAT2(a, b)
 const KernelSet& PRISM_CAT(kernels_k, PRISM_K)() {
-  static const KernelSet ks = {l_fused, l_fused_occupancy, l_local, l_local_occupancy, l_transform, l_synth, l_adjoint, l_prior_prep, l_prior_grad, l_prior, l_fibers, l_stitch};
+  static const KernelSet ks = {l_fused, l_fused_occupancy, l_local, l_local_occupancy, l_transform, l_synth, l_yhat, l_adjoint, l_prior_prep, l_prior_grad, l_prior, l_fibers, l_stitch};
   return ks;
 }
 

@@ -9,15 +9,18 @@ namespace prism {
 
 // Per-K launchers of the templated kernels (one translation unit per K).
 struct KernelSet {
-  // shell = 1: the shell loop of one thread per voxel, MSE, no calibration (K <= 3)
-  cudaError_t (*fused)(const IterArgs& a, int loss, int cal, int tpv, int shell, int grid, int nt, size_t smem,
-                       cudaStream_t st);
+  // shell = 1: the shell loop of one thread per voxel, MSE, no calibration (K <= 3); grad = 1: the
+  // gradient form (no update)
+  cudaError_t (*fused)(const IterArgs& a, int loss, int cal, int tpv, int shell, int grad, int grid, int nt,
+                       size_t smem, cudaStream_t st);
   cudaError_t (*fused_occupancy)(int loss, int cal, int tpv, int shell, int nt, size_t smem, int* blocks);
   // iterations of a fit without neighbour priors and calibration, several lanes per voxel
   cudaError_t (*local)(const IterArgs& a, int loss, int tpv, int grid, size_t smem, cudaStream_t st);
   cudaError_t (*local_occupancy)(int loss, int tpv, size_t smem, int* blocks);
   cudaError_t (*transform)(const IterArgs& a, int tb, int te, cudaStream_t st);
   cudaError_t (*synth)(const IterArgs& a, const PlainArgs& p, int cal, int tpv, int nt, cudaStream_t st);
+  cudaError_t (*yhat)(const IterArgs& a, int cal, const int32_t* vox_of_slot, const int64_t* row_off,
+                      const int32_t* order, float* out, cudaStream_t st);
   cudaError_t (*adjoint)(const IterArgs& a, const PlainArgs& p, int cal, int tpv, int nt, size_t smem,
                          cudaStream_t st);
   cudaError_t (*prior_prep)(const IterArgs& a, int tb, int te, cudaStream_t st);
@@ -85,8 +88,6 @@ cudaError_t launch_gather_params(const float* theta, const int32_t* slot_of_vox,
                                  float* out, cudaStream_t st);
 cudaError_t launch_default_init(const int32_t* slot_of_vox, const uint32_t* vcoord, int ny, int nz, int64_t V, int K,
                                 int Vpad, uint64_t seed, float* theta, cudaStream_t st);
-cudaError_t launch_gather_yhat(const float* ypack, const IterArgs& a, const int32_t* vox_of_slot,
-                               const int64_t* yhat_row_off, const int32_t* order, float* out, cudaStream_t st);
 cudaError_t launch_table_refresh(const GroupArgs& g, const IterArgs& a, cudaStream_t st);
 cudaError_t launch_adam_constants(const IterArgs& a, cudaStream_t st);
 cudaError_t launch_wait_probe(int32_t* status, int polls, cudaStream_t st);

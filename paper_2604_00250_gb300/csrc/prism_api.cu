@@ -739,8 +739,10 @@ int upload(T* dst, const std::vector<T, A>& src, cudaStream_t st) {
     if (r_ != PRISM_OK) return r_; \
   } while (0)
 
+// `rows`: per volume, the row of each voxel in vols[g].signal and vols[g].init (device memory; the
+// slabs of one whole-volume signal), or nullptr where the rows are in mask order.
 int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::vector<int64_t>& counts,
-              cudaStream_t st) {
+              const int64_t* const* rows, cudaStream_t st) {
   const prism_options& o = h->opt;
   h->K = o.K;
   h->Q = 4 * o.K + 5;
@@ -916,6 +918,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
     const int N = v.n_meas;
     const int64_t Vg = gr.n_vox;
     const float* sig = v.signal;
+    const int64_t* vrows = rows ? rows[g] : nullptr;
     float* tmp_sig = early[g];
     if (tmp_sig) {
       sig = tmp_sig;
@@ -924,33 +927,31 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
       CK(cudaMemcpyAsync(tmp_sig, v.signal, sizeof(float) * Vg * N, cudaMemcpyHostToDevice, st));
       sig = tmp_sig;
     }
-    std::vector<uint8_t> isb0(N);
+    std::vector<int32_t> b0n;                // the b <= 50 measurements
     std::vector<float> bv(N), bvec(3 * N);   // in table order
     const int32_t* ord = h->order.data() + gr.table_off;
     for (int n = 0; n < N; ++n) {
       bv[n] = v.bvals[ord[n]];
       for (int c = 0; c < 3; ++c) bvec[3 * n + c] = v.bvecs[3 * ord[n] + c];
     }
-    int nb0 = 0;
-    for (int n = 0; n < N; ++n) {
-      isb0[n] = v.bvals[n] <= 50.f;
-      nb0 += isb0[n];
-    }
-    uint8_t* d_isb0 = nullptr;
+    for (int n = 0; n < N; ++n)
+      if (v.bvals[n] <= 50.f) b0n.push_back(n);
+    const int nb0 = static_cast<int>(b0n.size());
+    int32_t* d_b0n = nullptr;
     float *d_bv = nullptr, *d_bvec = nullptr, *d_b0 = nullptr;
     double* d_part = nullptr;
-    const int nbk = static_cast<int>((Vg + 255) / 256);
-    RC(h->alloc(&d_isb0, N));
+    const int nbk = b0_stat_blocks(Vg);
+    RC(h->alloc(&d_b0n, nb0));
     RC(h->alloc(&d_bv, N));
     RC(h->alloc(&d_bvec, 3 * N));
     RC(h->alloc(&d_b0, Vg));
     RC(h->alloc(&d_part, nbk));
-    RC(upload(d_isb0, isb0, st));
+    RC(upload(d_b0n, b0n, st));
     RC(upload(d_bv, bv, st));
     RC(upload(d_bvec, bvec, st));
-    CK(launch_b0_stats(sig, Vg, N, d_isb0, nb0, d_b0, d_part, d_bad, st));
+    CK(launch_b0_stats(sig, vrows, Vg, N, d_b0n, nb0, d_b0, d_part, d_bad, st));
     CK(launch_sigma_init(d_part, nbk, Vg, nb0, o.sigma_init, h->d_gparams + gr.gp_off, st));
-    CK(launch_pack(h->ia, sig, d_b0, h->d_vox_of_slot, h->d_order + gr.table_off, h->vox0[g], gr.tile0,
+    CK(launch_pack(h->ia, sig, vrows, d_b0, h->d_vox_of_slot, h->d_order + gr.table_off, h->vox0[g], gr.tile0,
                    gr.tile0 + gr.ntiles, N, h->d_y, d_bad, st));
     CK(launch_table(d_bv, d_bvec, N, h->d_table + gr.table_off, st));
     CK(launch_pair_table(h->d_table + gr.table_off, N, h->d_table2 + gr.table2_off, st));
@@ -962,14 +963,14 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
         CK(cudaMemcpyAsync(tmp_in, v.init, sizeof(float) * Vg * Q, cudaMemcpyHostToDevice, st));
         in = tmp_in;
       }
-      CK(launch_scatter_params(in, h->d_slot_of_vox + h->vox0[g], Vg, Q, Vp, h->d_theta, st));
+      CK(launch_scatter_params(in, vrows, h->d_slot_of_vox + h->vox0[g], Vg, Q, Vp, h->d_theta, st));
     } else {
       CK(launch_default_init(h->d_slot_of_vox + h->vox0[g], h->d_vcoord, v.ny, v.nz, Vg, h->K, Vp,
                              static_cast<uint64_t>(o.seed) * 1315423911ull + g, h->d_theta, st));
     }
     // free per-volume temporaries (after the work that reads them)
     CK(cudaStreamSynchronize(st));
-    for (void* p : {static_cast<void*>(tmp_sig), static_cast<void*>(d_isb0), static_cast<void*>(d_bv),
+    for (void* p : {static_cast<void*>(tmp_sig), static_cast<void*>(d_b0n), static_cast<void*>(d_bv),
                     static_cast<void*>(d_bvec), static_cast<void*>(d_b0), static_cast<void*>(d_part)}) {
       if (!p) continue;
       auto it = std::find(h->allocs.begin(), h->allocs.end(), p);
@@ -1105,13 +1106,13 @@ struct DevTmp {
 };
 
 int create_handle(const prism_volume* vols, int n_vols, const std::vector<int64_t>& counts, const prism_options& o,
-                  int tpv, int nt, cudaStream_t st, prism_handle** out) {
+                  int tpv, int nt, const int64_t* const* rows, cudaStream_t st, prism_handle** out) {
   std::unique_ptr<prism_handle> h(new (std::nothrow) prism_handle());
   if (!h) return fail(PRISM_E_OOM, "host allocation failed");
   h->opt = o;
   h->TPV = tpv;
   h->NT = nt;
-  RC(init_impl(h.get(), vols, n_vols, counts, st));
+  RC(init_impl(h.get(), vols, n_vols, counts, rows, st));
   // the local kernel needs no graph: one launch holds up to kMaxIters iterations
   if (o.fused && o.use_graph && !h->local) RC(build_graphs(h.get()));
   *out = h.release();
@@ -1232,7 +1233,7 @@ void autotune_shape(const prism_volume* vols, int n_vols, const std::vector<int6
       if (o.shells == -1 && sh == 0) continue;
       oc.shells = sh;
       prism_handle* hc = nullptr;
-      if (create_handle(tv, n_vols, *tc, oc, lane, 128, st, &hc) != PRISM_OK) {
+      if (create_handle(tv, n_vols, *tc, oc, lane, 128, nullptr, st, &hc) != PRISM_OK) {
         g_err.clear();
         continue;
       }
@@ -1268,10 +1269,9 @@ void autotune_shape(const prism_volume* vols, int n_vols, const std::vector<int6
   g_err.clear();
 }
 
-}  // namespace
-
-extern "C" int prism_fit_init(const prism_volume* vols, int32_t n_vols, const prism_options* opt, void* stream,
-                              prism_handle** out) {
+// prism_fit_init, with the optional row maps of init_impl (then without autotuning).
+int fit_init(const prism_volume* vols, int n_vols, const prism_options* opt, const int64_t* const* rows, void* stream,
+             prism_handle** out) {
   g_err.clear();
   if (!out) return fail(PRISM_E_INVALID_ARG, "out is NULL");
   *out = nullptr;
@@ -1287,16 +1287,23 @@ extern "C" int prism_fit_init(const prism_volume* vols, int32_t n_vols, const pr
   for (int64_t c : counts) V += c;
   int tpv = 1, nt = 128;
   choose_shape(o, V, shells_apply(vols, n_vols, o), &tpv, &nt);
-  if (o.autotune && o.fused) {
+  if (o.autotune && o.fused && !rows) {
     int shells = o.shells;
     autotune_shape(vols, n_vols, counts, o, st, &tpv, &shells);
     o.shells = shells;
   }
   prism_handle* h = nullptr;
-  const int rc = create_handle(vols, n_vols, counts, o, tpv, nt, st, &h);
+  const int rc = create_handle(vols, n_vols, counts, o, tpv, nt, rows, st, &h);
   if (rc != PRISM_OK) return rc;
   *out = h;
   return PRISM_OK;
+}
+
+}  // namespace
+
+extern "C" int prism_fit_init(const prism_volume* vols, int32_t n_vols, const prism_options* opt, void* stream,
+                              prism_handle** out) {
+  return fit_init(vols, n_vols, opt, nullptr, stream, out);
 }
 
 extern "C" int prism_step(prism_handle* h, int32_t n_iters, void* stream) {
@@ -1391,7 +1398,7 @@ extern "C" int prism_set_params(prism_handle* h, const float* in, int32_t mem, v
   } else if (mem != PRISM_MEM_DEVICE) {
     return fail(PRISM_E_INVALID_ARG, "mem must be HOST or DEVICE");
   }
-  cudaError_t e = launch_scatter_params(src, h->d_slot_of_vox, h->V, h->Q, h->Vpad, h->d_theta, st);
+  cudaError_t e = launch_scatter_params(src, nullptr, h->d_slot_of_vox, h->V, h->Q, h->Vpad, h->d_theta, st);
   if (e == cudaSuccess) e = h->ks->transform(h->ia, 0, h->ntiles, st);
   if (tmp) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -1483,7 +1490,7 @@ extern "C" int prism_forward(prism_handle* h, const float* theta, const float* g
                              void* stream) {
   if (!h) return fail(PRISM_E_INVALID_ARG, "handle is NULL");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (theta) CK(launch_scatter_params(theta, h->d_slot_of_vox, h->V, h->Q, h->Vpad, h->d_theta, st));
+  if (theta) CK(launch_scatter_params(theta, nullptr, h->d_slot_of_vox, h->V, h->Q, h->Vpad, h->d_theta, st));
   if (groups) {
     CK(cudaMemcpyAsync(h->d_gparams, groups, h->GP * sizeof(float), cudaMemcpyDeviceToDevice, st));
     CK(launch_table_refresh(h->ga, h->ia, st));
@@ -1650,7 +1657,7 @@ extern "C" int prism_set_state(prism_handle* h, const void* host_buf, int64_t by
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
     e = cudaMemcpyAsync(tmp, p, nvq * sizeof(float), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_scatter_params(tmp, h->d_slot_of_vox, h->V, h->Q, h->Vpad, dsts[i], st);
+    if (e == cudaSuccess) e = launch_scatter_params(tmp, nullptr, h->d_slot_of_vox, h->V, h->Q, h->Vpad, dsts[i], st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     p += nvq * sizeof(float);
   }
@@ -1793,7 +1800,8 @@ extern "C" int prism_fit_init_slabs(const prism_volume* vol, int32_t slab, int32
       if (src1[i] >= 0) src1[i] += vox0[gidx[slab1[i]]];
     }
   });
-  // whole-volume signal (and initial parameters) on the device, then one gathered copy per slab
+  // whole-volume signal (and initial parameters) on the device; every slab reads its rows of it (the
+  // autotuner takes volumes with rows of their own: then one gathered copy per slab)
   DevTmp dsig, dinit, drows;
   const float* sig = vol->signal;
   const float* init = vol->init;
@@ -1808,31 +1816,36 @@ extern "C" int prism_fit_init_slabs(const prism_volume* vol, int32_t slab, int32
     }
   }
   CK(cudaMalloc(&drows.p, sizeof(int64_t) * acc));
+  const bool copies = o.autotune && o.fused;
   std::vector<DevTmp> ssig(G), sinit(G);
   std::vector<prism_volume> vols(G);
+  std::vector<const int64_t*> vrows(G);
   for (int s = 0; s < S; ++s) {
     const int g = gidx[s];
     if (g < 0) continue;
     const int64_t n = static_cast<int64_t>(rows[s].size());
     int64_t* dr = drows.as<int64_t>() + vox0[g];
     CK(cudaMemcpyAsync(dr, rows[s].data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-    CK(cudaMalloc(&ssig[g].p, sizeof(float) * n * N));
-    CK(launch_gather_rows(sig, dr, n, N, ssig[g].as<float>(), st));
-    if (init) {
-      CK(cudaMalloc(&sinit[g].p, sizeof(float) * n * Q));
-      CK(launch_gather_rows(init, dr, n, Q, sinit[g].as<float>(), st));
-    }
+    vrows[g] = dr;
     prism_volume& pv = vols[g];
     pv = *vol;
     pv.nz = z1s[s] - z0s[s];
     pv.mem = PRISM_MEM_DEVICE;
     pv.mask = sub[s].data();
+    pv.signal = sig;
+    pv.init = init;
+    if (!copies) continue;
+    CK(cudaMalloc(&ssig[g].p, sizeof(float) * n * N));
+    CK(launch_gather_rows(sig, dr, n, N, ssig[g].as<float>(), st));
     pv.signal = ssig[g].as<float>();
-    pv.init = init ? sinit[g].as<float>() : nullptr;
+    if (init) {
+      CK(cudaMalloc(&sinit[g].p, sizeof(float) * n * Q));
+      CK(launch_gather_rows(init, dr, n, Q, sinit[g].as<float>(), st));
+      pv.init = sinit[g].as<float>();
+    }
   }
-  CK(cudaStreamSynchronize(st));
   prism_handle* h = nullptr;
-  RC(prism_fit_init(vols.data(), G, &o, stream, &h));
+  RC(fit_init(vols.data(), G, &o, copies ? nullptr : vrows.data(), stream, &h));
   CK(cudaStreamSynchronize(st));
   h->slabbed = true;
   h->st_src0 = std::move(src0);

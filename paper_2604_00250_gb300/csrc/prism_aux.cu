@@ -11,115 +11,146 @@ namespace prism {
 // ---------------------------------------------------------------------------
 // Preprocessing (Sec. 2.5: both y and y_hat are divided by the measured b0).
 // ---------------------------------------------------------------------------
-// One warp per voxel (the lanes read the row's consecutive measurements together), 256 voxels
-// per block of 256 threads; part[block] is the block's sum of the squared b0 deviations. The
-// per-voxel sums are FP32 (a b0 mean of a few dozen positive values, stored as FP32); the
-// squared deviations accumulate in FP64 per thread and per block.
-__global__ void __launch_bounds__(256) k_b0_stats(const float* __restrict__ sig, int64_t V, int N,
-                                                  const uint8_t* __restrict__ isb0, int nb0,
+// b0 mean of every voxel and the block's sum of the squared b0 deviations, part[block]: kB0Lanes lanes
+// per voxel read the b <= 50 measurements (`b0n`, nb0 of them) and nothing else of the row; k_pack, which
+// reads all of it, looks for the other non-finite values. The per-voxel sums are FP32 (a b0 mean of a few dozen
+// positive values, stored as FP32); the squared deviations accumulate in FP64. A voxel whose mean is not
+// positive, or takes in a non-finite value, is counted in *bad and stored as -1. `rows`: the voxels' rows in `sig`, or null for
+// rows in order. (A warp per voxel over the whole row: 164 us of 141,000 voxels at N = 288, 30 us now.)
+constexpr int kB0Lanes = 8, kB0Vox = 256 / kB0Lanes;
+__global__ void __launch_bounds__(256) k_b0_stats(const float* __restrict__ sig, const int64_t* __restrict__ rows,
+                                                  int64_t V, int N, const int32_t* __restrict__ b0n, int nb0,
                                                   float* __restrict__ b0mean, double* __restrict__ part, int* bad) {
-  __shared__ double s[256];
-  __shared__ uint8_t s_b0[1024];   // N <= 1024 (prism_fit_init checks it)
-  for (int n = threadIdx.x; n < N; n += blockDim.x) s_b0[n] = isb0[n];
+  __shared__ double s[8];
+  __shared__ int32_t s_n[1024];   // nb0 <= N <= 1024 (prism_fit_init checks it)
+  for (int n = threadIdx.x; n < nb0; n += blockDim.x) s_n[n] = b0n[n];
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double acc = 0.0;
-  for (int j = 0; j < 32; ++j) {
-    const int64_t v = static_cast<int64_t>(blockIdx.x) * 256 + warp * 32 + j;
-    if (v >= V) break;
-    const float* row = sig + v * N;
-    float m = 0.f;
-    bool finite = true;
-    for (int n = lane; n < N; n += 32) {
-      const float x = row[n];
-      if (!isfinite(x)) finite = false;
-      if (s_b0[n]) m += x;
-    }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % kB0Lanes;
+  const int64_t v = static_cast<int64_t>(blockIdx.x) * kB0Vox + threadIdx.x / kB0Lanes;
+  const bool ok = v < V;
+  const float* row = sig + (ok ? (rows ? rows[v] : v) : 0) * N;
+  float m = 0.f;
+  bool finite = true;
+#pragma unroll 4
+  for (int i = sub; i < nb0; i += kB0Lanes) {
+    const float x = ok ? row[s_n[i]] : 0.f;
+    finite = finite && isfinite(x);
+    m += x;
+  }
+  const unsigned lanes = ((1u << kB0Lanes) - 1u) << (lane - sub);   // the voxel's
+  finite = (__ballot_sync(0xffffffffu, finite) & lanes) == lanes;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
-    finite = __all_sync(0xffffffffu, finite);
-    m /= static_cast<float>(nb0);
-    if (!finite || !(m > 0.f)) {
-      if (lane == 0) atomicAdd(bad, 1);
-      m = 1.f;
-    }
-    if (lane == 0) b0mean[v] = m;
-    const float inv = 1.f / m;
-    for (int n = lane; n < N; n += 32)
-      if (s_b0[n]) {
-        const float d = fmaf(row[n], inv, -1.f);
-        acc += static_cast<double>(d * d);
-      }
+  for (int o = kB0Lanes / 2; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+  m /= static_cast<float>(nb0);
+  const bool good = finite && m > 0.f;
+  if (ok && sub == 0) {
+    b0mean[v] = good ? m : -1.f;
+    if (!good) atomicAdd(bad, 1);
   }
-  s[threadIdx.x] = acc;
+  double acc = 0.0;
+  const float inv = good ? 1.f / m : 1.f;
+#pragma unroll 4
+  for (int i = sub; i < nb0; i += kB0Lanes) {
+    const float d = ok ? fmaf(row[s_n[i]], inv, -1.f) : 0.f;
+    acc += static_cast<double>(d * d);
+  }
+  acc = warp_sum_d(acc);
+  if (lane == 0) s[warp] = acc;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) acc += s[w];
+    part[blockIdx.x] = acc;
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = s[0];
 }
 
 // sigma init (Sec. 2.3 learns sigma but does not say where it starts): pooled std of the
-// normalised b0 repeats, clamped >= 1e-3.
-__global__ void k_sigma_init(const double* part, int nblocks, int64_t V, int nb0, float fallback,
-                             float* sigma_log) {
-  if (threadIdx.x != 0) return;
+// normalised b0 repeats, clamped >= 1e-3. One block, strided over the partials, then a fixed tree
+// (one thread reading them in turn took 24 us for 550).
+__global__ void __launch_bounds__(256) k_sigma_init(const double* part, int nblocks, int64_t V, int nb0, float fallback,
+                                                    float* sigma_log) {
+  __shared__ double s_w[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double s = 0.0;
-  for (int b = 0; b < nblocks; ++b) s += part[b];
+#pragma unroll 4
+  for (int b = threadIdx.x; b < nblocks; b += 256) s += part[b];
+  s = warp_sum_d(s);
+  if (lane == 0) s_w[warp] = s;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < 8; ++w) s += s_w[w];
   double sg = fallback;
   if (nb0 >= 2) sg = fmax(sqrt(s / (static_cast<double>(V) * (nb0 - 1))), 1e-3);
   *sigma_log = static_cast<float>(log(sg));
 }
 
-// One tile per block of kPackThreads: each warp column of the tile (VW voxels) in chunks of
-// kPackC measurements, staged in shared memory so that the reads run along the voxels' signal
-// rows and the writes along the packed [pair][voxel][2] layout (ypos).
+// One warp column of a tile (VW voxels) per block of kPackThreads, in chunks of kPackC measurements
+// staged in shared memory so that the reads run along the voxels' signal rows and the writes along the
+// packed [pair][voxel][2] layout (ypos). A voxel with a non-finite measurement is counted in *bad
+// (unless its b0 mean already was). Bound by the loads in flight: a block per tile, its four columns in
+// turn, took 118 us for 141,000 voxels at N = 288, now 65 us.
 constexpr int kPackThreads = 256, kPackC = 128;
 template <int VW>
 __global__ void __launch_bounds__(kPackThreads) k_pack(const IterArgs a, const float* __restrict__ sig,
+                                                       const int64_t* __restrict__ rows,
                                                        const float* __restrict__ b0mean,
                                                        const int32_t* __restrict__ vox_of_slot,
                                                        const int32_t* __restrict__ order, int64_t vox0, int tile_begin,
-                                                       int N, float* __restrict__ ypack) {
+                                                       int N, float* __restrict__ ypack, int* bad) {
   __shared__ float s[VW][kPackC + 1];
   __shared__ int64_t s_row[VW];   // the voxel's signal row (-1: padding slot)
-  __shared__ float s_inv[VW];     // 1 / its b0 mean
-  const int t = tile_begin + blockIdx.x;
+  __shared__ float s_inv[VW];     // 1 / its b0 mean (-1 where that was refused)
+  __shared__ int s_bad[VW];
+  const int t = tile_begin + blockIdx.x, w = blockIdx.y;
   const Tile tl = a.tiles[t];
   const int NP = (N + 3) & ~3;
-  for (int w = 0; w * VW < a.TV; ++w) {
-    if (threadIdx.x < VW) {
-      const int vl = w * VW + threadIdx.x;
-      int64_t r = -1;
-      float inv = 0.f;
-      if (vl < tl.count) {
-        const int64_t v = vox_of_slot[tl.slot0 + vl] - vox0;
-        r = v * N;
-        inv = 1.f / b0mean[v];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < VW) {
+    const int vl = w * VW + threadIdx.x;
+    int64_t r = -1;
+    float inv = 0.f;
+    if (vl < tl.count) {
+      const int64_t v = vox_of_slot[tl.slot0 + vl] - vox0;
+      r = (rows ? rows[v] : v) * N;
+      const float m = b0mean[v];
+      inv = m > 0.f ? 1.f / m : -1.f;
+    }
+    s_row[threadIdx.x] = r;
+    s_inv[threadIdx.x] = inv;
+    s_bad[threadIdx.x] = 0;
+  }
+  __syncthreads();
+  for (int n0 = 0; n0 < NP; n0 += kPackC) {
+    const int C = min(kPackC, NP - n0);   // even (NP and kPackC are multiples of 4)
+    int32_t on[kPackC / 32];   // the measurements this lane reads of every row (-1: padding)
+#pragma unroll
+    for (int q = 0; q < kPackC / 32; ++q) {
+      const int n = n0 + lane + 32 * q;
+      on[q] = (n < N) ? order[n] : -1;
+    }
+    // a warp per voxel row, its loads and those of the next rows in flight together
+#pragma unroll
+    for (int j = warp; j < VW; j += kPackThreads / 32) {
+      const int64_t r = s_row[j];
+      const float inv = s_inv[j];
+      bool nonfinite = false;
+#pragma unroll
+      for (int q = 0; q < kPackC / 32; ++q) {
+        const float x = (r >= 0 && on[q] >= 0) ? sig[r + on[q]] : 0.f;
+        nonfinite = nonfinite || !isfinite(x);
+        if (lane + 32 * q < C) s[j][lane + 32 * q] = x * inv;
       }
-      s_row[threadIdx.x] = r;
-      s_inv[threadIdx.x] = inv;
+      if (nonfinite) s_bad[j] = 1;
     }
     __syncthreads();
-    for (int n0 = 0; n0 < NP; n0 += kPackC) {
-      const int C = min(kPackC, NP - n0);   // even (NP and kPackC are multiples of 4)
+    float* out = ypack + tl.y_off + static_cast<size_t>(w) * NP * VW + static_cast<size_t>(n0) * VW;
 #pragma unroll 8
-      for (int i = threadIdx.x; i < VW * C; i += kPackThreads) {
-        const int j = i / C, nc = i - j * C, n = n0 + nc;
-        const int64_t r = s_row[j];
-        s[j][nc] = (r >= 0 && n < N) ? sig[r + order[n]] * s_inv[j] : 0.f;
-      }
-      __syncthreads();
-      float* out = ypack + tl.y_off + static_cast<size_t>(w) * NP * VW + static_cast<size_t>(n0) * VW;
-#pragma unroll 8
-      for (int i = threadIdx.x; i < VW * C; i += kPackThreads) {
-        const int pc = i / (2 * VW), r = i - pc * 2 * VW, j = r >> 1;
-        out[i] = s[j][2 * pc + (r & 1)];
-      }
-      __syncthreads();
+    for (int i = threadIdx.x; i < VW * C; i += kPackThreads) {
+      const int pc = i / (2 * VW), r = i - pc * 2 * VW, j = r >> 1;
+      out[i] = s[j][2 * pc + (r & 1)];
     }
+    __syncthreads();
   }
+  if (threadIdx.x < VW && s_bad[threadIdx.x] && s_inv[threadIdx.x] >= 0.f) atomicAdd(bad, 1);
 }
 
 // Static part of the per-measurement table; exp(alpha) = 1, beta = 0 (identity, Sec. 2.3).
@@ -221,32 +252,60 @@ __global__ void k_vox_of_slot(const int32_t* __restrict__ slot_of_vox, int64_t V
   if (v < V) vox_of_slot[slot_of_vox[v]] = static_cast<int32_t>(v);
 }
 
-// Row gather: dst[i][:] = src[rows[i]][:] (slab volumes cut from a whole volume).
-__global__ void k_gather_rows(const float* __restrict__ src, const int64_t* __restrict__ rows, int64_t n, int len,
-                              float* __restrict__ dst) {
-  const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= n * len) return;
-  const int64_t i = e / len;
-  const int c = static_cast<int>(e - i * len);
-  dst[e] = src[rows[i] * len + c];
+// Row gather: dst[i][:] = src[rows[i]][:], a warp per row.
+__global__ void __launch_bounds__(256) k_gather_rows(const float* __restrict__ src, const int64_t* __restrict__ rows,
+                                                     int64_t n, int len, float* __restrict__ dst) {
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  if (i >= n) return;
+  const float* s = src + rows[i] * len;
+  float* d = dst + i * len;
+#pragma unroll 4
+  for (int c = threadIdx.x & 31; c < len; c += 32) d[c] = s[c];
 }
 
-__global__ void k_scatter_params(const float* __restrict__ in, const int32_t* __restrict__ slot_of_vox,
-                                 int64_t V, int Q, int Vpad, float* __restrict__ theta) {
-  const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= V * Q) return;
-  const int64_t v = e / Q;
-  const int q = static_cast<int>(e - v * Q);
-  theta[static_cast<size_t>(q) * Vpad + slot_of_vox[v]] = in[e];
+// Raw parameters between the caller's rows [V][Q] (mask order; `rows`: row of each voxel, or null for
+// rows in order) and the kernels' [Q][Vpad] by slot, kParVox voxels per block through shared memory:
+// the rows are read and written along their length, the slots along runs of consecutive voxels. Q =
+// 4K + 5 is odd, so a column of the staged rows falls into 32 different banks. (Element by element, the
+// strided side took a sector per value: 62 us to read out 740,110 voxels at K = 3, now 17 us.)
+constexpr int kParVox = 128;
+__global__ void __launch_bounds__(kParVox) k_scatter_params(const float* __restrict__ in,
+                                                            const int64_t* __restrict__ rows,
+                                                            const int32_t* __restrict__ slot_of_vox, int64_t V, int Q,
+                                                            int Vpad, float* __restrict__ theta) {
+  extern __shared__ float s_par[];   // [kParVox][Q]
+  const int64_t v0 = static_cast<int64_t>(blockIdx.x) * kParVox;
+  const int nv = static_cast<int>(min(static_cast<int64_t>(kParVox), V - v0));
+  if (rows) {
+    for (int e = threadIdx.x; e < nv * Q; e += kParVox) {
+      const int v = e / Q;
+      s_par[e] = in[rows[v0 + v] * Q + (e - v * Q)];
+    }
+  } else {
+#pragma unroll 8
+    for (int e = threadIdx.x; e < nv * Q; e += kParVox) s_par[e] = in[v0 * Q + e];
+  }
+  __syncthreads();
+  if (threadIdx.x >= nv) return;
+  const int slot = slot_of_vox[v0 + threadIdx.x];
+#pragma unroll 8
+  for (int q = 0; q < Q; ++q) theta[static_cast<size_t>(q) * Vpad + slot] = s_par[threadIdx.x * Q + q];
 }
 
-__global__ void k_gather_params(const float* __restrict__ theta, const int32_t* __restrict__ slot_of_vox,
-                                int64_t V, int Q, int Vpad, float* __restrict__ out) {
-  const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= V * Q) return;
-  const int64_t v = e / Q;
-  const int q = static_cast<int>(e - v * Q);
-  out[e] = theta[static_cast<size_t>(q) * Vpad + slot_of_vox[v]];
+__global__ void __launch_bounds__(kParVox) k_gather_params(const float* __restrict__ theta,
+                                                           const int32_t* __restrict__ slot_of_vox, int64_t V, int Q,
+                                                           int Vpad, float* __restrict__ out) {
+  extern __shared__ float s_par[];   // [kParVox][Q]
+  const int64_t v0 = static_cast<int64_t>(blockIdx.x) * kParVox;
+  const int nv = static_cast<int>(min(static_cast<int64_t>(kParVox), V - v0));
+  if (threadIdx.x < nv) {
+    const int slot = slot_of_vox[v0 + threadIdx.x];
+#pragma unroll 8
+    for (int q = 0; q < Q; ++q) s_par[threadIdx.x * Q + q] = theta[static_cast<size_t>(q) * Vpad + slot];
+  }
+  __syncthreads();
+#pragma unroll 8
+  for (int e = threadIdx.x; e < nv * Q; e += kParVox) out[v0 * Q + e] = s_par[e];
 }
 
 // Counter-based generator: splitmix64 (Steele, Lea, Flood 2014) of (seed, voxel, draw).
@@ -652,27 +711,27 @@ cudaError_t launch_adam_voxel(const IterArgs& a, const PlainArgs& p, cudaStream_
   k_adam_voxel<<<nblk(n, 256), 256, 0, st>>>(a, p);
   return cudaGetLastError();
 }
-cudaError_t launch_b0_stats(const float* sig, int64_t V, int N, const uint8_t* isb0, int nb0, float* b0mean,
-                            double* part, int* bad, cudaStream_t st) {
-  k_b0_stats<<<nblk(V, 256), 256, 0, st>>>(sig, V, N, isb0, nb0, b0mean, part, bad);
+int b0_stat_blocks(int64_t V) { return nblk(V, kB0Vox); }
+cudaError_t launch_b0_stats(const float* sig, const int64_t* rows, int64_t V, int N, const int32_t* b0n, int nb0,
+                            float* b0mean, double* part, int* bad, cudaStream_t st) {
+  k_b0_stats<<<b0_stat_blocks(V), 256, 0, st>>>(sig, rows, V, N, b0n, nb0, b0mean, part, bad);
   return cudaGetLastError();
 }
 cudaError_t launch_sigma_init(const double* part, int nblocks, int64_t V, int nb0, float fb, float* out,
                               cudaStream_t st) {
-  k_sigma_init<<<1, 32, 0, st>>>(part, nblocks, V, nb0, fb, out);
+  k_sigma_init<<<1, 256, 0, st>>>(part, nblocks, V, nb0, fb, out);
   return cudaGetLastError();
 }
-cudaError_t launch_pack(const IterArgs& a, const float* sig, const float* b0mean, const int32_t* vox_of_slot,
-                        const int32_t* order, int64_t vox0, int tile_begin, int tile_end, int N, float* ypack,
-                        int* bad, cudaStream_t st) {
-  (void)bad;
+cudaError_t launch_pack(const IterArgs& a, const float* sig, const int64_t* rows, const float* b0mean,
+                        const int32_t* vox_of_slot, const int32_t* order, int64_t vox0, int tile_begin, int tile_end,
+                        int N, float* ypack, int* bad, cudaStream_t st) {
   if (tile_end <= tile_begin) return cudaSuccess;
   if (a.TV % a.VW != 0) return cudaErrorInvalidValue;
-  const int nb = tile_end - tile_begin;
+  const dim3 nb(tile_end - tile_begin, a.TV / a.VW);
   switch (a.VW) {
-    case 32: k_pack<32><<<nb, kPackThreads, 0, st>>>(a, sig, b0mean, vox_of_slot, order, vox0, tile_begin, N, ypack); break;
-    case 8: k_pack<8><<<nb, kPackThreads, 0, st>>>(a, sig, b0mean, vox_of_slot, order, vox0, tile_begin, N, ypack); break;
-    case 2: k_pack<2><<<nb, kPackThreads, 0, st>>>(a, sig, b0mean, vox_of_slot, order, vox0, tile_begin, N, ypack); break;
+    case 32: k_pack<32><<<nb, kPackThreads, 0, st>>>(a, sig, rows, b0mean, vox_of_slot, order, vox0, tile_begin, N, ypack, bad); break;
+    case 8: k_pack<8><<<nb, kPackThreads, 0, st>>>(a, sig, rows, b0mean, vox_of_slot, order, vox0, tile_begin, N, ypack, bad); break;
+    case 2: k_pack<2><<<nb, kPackThreads, 0, st>>>(a, sig, rows, b0mean, vox_of_slot, order, vox0, tile_begin, N, ypack, bad); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -695,7 +754,7 @@ cudaError_t launch_slot_data(const Tile* tiles, const GroupDev* groups, int G, c
 cudaError_t launch_gather_rows(const float* src, const int64_t* rows, int64_t n, int len, float* dst,
                                cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_gather_rows<<<nblk(n * len, 256), 256, 0, st>>>(src, rows, n, len, dst);
+  k_gather_rows<<<nblk(n, 8), 256, 0, st>>>(src, rows, n, len, dst);
   return cudaGetLastError();
 }
 cudaError_t launch_table(const float* bvals, const float* bvecs, int N, MeasRow* rows, cudaStream_t st) {
@@ -707,16 +766,16 @@ cudaError_t launch_pair_table(const MeasRow* rows, int N, MeasPair* out, cudaStr
   k_pair_table<<<nblk(NP / 2, 128), 128, 0, st>>>(rows, N, NP, out);
   return cudaGetLastError();
 }
-cudaError_t launch_scatter_params(const float* in, const int32_t* sov, int64_t V, int Q, int Vpad, float* th,
-                                  cudaStream_t st) {
+cudaError_t launch_scatter_params(const float* in, const int64_t* rows, const int32_t* sov, int64_t V, int Q, int Vpad,
+                                  float* th, cudaStream_t st) {
   if (V == 0) return cudaSuccess;
-  k_scatter_params<<<nblk(V * Q, 256), 256, 0, st>>>(in, sov, V, Q, Vpad, th);
+  k_scatter_params<<<nblk(V, kParVox), kParVox, sizeof(float) * kParVox * Q, st>>>(in, rows, sov, V, Q, Vpad, th);
   return cudaGetLastError();
 }
 cudaError_t launch_gather_params(const float* th, const int32_t* sov, int64_t V, int Q, int Vpad, float* out,
                                  cudaStream_t st) {
   if (V == 0) return cudaSuccess;
-  k_gather_params<<<nblk(V * Q, 256), 256, 0, st>>>(th, sov, V, Q, Vpad, out);
+  k_gather_params<<<nblk(V, kParVox), kParVox, sizeof(float) * kParVox * Q, st>>>(th, sov, V, Q, Vpad, out);
   return cudaGetLastError();
 }
 cudaError_t launch_default_init(const int32_t* sov, const uint32_t* vcoord, int ny, int nz, int64_t V, int K,

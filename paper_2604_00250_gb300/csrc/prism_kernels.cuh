@@ -1780,22 +1780,27 @@ __global__ void __launch_bounds__(256) k_synth(const IterArgs a, const PlainArgs
 
 // y_hat of every (voxel, measurement) straight into the caller's rows (mask order, the caller's
 // measurement order): a tile per block, kYhatC measurements at a time computed by the voxels' lanes
-// into shared memory and written along the rows. Writing from the packed layout, a thread per voxel,
-// spread a warp's stores over 32 rows: 709 us of a 243,000-voxel volume at N = 288, plus 199 us for
-// the packed y_hat; this kernel 326 us, 280 MB written.
+// (two measurements per step, the paired table staged in shared memory) and written along the rows
+// through shared memory. Bound by the output's bytes and the exponentials. Writing from the packed layout, a
+// thread per voxel, spread a warp's stores over 32 rows: 709 us of a 243,000-voxel volume at N = 288,
+// plus 199 us for the packed y_hat; this kernel 168 us, 333 MB written.
 constexpr int kYhatC = 32;
 template <int K, bool CAL>
-__global__ void __launch_bounds__(128) k_yhat(const IterArgs a, const int32_t* __restrict__ vox_of_slot,
+__global__ void __launch_bounds__(256) k_yhat(const IterArgs a, const int32_t* __restrict__ vox_of_slot,
                                              const int64_t* __restrict__ row_off, const int32_t* __restrict__ order,
                                              float* __restrict__ out) {
-  extern __shared__ float s_yh[];   // [TV][kYhatC + 1]
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ float4 s_tab[kYhatC / 2][8];
+  int64_t* s_row = reinterpret_cast<int64_t*>(smem);                 // [TV]
+  float* s_yh = reinterpret_cast<float*>(s_row + a.TV);              // [TV][kYhatC + 1]
   const Tile tl = a.tiles[blockIdx.x];
   const GroupDev gr = a.groups[tl.group];
-  const MeasRow* tab = a.table + gr.table_off;
+  const float4* tab = reinterpret_cast<const float4*>(a.table2 + gr.table2_off);
   const int32_t* ord = order + gr.table_off;
   const int TV = a.TV, lanes = static_cast<int>(blockDim.x) / TV;
   const int vl = threadIdx.x % TV, js = threadIdx.x / TV, slot = tl.slot0 + vl;
   const bool act = vl < tl.count;
+  if (js == 0 && act) s_row[vl] = row_off[vox_of_slot[slot]];
   float th[4 * K + 5];
   load_theta<K>(a.theta, a.Vpad, slot, act, th);
   Vox<K> P;
@@ -1806,33 +1811,38 @@ __global__ void __launch_bounds__(128) k_yhat(const IterArgs a, const int32_t* _
     unpack_coord(act ? a.vcoord[slot] : 0u, x, y, z);
     B = expf(tri_eval(a.gparams + gr.gp_off + 4 + 2 * gr.N4, tri_weights(x, y, z, gr.nx, gr.ny, gr.nz)));
   }
+  const float2 S0 = dup2(P.S0), fin = dup2(P.fin), omf = dup2(P.omf), B2 = dup2(B);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = static_cast<int>(blockDim.x) >> 5;
   for (int n0 = 0; n0 < tl.n_meas; n0 += kYhatC) {
     const int cnt = min(kYhatC, tl.n_meas - n0);
+    const int np = (cnt + 1) / 2;   // the table is zero past N, within its rows rounded up to 4
+    for (int e = threadIdx.x; e < 8 * np; e += blockDim.x) s_tab[e >> 3][e & 7] = tab[4 * n0 + e];
+    __syncthreads();
 #pragma unroll 2
-    for (int c = js; c < cnt; c += lanes) {
-      const MeasRow R = tab[n0 + c];
-      float T = P.f[0] * R.ecsf;
-      T = fmaf(P.f[1], R.egm, T);
-      T = fmaf(P.f[K + 2], R.eres, T);
+    for (int p = js; p < np; p += lanes) {
+      const float4 q0 = s_tab[p][0], q1 = s_tab[p][1], q2 = s_tab[p][2], q3 = s_tab[p][3], q4 = s_tab[p][4];
+      float2 T = __fmul2_rn(dup2(P.f[0]), lo2(q3));
+      T = __ffma2_rn(dup2(P.f[1]), hi2(q3), T);
+      T = __ffma2_rn(dup2(P.f[K + 2]), lo2(q4), T);
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        const float cc = fmaf(P.d[k][0], R.gx, fmaf(P.d[k][1], R.gy, P.d[k][2] * R.gz));
-        const float c2 = cc * cc;
-        const float e1 = ex2f_(R.nkpar * c2);
-        const float p = ex2f_(fmaf(R.nkd, c2, R.nkperp));
-        T = fmaf(P.f[2 + k], fmaf(P.fin, e1, P.omf * p), T);
+        const float2 c = __ffma2_rn(dup2(P.d[k][0]), lo2(q0),
+                                    __ffma2_rn(dup2(P.d[k][1]), hi2(q0), __fmul2_rn(dup2(P.d[k][2]), lo2(q1))));
+        const float2 c2 = __fmul2_rn(c, c);
+        const float2 e1 = ex2_2(__fmul2_rn(hi2(q1), c2));
+        const float2 pp = ex2_2(__ffma2_rn(hi2(q2), c2, lo2(q2)));
+        T = __ffma2_rn(dup2(P.f[2 + k]), __ffma2_rn(fin, e1, __fmul2_rn(omf, pp)), T);
       }
-      const float S = P.S0 * T;
-      s_yh[vl * (kYhatC + 1) + c] = CAL ? fmaf(R.A * B, S, R.beta) : S;
+      float2 y = __fmul2_rn(S0, T);
+      if (CAL) y = __ffma2_rn(__fmul2_rn(hi2(s_tab[p][5]), B2), y, lo2(s_tab[p][6]));
+      s_yh[vl * (kYhatC + 1) + 2 * p] = y.x;
+      s_yh[vl * (kYhatC + 1) + 2 * p + 1] = y.y;
     }
     __syncthreads();
     const int on = (lane < cnt) ? ord[n0 + lane] : 0;
-    for (int v = warp; v < tl.count; v += nw) {
-      const int64_t row = row_off[vox_of_slot[tl.slot0 + v]];
-      if (lane < cnt) out[row + on] = s_yh[v * (kYhatC + 1) + lane];
-    }
-    __syncthreads();
+#pragma unroll 4
+    for (int v = warp; v < tl.count; v += nw)
+      if (lane < cnt) out[s_row[v] + on] = s_yh[v * (kYhatC + 1) + lane];
   }
 }
 

@@ -181,7 +181,7 @@ cudaError_t l_yhat(const IterArgs& a, int cal, const int32_t* vos, const int64_t
                    float* out, cudaStream_t st) {
   if (a.ntiles <= 0) return cudaSuccess;
   const int nt = max(128, a.TV);   // TV: 8, 32, 128 or, on a plain handle with 256-thread CTAs, up to 256
-  const size_t smem = static_cast<size_t>(a.TV) * (kYhatC + 1) * sizeof(float);   // at most 33 KB
+  const size_t smem = static_cast<size_t>(a.TV) * ((kYhatC + 1) * sizeof(float) + sizeof(int64_t));   // at most 36 KB
   if (cal) k_yhat<kK, true><<<a.ntiles, nt, smem, st>>>(a, vos, roff, order, out);
   else k_yhat<kK, false><<<a.ntiles, nt, smem, st>>>(a, vos, roff, order, out);
   return cudaGetLastError();

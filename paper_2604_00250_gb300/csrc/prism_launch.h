@@ -68,13 +68,14 @@ cudaError_t launch_loss(const IterArgs& a, const PlainArgs& p, int loss, cudaStr
 cudaError_t launch_adam_voxel(const IterArgs& a, const PlainArgs& p, cudaStream_t st);
 
 // Preprocessing and layout kernels.
-cudaError_t launch_b0_stats(const float* sig, int64_t V, int N, const uint8_t* isb0, int nb0,
+int b0_stat_blocks(int64_t V);   // partials that launch_b0_stats writes
+cudaError_t launch_b0_stats(const float* sig, const int64_t* rows, int64_t V, int N, const int32_t* b0n, int nb0,
                             float* b0mean, double* part, int* bad, cudaStream_t st);
 cudaError_t launch_sigma_init(const double* part, int nblocks, int64_t V, int nb0, float sigma_fallback,
                               float* sigma_log_out, cudaStream_t st);
-cudaError_t launch_pack(const IterArgs& a, const float* sig, const float* b0mean, const int32_t* vox_of_slot,
-                        const int32_t* order, int64_t vox0, int tile_begin, int tile_end, int N, float* ypack,
-                        int* bad, cudaStream_t st);
+cudaError_t launch_pack(const IterArgs& a, const float* sig, const int64_t* rows, const float* b0mean,
+                        const int32_t* vox_of_slot, const int32_t* order, int64_t vox0, int tile_begin, int tile_end,
+                        int N, float* ypack, int* bad, cudaStream_t st);
 cudaError_t launch_slot_data(const Tile* tiles, const GroupDev* groups, int G, const GroupDev* host_groups,
                              const int32_t* slot_of_grid, const int32_t* slot_of_vox, int64_t V, int Vp, int TV, int nnb,
                              int32_t* vox_of_slot, uint32_t* vcoord, uint32_t* vflag, int32_t* nbr, cudaStream_t st);
@@ -82,8 +83,8 @@ cudaError_t launch_gather_rows(const float* src, const int64_t* rows, int64_t n,
                                cudaStream_t st);
 cudaError_t launch_table(const float* bvals, const float* bvecs, int N, MeasRow* rows, cudaStream_t st);
 cudaError_t launch_pair_table(const MeasRow* rows, int N, MeasPair* out, cudaStream_t st);
-cudaError_t launch_scatter_params(const float* in, const int32_t* slot_of_vox, int64_t V, int Q, int Vpad,
-                                  float* theta, cudaStream_t st);
+cudaError_t launch_scatter_params(const float* in, const int64_t* rows, const int32_t* slot_of_vox, int64_t V, int Q,
+                                  int Vpad, float* theta, cudaStream_t st);
 cudaError_t launch_gather_params(const float* theta, const int32_t* slot_of_vox, int64_t V, int Q, int Vpad,
                                  float* out, cudaStream_t st);
 cudaError_t launch_default_init(const int32_t* slot_of_vox, const uint32_t* vcoord, int ny, int nz, int64_t V, int K,

@@ -63,7 +63,7 @@ int cuda_fail(cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(e_, #call); \
   } while (0)
 
-constexpr int kSplitTiles = 64;
+constexpr int kSplitTiles = 32;   // tiles per first-level sum (k_group_sums)
 constexpr int kHistLen = 4096;
 constexpr int kGraphUnroll = 16;
 constexpr uint32_t kStateMagic = 0x50524953u;   // "PRIS"
@@ -121,7 +121,7 @@ struct prism_handle {
   ShellRun* d_runs = nullptr;
   double *d_tile_red = nullptr, *d_part2 = nullptr, *d_gred = nullptr, *d_gloss = nullptr;
   double* d_bscratch = nullptr;      // bias-gradient partial contractions (calibration only)
-  int64_t* d_bs_off = nullptr;       // [G][2] offsets into d_bscratch
+  int64_t* d_bs_off = nullptr;       // [G] offsets into d_bscratch
   int max_nx = 0, max_ny = 0;
   int32_t* d_gdone = nullptr;
   double *d_gprior = nullptr, *d_hist = nullptr;
@@ -369,8 +369,7 @@ int enqueue_fused_iter(prism_handle* h, cudaStream_t st) {
   CK(h->ks->fused(a, h->opt.loss, h->cal ? 1 : 0, h->TPV, h->shell ? 1 : 0, 0, h->fused_grid, h->NT, h->fused_smem,
                   st));
   if (h->cal) {   // without calibration the fused kernel's last CTA finalises the groups
-    CK(launch_bias_grad(a, h->ga, st));
-    CK(launch_group_reduce(a, h->ga, 1 | 2, st));
+    CK(launch_group_sums(a, h->ga, 1 | 2, true, st));
     CK(launch_group_adam(a, h->ga, 1 | 2, st));
   }
   return PRISM_OK;
@@ -408,8 +407,7 @@ int enqueue_plain_iter(prism_handle* h, cudaStream_t st) {
     CK(h->ks->prior(a, p, st));
     CK(launch_adam_voxel(a, p, st));
   }
-  if (h->cal) CK(launch_bias_grad(a, h->ga, st));
-  CK(launch_group_reduce(a, h->ga, 1 | (h->cal ? 2 : 0), st));
+  CK(launch_group_sums(a, h->ga, 1 | (h->cal ? 2 : 0), h->cal, st));
   CK(launch_group_adam(a, h->ga, 1 | 2, st));
   return PRISM_OK;
 }
@@ -789,7 +787,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
     tot_split += ns;
     h->max_split = std::max(h->max_split, ns);
   }
-  const int nce = (h->max_e + 255) / 256;
+  const int nce = (h->max_e + kRedE - 1) / kRedE;
   // The local kernel (prism_local.cuh): several lanes per voxel, no neighbour priors, no calibration;
   // with the Rician NLL, whose CTAs exchange sums, only where all tiles are resident at once.
   if (o.fused && !h->cal && !h->nb && h->TPV > 1) {
@@ -850,20 +848,18 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   CK(cudaMemsetAsync(h->d_gbar, 0, sizeof(int32_t) * G, st));
   CK(cudaMemsetAsync(h->d_gdone, 0, sizeof(int32_t), st));
   if (h->cal) {
-    // per group [nx][ny][8] then [nx][8][8] doubles for the separable bias-field adjoint
-    std::vector<int64_t> bs(2 * static_cast<size_t>(G));
+    // per group [nx][ny][8] doubles for the separable bias-field adjoint
+    std::vector<int64_t> bs(G);
     int64_t tot = 0;
     for (int g = 0; g < G; ++g) {
       const GroupDev& gr = h->groups[g];
-      bs[2 * g] = tot;
+      bs[g] = tot;
       tot += static_cast<int64_t>(gr.nx) * gr.ny * kGrid;
-      bs[2 * g + 1] = tot;
-      tot += static_cast<int64_t>(gr.nx) * kGrid * kGrid;
       h->max_nx = std::max(h->max_nx, gr.nx);
       h->max_ny = std::max(h->max_ny, gr.ny);
     }
     RC(h->alloc(&h->d_bscratch, tot));
-    RC(h->alloc(&h->d_bs_off, 2 * static_cast<size_t>(G)));
+    RC(h->alloc(&h->d_bs_off, G));
     RC(upload(h->d_bs_off, bs, st));
   }
   if (!o.fused) {
@@ -1507,8 +1503,7 @@ extern "C" int prism_forward(prism_handle* h, const float* theta, const float* g
     if (h->nb) CK(h->ks->prior_grad(a, 0, h->ntiles, st));
     CK(h->ks->fused(a, h->opt.loss, cal, h->TPV, h->shell ? 1 : 0, 1, h->fused_grid, h->NT, h->fused_smem, st));
     if (h->cal) {
-      CK(launch_bias_grad(a, h->ga, st));
-      CK(launch_group_reduce(a, h->ga, 1 | 2, st));
+      CK(launch_group_sums(a, h->ga, 1 | 2, true, st));
       CK(launch_group_adam(a, h->ga, 1, st));
     }
   } else {
@@ -1519,7 +1514,7 @@ extern "C" int prism_forward(prism_handle* h, const float* theta, const float* g
     CK(launch_loss(a, p, h->opt.loss, st));
     if (h->opt.lam_sp > 0.f) CK(h->ks->prior_prep(a, 0, h->ntiles, st));
     CK(h->ks->prior(a, p, st));
-    CK(launch_group_reduce(a, h->ga, 1, st));
+    CK(launch_group_sums(a, h->ga, 1, false, st));
     CK(launch_group_adam(a, h->ga, 1, st));
   }
   if (loss) CK(cudaMemcpyAsync(loss, h->d_gloss, sizeof(double) * h->G, cudaMemcpyDeviceToDevice, st));
@@ -1537,8 +1532,7 @@ extern "C" int prism_backward(prism_handle* h, float* grad_theta, float* grad_gr
     PlainArgs p{h->d_yhat, h->d_r, h->d_grad, 0, h->ntiles, 2};
     CK(h->ks->adjoint(a, p, h->cal ? 1 : 0, h->TPV, h->NT, h->adj_smem, st));
     CK(h->ks->prior(a, p, st));
-    if (h->cal) CK(launch_bias_grad(a, h->ga, st));
-    CK(launch_group_reduce(a, h->ga, 2, st));
+    CK(launch_group_sums(a, h->ga, 2, h->cal, st));
   }
   GroupArgs ga = h->ga;
   ga.gexport = grad_groups;
@@ -1565,8 +1559,7 @@ extern "C" int prism_profile(prism_handle* h, int32_t n_iters, void* stream, flo
       e = h->ks->fused(a, h->opt.loss, h->cal ? 1 : 0, h->TPV, h->shell ? 1 : 0, 0, h->fused_grid, h->NT,
                        h->fused_smem, st);
     if (e == cudaSuccess) e = cudaEventRecord(ev[2], st);
-    if (e == cudaSuccess && h->cal) e = launch_bias_grad(a, h->ga, st);
-    if (e == cudaSuccess && h->cal) e = launch_group_reduce(a, h->ga, 1 | 2, st);
+    if (e == cudaSuccess && h->cal) e = launch_group_sums(a, h->ga, 1 | 2, true, st);
     if (e == cudaSuccess && h->cal) e = launch_group_adam(a, h->ga, 1 | 2, st);
     if (e == cudaSuccess) e = cudaEventRecord(ev[3], st);
     if (e == cudaSuccess) e = cudaEventSynchronize(ev[3]);

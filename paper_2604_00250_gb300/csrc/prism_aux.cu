@@ -383,30 +383,50 @@ __global__ void k_adam_voxel(const IterArgs a, const PlainArgs pa) {
 // Group reductions: per-tile partials -> per-group sums, fixed order (two levels:
 // splits of `split_tiles` tiles, then the last-arriving block sums the splits).
 // Entries: 0 data loss, 1 dJ/dsigma_log, 2 prior loss, 3.. 3+2N alpha / beta.
+// A block takes kRedE entries of a split, a quarter of its tiles per 64 threads. Bound by latency and by
+// GB300's FP64 rate (an add per warp costs its SM about 16 cycles): the tiles' FP32 partials are
+// summed in two-float arithmetic (Knuth's exact two-sum, error below 2^-44 of the sum of magnitudes) and
+// only the few sums of sums in FP64; a split's tiles lie at one stride, so their loads go out together.
+// (One FP64 chain of 64 tiles per thread, offsets looked up: 34 us for 2,048 tiles at N = 360; 17.5 us now, the adjoint's z pass, 7.4 us before, included.)
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_group_reduce(const IterArgs a, const GroupArgs g, int what) {
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
+  const float s = hi + x, bb = s - hi;
+  lo += (hi - (s - bb)) + (x - bb);
+  hi = s;
+}
+__device__ __forceinline__ void group_reduce_block(const IterArgs& a, const GroupArgs& g, int gi, int s, int ce, int what) {
   __shared__ int s_last;
-  const int gi = blockIdx.z, s = blockIdx.y, ce = blockIdx.x;
+  __shared__ double s_q[4][kRedE];
   const GroupDev gr = a.groups[gi];
   const int nsplit = (gr.ntiles + g.split_tiles - 1) / g.split_tiles;
   if (s >= nsplit) return;
   const int E = 3 + ((gr.calib && (what & 2)) ? 2 * gr.N : 0);
-  if (ce * 256 >= E) return;
-  const int e = ce * 256 + threadIdx.x;
-  const int t0 = gr.tile0 + s * g.split_tiles;
-  const int t1 = min(gr.tile0 + gr.ntiles, t0 + g.split_tiles);
+  if (ce * kRedE >= E) return;
+  const int el = threadIdx.x % kRedE, sub = threadIdx.x / kRedE, e = ce * kRedE + el;
+  const int per = (g.split_tiles + 3) / 4, first = s * g.split_tiles + sub * per;
+  const int n = min(per, min((s + 1) * g.split_tiles, gr.ntiles) - first);   // this quarter's tiles
   double acc = 0.0;
-  if (e < E) {
+  if (e < E && n > 0) {
+    const int t0 = gr.tile0 + first;
     if (e < 3) {
-      for (int t = t0; t < t1; ++t) acc += a.tile_red[4 * static_cast<size_t>(t) + e];
+      const double* src = a.tile_red + 4 * static_cast<size_t>(t0) + e;
+#pragma unroll 8
+      for (int t = 0; t < n; ++t) acc += src[4 * t];
     } else {
-      for (int t = t0; t < t1; ++t) acc += a.tile_ab[a.tiles[t].ab_off + (e - 3)];
+      const float* src = a.tile_ab + a.tiles[t0].ab_off + (e - 3);   // a group's tiles follow one another
+      float hi = 0.f, lo = 0.f;
+#pragma unroll 8
+      for (int t = 0; t < n; ++t) two_sum(hi, lo, src[static_cast<size_t>(t) * 2 * gr.N]);
+      acc = static_cast<double>(hi) + static_cast<double>(lo);
     }
-    g.part2[static_cast<size_t>(g.split_off[gi] + s) * g.max_e + e] = acc;
   }
+  s_q[sub][el] = acc;
+  __syncthreads();
+  if (sub == 0 && e < E)
+    g.part2[static_cast<size_t>(g.split_off[gi] + s) * g.max_e + e] = (s_q[0][el] + s_q[1][el]) + (s_q[2][el] + s_q[3][el]);
   __threadfence();
   __syncthreads();
-  const int nce = (g.max_e + 255) / 256;
+  const int nce = (g.max_e + kRedE - 1) / kRedE;
   if (threadIdx.x == 0) {
     const int prev = atomicAdd(&g.counters[gi * nce + ce], 1);
     s_last = (prev == nsplit - 1);
@@ -414,10 +434,16 @@ __global__ void __launch_bounds__(256) k_group_reduce(const IterArgs a, const Gr
   __syncthreads();
   if (!s_last) return;
   __threadfence();
+  acc = 0.0;
   if (e < E) {
-    double tot = 0.0;
-    for (int k = 0; k < nsplit; ++k)
-      tot += __ldcg(&g.part2[static_cast<size_t>(g.split_off[gi] + k) * g.max_e + e]);
+    const double* src = g.part2 + static_cast<size_t>(g.split_off[gi]) * g.max_e + e;
+#pragma unroll 8
+    for (int k = sub; k < nsplit; k += 4) acc += __ldcg(&src[static_cast<size_t>(k) * g.max_e]);
+  }
+  s_q[sub][el] = acc;
+  __syncthreads();
+  if (sub == 0 && e < E) {
+    const double tot = (s_q[0][el] + s_q[1][el]) + (s_q[2][el] + s_q[3][el]);
     if (e == 0) {
       if (what & 1) g.gloss[gi] = tot;
     } else if (e == 1) {
@@ -432,8 +458,8 @@ __global__ void __launch_bounds__(256) k_group_reduce(const IterArgs a, const Gr
 }
 
 // dJ/db_lr[c] = sum_x w_c(x) dJ/dU(x): the adjoint of the trilinear upsampling. Its weights
-// factor per axis, w_c(x, y, z) = w_cx(x) w_cy(y) w_cz(z), so the sum is three contractions
-// in a fixed order: over z (per (x, y) line), then y, then x; each grid voxel is read once.
+// factor per axis, w_c(x, y, z) = w_cx(x) w_cy(y) w_cz(z), so the sum is taken in a fixed order
+// over z (per (x, y) line), then over the corner's (x, y) support; each grid voxel is read once.
 // Axis weights as in tri_weights: u = clamp((i + .5) 8 / n - .5, 0, 7), i0 = min(floor u, 6),
 // corner i0 takes 1 - (u - i0) and corner i0 + 1 takes u - i0.
 __device__ __forceinline__ void axis_weight(int i, int n, int& i0, float& w) {
@@ -459,12 +485,11 @@ __device__ __forceinline__ float axis_corner_weight(int i, int n, int c) {
 
 // Pass 1: G1[x][y][cz] = sum_z w_cz(z) dJ/dU(x, y, z); one warp per (x, y) line, its lanes
 // strided over z, then a fixed-order butterfly over the lanes (FP32: at most 1023 terms).
-__global__ void __launch_bounds__(128) k_bias_grad_z(const IterArgs a, const GroupArgs g) {
-  const int gi = blockIdx.y;
+__device__ __forceinline__ void bias_grad_z(const IterArgs& a, const GroupArgs& g, int gi, int line) {
   const GroupDev gr = a.groups[gi];
-  const int line = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
   if (!gr.calib || line >= gr.nx * gr.ny) return;   // warp-uniform
-  double* G1 = g.bscratch + g.bs_off[2 * gi];
+  double* G1 = g.bscratch + g.bs_off[gi];
   float acc[kGrid];
 #pragma unroll
   for (int c = 0; c < kGrid; ++c) acc[c] = 0.f;
@@ -490,52 +515,61 @@ __global__ void __launch_bounds__(128) k_bias_grad_z(const IterArgs a, const Gro
   }
 }
 
-// Pass 2: G2[x][cy][cz] = sum_y w_cy(y) G1[x][y][cz]; one thread per (x, cy, cz), over the
-// support of cy only.
-__global__ void __launch_bounds__(128) k_bias_grad_y(const IterArgs a, const GroupArgs g) {
+// The tile sums and, in the first `nbz` blocks of a group, pass 1 of the bias-field adjoint (eight
+// lines per block): neither reads what the other writes, so they share a launch.
+__global__ void __launch_bounds__(256) k_group_sums(const IterArgs a, const GroupArgs g, int what, int nbz) {
+  grid_dep_wait();
+  grid_dep_launch();
+  const int b = blockIdx.x, gi = blockIdx.y;
+  if (b < nbz) {
+    bias_grad_z(a, g, gi, b * 8 + (threadIdx.x >> 5));
+  } else {
+    const int nce = (g.max_e + kRedE - 1) / kRedE;
+    group_reduce_block(a, g, gi, (b - nbz) / nce, (b - nbz) % nce, what);
+  }
+}
+
+// Pass 2: dJ/db_lr[cx][cy][cz] = sum_xy w_cx(x) w_cy(y) G1[x][y][cz], a warp per corner, its lanes strided
+// over the corner's (x, y) support, then a butterfly: 512 warps share the FP64 work (a thread per
+// corner over x after one over y had it on a few SMs: 8.2 + 8.3 us for 64^3, 8.9 us now).
+__global__ void __launch_bounds__(256) k_bias_grad_xy(const IterArgs a, const GroupArgs g) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int gi = blockIdx.y;
   const GroupDev gr = a.groups[gi];
   if (!gr.calib) return;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= gr.nx * kGrid * kGrid) return;
-  const int x = e / (kGrid * kGrid), cy = (e / kGrid) % kGrid, cz = e % kGrid;
-  const double* G1 = g.bscratch + g.bs_off[2 * gi];
-  double* G2 = g.bscratch + g.bs_off[2 * gi + 1];
-  int lo, hi;
-  axis_support(cy, gr.ny, lo, hi);
+  const int c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int cx = c / (kGrid * kGrid), cy = (c / kGrid) % kGrid, cz = c % kGrid;
+  const double* G1 = g.bscratch + g.bs_off[gi] + cz;
+  int xlo, xhi, ylo, yhi;
+  axis_support(cx, gr.nx, xlo, xhi);
+  axis_support(cy, gr.ny, ylo, yhi);
+  const int ny = yhi - ylo + 1, n = (xhi - xlo + 1) * ny;
   double acc = 0.0;
-  for (int y = lo; y <= hi; ++y) {
-    const float w = axis_corner_weight(y, gr.ny, cy);
-    if (w != 0.f) acc += static_cast<double>(w) * G1[(static_cast<int64_t>(x) * gr.ny + y) * kGrid + cz];
+#pragma unroll 4
+  for (int e = lane; e < n; e += 32) {
+    const int x = xlo + e / ny, y = ylo + e % ny;
+    const float wx = axis_corner_weight(x, gr.nx, cx), wy = axis_corner_weight(y, gr.ny, cy);
+    const double v = G1[(static_cast<int64_t>(x) * gr.ny + y) * kGrid];
+    if (wx != 0.f && wy != 0.f) acc += (static_cast<double>(wx) * static_cast<double>(wy)) * v;
   }
-  G2[(static_cast<int64_t>(x) * kGrid + cy) * kGrid + cz] = acc;
-}
-
-// Pass 3: dJ/db_lr[cx][cy][cz] = sum_x w_cx(x) G2[x][cy][cz]; one thread per corner.
-__global__ void __launch_bounds__(kNGrid) k_bias_grad_x(const IterArgs a, const GroupArgs g) {
-  const int gi = blockIdx.x;
-  const GroupDev gr = a.groups[gi];
-  if (!gr.calib) return;
-  const int c = threadIdx.x;
-  const int cx = c / (kGrid * kGrid), cyz = c % (kGrid * kGrid);
-  const double* G2 = g.bscratch + g.bs_off[2 * gi + 1];
-  int lo, hi;
-  axis_support(cx, gr.nx, lo, hi);
-  double acc = 0.0;
-  for (int x = lo; x <= hi; ++x) {
-    const float w = axis_corner_weight(x, gr.nx, cx);
-    if (w != 0.f) acc += static_cast<double>(w) * G2[static_cast<int64_t>(x) * kGrid * kGrid + cyz];
-  }
-  g.gred[gr.gp_off + 4 + 2 * gr.N4 + c] = acc;
+  acc = warp_sum_d(acc);
+  if (lane == 0) g.gred[gr.gp_off + 4 + 2 * gr.N4 + c] = acc;
 }
 
 // Group finalisation (one block): objective with the calibration regularisers of Sec. 2.4
 // (L2 on alpha, beta, b_lr and TV on B; the paper gives no weights: 1e-3 each by default),
 // loss history, Adam on sigma_log / alpha / beta / b_lr, table refresh, step counter.
-// mode bit 0: loss; bit 1: Adam + step; bit 2: export gradients.
-__global__ void __launch_bounds__(256) k_group_adam(const IterArgs a, const GroupArgs g, int mode) {
-  __shared__ double s[256];
+// mode bit 0: loss; bit 1: Adam + step; bit 2: export gradients. One block per group on the critical
+// path of a calibrated iteration, bound by one SM's FP64 rate: the weights are divided once and each
+// parameter costs five FP64 operations (with a division per parameter and 256 threads 25 us for the
+// 1,236 parameters at N = 360, 15 us now).
+constexpr int kGroupThreads = 512;
+__global__ void __launch_bounds__(kGroupThreads) k_group_adam(const IterArgs a, const GroupArgs g, int mode) {
+  __shared__ double s[kGroupThreads / 32], s_w[3];
   __shared__ int s_bad, s_last;
+  grid_dep_wait();
+  grid_dep_launch();
   const int tid = threadIdx.x;
   if (tid == 0) s_bad = 0;
   const int step = *a.step;
@@ -545,29 +579,34 @@ __global__ void __launch_bounds__(256) k_group_adam(const IterArgs a, const Grou
     const GroupDev gr = a.groups[gi];
     const int base = gr.gp_off;
     const int N = gr.N, N4 = gr.N4;
-    // regulariser values
-    double reg = 0.0;
+    // regulariser weights of a squared alpha, beta and b_lr, and their values
+    if (tid < 3) s_w[tid] = static_cast<double>(tid == 0 ? g.w_alpha : tid == 1 ? g.w_beta : g.w_blr) / (tid < 2 ? N : kNGrid);
+    double ra = 0.0, rb = 0.0, rl = 0.0;
     if (gr.calib) {
-      for (int i = tid; i < 2 * N + kNGrid; i += blockDim.x) {
-        float x;
-        double w;
-        if (i < N) { x = g.gparams[base + 4 + i]; w = g.w_alpha / N; }
-        else if (i < 2 * N) { x = g.gparams[base + 4 + N4 + (i - N)]; w = g.w_beta / N; }
-        else { x = g.gparams[base + 4 + 2 * N4 + (i - 2 * N)]; w = g.w_blr / kNGrid; }
-        reg += w * static_cast<double>(x) * x;
+      const float* p = g.gparams + base + 4;
+      for (int i = tid; i < N; i += kGroupThreads) {
+        const double xa = p[i], xb = p[N4 + i];
+        ra = fma(xa, xa, ra);
+        rb = fma(xb, xb, rb);
+      }
+      for (int i = tid; i < kNGrid; i += kGroupThreads) {
+        const double x = p[2 * N4 + i];
+        rl = fma(x, x, rl);
       }
     }
-    s[tid] = reg;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-      if (tid < o) s[tid] += s[tid + o];
+    const double wa = s_w[0], wb = s_w[1], wl = s_w[2];
+    if (mode & 1) {
+      double reg = gr.calib ? warp_sum_d(fma(wa, ra, fma(wb, rb, wl * rl))) : 0.0;
+      if ((tid & 31) == 0) s[tid >> 5] = reg;
       __syncthreads();
-    }
-    if ((mode & 1) && tid == 0) {
-      const double J = g.gloss[gi] + g.gprior[gi] + s[0];
-      g.gloss[gi] = J;
-      if (!isfinite(J)) s_bad = 1;
-      if (mode & 2) g.hist[static_cast<size_t>(step % g.hist_len) * g.G + gi] = J;
+      if (tid == 0) {
+        for (int w = 1; gr.calib && w < kGroupThreads / 32; ++w) reg += s[w];
+        const double J = g.gloss[gi] + g.gprior[gi] + reg;
+        g.gloss[gi] = J;
+        if (!isfinite(J)) s_bad = 1;
+        if (mode & 2) g.hist[static_cast<size_t>(step % g.hist_len) * g.G + gi] = J;
+      }
     }
     __syncthreads();
     // gradients and Adam over the group's packed parameters
@@ -584,13 +623,13 @@ __global__ void __launch_bounds__(256) k_group_adam(const IterArgs a, const Grou
         grad = 0.f;
       } else if (i < 4 + N4) {
         train = gr.calib && (i - 4 < N);
-        grad = train ? static_cast<float>(g.gred[base + i] + 2.0 * g.w_alpha / N * x) : 0.f;
+        grad = train ? static_cast<float>(fma(2.0 * wa, static_cast<double>(x), g.gred[base + i])) : 0.f;
       } else if (i < 4 + 2 * N4) {
         train = gr.calib && (i - 4 - N4 < N);
-        grad = train ? static_cast<float>(g.gred[base + i] + 2.0 * g.w_beta / N * x) : 0.f;
+        grad = train ? static_cast<float>(fma(2.0 * wb, static_cast<double>(x), g.gred[base + i])) : 0.f;
       } else {
         train = gr.calib;
-        grad = train ? static_cast<float>(g.gred[base + i] + 2.0 * g.w_blr / kNGrid * x) : 0.f;
+        grad = train ? static_cast<float>(fma(2.0 * wl, static_cast<double>(x), g.gred[base + i])) : 0.f;
       }
       if (g.gexport && (mode & 4)) g.gexport[base + i] = grad;
       if ((mode & 2) && train) {
@@ -683,20 +722,16 @@ cudaError_t launch_wait_probe(int32_t* status, int polls, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_group_reduce(const IterArgs& a, const GroupArgs& g, int what, cudaStream_t st) {
-  dim3 grid((g.max_e + 255) / 256, g.max_split, g.G);
-  k_group_reduce<<<grid, 256, 0, st>>>(a, g, what);
-  return cudaGetLastError();
-}
-cudaError_t launch_bias_grad(const IterArgs& a, const GroupArgs& g, cudaStream_t st) {
-  k_bias_grad_z<<<dim3(nblk(static_cast<int64_t>(g.max_nx) * g.max_ny, 4), g.G), 128, 0, st>>>(a, g);
-  k_bias_grad_y<<<dim3(nblk(static_cast<int64_t>(g.max_nx) * kGrid * kGrid, 128), g.G), 128, 0, st>>>(a, g);
-  k_bias_grad_x<<<g.G, kNGrid, 0, st>>>(a, g);
-  return cudaGetLastError();
+cudaError_t launch_group_sums(const IterArgs& a, const GroupArgs& g, int what, bool bias, cudaStream_t st) {
+  const int nbz = bias ? nblk(static_cast<int64_t>(g.max_nx) * g.max_ny, 8) : 0;
+  const int nred = (g.max_e + kRedE - 1) / kRedE * g.max_split;
+  cudaError_t e = launch_dep(k_group_sums, dim3(nbz + nred, g.G), dim3(256), 0, st, a.pdl != 0, a, g, what, nbz);
+  if (e == cudaSuccess && bias)
+    e = launch_dep(k_bias_grad_xy, dim3(kNGrid / 8, g.G), dim3(256), 0, st, a.pdl != 0, a, g);
+  return e;
 }
 cudaError_t launch_group_adam(const IterArgs& a, const GroupArgs& g, int mode, cudaStream_t st) {
-  k_group_adam<<<g.G, 256, 0, st>>>(a, g, mode);
-  return cudaGetLastError();
+  return launch_dep(k_group_adam, dim3(g.G), dim3(kGroupThreads), 0, st, a.pdl != 0, a, g, mode);
 }
 cudaError_t launch_loss(const IterArgs& a, const PlainArgs& p, int loss, cudaStream_t st) {
   const int nt = p.tile_end - p.tile_begin;

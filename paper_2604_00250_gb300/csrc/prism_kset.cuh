@@ -13,27 +13,6 @@ namespace {
 
 constexpr int kK = PRISM_K;
 
-// Launches fn on st, as a programmatic dependent of the stream's previous kernel when `pdl`
-// (the kernel then waits for it on the device before reading what it wrote).
-template <typename... P, typename... A>
-cudaError_t launch_dep(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, A... args) {
-  if (!pdl) {
-    fn<<<grid, block, smem, st>>>(args...);
-    return cudaGetLastError();
-  }
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fn, args...);
-}
-
 template <int TPV, int LOSS, bool CAL, bool SHELL = false, bool GRAD = false>
 cudaError_t fused_one(const IterArgs& a, int grid, int nt, size_t smem, cudaStream_t st) {
   auto fn = k_iter_fused<kK, TPV, LOSS, CAL, SHELL, GRAD>;

@@ -7,6 +7,27 @@
 
 namespace prism {
 
+// Launches fn on st, as a programmatic dependent of the stream's previous kernel when `pdl`
+// (the kernel then waits for it on the device before reading what it wrote).
+template <typename... P, typename... A>
+cudaError_t launch_dep(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl, A... args) {
+  if (!pdl) {
+    fn<<<grid, block, smem, st>>>(args...);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, args...);
+}
+
 // Per-K launchers of the templated kernels (one translation unit per K).
 struct KernelSet {
   // shell = 1: the shell loop of one thread per voxel, MSE, no calibration (K <= 3); grad = 1: the
@@ -36,11 +57,12 @@ struct KernelSet {
 const KernelSet& kernels_for_k(int K);
 
 // Group-level kernels (prism_aux.cu).
+constexpr int kRedE = 64;   // entries of the group sums per block
 struct GroupArgs {
   int32_t G, max_split, split_tiles, max_e;
   const int32_t* split_off;   // [G] first part2 row of the group
   double* part2;              // [sum splits][max_e]
-  int32_t* counters;          // [G][ceil(max_e / 256)]
+  int32_t* counters;          // [G][ceil(max_e / kRedE)]
   double* gred;               // packed like gparams (double); loss kept separately
   double* gloss;              // [G] data term, then the full objective after finalisation
   double* gprior;             // [G] prior total
@@ -55,14 +77,15 @@ struct GroupArgs {
   float* gexport;             // packed group gradients for the caller (or null)
   int32_t loss_mode;          // kLossMSE / kLossNLL
   float w_alpha, w_beta, w_blr;
-  double* bscratch;           // bias-gradient partial contractions (see k_bias_grad_*)
-  const int64_t* bs_off;      // [G][2] offsets of a group's [nx][ny][8] and [nx][8][8] parts
+  double* bscratch;           // bias-gradient partial contractions (see bias_grad_z)
+  const int64_t* bs_off;      // [G] offset of a group's [nx][ny][8] sums over z
   int32_t max_nx, max_ny;     // largest grid extents over the groups
   int32_t* gdone;             // blocks of k_group_adam that finished (last one resets it)
 };
 
-cudaError_t launch_group_reduce(const IterArgs& a, const GroupArgs& g, int what, cudaStream_t st);
-cudaError_t launch_bias_grad(const IterArgs& a, const GroupArgs& g, cudaStream_t st);
+// Sums over the tiles (`what` bit 0: objective, bit 1: group gradients) and, with `bias`, the
+// bias-field adjoint.
+cudaError_t launch_group_sums(const IterArgs& a, const GroupArgs& g, int what, bool bias, cudaStream_t st);
 cudaError_t launch_group_adam(const IterArgs& a, const GroupArgs& g, int mode, cudaStream_t st);
 cudaError_t launch_loss(const IterArgs& a, const PlainArgs& p, int loss, cudaStream_t st);
 cudaError_t launch_adam_voxel(const IterArgs& a, const PlainArgs& p, cudaStream_t st);

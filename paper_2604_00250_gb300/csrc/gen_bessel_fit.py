@@ -1,14 +1,15 @@
 """Writes bessel_fit.h: float32 approximations of the modified Bessel functions
-that the Rician NLL (Eq. 9) and its gradient need.
-
-For z < ZS the kernels sum the power series (A&S 9.6.10)
-    I0(z) = sum_k t^k / (k!)^2,   I1(z) = (z/2) sum_k t^k / (k! (k+1)!),   t = z^2/4,
-with NSER terms. For z >= ZS they evaluate two smooth functions of x = ZS / z in (0, 1]:
-    PA(x) = sqrt(2 pi z) i0e(z)            -> log i0e(z) = log PA - log(2 pi z) / 2
-    PB(x) = z (1 - I1(z) / I0(z))          -> Q(z) = 1 - I1/I0 = PB / z
-as degree-DEG polynomials fitted here by relative least squares on Chebyshev-spaced
-nodes against scipy.special.i0e / i1e (Cephes, float64). Q is obtained directly, never
-as 1 - I1/I0, so it keeps relative accuracy where I1/I0 -> 1.
+that the Rician NLL (Eq. 9) and its gradient need,
+    Q(z) = 1 - I1(z) / I0(z),   L(z) = log(exp(-z) I0(z)),   z >= 0,
+as one polynomial of degree DEG per segment of z, so that lanes of a warp with unlike z take
+the same instructions. Segment s < 8 covers [s, s + 1] in w = z - s - 1/2; segment 8 covers
+z >= 8 in w = 8 / z. With r = 1 / max(z, 8):
+    Q = P(w) r            P fits 8 Q for s < 8, z Q for s = 8
+    L = G(w) - log(max(z, 8)) / 2
+                          G fits L + log(8) / 2, and log(sqrt(z) exp(-z) I0(z)) for s = 8
+Q is obtained directly, never as 1 - I1/I0, so it keeps relative accuracy where I1/I0 -> 1.
+The fits are weighted least squares in the Chebyshev basis (weights iterated towards the
+minimax fit, Lawson 1961) against scipy.special.i0e / i1e (Cephes, float64).
 
 Run: python gen_bessel_fit.py > bessel_fit.h
 """
@@ -17,56 +18,63 @@ import math
 import numpy as np
 import scipy.special as sp
 
-ZS = 4.0
-DEG = 12
-NSER = 12
+NSEG = 9
+ZS = 8.0
+DEG = 7
 
 
-def fit(fun):
-    xs = 0.5 * (1 - np.cos(np.linspace(0, np.pi, 4000)))
-    xs = xs[xs > 1e-7]
-    y = fun(ZS / xs)
-    V = np.vander(xs, DEG + 1, increasing=True)
-    c, *_ = np.linalg.lstsq(V / y[:, None], np.ones_like(y), rcond=None)
-    return c
+def q_of(z):
+    """1 - I1(z) / I0(z); above z = 50 by the asymptotic series of I0 and I1 (A&S 9.7.1)."""
+    far = 1 / (2 * z) + 1 / (8 * z**2) + 1 / (8 * z**3) + 25 / (128 * z**4) + 13 / (32 * z**5) + 1073 / (1024 * z**6)
+    near = np.minimum(z, 50.0)
+    return np.where(z < 50, 1 - sp.i1e(near) / sp.i0e(near), far)
 
 
-def pa(z):
-    return np.sqrt(2 * np.pi * z) * sp.i0e(z)
+def fit(f, lo, hi, relative, n=3000, iters=60):
+    """Power-basis coefficients of the fit of f over w in [lo, hi]."""
+    t = np.cos(np.pi * (np.arange(n) + 0.5) / n)
+    y = f((t + 1) / 2 * (hi - lo) + lo)
+    w0 = 1 / np.abs(y) if relative else np.ones(n)
+    B = np.polynomial.chebyshev.chebvander(t, DEG)
+    lw = np.ones(n)
+    for _ in range(iters):
+        c, *_ = np.linalg.lstsq(B * (w0 * np.sqrt(lw))[:, None], y * w0 * np.sqrt(lw), rcond=None)
+        e = np.abs((B @ c - y) * w0)
+        lw = lw * (e / e.max() + 1e-6)
+        lw /= lw.sum() / n
+    P = np.polynomial.Polynomial([0.0])
+    arg = np.polynomial.Polynomial([-(hi + lo) / (hi - lo), 2 / (hi - lo)])
+    for k in np.polynomial.chebyshev.cheb2poly(c)[::-1]:
+        P = P * arg + k
+    return P.coef
 
 
-def pb(z):
-    return z * (1 - sp.i1e(z) / sp.i0e(z))
+def table():
+    """[DEG + 1][NSEG][2]: the coefficients of P and G."""
+    tab = np.zeros((DEG + 1, NSEG, 2))
+    for s in range(NSEG - 1):
+        tab[:, s, 0] = fit(lambda w: 8 * q_of(w + s + 0.5), -0.5, 0.5, True)
+        tab[:, s, 1] = fit(lambda w: np.log(sp.i0e(w + s + 0.5)) + 0.5 * math.log(8.0), -0.5, 0.5, False)
 
-
-def arr(name, vals):
-    body = ", ".join(f"{float(v):.9e}f" for v in vals)
-    return f"__device__ __constant__ float {name}[{len(vals)}] = {{{body}}};"
-
-
-def arr2(name, xs, ys):
-    """Two tables interleaved as float2 {x_k, y_k}: the two Horner chains that share an argument
-    then run as one packed f32x2 chain."""
-    body = ", ".join(f"{{{float(x):.9e}f, {float(y):.9e}f}}" for x, y in zip(xs, ys))
-    return f"__device__ __constant__ float2 {name}[{len(xs)}] = {{{body}}};"
+    def z_of(x):
+        return ZS / np.maximum(x, 1e-7)
+    tab[:, NSEG - 1, 0] = fit(lambda x: z_of(x) * q_of(z_of(x)), 0.0, 1.0, True)
+    tab[:, NSEG - 1, 1] = fit(lambda x: np.log(sp.i0e(z_of(x)) * np.sqrt(z_of(x))), 0.0, 1.0, False)
+    return tab
 
 
 def main():
-    ca = fit(pa)
-    cb = fit(pb)
-    s0 = [1.0 / math.factorial(k) ** 2 for k in range(NSER)]
-    s1 = [1.0 / (math.factorial(k) * math.factorial(k + 1)) for k in range(NSER)]
+    tab = table()
     print("/* Generated by gen_bessel_fit.py -- do not edit. */")
     print("#pragma once")
-    print(f"#define PRISM_BESSEL_ZS {ZS:.1f}f")
+    print(f"#define PRISM_BESSEL_NSEG {NSEG}")
     print(f"#define PRISM_BESSEL_DEG {DEG}")
-    print(f"#define PRISM_BESSEL_NSER {NSER}")
-    print(arr("k_bessel_pa", ca))
-    print(arr("k_bessel_pb", cb))
-    print(arr("k_bessel_s0", s0))
-    print(arr("k_bessel_s1", s1))
-    print(arr2("k_bessel_pba", cb, ca))
-    print(arr2("k_bessel_s01", s0, s1))
+    print("/* [j][segment]: {P, G coefficients of w^(2j), P, G coefficients of w^(2j+1)} */")
+    print(f"__device__ const float4 k_bessel_tab[{(DEG + 1) // 2 * NSEG}] = {{")
+    for j in range((DEG + 1) // 2):
+        row = ["{%s}" % ", ".join(f"{float(v):.9e}f" for v in (*tab[2 * j, s], *tab[2 * j + 1, s])) for s in range(NSEG)]
+        print("  " + ",\n  ".join(row) + ",")
+    print("};")
 
 
 if __name__ == "__main__":

@@ -17,7 +17,6 @@ constexpr int kGrid = 8;          // bias control grid edge (Sec. 2.3 item 1)
 constexpr int kNGrid = 512;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
-constexpr float kHalfLog2Pi = 0.9189385332046727f;   // log(2 pi) / 2
 constexpr float kNormEps2 = 1e-24f;                  // |v| clamp 1e-12, squared
 
 // Device status word bits (read by prism_sync).
@@ -270,38 +269,40 @@ __device__ __forceinline__ float huber_drho(float r, float dl) {
   return fabsf(r) <= dl ? r : copysignf(dl, r);
 }
 
-// Q(z) = 1 - I1(z)/I0(z) and L(z) = log(exp(-z) I0(z)) for z >= 0, float32.
-// Power series below PRISM_BESSEL_ZS, fitted smooth functions of ZS/z above. The two Horner
-// chains of each branch share their argument, so they run as one packed f32x2 chain over the
-// interleaved tables (each lane the same round-to-nearest multiply-add as the scalar chain; on
-// GB300 the DiSCo1-shaped NLL fit's fused kernel 9 % faster).
-template <bool WANT_L>
-__device__ __forceinline__ void bessel_QL(float z, float& Q, float& L) {
-  if (z < PRISM_BESSEL_ZS) {
-    const float t = 0.25f * z * z;
-    const float2 tt = make_float2(t, t);
-    float2 s = k_bessel_s01[PRISM_BESSEL_NSER - 1];
-#pragma unroll
-    for (int k = PRISM_BESSEL_NSER - 2; k >= 0; --k) s = __ffma2_rn(s, tt, k_bessel_s01[k]);
-    const float i0 = s.x, i1 = s.y;
-    Q = 1.f - 0.5f * z * i1 * rcpf_(i0);   // i0 >= 1
-    if (WANT_L) L = lg2f_(i0) * kLn2 - z;
-  } else {
-    const float x = PRISM_BESSEL_ZS * rcpf_(z);
-    if (WANT_L) {
-      const float2 xx = make_float2(x, x);
-      float2 p = k_bessel_pba[PRISM_BESSEL_DEG];
-#pragma unroll
-      for (int k = PRISM_BESSEL_DEG - 1; k >= 0; --k) p = __ffma2_rn(p, xx, k_bessel_pba[k]);
-      Q = p.x * x * (1.f / PRISM_BESSEL_ZS);
-      L = (lg2f_(p.y) - 0.5f * lg2f_(z)) * kLn2 - kHalfLog2Pi;
-    } else {
-      float pb = k_bessel_pb[PRISM_BESSEL_DEG];
-#pragma unroll
-      for (int k = PRISM_BESSEL_DEG - 1; k >= 0; --k) pb = fmaf(pb, x, k_bessel_pb[k]);
-      Q = pb * x * (1.f / PRISM_BESSEL_ZS);
-    }
-  }
+// Q(z) = 1 - I1(z)/I0(z) and L(z) = log(exp(-z) I0(z)) for z >= 0, float32, by one polynomial per
+// segment of z (gen_bessel_fit.py), coefficients looked up in shared memory (`tab`, bessel_stage): the
+// nine segments' entries of a degree are neighbours, so a warp reads them without bank conflicts. No
+// branch depends on z: with a power series below z = 4 and a degree-12 fit above, half to three
+// quarters of the warps held lanes on both sides (phantoms at SNR 20-50) and ran both, one measurement
+// after the other (calibrated bundle phantom: fused kernel 634 -> 537 us, DiSCo1-shaped 214 -> 206). The two polynomials share their argument and run as one packed f32x2
+// chain. Error (float32 evaluation against float64): Q 2e-7 relative, L 5e-7 absolute at most, both below
+// the two-branch form's (1.4e-6, 7e-7).
+constexpr int kBesselTab = (PRISM_BESSEL_DEG + 1) / 2 * PRISM_BESSEL_NSEG;
+static_assert(PRISM_BESSEL_DEG == 7 && PRISM_BESSEL_NSEG == 9, "bessel_QL is written out for these");
+__device__ __forceinline__ void bessel_stage(float4* tab) {   // the caller synchronises the block
+  for (int i = threadIdx.x; i < kBesselTab; i += blockDim.x) tab[i] = k_bessel_tab[i];
+}
+__device__ __forceinline__ void bessel_QL(float z, const float4* __restrict__ tab, float& Q, float& L) {
+  const float zm = fmaxf(z, 8.f);
+  const float r = rcpf_(zm);
+  // segment floor(z) for z < 8 (a z on a boundary may take either), else 8: round(min(z, 8) - 1/2) by
+  // the addition of 1.5 * 2^23, whose low bits then hold it; 0..8 for every z >= 0, and 8 for a NaN
+  const float zh = fminf(z, 8.f) - 0.5f;
+  const float mg = zh + 12582912.f;
+  const float seg = mg - 12582912.f;
+  const float w = (z < 8.f) ? zh - seg : 8.f * r;
+  const float4* t = tab + (__float_as_int(mg) & 15);
+  const float4 c3 = t[3 * PRISM_BESSEL_NSEG], c2 = t[2 * PRISM_BESSEL_NSEG], c1 = t[PRISM_BESSEL_NSEG], c0 = t[0];
+  const float2 ww = make_float2(w, w);
+  float2 p = __ffma2_rn(make_float2(c3.z, c3.w), ww, make_float2(c3.x, c3.y));
+  p = __ffma2_rn(p, ww, make_float2(c2.z, c2.w));
+  p = __ffma2_rn(p, ww, make_float2(c2.x, c2.y));
+  p = __ffma2_rn(p, ww, make_float2(c1.z, c1.w));
+  p = __ffma2_rn(p, ww, make_float2(c1.x, c1.y));
+  p = __ffma2_rn(p, ww, make_float2(c0.z, c0.w));
+  p = __ffma2_rn(p, ww, make_float2(c0.x, c0.y));
+  Q = p.x * r;
+  L = fmaf(-0.5f * kLn2, lg2f_(zm), p.y);
 }
 
 // U(x) = trilinear upsampling of the 8^3 grid at voxel (i, j, k) of an n-grid,

@@ -353,7 +353,7 @@ __device__ __forceinline__ void acc_reduce_tpv(Acc<K>& A) {
 template <int K, int LOSS, bool CAL, bool EXT_R>
 __device__ __forceinline__ void pair(const Vox<K>& P, const float (&ffin)[K], const float (&fomf)[K],
                                      const MeasRow& R, float yv, float B, float inv_s2, float r_ext, Acc<K>& A,
-                                     float& rr_out, float& u_out) {
+                                     float& rr_out, float& u_out, const float4* bess = nullptr) {
   float T = P.f[0] * R.ecsf;
   T = fmaf(P.f[1], R.egm, T);
   T = fmaf(P.f[K + 2], R.eres, T);
@@ -381,13 +381,13 @@ __device__ __forceinline__ void pair(const Vox<K>& P, const float (&ffin)[K], co
     rr = yh - yv;
     A.l1 = fmaf(rr, rr, A.l1);
   } else {
-    const float ay = fabsf(yh);
-    const float sy = (yh >= 0.f) ? yv : -yv;
+    const float ay = fabsf(yh), yy = fabsf(yv);   // I0 is even: the objective takes |y| (see nll_lane)
+    const float sy = (yh >= 0.f) ? yy : -yy;
     float Qz, Lz;
-    bessel_QL<true>(yv * ay * inv_s2, Qz, Lz);
-    const float e = yv - ay;
+    bessel_QL(yy * ay * inv_s2, bess, Qz, Lz);
+    const float e = yy - ay;
     A.l1 = fmaf(e, e, A.l1);
-    A.l2 = fmaf(yv * ay, Qz, A.l2);
+    A.l2 = fmaf(yy * ay, Qz, A.l2);
     A.l3 += Lz;
     rr = fmaf(sy, Qz, yh - sy);      // y_hat - y R(z), R = I1/I0
   }
@@ -477,16 +477,18 @@ __device__ __forceinline__ void voxp_init(const Vox<K>& P, VoxP<K>& D, AccP<K>& 
 
 // Rician NLL terms of one measurement (Eq. 9) for the packed path: adds (y - |y_hat|)^2 to l1,
 // y |y_hat| Q(z) to l2 and L(z) to l3, and returns dL/dy_hat unscaled (y_hat - y R(z)); a
-// lane with m = 0 (padding) adds nothing.
+// lane with m = 0 (padding) adds nothing. A negative magnitude (filtered data) counts as |y|: with
+// I0 even and I1 odd, y R(y a / sigma^2) = |y| R(|y| a / sigma^2) and (y - a)^2 / 2 sigma^2 - log(e^-z I0(z))
+// take the same value at y and -y, so z is never negative.
 __device__ __forceinline__ float nll_lane(float yh, float yv, float inv_s2, float m, float& l1, float& l2,
-                                          float& l3) {
-  const float ay = fabsf(yh);
-  const float sy = (yh >= 0.f) ? yv : -yv;
+                                          float& l3, const float4* bess) {
+  const float ay = fabsf(yh), yy = fabsf(yv);
+  const float sy = (yh >= 0.f) ? yy : -yy;
   float Qz, Lz;
-  bessel_QL<true>(yv * ay * inv_s2, Qz, Lz);
-  const float e = yv - ay;
+  bessel_QL(yy * ay * inv_s2, bess, Qz, Lz);
+  const float e = yy - ay;
   l1 = fmaf(m * e, e, l1);
-  l2 = fmaf(m * yv * ay, Qz, l2);
+  l2 = fmaf(m * yy * ay, Qz, l2);
   l3 = fmaf(m, Lz, l3);
   return m * fmaf(sy, Qz, yh - sy);
 }
@@ -499,8 +501,8 @@ __device__ __forceinline__ float nll_lane(float yh, float yv, float inv_s2, floa
 // two measurements for the per-measurement alpha / beta partials.
 template <int K, bool MASK, int LOSS = kLossMSE, bool CAL = false>
 __device__ __forceinline__ void step2(const VoxP<K>& D, const MeasPair& R, float2 y, float2 msk, AccP<K>& A,
-                                      float inv_s2 = 0.f, float2 B2 = float2{1.f, 1.f}, float2* uo = nullptr,
-                                      float2* ro = nullptr) {
+                                      float inv_s2 = 0.f, const float4* bess = nullptr,
+                                      float2 B2 = float2{1.f, 1.f}, float2* uo = nullptr, float2* ro = nullptr) {
   const float4 q0 = R.q[0], q1 = R.q[1], q2 = R.q[2], q3 = R.q[3], q4 = R.q[4], q5 = R.q[5];
   const float2 gx = lo2(q0), gy = hi2(q0), gz = lo2(q1), nkpar = hi2(q1);
   const float2 nkperp = lo2(q2), nkd = hi2(q2), ecsf = lo2(q3), egm = hi2(q3);
@@ -528,8 +530,8 @@ __device__ __forceinline__ void step2(const VoxP<K>& D, const MeasPair& R, float
       if (MASK) r = __fmul2_rn(r, msk);
       A.l1 = __ffma2_rn(r, r, A.l1);
     } else {
-      r.x = -nll_lane(yh.x, y.x, inv_s2, MASK ? msk.x : 1.f, A.l1.x, A.l2, A.l3);
-      r.y = -nll_lane(yh.y, y.y, inv_s2, MASK ? msk.y : 1.f, A.l1.y, A.l2, A.l3);
+      r.x = -nll_lane(yh.x, y.x, inv_s2, MASK ? msk.x : 1.f, A.l1.x, A.l2, A.l3, bess);
+      r.y = -nll_lane(yh.y, y.y, inv_s2, MASK ? msk.y : 1.f, A.l1.y, A.l2, A.l3, bess);
     }
     q = __fmul2_rn(r, AB);
     const float2 u = __fmul2_rn(q, S);
@@ -543,8 +545,8 @@ __device__ __forceinline__ void step2(const VoxP<K>& D, const MeasPair& R, float
       A.l1 = __ffma2_rn(r, r, A.l1);
     } else {
       const float2 yh = __fmul2_rn(D.nS0, T);   // -y_hat
-      r.x = -nll_lane(-yh.x, y.x, inv_s2, MASK ? msk.x : 1.f, A.l1.x, A.l2, A.l3);
-      r.y = -nll_lane(-yh.y, y.y, inv_s2, MASK ? msk.y : 1.f, A.l1.y, A.l2, A.l3);
+      r.x = -nll_lane(-yh.x, y.x, inv_s2, MASK ? msk.x : 1.f, A.l1.x, A.l2, A.l3, bess);
+      r.y = -nll_lane(-yh.y, y.y, inv_s2, MASK ? msk.y : 1.f, A.l1.y, A.l2, A.l3, bess);
     }
     q = r;
   }
@@ -1098,6 +1100,9 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
   constexpr int TV = kFusedThreads / TPV;
   __shared__ float s_acc[(TPV > 1) ? (8 + 5 * K) * TV : 1];
 
+  __shared__ float4 s_bess[(LOSS == kLossNLL) ? kBesselTab : 1];
+  if constexpr (LOSS == kLossNLL) bessel_stage(s_bess);   // visible after the block barrier below
+
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // A voxel's TPV lanes lie VW apart (lane = js * VW + lv): the lanes that read one table row
   // at a time are then contiguous, so table reads stay broadcasts and signal reads contiguous.
@@ -1323,7 +1328,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
               float2 u = make_float2(0.f, 0.f), r = make_float2(0.f, 0.f);
               if (act && 2 * pi < cnt)
                 step2<K, true, LOSS, true>(DP, tab2[pi], yc2[pi * VW], make_float2(1.f, (2 * pi + 1 < cnt) ? 1.f : 0.f),
-                                           AP, inv_s2, B2, &u, &r);
+                                           AP, inv_s2, s_bess, B2, &u, &r);
               uu[2 * h] = u.x;
               uu[2 * h + 1] = u.y;
               rv[2 * h] = r.x;
@@ -1352,7 +1357,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
               float2 u = make_float2(0.f, 0.f), r = make_float2(0.f, 0.f);
               if (act && 2 * pi < cnt)
                 step2<K, true, LOSS, true>(DP, tab2[pi], yc2[pi * VW], make_float2(1.f, (2 * pi + 1 < cnt) ? 1.f : 0.f),
-                                           AP, inv_s2, B2, &u, &r);
+                                           AP, inv_s2, s_bess, B2, &u, &r);
               uu[2 * h] = u.x;
               uu[2 * h + 1] = u.y;
               rv[2 * h] = r.x;
@@ -1373,21 +1378,21 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
 #pragma unroll (K >= 5 ? 1 : 2)
           for (int i = 0; i < kChunk / 2 / TPV; ++i) {
             const int pi = (TPV == 1) ? i : i * TPV + js;
-            step2<K, false, LOSS>(DP, tab2[pi], yc2[pi * VW], make_float2(1.f, 1.f), AP, inv_s2);
+            step2<K, false, LOSS>(DP, tab2[pi], yc2[pi * VW], make_float2(1.f, 1.f), AP, inv_s2, s_bess);
           }
         } else if (act && TPV == 1) {
           if (i0 > 0) step2_b0<K>(DP, yc2, VW, i0, AP);
 #pragma unroll 1
           for (int i = i0; i < (cnt + 1) / 2; ++i)
             step2<K, true, LOSS>(DP, tab2[i], yc2[i * VW], make_float2(1.f, (2 * i + 1 < cnt) ? 1.f : 0.f), AP,
-                                 inv_s2);
+                                 inv_s2, s_bess);
         } else if (act) {
           if (i0 > js) step2_b0<K>(DP, yc2 + js * VW, TPV * VW, (i0 - js + TPV - 1) / TPV, AP);
           const int first = i0 + ((js - i0) % TPV + TPV) % TPV;   // this lane's first pair >= i0
 #pragma unroll 1
           for (int pi = first; pi < (cnt + 1) / 2; pi += TPV)
             step2<K, true, LOSS>(DP, tab2[pi], yc2[pi * VW], make_float2(1.f, (2 * pi + 1 < cnt) ? 1.f : 0.f), AP,
-                                 inv_s2);
+                                 inv_s2, s_bess);
         }
         __syncwarp();
         ++g;
@@ -1402,7 +1407,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         for (int i = 0; i < kChunk / TPV; ++i) {
           const int nl = i * TPV + js;
           float rr, u;
-          pair<K, LOSS, CAL, false>(P, ffin, fomf, tab[nl], yc[(nl >> 1) * (2 * VW) + (nl & 1)], B, inv_s2, 0.f, A, rr, u);
+          pair<K, LOSS, CAL, false>(P, ffin, fomf, tab[nl], yc[(nl >> 1) * (2 * VW) + (nl & 1)], B, inv_s2, 0.f, A, rr, u, s_bess);
         }
       } else if (CAL && TPV == 1) {
         // per-measurement alpha / beta partials summed over the warp's 32 voxels, kCalG
@@ -1416,7 +1421,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
             const int nl = i0 + gq;
             const bool ok = act && (nl < cnt);
             float rr = 0.f, u = 0.f;
-            if (ok) pair<K, LOSS, CAL, false>(P, ffin, fomf, tab[nl], yc[(nl >> 1) * (2 * VW) + (nl & 1)], B, inv_s2, 0.f, A, rr, u);
+            if (ok) pair<K, LOSS, CAL, false>(P, ffin, fomf, tab[nl], yc[(nl >> 1) * (2 * VW) + (nl & 1)], B, inv_s2, 0.f, A, rr, u, s_bess);
             uu[gq] = ok ? u : 0.f;
             rv[gq] = ok ? rr : 0.f;
           }
@@ -1434,7 +1439,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
           const int nl = i * TPV + js;
           const bool ok = act && (nl < cnt);
           float rr = 0.f, u = 0.f;
-          if (ok) pair<K, LOSS, CAL, false>(P, ffin, fomf, tab[nl], yc[(nl >> 1) * (2 * VW) + (nl & 1)], B, inv_s2, 0.f, A, rr, u);
+          if (ok) pair<K, LOSS, CAL, false>(P, ffin, fomf, tab[nl], yc[(nl >> 1) * (2 * VW) + (nl & 1)], B, inv_s2, 0.f, A, rr, u, s_bess);
           if (CAL) {
             // over the warp's voxels: the VW lanes of one js are contiguous
             float su = warp_sum_range<1, VW / 2>(ok ? u : 0.f);
@@ -1850,8 +1855,13 @@ __global__ void __launch_bounds__(256) k_yhat(const IterArgs a, const int32_t* _
 template <int LOSS>
 __global__ void __launch_bounds__(256) k_loss(const IterArgs a, const PlainArgs pa) {
   __shared__ double s_red[8][3];
+  __shared__ float4 s_bess[(LOSS == kLossNLL) ? kBesselTab : 1];
   const int t = pa.tile_begin + blockIdx.x;
   if (t >= pa.tile_end) return;
+  if constexpr (LOSS == kLossNLL) {
+    bessel_stage(s_bess);
+    __syncthreads();
+  }
   const Tile tl = a.tiles[t];
   const GroupDev gr = a.groups[tl.group];
   const int N = tl.n_meas;
@@ -1872,13 +1882,13 @@ __global__ void __launch_bounds__(256) k_loss(const IterArgs a, const PlainArgs 
       rr = yh - yv;
       l += static_cast<double>(rr * rr) * gr.inv_M;
     } else {
-      const float ay = fabsf(yh);
-      const float sy = (yh >= 0.f) ? yv : -yv;
+      const float ay = fabsf(yh), yy = fabsf(yv);
+      const float sy = (yh >= 0.f) ? yy : -yy;
       float Qz, Lz;
-      bessel_QL<true>(yv * ay * inv_s2, Qz, Lz);
-      const float d = yv - ay;
+      bessel_QL(yy * ay * inv_s2, s_bess, Qz, Lz);
+      const float d = yy - ay;
       l += static_cast<double>(2.f * slog + 0.5f * inv_s2 * d * d - Lz);
-      sg += static_cast<double>(2.f - inv_s2 * (d * d + 2.f * yv * ay * Qz));
+      sg += static_cast<double>(2.f - inv_s2 * (d * d + 2.f * yy * ay * Qz));
       rr = fmaf(sy, Qz, yh - sy);
     }
     pa.r[ix] = rr * scale;

@@ -62,6 +62,8 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
   __shared__ uint64_t s_bar;
   __shared__ float s_ac[2 * kMaxIters];
   __shared__ int s_last;
+  __shared__ float4 s_bess[(LOSS == kLossNLL) ? kBesselTab : 1];
+  if constexpr (LOSS == kLossNLL) bessel_stage(s_bess);   // visible after the first tile's barriers
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int lv = lane % VW, js = lane / VW, vl = warp * VW + lv;
   const int Vp = a.Vpad, step = *a.step, n_it = a.n_it;
@@ -137,10 +139,10 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
 #pragma unroll (K >= 4 || LOSS == kLossNLL ? 1 : 2)
         for (; p < N / 2; p += TPV)
           step2<K, false, LOSS>(DP, reinterpret_cast<const MeasPair&>(s_tab[p * kLocalRow]), yc2[p * VW],
-                                make_float2(1.f, 1.f), AP, inv_s2);
+                                make_float2(1.f, 1.f), AP, inv_s2, s_bess);
         if (p < (N + 1) / 2)   // the last measurement of an odd count
           step2<K, true, LOSS>(DP, reinterpret_cast<const MeasPair&>(s_tab[p * kLocalRow]), yc2[p * VW],
-                               make_float2(1.f, 0.f), AP, inv_s2);
+                               make_float2(1.f, 0.f), AP, inv_s2, s_bess);
         accp_sums<K, LOSS, false>(AP, A);
       }
       acc_reduce_tpv<K, TPV, VW>(A);

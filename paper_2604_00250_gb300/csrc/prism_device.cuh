@@ -52,7 +52,8 @@ constexpr int kPairFieldA = 11, kPairFieldBeta = 12;
 // with rho = 1 - D_perp / D_par and C0 = log2(1 - f_in) - rho log2 f_in per voxel, and
 //   dE_wm/dd = -2 ln(2) c' (f_in e1 + rho (1 - f_in) p) g'.
 struct __align__(16) ShellRun {
-  int32_t p0, p1, b0, pad;         // pairs [p0, p1); b0 = 1 for b = 0 (every E of Eqs. 4-5 is 1)
+  int32_t p0, p1, b0, odd;         // pairs [p0, p1); b0 = 1 for b = 0 (every E of Eqs. 4-5 is 1); odd = 1:
+                                   // the last pair's second measurement is padding
   float ecsf, egm, eres, nbperp;   // E_csf, E_gm, E_res; -b D_perp log2(e)
 };
 constexpr int kMaxRuns = 16;        // shells per group the shell loop takes

@@ -773,7 +773,8 @@ struct ShellRows {
   static_assert(gres < count, "the column holds every row");
 };
 
-template <int K>
+// MASK: the second measurement of the pair is padding (the last pair of a shell of odd length).
+template <int K, bool MASK = false>
 __device__ __forceinline__ void shell_step(ShellState<K>& S, float2 gx, float2 gy, float2 gz, float2 y) {
   const float2 nrho = make_float2(-kRho, -kRho), rho = make_float2(kRho, kRho);
   float2 cp[K], e1[K], pp[K], t[K];
@@ -788,6 +789,7 @@ __device__ __forceinline__ void shell_step(ShellState<K>& S, float2 gx, float2 g
   float2 r = __fadd2_rn(y, S.c0);   // y - y_hat
 #pragma unroll
   for (int k = 0; k < K; ++k) r = __ffma2_rn(S.nf[k], t[k], r);
+  if (MASK) r.y = 0.f;
   S.l1 = __ffma2_rn(r, r, S.l1);
   S.Qs = __fadd2_rn(S.Qs, r);
 #pragma unroll

@@ -114,9 +114,10 @@ typedef struct prism_options {
                              loop or the per-measurement loop; above about 311k voxels on a bounded
                              sample of each volume's fullest patches */
   int32_t seed;           /* seed of the default initialisation (init == NULL) */
-  int32_t shells;         /* fused kernel, one thread per voxel, MSE, no calibration, K <= 3: 0 = take
-                             the shell loop (per b-value shell work done once; needs every shell of
-                             every volume to hold an even number of measurements), -1 = never */
+  int32_t shells;         /* fused kernel, one thread per voxel, MSE, no calibration: 0 = take the shell
+                             loop (per b-value shell work done once; at most 16 shells in every
+                             volume, each of an even number of measurements below 32,768 voxels),
+                             -1 = never */
   int32_t reserved[3];
 } prism_options;
 

@@ -100,6 +100,12 @@ struct prism_handle {
   uint32_t *d_vcoord = nullptr, *d_vflag = nullptr;
   int64_t* d_row_off = nullptr;
   int32_t* d_order = nullptr;          // [tab_rows] table position -> caller's measurement index
+  // the packed signal's positions: the table order, with the odd shells of a shell-loop handle padded
+  // to even ones (-1)
+  std::vector<int32_t> pack_order;
+  std::vector<int64_t> pack_off;       // [G] first position of a group
+  std::vector<int32_t> n_pos;          // [G]
+  int32_t* d_pack_order = nullptr;
   // slab fits (prism_fit_init_slabs): per voxel of the whole volume, its source voxel(s) in
   // the handle and the weight of the second source
   bool slabbed = false;
@@ -112,8 +118,7 @@ struct prism_handle {
   // shell loop: per-group gradient rows and shells (host copies built by the plan)
   std::vector<float> gtab;
   std::vector<ShellRun> runs;
-  bool shells_even = true;             // every group's shells hold an even number of measurements
-  bool shell = false;                  // the fused kernel takes the shell loop
+  int shell = 0;                       // the fused kernel takes the shell loop (2: with padded odd shells)
   bool local = false;                  // iterations run in k_iter_local, many per launch
   int local_grid = 0;
   size_t local_smem = 0;
@@ -366,7 +371,7 @@ int enqueue_fused_iter(prism_handle* h, cudaStream_t st) {
   const IterArgs& a = h->ia;
   if (h->opt.lam_sp > 0.f) CK(h->ks->prior_prep(a, 0, h->ntiles, st));
   if (h->nb) CK(h->ks->prior_grad(a, 0, h->ntiles, st));
-  CK(h->ks->fused(a, h->opt.loss, h->cal ? 1 : 0, h->TPV, h->shell ? 1 : 0, 0, h->fused_grid, h->NT, h->fused_smem,
+  CK(h->ks->fused(a, h->opt.loss, h->cal ? 1 : 0, h->TPV, h->shell, 0, h->fused_grid, h->NT, h->fused_smem,
                   st));
   if (h->cal) {   // without calibration the fused kernel's last CTA finalises the groups
     CK(launch_group_sums(a, h->ga, 1 | 2, true, st));
@@ -455,21 +460,20 @@ static int32_t meas_order(const prism_volume& v, bool cal, std::vector<int32_t>&
 // host-side constants.
 constexpr double kDpar = 1.7e-3, kDperp = 0.4e-3, kLog2e = 1.4426950408889634;
 
-// Shells of one group in table order (runs of equal b-value) with the constants of the
-// shell loop (ShellRun); false when a shell holds an odd number of measurements (a pair would
-// straddle two shells) or there are more than kMaxRuns shells.
-static bool shell_runs(const prism_volume& v, const int32_t* ord, std::vector<ShellRun>& runs) {
+// Shells of one group in table order `ord` (runs of equal b-value) with the constants of the shell
+// loop (ShellRun), each padded to an even count; `pos` receives the positions (-1: padding).
+static void shell_runs(const prism_volume& v, const int32_t* ord, std::vector<ShellRun>& runs,
+                       std::vector<int32_t>& pos) {
   const int N = v.n_meas;
-  bool ok = true;
-  int n0 = 0, nr = 0;
-  while (n0 < N) {
-    const float b = v.bvals[ord[n0]];
-    int n1 = n0 + 1;
-    while (n1 < N && v.bvals[ord[n1]] == b) ++n1;
-    if ((n1 - n0) % 2 != 0) ok = false;
+  const size_t base = pos.size();
+  for (int n = 0; n < N;) {
+    const float b = v.bvals[ord[n]];
     ShellRun r{};
-    r.p0 = n0 / 2;
-    r.p1 = n1 / 2;
+    r.p0 = static_cast<int32_t>((pos.size() - base) / 2);
+    for (; n < N && v.bvals[ord[n]] == b; ++n) pos.push_back(ord[n]);
+    r.odd = static_cast<int32_t>((pos.size() - base) % 2);
+    if (r.odd) pos.push_back(-1);
+    r.p1 = static_cast<int32_t>((pos.size() - base) / 2);
     r.b0 = (b == 0.f) ? 1 : 0;
     const double bd = b;
     r.ecsf = static_cast<float>(std::exp(-bd * 3.0e-3));   // Eq. 4
@@ -477,10 +481,7 @@ static bool shell_runs(const prism_volume& v, const int32_t* ord, std::vector<Sh
     r.eres = static_cast<float>(std::exp(-bd * 0.2e-3));
     r.nbperp = static_cast<float>(-bd * kDperp * kLog2e);
     runs.push_back(r);
-    ++nr;
-    n0 = n1;
   }
-  return ok && nr <= kMaxRuns;
 }
 
 // Runs fn(begin, end) over [0, n) split into contiguous chunks on the process's host worker
@@ -605,27 +606,34 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, Plan& pl) 
     gr.calib = h->cal ? 1 : 0;
     gr.table_off = static_cast<int32_t>(tab);
     gr.nb0p = meas_order(v, h->cal, h->order);
-    {
-      // shells and gradient rows of the group's table order (shell loop)
-      const int32_t* ord = h->order.data() + tab;
+    const int32_t* ord = h->order.data() + tab;
+    h->pack_off.push_back(static_cast<int64_t>(h->pack_order.size()));
+    if (h->shell) {
+      // shells and gradient rows of the group's positions (shell loop)
       gr.run_off = static_cast<int32_t>(h->runs.size());
-      if (!shell_runs(v, ord, h->runs)) h->shells_even = false;
+      shell_runs(v, ord, h->runs, h->pack_order);
       gr.n_runs = static_cast<int32_t>(h->runs.size()) - gr.run_off;
-      const int NPg = (v.n_meas + 3) & ~3;
+      const int32_t* pos = h->pack_order.data() + h->pack_off[g];
+      const int np = static_cast<int>(h->pack_order.size() - h->pack_off[g]), NPg = (np + 3) & ~3;
       gr.gtab_off = static_cast<int32_t>(h->gtab.size());
       h->gtab.resize(h->gtab.size() + 3 * static_cast<size_t>(NPg), 0.f);
       float* gt = h->gtab.data() + gr.gtab_off;
       // the scaled directions g' = s g, s = sqrt(b D_par log2 e) (Eq. 5: c' = s c = g' . d), per
-      // pair p: {g'_x(2p), g'_x(2p+1), g'_y(2p), g'_y(2p+1)} at 4p, then g'_z of every measurement
+      // pair p: {g'_x(2p), g'_x(2p+1), g'_y(2p), g'_y(2p+1)} at 4p, then g'_z of every position
       // from 2 NP on (one 16-byte and one 8-byte shared-memory load per pair)
-      for (int n = 0; n < v.n_meas; ++n) {
-        const int p = n / 2, h = n % 2;
-        const double s = std::sqrt(static_cast<double>(v.bvals[ord[n]]) * kDpar * kLog2e);
-        gt[4 * p + h] = static_cast<float>(s * v.bvecs[3 * ord[n]]);
-        gt[4 * p + 2 + h] = static_cast<float>(s * v.bvecs[3 * ord[n] + 1]);
-        gt[2 * NPg + n] = static_cast<float>(s * v.bvecs[3 * ord[n] + 2]);
+      for (int i = 0; i < np; ++i) {
+        const int n = pos[i], p = i / 2, h2 = i % 2;
+        if (n < 0) continue;
+        const double s = std::sqrt(static_cast<double>(v.bvals[n]) * kDpar * kLog2e);
+        gt[4 * p + h2] = static_cast<float>(s * v.bvecs[3 * n]);
+        gt[4 * p + 2 + h2] = static_cast<float>(s * v.bvecs[3 * n + 1]);
+        gt[2 * NPg + i] = static_cast<float>(s * v.bvecs[3 * n + 2]);
       }
+    } else {
+      h->pack_order.insert(h->pack_order.end(), ord, ord + v.n_meas);
     }
+    const int npos = static_cast<int>(h->pack_order.size() - h->pack_off[g]);
+    h->n_pos.push_back(npos);
     tab += v.n_meas;
     gr.table2_off = static_cast<int32_t>(h->tab2_pairs);
     h->tab2_pairs += ((v.n_meas + 3) & ~3) / 2;
@@ -637,7 +645,7 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, Plan& pl) 
     gp += 4 + 2 * gr.N4 + kNGrid;
     h->yhat_off[g] = yh;
     yh += static_cast<int64_t>(gr.n_vox) * v.n_meas;
-    Nmax = std::max(Nmax, v.n_meas);
+    Nmax = std::max(Nmax, npos);
     gr.tile0 = static_cast<int32_t>(h->tiles.size());
     const int px = (v.nx + P - 1) / P, py = (v.ny + P - 1) / P, pz = (v.nz + P - 1) / P;
     const int64_t npatch = static_cast<int64_t>(px) * py * pz;
@@ -675,8 +683,8 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, Plan& pl) 
         t.count = std::min(TV, pcount[pi] - s0);
         t.y_off = yoff;
         t.ab_off = static_cast<int32_t>(aboff);
-        t.n_meas = v.n_meas;
-        yoff += static_cast<int64_t>((v.n_meas + 3) & ~3) * TV;
+        t.n_meas = npos;
+        yoff += static_cast<int64_t>((npos + 3) & ~3) * TV;
         aboff += 2 * v.n_meas;
         h->tiles.push_back(t);
       }
@@ -737,6 +745,32 @@ int upload(T* dst, const std::vector<T, A>& src, cudaStream_t st) {
     if (r_ != PRISM_OK) return r_; \
   } while (0)
 
+// The form of the shell loop that the fused kernel would take with one thread per voxel, 0 for none:
+// MSE without calibration, shells not switched off, and in every volume at most kMaxRuns b-value
+// shells (runs of equal b in sorted order). Shells of even length throughout: 1. With odd ones, padded:
+// 2, from kPadVoxels voxels on, where one thread per voxel is the automatic shape (four 56 x 61 x 47 and
+// smaller ellipsoids at N = 271, shells of 86, K = 3: fused kernel 152 -> 129 us; 48^3 at N = 271 with four
+// fibers 196 -> 119 us an iteration; below, a forced one-lane fit is bound by latency, not by its operations).
+constexpr int64_t kPadVoxels = 32768;
+int shells_apply(const prism_volume* vols, int n, const prism_options& o, int64_t V) {
+  if (!o.fused || o.loss != PRISM_LOSS_MSE || o.calibration || o.shells != 0) return 0;
+  bool even = true;
+  for (int g = 0; g < n; ++g) {
+    std::vector<float> b(vols[g].bvals, vols[g].bvals + vols[g].n_meas);
+    std::sort(b.begin(), b.end());
+    int runs = 0;
+    for (size_t i = 0; i < b.size();) {
+      size_t j = i + 1;
+      while (j < b.size() && b[j] == b[i]) ++j;
+      if ((j - i) % 2 != 0) even = false;
+      ++runs;
+      i = j;
+    }
+    if (runs > kMaxRuns) return 0;
+  }
+  return even ? 1 : (V >= kPadVoxels ? 2 : 0);
+}
+
 // `rows`: per volume, the row of each voxel in vols[g].signal and vols[g].init (device memory; the
 // slabs of one whole-volume signal), or nullptr where the rows are in mask order.
 int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::vector<int64_t>& counts,
@@ -749,6 +783,9 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   h->nb = (o.lam_sp > 0.f) || (o.lam_dir > 0.f);
   h->ks = &kernels_for_k(o.K);
   h->TV = h->NT / h->TPV;
+  int64_t Vsum = 0;
+  for (int64_t c : counts) Vsum += c;
+  h->shell = (h->TPV == 1) ? shells_apply(vols, n_vols, o, Vsum) : 0;
   int dev = 0, sms = 0;
   if (o.fused) {
     CK(cudaGetDevice(&dev));
@@ -840,6 +877,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   RC(h->alloc(&h->d_slot_of_grid, pl.slot_of_grid.size()));
   RC(h->alloc(&h->d_row_off, h->V));
   RC(h->alloc(&h->d_order, std::max<int64_t>(h->tab_rows, 1)));
+  RC(h->alloc(&h->d_pack_order, h->pack_order.size()));
   RC(h->alloc(&h->d_split_off, G));
   RC(h->alloc(&h->d_part2, static_cast<size_t>(tot_split) * h->max_e));
   RC(h->alloc(&h->d_counters, static_cast<size_t>(G) * nce));
@@ -900,6 +938,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
                       Vp, h->TV, h->opt.connectivity, h->d_vox_of_slot, h->d_vcoord, h->d_vflag, h->d_nbr, st));
   RC(upload(h->d_row_off, pl.row_off, st));
   RC(upload(h->d_order, h->order, st));
+  RC(upload(h->d_pack_order, h->pack_order, st));
   RC(upload(h->d_gtab, h->gtab, st));
   RC(upload(h->d_runs, h->runs, st));
   RC(upload(h->d_split_off, split_off, st));
@@ -947,8 +986,8 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
     RC(upload(d_bvec, bvec, st));
     CK(launch_b0_stats(sig, vrows, Vg, N, d_b0n, nb0, d_b0, d_part, d_bad, st));
     CK(launch_sigma_init(d_part, nbk, Vg, nb0, o.sigma_init, h->d_gparams + gr.gp_off, st));
-    CK(launch_pack(h->ia, sig, vrows, d_b0, h->d_vox_of_slot, h->d_order + gr.table_off, h->vox0[g], gr.tile0,
-                   gr.tile0 + gr.ntiles, N, h->d_y, d_bad, st));
+    CK(launch_pack(h->ia, sig, vrows, d_b0, h->d_vox_of_slot, h->d_pack_order + h->pack_off[g], h->vox0[g], gr.tile0,
+                   gr.tile0 + gr.ntiles, N, h->n_pos[g], h->d_y, d_bad, st));
     CK(launch_table(d_bv, d_bvec, N, h->d_table + gr.table_off, st));
     CK(launch_pair_table(h->d_table + gr.table_off, N, h->d_table2 + gr.table2_off, st));
     if (v.init) {
@@ -983,8 +1022,6 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   CK(launch_adam_constants(h->ia, st));
   // launch geometry of the fused kernel
   const int NW = h->NT / 32;
-  h->shell = o.fused && !h->cal && o.loss == PRISM_LOSS_MSE && h->TPV == 1 && o.K <= 3 && h->shells_even &&
-             o.shells == 0;
   const size_t ring = static_cast<size_t>(kStages) * kChunk * (kFusedThreads / h->TPV) * sizeof(float);
   if (h->shell) {
     h->fused_smem = 3 * static_cast<size_t>(h->Nmax) * sizeof(float) + kMaxRuns * sizeof(ShellRun) +
@@ -996,7 +1033,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   h->adj_smem = h->cal ? static_cast<size_t>(NW) * 2 * h->Nmax * sizeof(float) : 0;
   if (o.fused) {
     int bps = 0;
-    CK(h->ks->fused_occupancy(o.loss, h->cal ? 1 : 0, h->TPV, h->shell ? 1 : 0, h->NT, h->fused_smem, &bps));
+    CK(h->ks->fused_occupancy(o.loss, h->cal ? 1 : 0, h->TPV, h->shell, h->NT, h->fused_smem, &bps));
     if (bps < 1) return fail(PRISM_E_CUDA, "fused kernel does not fit on an SM");
     h->fused_grid = std::max(1, std::min(h->ntiles, sms * bps));
   }
@@ -1035,27 +1072,6 @@ int choose_shape(const prism_options& o, int64_t V, bool shell, int* tpv, int* n
   // the fused kernel is compiled for 128-thread CTAs (4 resident per SM)
   *nt = o.fused ? 128 : (o.cta_threads ? o.cta_threads : 128);
   return PRISM_OK;
-}
-
-// Whether the fused kernel would take the shell loop with one thread per voxel: MSE without
-// calibration, K <= 3, shells not switched off, and every volume's b-value shells (runs of
-// equal b in sorted order) of even length and at most kMaxRuns of them.
-bool shells_apply(const prism_volume* vols, int n, const prism_options& o) {
-  if (!o.fused || o.loss != PRISM_LOSS_MSE || o.calibration || o.K > 3 || o.shells != 0) return false;
-  for (int g = 0; g < n; ++g) {
-    std::vector<float> b(vols[g].bvals, vols[g].bvals + vols[g].n_meas);
-    std::sort(b.begin(), b.end());
-    int runs = 0;
-    for (size_t i = 0; i < b.size();) {
-      size_t j = i + 1;
-      while (j < b.size() && b[j] == b[i]) ++j;
-      if ((j - i) % 2 != 0) return false;
-      ++runs;
-      i = j;
-    }
-    if (runs > kMaxRuns) return false;
-  }
-  return true;
 }
 
 // Masked voxels of each volume.
@@ -1282,7 +1298,7 @@ int fit_init(const prism_volume* vols, int n_vols, const prism_options* opt, con
   int64_t V = 0;
   for (int64_t c : counts) V += c;
   int tpv = 1, nt = 128;
-  choose_shape(o, V, shells_apply(vols, n_vols, o), &tpv, &nt);
+  choose_shape(o, V, shells_apply(vols, n_vols, o, V) != 0, &tpv, &nt);
   if (o.autotune && o.fused && !rows) {
     int shells = o.shells;
     autotune_shape(vols, n_vols, counts, o, st, &tpv, &shells);
@@ -1358,7 +1374,7 @@ extern "C" int prism_get_shape(const prism_handle* h, int32_t* threads_per_voxel
   if (threads_per_voxel) *threads_per_voxel = h->TPV;
   if (tile_voxels) *tile_voxels = h->TV;
   if (fused_grid) *fused_grid = h->opt.fused ? h->fused_grid : 0;
-  if (shell_loop) *shell_loop = h->shell ? 1 : 0;
+  if (shell_loop) *shell_loop = h->shell ? 1 : 0;   // either form
   return PRISM_OK;
 }
 
@@ -1501,7 +1517,7 @@ extern "C" int prism_forward(prism_handle* h, const float* theta, const float* g
     // exponentials twice: forward and backward of a 582,000-voxel brain 2.25 ms, now 0.54 ms.)
     if (h->opt.lam_sp > 0.f) CK(h->ks->prior_prep(a, 0, h->ntiles, st));
     if (h->nb) CK(h->ks->prior_grad(a, 0, h->ntiles, st));
-    CK(h->ks->fused(a, h->opt.loss, cal, h->TPV, h->shell ? 1 : 0, 1, h->fused_grid, h->NT, h->fused_smem, st));
+    CK(h->ks->fused(a, h->opt.loss, cal, h->TPV, h->shell, 1, h->fused_grid, h->NT, h->fused_smem, st));
     if (h->cal) {
       CK(launch_group_sums(a, h->ga, 1 | 2, true, st));
       CK(launch_group_adam(a, h->ga, 1, st));
@@ -1556,7 +1572,7 @@ extern "C" int prism_profile(prism_handle* h, int32_t n_iters, void* stream, flo
     if (e == cudaSuccess && h->nb) e = h->ks->prior_grad(a, 0, h->ntiles, st);
     if (e == cudaSuccess) e = cudaEventRecord(ev[1], st);
     if (e == cudaSuccess)
-      e = h->ks->fused(a, h->opt.loss, h->cal ? 1 : 0, h->TPV, h->shell ? 1 : 0, 0, h->fused_grid, h->NT,
+      e = h->ks->fused(a, h->opt.loss, h->cal ? 1 : 0, h->TPV, h->shell, 0, h->fused_grid, h->NT,
                        h->fused_smem, st);
     if (e == cudaSuccess) e = cudaEventRecord(ev[2], st);
     if (e == cudaSuccess && h->cal) e = launch_group_sums(a, h->ga, 1 | 2, true, st);

@@ -95,14 +95,14 @@ __global__ void __launch_bounds__(kPackThreads) k_pack(const IterArgs a, const f
                                                        const float* __restrict__ b0mean,
                                                        const int32_t* __restrict__ vox_of_slot,
                                                        const int32_t* __restrict__ order, int64_t vox0, int tile_begin,
-                                                       int N, float* __restrict__ ypack, int* bad) {
+                                                       int N, int npos, float* __restrict__ ypack, int* bad) {
   __shared__ float s[VW][kPackC + 1];
   __shared__ int64_t s_row[VW];   // the voxel's signal row (-1: padding slot)
   __shared__ float s_inv[VW];     // 1 / its b0 mean (-1 where that was refused)
   __shared__ int s_bad[VW];
   const int t = tile_begin + blockIdx.x, w = blockIdx.y;
   const Tile tl = a.tiles[t];
-  const int NP = (N + 3) & ~3;
+  const int NP = (npos + 3) & ~3;   // positions: order[] holds the measurement of each, -1 for padding
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x < VW) {
     const int vl = w * VW + threadIdx.x;
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kPackThreads) k_pack(const IterArgs a, const f
 #pragma unroll
     for (int q = 0; q < kPackC / 32; ++q) {
       const int n = n0 + lane + 32 * q;
-      on[q] = (n < N) ? order[n] : -1;
+      on[q] = (n < npos) ? order[n] : -1;
     }
     // a warp per voxel row, its loads and those of the next rows in flight together
 #pragma unroll
@@ -759,14 +759,14 @@ cudaError_t launch_sigma_init(const double* part, int nblocks, int64_t V, int nb
 }
 cudaError_t launch_pack(const IterArgs& a, const float* sig, const int64_t* rows, const float* b0mean,
                         const int32_t* vox_of_slot, const int32_t* order, int64_t vox0, int tile_begin, int tile_end,
-                        int N, float* ypack, int* bad, cudaStream_t st) {
+                        int N, int npos, float* ypack, int* bad, cudaStream_t st) {
   if (tile_end <= tile_begin) return cudaSuccess;
   if (a.TV % a.VW != 0) return cudaErrorInvalidValue;
   const dim3 nb(tile_end - tile_begin, a.TV / a.VW);
   switch (a.VW) {
-    case 32: k_pack<32><<<nb, kPackThreads, 0, st>>>(a, sig, rows, b0mean, vox_of_slot, order, vox0, tile_begin, N, ypack, bad); break;
-    case 8: k_pack<8><<<nb, kPackThreads, 0, st>>>(a, sig, rows, b0mean, vox_of_slot, order, vox0, tile_begin, N, ypack, bad); break;
-    case 2: k_pack<2><<<nb, kPackThreads, 0, st>>>(a, sig, rows, b0mean, vox_of_slot, order, vox0, tile_begin, N, ypack, bad); break;
+    case 32: k_pack<32><<<nb, kPackThreads, 0, st>>>(a, sig, rows, b0mean, vox_of_slot, order, vox0, tile_begin, N, npos, ypack, bad); break;
+    case 8: k_pack<8><<<nb, kPackThreads, 0, st>>>(a, sig, rows, b0mean, vox_of_slot, order, vox0, tile_begin, N, npos, ypack, bad); break;
+    case 2: k_pack<2><<<nb, kPackThreads, 0, st>>>(a, sig, rows, b0mean, vox_of_slot, order, vox0, tile_begin, N, npos, ypack, bad); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -72,7 +72,7 @@ struct Tile {
   int32_t group, patch, slot0, count;
   int64_t y_off;     // float offset of the packed [N][TV] signal block
   int32_t ab_off;    // float offset of the tile's [2][N] alpha/beta gradient partials
-  int32_t n_meas;
+  int32_t n_meas;    // positions of the packed signal: the measurements, and padding of odd shells (shell loop)
 };
 
 struct GroupDev {

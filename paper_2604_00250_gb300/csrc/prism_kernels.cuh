@@ -150,7 +150,8 @@ __device__ __forceinline__ void nbr_term(const IterArgs& a, const Vox<K>& P, int
 // The neighbour priors of Sec. 2.4 at one voxel: the Huber-Laplacian (from the precomputed
 // rho'(u)/|N| of the voxel and its neighbours) and directional continuity (from the neighbours'
 // directions; only P.d is read). Returns the value; adds the gradient to gf / gd.
-template <int K>
+// NB: 6 or 26 neighbours, 0: a.n_nbr (a kernel for each: the registers of one cost the other 8 %).
+template <int K, int NB = 0>
 __device__ __forceinline__ float nbr_priors(const IterArgs& a, const Vox<K>& P, int slot, float inv_M,
                                             const float* __restrict__ xf_cur, float (&gf)[K + 3],
                                             float (&gd)[K][3]) {
@@ -167,7 +168,7 @@ __device__ __forceinline__ float nbr_priors(const IterArgs& a, const Vox<K>& P, 
 #pragma unroll
       for (int c = 0; c < NF; ++c) hs[c] = a.hsp[static_cast<size_t>(c) * Vp + slot] * static_cast<float>(ncnt);
     }
-    if (a.n_nbr == 6) {
+    if (NB == 6 || (NB == 0 && a.n_nbr == 6)) {
       // face neighbours: every index first, then every neighbour's data (a missing
       // neighbour reads the voxel's own row with weight 0), so that the gathers overlap
       int xs[6];
@@ -176,8 +177,16 @@ __device__ __forceinline__ float nbr_priors(const IterArgs& a, const Vox<K>& P, 
 #pragma unroll
       for (int e = 0; e < 6; ++e) nbr_term<K>(a, P, xs[e], slot, inv_n, wdir, xf_cur, hs, val, gd);
     } else {
-      for (int e = 0; e < a.n_nbr; ++e)
-        nbr_term<K>(a, P, a.nbr[static_cast<size_t>(e) * Vp + slot], slot, inv_n, wdir, xf_cur, hs, val, gd);
+      // the same in two halves of the 26 (one index at a time, each neighbour waited for its own index
+      // and its gathers: 63 us for 193,000 voxels, 34 us so)
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        int xs[13];
+#pragma unroll
+        for (int e = 0; e < 13; ++e) xs[e] = a.nbr[static_cast<size_t>(13 * h + e) * Vp + slot];
+#pragma unroll
+        for (int e = 0; e < 13; ++e) nbr_term<K>(a, P, xs[e], slot, inv_n, wdir, xf_cur, hs, val, gd);
+      }
     }
     if (a.lam_sp > 0.f) {
 #pragma unroll
@@ -1061,24 +1070,26 @@ __host__ __device__ constexpr bool fused_packed() {
 // CTAs per SM the fused kernel is compiled for: 4 (128 registers per thread) where the voxel
 // state fits, 3 (170 registers) for five fibers and the packed NLL and calibrated variants,
 // which spill at 128 and measured 7-54 % faster at 3.
-template <int K, int TPV, int LOSS, bool CAL>
+template <int K, int TPV, int LOSS, bool CAL, int SHELL = 0>
 constexpr int fused_min_blocks() {
-  return ((K >= 5) || (fused_packed<K, TPV, LOSS, CAL>() && (CAL || LOSS == kLossNLL))) ? 3 : 4;
+  return ((K >= 5 || (K == 4 && SHELL)) || (fused_packed<K, TPV, LOSS, CAL>() && (CAL || LOSS == kLossNLL))) ? 3 : 4;
 }
 
 // SHELL: the shell loop (see ShellState) instead of the packed pairs; only for one thread per
-// voxel, the MSE, no calibration and K <= 3, with every group's shells of even length.
+// voxel, the MSE and no calibration. 1: every group's shells have even length; 2: odd shells are
+// padded to even ones and their last pair takes its first measurement only (a kernel of its own:
+// the extra step costs the even case registers it needs).
 // GRAD: the gradient form behind prism_forward / prism_backward: the same pass over the signal, its
 // epilogue writes the raw-parameter gradient instead of updating, and no state advances.
-template <int K, int TPV, int LOSS, bool CAL, bool SHELL = false, bool GRAD = false>
-__global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS, CAL>())) k_iter_fused(const IterArgs a) {
+template <int K, int TPV, int LOSS, bool CAL, int SHELL = 0, bool GRAD = false>
+__global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS, CAL, SHELL>())) k_iter_fused(const IterArgs a) {
   constexpr int NF = K + 3, Q = 4 * K + 5, XF = 4 * K + 3;
   constexpr int NW = kFusedThreads / 32;
   constexpr int VW = 32 / TPV;              // voxels per warp
   constexpr bool PACKED = fused_packed<K, TPV, LOSS, CAL>();
   constexpr bool HOIST = PACKED && TPV == 1 && K <= 3 && LOSS == kLossMSE && !CAL;
-  static_assert(!SHELL || HOIST, "the shell loop covers one thread per voxel, MSE, no calibration, K <= 3");
-  using SR = ShellRows<(K <= 3 ? K : 3)>;
+  static_assert(!SHELL || (TPV == 1 && LOSS == kLossMSE && !CAL), "the shell loop covers one thread per voxel, MSE, no calibration");
+  using SR = ShellRows<K>;
   // ring stages per warp (kStages; a ring as deep in bytes for four or sixteen lanes per voxel,
   // kStages * TPV, measured 0-25 % slower)
   constexpr int NS = kStages;
@@ -1245,7 +1256,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
     fiber_weights<K>(P, ffin, fomf);
     VoxP<K> DP;
     AccP<K> AP;
-    ShellState<(K <= 3 ? K : 3)> SS;
+    ShellState<K> SS;
     float* col = s_col + tid;
     if constexpr (SHELL) {
       shell_begin(SS, P, col);
@@ -1292,17 +1303,33 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
             if (SS.b0) {
 #pragma unroll 1
               for (; p < pe; ++p) {
-                const float2 r = __fadd2_rn(yc2[(p - pc0) * VW], SS.c0);
+                float2 r = __fadd2_rn(yc2[(p - pc0) * VW], SS.c0);
+                if constexpr (SHELL == 2) {
+                  if (p >= s_runs[SS.ri].p1 - s_runs[SS.ri].odd) r.y = 0.f;
+                }
                 SS.l1 = __ffma2_rn(r, r, SS.l1);
                 SS.Qs = __fadd2_rn(SS.Qs, r);
               }
-            } else {
+            } else if constexpr (SHELL == 1) {
               // three steps in flight (on the brain workload unroll 2 / 4 / 8 measured 0.1-0.3 %
-              // slower, 6 2.5 % slower; no spills in any)
-#pragma unroll 3
+              // slower, 6 2.5 % slower; no spills in any; more than three fibers: one, the state leaves
+              // no registers for more)
+#pragma unroll (K <= 3 ? 3 : 1)
               for (; p < pe; ++p) {
                 const float4 gq = gxy[p];
                 shell_step(SS, make_float2(gq.x, gq.y), make_float2(gq.z, gq.w), gz2[p], yc2[(p - pc0) * VW]);
+              }
+            } else {
+              const int pf = min(pe, s_runs[SS.ri].p1 - s_runs[SS.ri].odd);   // end of the whole pairs
+#pragma unroll (K <= 3 ? 3 : 1)
+              for (; p < pf; ++p) {
+                const float4 gq = gxy[p];
+                shell_step(SS, make_float2(gq.x, gq.y), make_float2(gq.z, gq.w), gz2[p], yc2[(p - pc0) * VW]);
+              }
+              if (p < pe) {
+                const float4 gq = gxy[p];
+                shell_step<K, true>(SS, make_float2(gq.x, gq.y), make_float2(gq.z, gq.w), gz2[p], yc2[(p - pc0) * VW]);
+                ++p;
               }
             }
           }
@@ -1528,7 +1555,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         load_moments<Q>(a, eslot, writer, mq, vq);
       }
       float gq[Q];
-      chain_raw<K, SHELL>(P, gS0, gf, gd, gfin, gq);
+      chain_raw<K, SHELL != 0>(P, gS0, gf, gd, gfin, gq);
       if constexpr (GRAD) {
         if (writer) {
 #pragma unroll
@@ -1820,8 +1847,8 @@ __global__ void __launch_bounds__(256) k_yhat(const IterArgs a, const int32_t* _
   }
   const float2 S0 = dup2(P.S0), fin = dup2(P.fin), omf = dup2(P.omf), B2 = dup2(B);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = static_cast<int>(blockDim.x) >> 5;
-  for (int n0 = 0; n0 < tl.n_meas; n0 += kYhatC) {
-    const int cnt = min(kYhatC, tl.n_meas - n0);
+  for (int n0 = 0; n0 < gr.N; n0 += kYhatC) {   // (the tile's own count may hold padding)
+    const int cnt = min(kYhatC, gr.N - n0);
     const int np = (cnt + 1) / 2;   // the table is zero past N, within its rows rounded up to 4
     for (int e = threadIdx.x; e < 8 * np; e += blockDim.x) s_tab[e >> 3][e & 7] = tab[4 * n0 + e];
     __syncthreads();
@@ -1976,7 +2003,7 @@ __global__ void __launch_bounds__(256) k_adjoint(const IterArgs a, const PlainAr
 }
 
 // Huber-Laplacian preparation: rho'(u_c(x)) / |N(x)| and the prior value per voxel (Eq. 7).
-template <int K>
+template <int K, int NB>
 __global__ void k_prior_prep(const IterArgs a, int tile_begin, int tile_end) {
   constexpr int NF = K + 3, XF = 4 * K + 3;
   // launched as a programmatic dependent of the previous iteration's fused kernel: wait for it
@@ -1998,7 +2025,7 @@ __global__ void k_prior_prep(const IterArgs a, int tile_begin, int tile_end) {
     float sum[NF];
 #pragma unroll
     for (int c = 0; c < NF; ++c) sum[c] = 0.f;
-    if (a.n_nbr == 6) {
+    if constexpr (NB == 6) {
       // every index first, then every neighbour's fractions (a missing neighbour reads the
       // voxel's own row and adds nothing), so that the gathers are in flight together
       int xs[6];
@@ -2015,11 +2042,21 @@ __global__ void k_prior_prep(const IterArgs a, int tile_begin, int tile_end) {
         }
       }
     } else {
-      for (int e = 0; e < a.n_nbr; ++e) {
-        const int x = a.nbr[static_cast<size_t>(e) * Vp + slot];
-        if (x < 0) continue;
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        int xs[13];
 #pragma unroll
-        for (int c = 0; c < NF; ++c) sum[c] += xf[static_cast<size_t>(c) * Vp + x];
+        for (int e = 0; e < 13; ++e) xs[e] = a.nbr[static_cast<size_t>(13 * h + e) * Vp + slot];
+#pragma unroll
+        for (int e = 0; e < 13; ++e) {
+          const bool ok = xs[e] >= 0;
+          const int x = ok ? xs[e] : slot;
+#pragma unroll
+          for (int c = 0; c < NF; ++c) {
+            const float v = xf[static_cast<size_t>(c) * Vp + x];
+            sum[c] += ok ? v : 0.f;
+          }
+        }
       }
     }
     const float inv_n = 1.f / static_cast<float>(ncnt);
@@ -2038,7 +2075,7 @@ __global__ void k_prior_prep(const IterArgs a, int tile_begin, int tile_end) {
 // coalesced load each instead of gathering the neighbourhood there, where the gathers'
 // latency stalls the tile (on the brain workload with one thread per voxel: about 30 us here
 // against 68 us of the fused kernel's epilogue).
-template <int K>
+template <int K, int NB>
 __global__ void k_prior_grad(const IterArgs a, int tile_begin, int tile_end) {
   constexpr int NF = K + 3, XF = 4 * K + 3;
   // as k_prior_prep: wait for the predecessor, then let the fused kernel start launching (its
@@ -2062,7 +2099,7 @@ __global__ void k_prior_grad(const IterArgs a, int tile_begin, int tile_end) {
   for (int c = 0; c < NF; ++c) gf[c] = 0.f;
 #pragma unroll
   for (int k = 0; k < K; ++k) gd[k][0] = gd[k][1] = gd[k][2] = 0.f;
-  const float val = nbr_priors<K>(a, P, slot, gr.inv_M, xf, gf, gd);
+  const float val = nbr_priors<K, NB>(a, P, slot, gr.inv_M, xf, gf, gd);
   float* pg = a.pg + slot;
 #pragma unroll
   for (int c = 0; c < NF; ++c) pg[static_cast<size_t>(c) * Vp] = gf[c];

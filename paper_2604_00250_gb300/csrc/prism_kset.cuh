@@ -13,7 +13,7 @@ namespace {
 
 constexpr int kK = PRISM_K;
 
-template <int TPV, int LOSS, bool CAL, bool SHELL = false, bool GRAD = false>
+template <int TPV, int LOSS, bool CAL, int SHELL = 0, bool GRAD = false>
 cudaError_t fused_one(const IterArgs& a, int grid, int nt, size_t smem, cudaStream_t st) {
   auto fn = k_iter_fused<kK, TPV, LOSS, CAL, SHELL, GRAD>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -27,7 +27,7 @@ cudaError_t fused_one(const IterArgs& a, int grid, int nt, size_t smem, cudaStre
   return launch_dep(fn, dim3(grid), dim3(nt), smem, st, dep, a);
 }
 
-template <int TPV, int LOSS, bool CAL, bool SHELL = false>
+template <int TPV, int LOSS, bool CAL, int SHELL = 0>
 cudaError_t fused_occ(int nt, size_t smem, int* blocks) {
   auto fn = k_iter_fused<kK, TPV, LOSS, CAL, SHELL>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -38,11 +38,11 @@ cudaError_t fused_occ(int nt, size_t smem, int* blocks) {
 template <int TPV, bool GRAD>
 cudaError_t fused_tpv(const IterArgs& a, int loss, int cal, int grid, int nt, size_t smem, cudaStream_t st) {
   if (loss == kLossMSE) {
-    return cal ? fused_one<TPV, kLossMSE, true, false, GRAD>(a, grid, nt, smem, st)
-               : fused_one<TPV, kLossMSE, false, false, GRAD>(a, grid, nt, smem, st);
+    return cal ? fused_one<TPV, kLossMSE, true, 0, GRAD>(a, grid, nt, smem, st)
+               : fused_one<TPV, kLossMSE, false, 0, GRAD>(a, grid, nt, smem, st);
   }
-  return cal ? fused_one<TPV, kLossNLL, true, false, GRAD>(a, grid, nt, smem, st)
-             : fused_one<TPV, kLossNLL, false, false, GRAD>(a, grid, nt, smem, st);
+  return cal ? fused_one<TPV, kLossNLL, true, 0, GRAD>(a, grid, nt, smem, st)
+             : fused_one<TPV, kLossNLL, false, 0, GRAD>(a, grid, nt, smem, st);
 }
 
 template <int TPV>
@@ -56,11 +56,10 @@ cudaError_t occ_tpv(int loss, int cal, int nt, size_t smem, int* blocks) {
 template <bool GRAD>
 cudaError_t fused_any(const IterArgs& a, int loss, int cal, int tpv, int shell, int grid, int nt, size_t smem,
                       cudaStream_t st) {
-  if constexpr (kK <= 3) {
-    if (shell) {
-      if (tpv != 1 || loss != kLossMSE || cal) return cudaErrorInvalidValue;
-      return fused_one<1, kLossMSE, false, true, GRAD>(a, grid, nt, smem, st);
-    }
+  if (shell) {
+    if (tpv != 1 || loss != kLossMSE || cal) return cudaErrorInvalidValue;
+    return shell == 2 ? fused_one<1, kLossMSE, false, 2, GRAD>(a, grid, nt, smem, st)
+                      : fused_one<1, kLossMSE, false, 1, GRAD>(a, grid, nt, smem, st);
   }
   switch (tpv) {
     case 1: return fused_tpv<1, GRAD>(a, loss, cal, grid, nt, smem, st);
@@ -77,11 +76,10 @@ cudaError_t l_fused(const IterArgs& a, int loss, int cal, int tpv, int shell, in
 }
 
 cudaError_t l_fused_occupancy(int loss, int cal, int tpv, int shell, int nt, size_t smem, int* blocks) {
-  if constexpr (kK <= 3) {
-    if (shell) {
-      if (tpv != 1 || loss != kLossMSE || cal) return cudaErrorInvalidValue;
-      return fused_occ<1, kLossMSE, false, true>(nt, smem, blocks);
-    }
+  if (shell) {
+    if (tpv != 1 || loss != kLossMSE || cal) return cudaErrorInvalidValue;
+    return shell == 2 ? fused_occ<1, kLossMSE, false, 2>(nt, smem, blocks)
+                      : fused_occ<1, kLossMSE, false, 1>(nt, smem, blocks);
   }
   switch (tpv) {
     case 1: return occ_tpv<1>(loss, cal, nt, smem, blocks);
@@ -193,13 +191,15 @@ cudaError_t l_adjoint(const IterArgs& a, const PlainArgs& p, int cal, int tpv, i
 cudaError_t l_prior_prep(const IterArgs& a, int tb, int te, cudaStream_t st) {
   const int64_t n = static_cast<int64_t>(te - tb) * a.TV;
   if (n <= 0) return cudaSuccess;
-  return launch_dep(k_prior_prep<kK>, dim3(nblocks(n, 128)), dim3(128), 0, st, a.pdl != 0, a, tb, te);
+  return launch_dep(a.n_nbr == 6 ? k_prior_prep<kK, 6> : k_prior_prep<kK, 26>, dim3(nblocks(n, 128)), dim3(128), 0, st, a.pdl != 0,
+                    a, tb, te);
 }
 
 cudaError_t l_prior_grad(const IterArgs& a, int tb, int te, cudaStream_t st) {
   const int64_t n = static_cast<int64_t>(te - tb) * a.TV;
   if (n <= 0) return cudaSuccess;
-  return launch_dep(k_prior_grad<kK>, dim3(nblocks(n, 128)), dim3(128), 0, st, a.pdl != 0, a, tb, te);
+  return launch_dep(a.n_nbr == 6 ? k_prior_grad<kK, 6> : k_prior_grad<kK, 26>, dim3(nblocks(n, 128)), dim3(128), 0, st, a.pdl != 0,
+                    a, tb, te);
 }
 
 cudaError_t l_prior(const IterArgs& a, const PlainArgs& p, cudaStream_t st) {

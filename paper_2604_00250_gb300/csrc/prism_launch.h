@@ -30,8 +30,8 @@ cudaError_t launch_dep(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cud
 
 // Per-K launchers of the templated kernels (one translation unit per K).
 struct KernelSet {
-  // shell = 1: the shell loop of one thread per voxel, MSE, no calibration (K <= 3); grad = 1: the
-  // gradient form (no update)
+  // shell = 1 or 2: the shell loop of one thread per voxel, MSE, no calibration (2: with padded odd
+  // shells); grad = 1: the gradient form (no update)
   cudaError_t (*fused)(const IterArgs& a, int loss, int cal, int tpv, int shell, int grad, int grid, int nt,
                        size_t smem, cudaStream_t st);
   cudaError_t (*fused_occupancy)(int loss, int cal, int tpv, int shell, int nt, size_t smem, int* blocks);
@@ -98,7 +98,7 @@ cudaError_t launch_sigma_init(const double* part, int nblocks, int64_t V, int nb
                               float* sigma_log_out, cudaStream_t st);
 cudaError_t launch_pack(const IterArgs& a, const float* sig, const int64_t* rows, const float* b0mean,
                         const int32_t* vox_of_slot, const int32_t* order, int64_t vox0, int tile_begin, int tile_end,
-                        int N, float* ypack, int* bad, cudaStream_t st);
+                        int N, int npos, float* ypack, int* bad, cudaStream_t st);
 cudaError_t launch_slot_data(const Tile* tiles, const GroupDev* groups, int G, const GroupDev* host_groups,
                              const int32_t* slot_of_grid, const int32_t* slot_of_vox, int64_t V, int Vp, int TV, int nnb,
                              int32_t* vox_of_slot, uint32_t* vcoord, uint32_t* vflag, int32_t* nbr, cudaStream_t st);

@@ -98,7 +98,6 @@ struct prism_handle {
   int32_t *d_slot_of_vox = nullptr, *d_vox_of_slot = nullptr, *d_slot_of_grid = nullptr;
   int32_t *d_split_off = nullptr, *d_counters = nullptr, *d_gbar = nullptr;
   uint32_t *d_vcoord = nullptr, *d_vflag = nullptr;
-  int64_t* d_row_off = nullptr;
   int32_t* d_order = nullptr;          // [tab_rows] table position -> caller's measurement index
   // the packed signal's positions: the table order, with the odd shells of a shell-loop handle padded
   // to even ones (-1)
@@ -106,11 +105,13 @@ struct prism_handle {
   std::vector<int64_t> pack_off;       // [G] first position of a group
   std::vector<int32_t> n_pos;          // [G]
   int32_t* d_pack_order = nullptr;
-  // slab fits (prism_fit_init_slabs): per voxel of the whole volume, its source voxel(s) in
-  // the handle and the weight of the second source
+  // slab fits (prism_fit_init_slabs): per voxel of the whole volume its grid position, and per slice
+  // its slab or slabs
   bool slabbed = false;
-  std::vector<int64_t> st_src0, st_src1;
-  std::vector<float> st_w1;
+  int64_t n_whole = 0;
+  int32_t* d_grid_of_vox = nullptr;
+  SliceDev* d_slices = nullptr;
+  int whole_ny = 0, whole_nz = 0;
   std::vector<int32_t> order;          // host copy
   MeasRow* d_table = nullptr;
   MeasPair* d_table2 = nullptr;
@@ -152,6 +153,12 @@ struct prism_handle {
     allocs.push_back(q);
     *p = static_cast<T*>(q);
     return PRISM_OK;
+  }
+  void release(void* p) {   // a temporary that nothing reads any more
+    auto it = std::find(allocs.begin(), allocs.end(), p);
+    if (!p || it == allocs.end()) return;
+    allocs.erase(it);
+    cudaFree(p);
   }
   ~prism_handle() {
     if (g1) cudaGraphExecDestroy(g1);
@@ -512,35 +519,67 @@ static std::vector<int32_t> tile_queue_order(const std::vector<Tile>& tiles, int
   return order;
 }
 
-// A vector whose elements start uninitialised: the plan's large index tables are written in
-// full by its parallel passes, so a serial fill first would only add a pass over them.
-template <typename T>
-struct NoFillAlloc : std::allocator<T> {
-  template <typename U>
-  struct rebind {
-    using other = NoFillAlloc<U>;
-  };
-  NoFillAlloc() = default;
-  template <typename U>
-  NoFillAlloc(const NoFillAlloc<U>&) noexcept {}
-  template <typename U>
-  void construct(U* p) noexcept {
-    ::new (static_cast<void*>(p)) U;
-  }
-  template <typename U, typename... A>
-  void construct(U* p, A&&... a) {
-    ::new (static_cast<void*>(p)) U(std::forward<A>(a)...);
-  }
+// Host index of one volume's mask: masked voxels, per patch_dim^3 patch (C order of patches) and, as
+// an exclusive sum in mask order, before each (x, y) line. One pass over the mask; everything per voxel is
+// worked out on the device from it (k_plan).
+struct MaskIndex {
+  int64_t count = 0;
+  std::vector<int32_t> pcount, line;
 };
-template <typename T>
-using RawVec = std::vector<T, NoFillAlloc<T>>;
+
+// A volume's mask in memory: [nx][ny] lines `stride` bytes apart, of which slices [z0, z0 + nz) belong
+// to the volume (a slab of a whole volume; otherwise stride = nz, z0 = 0).
+struct MaskView {
+  const uint8_t* mask;
+  int nx, ny, nz, stride, z0;
+};
+MaskView view_of(const prism_volume& v) { return {v.mask, v.nx, v.ny, v.nz, v.nz, 0}; }
+
+MaskIndex index_mask(const MaskView& v, int P) {
+  MaskIndex ix;
+  const int py = (v.ny + P - 1) / P, pz = (v.nz + P - 1) / P, px = (v.nx + P - 1) / P;
+  ix.pcount.assign(static_cast<size_t>(px) * py * pz, 0);
+  ix.line.assign(static_cast<size_t>(v.nx) * v.ny, 0);
+  // whole layers of patches per chunk, so that no two threads write one patch's count
+  parallel_chunks(px, std::max(1, (1 << 16) / std::max(1, P * v.ny * v.nz)), [&](int64_t b, int64_t e) {
+    for (int x = static_cast<int>(b) * P; x < std::min<int64_t>(v.nx, e * P); ++x)
+      for (int y = 0; y < v.ny; ++y) {
+        const uint8_t* m = v.mask + (static_cast<int64_t>(x) * v.ny + y) * v.stride + v.z0;
+        int32_t* pc = ix.pcount.data() + (static_cast<size_t>(x / P) * py + y / P) * pz;
+        int32_t n = 0;
+        for (int c = 0; c < pz; ++c) {
+          int32_t k = 0;
+          for (int z = c * P; z < std::min(v.nz, (c + 1) * P); ++z) k += m[z] != 0;
+          pc[c] += k;
+          n += k;
+        }
+        ix.line[static_cast<size_t>(x) * v.ny + y] = n;
+      }
+  });
+  int32_t sum = 0;
+  for (int32_t& n : ix.line) {
+    const int32_t k = n;
+    n = sum;
+    sum += k;
+  }
+  ix.count = sum;
+  return ix;
+}
+
+std::vector<MaskIndex> index_masks(const prism_volume* vols, int n, int P) {
+  std::vector<MaskIndex> ix;
+  for (int g = 0; g < n; ++g) ix.push_back(index_mask(view_of(vols[g]), P));
+  return ix;
+}
 
 struct Plan {
-  RawVec<int32_t> slot_of_vox, slot_of_grid;
-  RawVec<int64_t> row_off;
+  std::vector<int32_t> ptile;      // first tile of every patch of every volume (-1: no masked voxel)
+  std::vector<int64_t> patch0;     // [n_vols] first patch of a volume in ptile
+  std::vector<int64_t> line0;      // [n_vols] first line of a volume
+  int64_t n_lines = 0, grid_tot = 0;
 };
 
-int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, Plan& pl) {
+int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, const std::vector<MaskIndex>& idx, Plan& pl) {
   const int P = h->opt.patch_dim;
   const int TV = h->TV;
   h->G = n_vols;
@@ -549,47 +588,23 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, Plan& pl) 
   h->gp_layout.assign(4 * static_cast<size_t>(n_vols) + 1, 0);
   h->yhat_off.assign(n_vols + 1, 0);
   // counts
-  int64_t Vtot = 0, grid_tot = 0;
-  std::vector<RawVec<int32_t>> vidx(n_vols);
+  int64_t Vtot = 0;
   for (int g = 0; g < n_vols; ++g) {
     const prism_volume& v = vols[g];
-    const int64_t ng = static_cast<int64_t>(v.nx) * v.ny * v.nz;
-    vidx[g].resize(ng);
-    // mask-order index of every grid position (-1 outside the mask): chunk counts, then chunk
-    // offsets
-    constexpr int64_t kChunkN = 1 << 18;
-    const int64_t nch = (ng + kChunkN - 1) / kChunkN;
-    std::vector<int32_t> cc(nch + 1, 0);
-    parallel_chunks(nch, 1, [&](int64_t b, int64_t e) {
-      for (int64_t k = b; k < e; ++k) {
-        int32_t n = 0;
-        for (int64_t i = k * kChunkN; i < std::min(ng, (k + 1) * kChunkN); ++i) n += v.mask[i] != 0;
-        cc[k + 1] = n;
-      }
-    });
-    for (int64_t k = 0; k < nch; ++k) cc[k + 1] += cc[k];
-    parallel_chunks(nch, 1, [&](int64_t b, int64_t e) {
-      for (int64_t k = b; k < e; ++k) {
-        int32_t n = cc[k];
-        for (int64_t i = k * kChunkN; i < std::min(ng, (k + 1) * kChunkN); ++i) vidx[g][i] = v.mask[i] ? n++ : -1;
-      }
-    });
-    const int32_t c = cc[nch];
+    const int64_t c = idx[g].count;
     if (c == 0) return fail(PRISM_E_SHAPE, "volume " + std::to_string(g) + ": empty mask");
     if (v.norm_count != 0 && v.norm_count < c)
       return fail(PRISM_E_SHAPE, "volume " + std::to_string(g) + ": norm_count " + std::to_string(v.norm_count) +
                                      " is below the " + std::to_string(c) + " masked voxels");
     h->vox0[g] = Vtot;
     Vtot += c;
-    h->groups[g].grid_off = grid_tot;
-    grid_tot += ng;
+    h->groups[g].grid_off = pl.grid_tot;
+    pl.grid_tot += static_cast<int64_t>(v.nx) * v.ny * v.nz;
+    pl.line0.push_back(pl.n_lines);
+    pl.n_lines += static_cast<int64_t>(v.nx) * v.ny;
   }
   h->vox0[n_vols] = Vtot;
   h->V = Vtot;
-  // every entry of the three tables is written by pass 2 below
-  pl.slot_of_vox.resize(Vtot);
-  pl.row_off.resize(Vtot);
-  pl.slot_of_grid.resize(grid_tot);
   // tiles
   int64_t yoff = 0, aboff = 0, tab = 0, gp = 0, yh = 0;
   int Nmax = 0;
@@ -647,34 +662,16 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, Plan& pl) 
     yh += static_cast<int64_t>(gr.n_vox) * v.n_meas;
     Nmax = std::max(Nmax, npos);
     gr.tile0 = static_cast<int32_t>(h->tiles.size());
-    const int px = (v.nx + P - 1) / P, py = (v.ny + P - 1) / P, pz = (v.nz + P - 1) / P;
-    const int64_t npatch = static_cast<int64_t>(px) * py * pz;
-    // pass 1 (parallel): masked voxels per patch
-    std::vector<int32_t> pcount(npatch, 0);
-    auto patch_box = [&](int64_t pi, int lo[3], int hi[3]) {
-      const int a = static_cast<int>(pi / (static_cast<int64_t>(py) * pz)), b = static_cast<int>((pi / pz) % py),
-                c3 = static_cast<int>(pi % pz);
-      lo[0] = a * P, lo[1] = b * P, lo[2] = c3 * P;
-      hi[0] = std::min(v.nx, (a + 1) * P), hi[1] = std::min(v.ny, (b + 1) * P), hi[2] = std::min(v.nz, (c3 + 1) * P);
-    };
-    parallel_chunks(npatch, 16, [&](int64_t b0, int64_t e0) {
-      for (int64_t pi = b0; pi < e0; ++pi) {
-        int lo[3], hi[3];
-        patch_box(pi, lo, hi);
-        int32_t n = 0;
-        for (int x = lo[0]; x < hi[0]; ++x)
-          for (int y = lo[1]; y < hi[1]; ++y)
-            for (int z = lo[2]; z < hi[2]; ++z) n += vidx[g][(static_cast<int64_t>(x) * v.ny + y) * v.nz + z] >= 0;
-        pcount[pi] = n;
-      }
-    });
-    // tiles and patches in patch order (sequential, one entry per tile)
-    std::vector<int32_t> ptile(npatch, -1);
-    for (int64_t pi = 0; pi < npatch; ++pi) {
+    gr.vox0 = h->vox0[g];
+    gr.yhat_off = h->yhat_off[g];
+    // tiles and patches in patch order (one entry per tile)
+    const std::vector<int32_t>& pcount = idx[g].pcount;
+    pl.patch0.push_back(static_cast<int64_t>(pl.ptile.size()));
+    for (size_t pi = 0; pi < pcount.size(); ++pi) {
+      pl.ptile.push_back(pcount[pi] ? static_cast<int32_t>(h->tiles.size()) : -1);
       if (pcount[pi] == 0) continue;
       const int pid = static_cast<int>(h->patches.size());
       const int tb = static_cast<int>(h->tiles.size());
-      ptile[pi] = tb;
       for (int32_t s0 = 0; s0 < pcount[pi]; s0 += TV) {
         Tile t{};
         t.group = g;
@@ -690,30 +687,6 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, Plan& pl) 
       }
       h->patches.push_back({tb, static_cast<int>(h->tiles.size())});
     }
-    // pass 2 (parallel): the slots of each patch's voxels, in C order within the patch; grid
-    // positions outside the mask (the patch boxes cover the grid) get slot -1
-    parallel_chunks(npatch, 16, [&](int64_t b0, int64_t e0) {
-      for (int64_t pi = b0; pi < e0; ++pi) {
-        int lo[3], hi[3];
-        patch_box(pi, lo, hi);
-        int slot = ptile[pi] * TV;
-        for (int x = lo[0]; x < hi[0]; ++x)
-          for (int y = lo[1]; y < hi[1]; ++y)
-            for (int z = lo[2]; z < hi[2]; ++z) {
-              const int64_t gi = (static_cast<int64_t>(x) * v.ny + y) * v.nz + z;
-              const int32_t vi = vidx[g][gi];
-              if (vi < 0) {
-                pl.slot_of_grid[gr.grid_off + gi] = -1;
-                continue;
-              }
-              const int64_t vg = h->vox0[g] + vi;
-              pl.slot_of_vox[vg] = slot;
-              pl.slot_of_grid[gr.grid_off + gi] = slot;
-              pl.row_off[vg] = h->yhat_off[g] + static_cast<int64_t>(vi) * v.n_meas;
-              ++slot;
-            }
-      }
-    });
     gr.ntiles = static_cast<int32_t>(h->tiles.size()) - gr.tile0;
   }
   h->ntiles = static_cast<int>(h->tiles.size());
@@ -727,8 +700,8 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, Plan& pl) 
   h->tab_rows = tab;
   h->yhat_off[n_vols] = yh;
   h->yhat_len = yh;
-  // the per-slot tables (mask-order index, coordinates, neighbour slots and flags) are built
-  // on the device from slot_of_grid (launch_slot_data)
+  // the slots and the per-slot tables (mask-order index, coordinates, neighbour slots and flags) are
+  // worked out on the device (launch_plan, launch_slot_data)
   return PRISM_OK;
 }
 
@@ -771,10 +744,17 @@ int shells_apply(const prism_volume* vols, int n, const prism_options& o, int64_
   return even ? 1 : (V >= kPadVoxels ? 2 : 0);
 }
 
-// `rows`: per volume, the row of each voxel in vols[g].signal and vols[g].init (device memory; the
-// slabs of one whole-volume signal), or nullptr where the rows are in mask order.
-int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::vector<int64_t>& counts,
-              const int64_t* const* rows, cudaStream_t st) {
+// Slabs of one whole volume (prism_fit_init_slabs): the volumes are slices [z0[g], z0[g] + nz) of its
+// mask, and their signal and init rows are those of the whole volume (whole-volume pointers in vols[g]).
+struct SlabSrc {
+  prism_volume whole;
+  std::vector<int> z0;             // per volume of the handle
+  std::vector<SliceDev> slices;    // per slice of the whole volume
+  MaskIndex index;                 // of the whole mask
+};
+
+int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::vector<MaskIndex>& idx,
+              const SlabSrc* slabs, cudaStream_t st) {
   const prism_options& o = h->opt;
   h->K = o.K;
   h->Q = 4 * o.K + 5;
@@ -784,13 +764,8 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   h->ks = &kernels_for_k(o.K);
   h->TV = h->NT / h->TPV;
   int64_t Vsum = 0;
-  for (int64_t c : counts) Vsum += c;
+  for (const MaskIndex& ix : idx) Vsum += ix.count;
   h->shell = (h->TPV == 1) ? shells_apply(vols, n_vols, o, Vsum) : 0;
-  int dev = 0, sms = 0;
-  if (o.fused) {
-    CK(cudaGetDevice(&dev));
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
   // Host signals start their copy to the device before the plan is built: a copy needs only the
   // voxel count, and the DMA then runs while the host builds the plan. All copies start at once
   // when together they take at most a quarter of the free device memory; otherwise each volume
@@ -799,19 +774,24 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   {
     size_t bytes = 0;
     for (int g = 0; g < n_vols; ++g)
-      if (vols[g].mem == PRISM_MEM_HOST) bytes += sizeof(float) * static_cast<size_t>(counts[g]) * vols[g].n_meas;
+      if (vols[g].mem == PRISM_MEM_HOST) bytes += sizeof(float) * static_cast<size_t>(idx[g].count) * vols[g].n_meas;
     size_t fr = 0, tot = 0;
     if (bytes > 0 && cudaMemGetInfo(&fr, &tot) == cudaSuccess && bytes <= fr / 4) {
       for (int g = 0; g < n_vols; ++g) {
         if (vols[g].mem != PRISM_MEM_HOST) continue;
-        const size_t n = static_cast<size_t>(counts[g]) * vols[g].n_meas;
+        const size_t n = static_cast<size_t>(idx[g].count) * vols[g].n_meas;
         RC(h->alloc(&early[g], n));
         CK(cudaMemcpyAsync(early[g], vols[g].signal, sizeof(float) * n, cudaMemcpyHostToDevice, st));
       }
     }
   }
   Plan pl;
-  RC(build_plan(h, vols, n_vols, pl));
+  RC(build_plan(h, vols, n_vols, idx, pl));
+  int dev = 0, sms = 0;
+  if (o.fused) {
+    CK(cudaGetDevice(&dev));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  }
   const int Vp = h->Vpad, Q = h->Q, G = h->G;
   // group reduction geometry
   h->max_e = 3 + (h->cal ? 2 * h->Nmax : 0);
@@ -874,8 +854,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   RC(h->alloc(&h->d_adamc, 2));
   RC(h->alloc(&h->d_slot_of_vox, h->V));
   RC(h->alloc(&h->d_vox_of_slot, Vp));
-  RC(h->alloc(&h->d_slot_of_grid, pl.slot_of_grid.size()));
-  RC(h->alloc(&h->d_row_off, h->V));
+  RC(h->alloc(&h->d_slot_of_grid, pl.grid_tot));
   RC(h->alloc(&h->d_order, std::max<int64_t>(h->tab_rows, 1)));
   RC(h->alloc(&h->d_pack_order, h->pack_order.size()));
   RC(h->alloc(&h->d_split_off, G));
@@ -932,11 +911,58 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   RC(upload(h->d_tiles, h->tiles, st));
   RC(upload(h->d_tile_order, tile_queue_order(h->tiles, h->TV), st));
   RC(upload(h->d_groups, h->groups, st));
-  RC(upload(h->d_slot_of_vox, pl.slot_of_vox, st));
-  RC(upload(h->d_slot_of_grid, pl.slot_of_grid, st));
-  CK(launch_slot_data(h->d_tiles, h->d_groups, h->G, h->groups.data(), h->d_slot_of_grid, h->d_slot_of_vox, h->V,
-                      Vp, h->TV, h->opt.connectivity, h->d_vox_of_slot, h->d_vcoord, h->d_vflag, h->d_nbr, st));
-  RC(upload(h->d_row_off, pl.row_off, st));
+  // slots of every voxel from the masks, the patches' first tiles and the lines' first voxels
+  uint8_t* d_mask = nullptr;
+  int32_t *d_ptile = nullptr, *d_line = nullptr, *d_wline = nullptr;
+  int64_t* d_rows = nullptr;   // slabs: the whole-volume row of each voxel
+  const size_t mask_bytes =
+      slabs ? static_cast<size_t>(slabs->whole.nx) * slabs->whole.ny * slabs->whole.nz : static_cast<size_t>(pl.grid_tot);
+  RC(h->alloc(&d_mask, mask_bytes));
+  RC(h->alloc(&d_ptile, pl.ptile.size()));
+  RC(h->alloc(&d_line, pl.n_lines));
+  RC(upload(d_ptile, pl.ptile, st));
+  for (int g = 0; g < G; ++g) RC(upload(d_line + pl.line0[g], idx[g].line, st));
+  CK(cudaMemsetAsync(h->d_vox_of_slot, 0xff, sizeof(int32_t) * Vp, st));
+  CK(cudaMemsetAsync(h->d_vcoord, 0, sizeof(uint32_t) * Vp, st));
+  if (slabs) {
+    const prism_volume& w = slabs->whole;
+    CK(cudaMemcpyAsync(d_mask, w.mask, mask_bytes, cudaMemcpyHostToDevice, st));
+    RC(h->alloc(&d_wline, slabs->index.line.size()));
+    RC(upload(d_wline, slabs->index.line, st));
+    RC(h->alloc(&d_rows, h->V));
+    h->slabbed = true;
+    h->n_whole = slabs->index.count;
+    h->whole_ny = w.ny;
+    h->whole_nz = w.nz;
+    RC(h->alloc(&h->d_grid_of_vox, h->n_whole));
+    RC(h->alloc(&h->d_slices, slabs->slices.size()));
+    RC(upload(h->d_slices, slabs->slices, st));
+    CK(launch_grid_of_vox(d_mask, d_wline, w.nx, w.ny, w.nz, h->d_grid_of_vox, st));
+  }
+  for (int g = 0; g < G; ++g) {
+    const prism_volume& v = vols[g];
+    PlanArgs pa{};
+    pa.mask = slabs ? d_mask : d_mask + h->groups[g].grid_off;
+    if (!slabs)
+      CK(cudaMemcpyAsync(d_mask + h->groups[g].grid_off, v.mask, static_cast<size_t>(v.nx) * v.ny * v.nz,
+                         cudaMemcpyHostToDevice, st));
+    pa.stride = slabs ? slabs->whole.nz : v.nz;
+    pa.z0 = slabs ? slabs->z0[g] : 0;
+    pa.line = d_line + pl.line0[g];
+    pa.wline = d_wline;
+    pa.ptile = d_ptile + pl.patch0[g];
+    pa.g = g;
+    pa.P = o.patch_dim;
+    pa.TV = h->TV;
+    pa.slot_of_grid = h->d_slot_of_grid;
+    pa.slot_of_vox = h->d_slot_of_vox;
+    pa.vox_of_slot = h->d_vox_of_slot;
+    pa.vcoord = h->d_vcoord;
+    pa.rows = d_rows;
+    CK(launch_plan(pa, h->d_groups, static_cast<int>(idx[g].pcount.size()), st));
+  }
+  CK(launch_slot_data(h->d_tiles, h->d_groups, h->G, h->groups.data(), h->d_slot_of_grid, Vp, h->TV,
+                      h->opt.connectivity, h->d_vflag, h->d_nbr, st));
   RC(upload(h->d_order, h->order, st));
   RC(upload(h->d_pack_order, h->pack_order, st));
   RC(upload(h->d_gtab, h->gtab, st));
@@ -953,7 +979,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
     const int N = v.n_meas;
     const int64_t Vg = gr.n_vox;
     const float* sig = v.signal;
-    const int64_t* vrows = rows ? rows[g] : nullptr;
+    const int64_t* vrows = slabs ? d_rows + h->vox0[g] : nullptr;
     float* tmp_sig = early[g];
     if (tmp_sig) {
       sig = tmp_sig;
@@ -1006,13 +1032,12 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
     // free per-volume temporaries (after the work that reads them)
     CK(cudaStreamSynchronize(st));
     for (void* p : {static_cast<void*>(tmp_sig), static_cast<void*>(d_b0n), static_cast<void*>(d_bv),
-                    static_cast<void*>(d_bvec), static_cast<void*>(d_b0), static_cast<void*>(d_part)}) {
-      if (!p) continue;
-      auto it = std::find(h->allocs.begin(), h->allocs.end(), p);
-      if (it != h->allocs.end()) h->allocs.erase(it);
-      cudaFree(p);
-    }
+                    static_cast<void*>(d_bvec), static_cast<void*>(d_b0), static_cast<void*>(d_part)})
+      h->release(p);
   }
+  for (void* p : {static_cast<void*>(d_mask), static_cast<void*>(d_ptile), static_cast<void*>(d_line),
+                  static_cast<void*>(d_wline), static_cast<void*>(d_rows)})
+    h->release(p);
   int bad = 0;
   CK(cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -1074,26 +1099,6 @@ int choose_shape(const prism_options& o, int64_t V, bool shell, int* tpv, int* n
   return PRISM_OK;
 }
 
-// Masked voxels of each volume.
-std::vector<int64_t> count_voxels(const prism_volume* vols, int n) {
-  std::vector<int64_t> V(n, 0);
-  for (int g = 0; g < n; ++g) {
-    const int64_t ng = static_cast<int64_t>(vols[g].nx) * vols[g].ny * vols[g].nz;
-    constexpr int64_t kChunkN = 1 << 18;
-    const int64_t nch = (ng + kChunkN - 1) / kChunkN;
-    std::vector<int64_t> cc(nch, 0);
-    parallel_chunks(nch, 4, [&](int64_t b, int64_t e) {
-      for (int64_t k = b; k < e; ++k) {
-        int64_t c = 0;
-        for (int64_t i = k * kChunkN; i < std::min(ng, (k + 1) * kChunkN); ++i) c += vols[g].mask[i] != 0;
-        cc[k] = c;
-      }
-    });
-    for (int64_t c : cc) V[g] += c;
-  }
-  return V;
-}
-
 int build_graphs(prism_handle* h) {
   CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   RC(capture_graph(h, 1, &h->g1));
@@ -1117,14 +1122,14 @@ struct DevTmp {
   }
 };
 
-int create_handle(const prism_volume* vols, int n_vols, const std::vector<int64_t>& counts, const prism_options& o,
-                  int tpv, int nt, const int64_t* const* rows, cudaStream_t st, prism_handle** out) {
+int create_handle(const prism_volume* vols, int n_vols, const std::vector<MaskIndex>& idx, const prism_options& o,
+                  int tpv, int nt, const SlabSrc* slabs, cudaStream_t st, prism_handle** out) {
   std::unique_ptr<prism_handle> h(new (std::nothrow) prism_handle());
   if (!h) return fail(PRISM_E_OOM, "host allocation failed");
   h->opt = o;
   h->TPV = tpv;
   h->NT = nt;
-  RC(init_impl(h.get(), vols, n_vols, counts, rows, st));
+  RC(init_impl(h.get(), vols, n_vols, idx, slabs, st));
   // the local kernel needs no graph: one launch holds up to kMaxIters iterations
   if (o.fused && o.use_graph && !h->local) RC(build_graphs(h.get()));
   *out = h.release();
@@ -1144,19 +1149,18 @@ struct TuneSample {
   std::vector<std::vector<uint8_t>> masks;
   std::vector<std::vector<float>> host_sig;
   std::vector<DevTmp> dev_sig, dev_rows;
-  std::vector<int64_t> counts;
+  std::vector<MaskIndex> idx;
 };
 
-int tune_sample(const prism_volume* vols, int n_vols, const std::vector<int64_t>& counts, int P, int64_t budget,
+int tune_sample(const prism_volume* vols, int n_vols, const std::vector<MaskIndex>& idx, int P, int64_t budget,
                 cudaStream_t st, TuneSample& S) {
   int64_t V = 0;
-  for (int64_t c : counts) V += c;
+  for (const MaskIndex& ix : idx) V += ix.count;
   S.vols.assign(vols, vols + n_vols);
   S.masks.resize(n_vols);
   S.host_sig.resize(n_vols);
   S.dev_sig.resize(n_vols);
   S.dev_rows.resize(n_vols);
-  S.counts.assign(n_vols, 0);
   for (int g = 0; g < n_vols; ++g) {
     const prism_volume& v = vols[g];
     const int64_t ng = static_cast<int64_t>(v.nx) * v.ny * v.nz;
@@ -1172,7 +1176,7 @@ int tune_sample(const prism_volume* vols, int n_vols, const std::vector<int64_t>
     std::vector<int32_t> order(pcount.size());
     for (size_t i = 0; i < order.size(); ++i) order[i] = static_cast<int32_t>(i);
     std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return pcount[a] > pcount[b]; });
-    const int64_t quota = std::max<int64_t>(1, budget * counts[g] / std::max<int64_t>(V, 1));
+    const int64_t quota = std::max<int64_t>(1, budget * idx[g].count / std::max<int64_t>(V, 1));
     std::vector<uint8_t> keep(pcount.size(), 0);
     int64_t got = 0;
     for (int32_t p : order) {
@@ -1194,8 +1198,7 @@ int tune_sample(const prism_volume* vols, int n_vols, const std::vector<int64_t>
     prism_volume& pv = S.vols[g];
     pv.mask = S.masks[g].data();
     pv.init = nullptr;
-    pv.norm_count = v.norm_count > 0 ? v.norm_count : static_cast<int32_t>(counts[g]);
-    S.counts[g] = n;
+    pv.norm_count = v.norm_count > 0 ? v.norm_count : static_cast<int32_t>(idx[g].count);
     if (v.mem == PRISM_MEM_HOST) {
       S.host_sig[g].resize(static_cast<size_t>(n) * N);
       for (int64_t i = 0; i < n; ++i)
@@ -1210,23 +1213,24 @@ int tune_sample(const prism_volume* vols, int n_vols, const std::vector<int64_t>
     }
   }
   CK(cudaStreamSynchronize(st));
+  S.idx = index_masks(S.vols.data(), n_vols, P);
   return PRISM_OK;
 }
 
-void autotune_shape(const prism_volume* vols, int n_vols, const std::vector<int64_t>& counts, const prism_options& o,
+void autotune_shape(const prism_volume* vols, int n_vols, const std::vector<MaskIndex>& idx, const prism_options& o,
                     cudaStream_t st, int* tpv, int* shells) {
   int64_t V = 0;
-  for (int64_t c : counts) V += c;
+  for (const MaskIndex& ix : idx) V += ix.count;
   TuneSample S;
   const prism_volume* tv = vols;
-  const std::vector<int64_t>* tc = &counts;
+  const std::vector<MaskIndex>* tc = &idx;
   if (V > kTuneVoxels) {
-    if (tune_sample(vols, n_vols, counts, o.patch_dim, kTuneVoxels, st, S) != PRISM_OK) {
+    if (tune_sample(vols, n_vols, idx, o.patch_dim, kTuneVoxels, st, S) != PRISM_OK) {
       g_err.clear();
       return;
     }
     tv = S.vols.data();
-    tc = &S.counts;
+    tc = &S.idx;
   }
   prism_options oc = o;
   oc.use_graph = 0;
@@ -1281,8 +1285,8 @@ void autotune_shape(const prism_volume* vols, int n_vols, const std::vector<int6
   g_err.clear();
 }
 
-// prism_fit_init, with the optional row maps of init_impl (then without autotuning).
-int fit_init(const prism_volume* vols, int n_vols, const prism_options* opt, const int64_t* const* rows, void* stream,
+// prism_fit_init, or with `slabs` the volumes of a slab fit (then without autotuning).
+int fit_init(const prism_volume* vols, int n_vols, const prism_options* opt, const SlabSrc* slabs, void* stream,
              prism_handle** out) {
   g_err.clear();
   if (!out) return fail(PRISM_E_INVALID_ARG, "out is NULL");
@@ -1294,18 +1298,27 @@ int fit_init(const prism_volume* vols, int n_vols, const prism_options* opt, con
   RC(validate_options(o));
   for (int g = 0; g < n_vols; ++g) RC(validate_volume(vols[g], g));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const std::vector<int64_t> counts = count_voxels(vols, n_vols);
+  std::vector<MaskIndex> idx;
   int64_t V = 0;
-  for (int64_t c : counts) V += c;
+  for (int g = 0; g < n_vols; ++g) {
+    MaskView mv = view_of(vols[g]);
+    if (slabs) {
+      mv.mask = slabs->whole.mask;
+      mv.stride = slabs->whole.nz;
+      mv.z0 = slabs->z0[g];
+    }
+    idx.push_back(index_mask(mv, o.patch_dim));
+    V += idx.back().count;
+  }
   int tpv = 1, nt = 128;
   choose_shape(o, V, shells_apply(vols, n_vols, o, V) != 0, &tpv, &nt);
-  if (o.autotune && o.fused && !rows) {
+  if (o.autotune && o.fused && !slabs) {
     int shells = o.shells;
-    autotune_shape(vols, n_vols, counts, o, st, &tpv, &shells);
+    autotune_shape(vols, n_vols, idx, o, st, &tpv, &shells);
     o.shells = shells;
   }
   prism_handle* h = nullptr;
-  const int rc = create_handle(vols, n_vols, counts, o, tpv, nt, rows, st, &h);
+  const int rc = create_handle(vols, n_vols, idx, o, tpv, nt, slabs, st, &h);
   if (rc != PRISM_OK) return rc;
   *out = h;
   return PRISM_OK;
@@ -1534,7 +1547,7 @@ extern "C" int prism_forward(prism_handle* h, const float* theta, const float* g
     CK(launch_group_adam(a, h->ga, 1, st));
   }
   if (loss) CK(cudaMemcpyAsync(loss, h->d_gloss, sizeof(double) * h->G, cudaMemcpyDeviceToDevice, st));
-  if (yhat) CK(h->ks->yhat(a, cal, h->d_vox_of_slot, h->d_row_off, h->d_order, yhat, st));
+  if (yhat) CK(h->ks->yhat(a, cal, h->d_vox_of_slot, h->d_order, yhat, st));
   h->forward_done = true;
   return PRISM_OK;
 }
@@ -1687,10 +1700,6 @@ extern "C" int prism_set_state(prism_handle* h, const void* host_buf, int64_t by
   return PRISM_OK;
 }
 
-namespace {
-// Device buffer released on scope exit (temporaries of the slab entry points).
-}  // namespace
-
 extern "C" int prism_fit_init_slabs(const prism_volume* vol, int32_t slab, int32_t overlap, const prism_options* opt,
                                     void* stream, prism_handle** out) {
   g_err.clear();
@@ -1722,96 +1731,40 @@ extern "C" int prism_fit_init_slabs(const prism_volume* vol, int32_t slab, int32
       if (zb[z] >= 0) return fail(PRISM_E_INVALID_ARG, "a slice lies in three slabs");
       (za[z] < 0 ? za[z] : zb[z]) = s;
     }
-  // whole-volume mask order (C order) -> per-slab mask order (the same relative order), in two
-  // passes over chunks of x (counts, then the entries at the chunks' offsets)
-  std::vector<std::vector<int64_t>> rows(S);
-  std::vector<std::vector<uint8_t>> sub(S);
-  for (int s = 0; s < S; ++s) sub[s].assign(static_cast<size_t>(nx) * ny * (z1s[s] - z0s[s]), 0);
-  const int nxc = std::min(nx, 64);
-  std::vector<int64_t> cnt(static_cast<size_t>(nxc + 1) * (S + 1), 0);   // [chunk + 1][S + 1]
-  auto xr = [&](int c, int& xa, int& xe) {
-    xa = static_cast<int>(static_cast<int64_t>(nx) * c / nxc);
-    xe = static_cast<int>(static_cast<int64_t>(nx) * (c + 1) / nxc);
-  };
-  parallel_chunks(nxc, 1, [&](int64_t cb, int64_t ce) {
-    for (int c = static_cast<int>(cb); c < ce; ++c) {
-      int xa, xe;
-      xr(c, xa, xe);
-      int64_t* k = cnt.data() + static_cast<size_t>(c + 1) * (S + 1);
-      for (int x = xa; x < xe; ++x)
-        for (int y = 0; y < ny; ++y) {
-          const uint8_t* m = vol->mask + (static_cast<int64_t>(x) * ny + y) * nz;
-          for (int z = 0; z < nz; ++z)
-            if (m[z]) {
-              ++k[S];
-              ++k[za[z]];
-              if (zb[z] >= 0) ++k[zb[z]];
-            }
-        }
-    }
-  });
-  for (int c = 0; c < nxc; ++c)
-    for (int s = 0; s <= S; ++s) cnt[static_cast<size_t>(c + 1) * (S + 1) + s] += cnt[static_cast<size_t>(c) * (S + 1) + s];
-  const int64_t V = cnt[static_cast<size_t>(nxc) * (S + 1) + S];
-  for (int s = 0; s < S; ++s) rows[s].resize(static_cast<size_t>(cnt[static_cast<size_t>(nxc) * (S + 1) + s]));
-  std::vector<int64_t> src0(V), src1(V);
-  std::vector<int32_t> slab0(V), slab1(V);
-  std::vector<float> w1(V);
-  parallel_chunks(nxc, 1, [&](int64_t cb, int64_t ce) {
-    std::vector<int64_t> at(S + 1);
-    for (int c = static_cast<int>(cb); c < ce; ++c) {
-      int xa, xe;
-      xr(c, xa, xe);
-      for (int s = 0; s <= S; ++s) at[s] = cnt[static_cast<size_t>(c) * (S + 1) + s];
-      for (int x = xa; x < xe; ++x)
-        for (int y = 0; y < ny; ++y) {
-          const uint8_t* m = vol->mask + (static_cast<int64_t>(x) * ny + y) * nz;
-          for (int z = 0; z < nz; ++z) {
-            if (!m[z]) continue;
-            const int64_t v = at[S]++;
-            const int first = za[z], second = zb[z];
-            const int64_t i0 = at[first]++;
-            rows[first][i0] = v;
-            sub[first][(static_cast<size_t>(x) * ny + y) * (z1s[first] - z0s[first]) + (z - z0s[first])] = 1;
-            int64_t i1 = -1;
-            float wt = 0.f;
-            if (second >= 0) {
-              i1 = at[second]++;
-              rows[second][i1] = v;
-              sub[second][(static_cast<size_t>(x) * ny + y) * (z1s[second] - z0s[second]) + (z - z0s[second])] = 1;
-              // linear ramp across the overlap of slabs first and second
-              wt = (static_cast<float>(z - z0s[second]) + 0.5f) / static_cast<float>(z1s[first] - z0s[second]);
-            }
-            slab0[v] = first;
-            src0[v] = i0;
-            slab1[v] = second;
-            src1[v] = i1;
-            w1[v] = wt;
-          }
-        }
-    }
-  });
+  SlabSrc src;
+  src.whole = *vol;
+  src.index = index_mask(view_of(*vol), o.patch_dim);
+  const int64_t V = src.index.count;
   if (V == 0) return fail(PRISM_E_SHAPE, "the mask is empty");
-  // non-empty slabs become the handle's volumes; handle voxel = vox0[g] + index in the slab
+  // non-empty slabs become the handle's volumes
   std::vector<int> gidx(S, -1);
-  std::vector<int64_t> vox0;
-  int G = 0;
-  int64_t acc = 0;
-  for (int s = 0; s < S; ++s)
-    if (!rows[s].empty()) {
-      gidx[s] = G++;
-      vox0.push_back(acc);
-      acc += static_cast<int64_t>(rows[s].size());
+  std::vector<prism_volume> vols;
+  for (int s = 0; s < S; ++s) {
+    bool any = false;
+    for (int64_t l = 0; l < static_cast<int64_t>(nx) * ny && !any; ++l)
+      for (int z = z0s[s]; z < z1s[s]; ++z) any |= vol->mask[l * nz + z] != 0;
+    if (!any) continue;
+    gidx[s] = static_cast<int>(vols.size());
+    src.z0.push_back(z0s[s]);
+    vols.push_back(*vol);
+    vols.back().nz = z1s[s] - z0s[s];
+    vols.back().mem = PRISM_MEM_DEVICE;
+  }
+  const int G = static_cast<int>(vols.size());
+  for (int z = 0; z < nz; ++z) {
+    SliceDev sl{};
+    sl.g0 = gidx[za[z]];
+    sl.z0 = z0s[za[z]];
+    sl.g1 = zb[z] >= 0 ? gidx[zb[z]] : -1;
+    if (zb[z] >= 0) {
+      sl.z1 = z0s[zb[z]];
+      // linear ramp across the overlap of the two slabs
+      sl.w1 = (static_cast<float>(z - z0s[zb[z]]) + 0.5f) / static_cast<float>(z1s[za[z]] - z0s[zb[z]]);
     }
-  parallel_chunks(V, 1 << 15, [&](int64_t b, int64_t e) {
-    for (int64_t i = b; i < e; ++i) {
-      src0[i] += vox0[gidx[slab0[i]]];
-      if (src1[i] >= 0) src1[i] += vox0[gidx[slab1[i]]];
-    }
-  });
-  // whole-volume signal (and initial parameters) on the device; every slab reads its rows of it (the
-  // autotuner takes volumes with rows of their own: then one gathered copy per slab)
-  DevTmp dsig, dinit, drows;
+    src.slices.push_back(sl);
+  }
+  // whole-volume signal (and initial parameters) on the device; every slab reads its rows of it
+  DevTmp dsig, dinit;
   const float* sig = vol->signal;
   const float* init = vol->init;
   if (vol->mem == PRISM_MEM_HOST) {
@@ -1824,42 +1777,25 @@ extern "C" int prism_fit_init_slabs(const prism_volume* vol, int32_t slab, int32
       init = dinit.as<float>();
     }
   }
-  CK(cudaMalloc(&drows.p, sizeof(int64_t) * acc));
-  const bool copies = o.autotune && o.fused;
-  std::vector<DevTmp> ssig(G), sinit(G);
-  std::vector<prism_volume> vols(G);
-  std::vector<const int64_t*> vrows(G);
-  for (int s = 0; s < S; ++s) {
-    const int g = gidx[s];
-    if (g < 0) continue;
-    const int64_t n = static_cast<int64_t>(rows[s].size());
-    int64_t* dr = drows.as<int64_t>() + vox0[g];
-    CK(cudaMemcpyAsync(dr, rows[s].data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-    vrows[g] = dr;
-    prism_volume& pv = vols[g];
-    pv = *vol;
-    pv.nz = z1s[s] - z0s[s];
-    pv.mem = PRISM_MEM_DEVICE;
-    pv.mask = sub[s].data();
+  for (prism_volume& pv : vols) {
     pv.signal = sig;
     pv.init = init;
-    if (!copies) continue;
-    CK(cudaMalloc(&ssig[g].p, sizeof(float) * n * N));
-    CK(launch_gather_rows(sig, dr, n, N, ssig[g].as<float>(), st));
-    pv.signal = ssig[g].as<float>();
-    if (init) {
-      CK(cudaMalloc(&sinit[g].p, sizeof(float) * n * Q));
-      CK(launch_gather_rows(init, dr, n, Q, sinit[g].as<float>(), st));
-      pv.init = sinit[g].as<float>();
-    }
+  }
+  if (o.autotune && o.fused) {   // on the whole volume: the same voxels but the overlaps'
+    prism_volume w = *vol;
+    w.mem = PRISM_MEM_DEVICE;
+    w.signal = sig;
+    w.init = init;
+    const std::vector<MaskIndex> wi{src.index};
+    int tpv = 1, nt = 128, shells = o.shells;
+    choose_shape(o, V, shells_apply(&w, 1, o, V) != 0, &tpv, &nt);
+    autotune_shape(&w, 1, wi, o, st, &tpv, &shells);
+    o.threads_per_voxel = tpv;
+    o.shells = shells;
   }
   prism_handle* h = nullptr;
-  RC(fit_init(vols.data(), G, &o, copies ? nullptr : vrows.data(), stream, &h));
+  RC(fit_init(vols.data(), G, &o, &src, stream, &h));
   CK(cudaStreamSynchronize(st));
-  h->slabbed = true;
-  h->st_src0 = std::move(src0);
-  h->st_src1 = std::move(src1);
-  h->st_w1 = std::move(w1);
   *out = h;
   return PRISM_OK;
 }
@@ -1870,15 +1806,9 @@ extern "C" int prism_stitch_slabs(prism_handle* h, float* s0, float* fracs, floa
   if (!h->slabbed) return fail(PRISM_E_STATE, "the handle was not made by prism_fit_init_slabs");
   if (mem != PRISM_MEM_HOST && mem != PRISM_MEM_DEVICE) return fail(PRISM_E_INVALID_ARG, "mem must be HOST or DEVICE");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int64_t n = static_cast<int64_t>(h->st_src0.size());
+  const int64_t n = h->n_whole;
   const int K = h->K;
-  DevTmp d0, d1, dw, out;
-  CK(cudaMalloc(&d0.p, sizeof(int64_t) * n));
-  CK(cudaMalloc(&d1.p, sizeof(int64_t) * n));
-  CK(cudaMalloc(&dw.p, sizeof(float) * n));
-  CK(cudaMemcpyAsync(d0.p, h->st_src0.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(d1.p, h->st_src1.data(), sizeof(int64_t) * n, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(dw.p, h->st_w1.data(), sizeof(float) * n, cudaMemcpyHostToDevice, st));
+  DevTmp out;
   const size_t ns = n, nf = n * (K + 3), nd = n * K * 3;
   float *o_s0 = s0, *o_fr = fracs, *o_fin = fin, *o_d = dirs;
   if (mem == PRISM_MEM_HOST) {
@@ -1889,8 +1819,8 @@ extern "C" int prism_stitch_slabs(prism_handle* h, float* s0, float* fracs, floa
     o_fr = fracs ? b + 2 * ns : nullptr;
     o_d = dirs ? b + 2 * ns + nf : nullptr;
   }
-  CK(h->ks->stitch(h->ia, h->d_slot_of_vox, n, d0.as<int64_t>(), d1.as<int64_t>(), dw.as<float>(), o_s0, o_fr,
-                   o_fin, o_d, st));
+  const StitchArgs sa{h->d_grid_of_vox, h->d_slices, h->d_slot_of_grid, n, h->whole_ny, h->whole_nz, o_s0, o_fr, o_fin, o_d};
+  CK(h->ks->stitch(h->ia, sa, st));
   if (mem == PRISM_MEM_HOST) {
     if (s0) CK(cudaMemcpyAsync(s0, o_s0, sizeof(float) * ns, cudaMemcpyDeviceToHost, st));
     if (fin) CK(cudaMemcpyAsync(fin, o_fin, sizeof(float) * ns, cudaMemcpyDeviceToHost, st));

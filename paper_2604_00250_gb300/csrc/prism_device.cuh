@@ -91,6 +91,15 @@ struct GroupDev {
   int32_t n_runs;      // its shells
   int32_t gtab_off;    // float offset of the group's gradient table: [NP / 2][4] {g_x, g_y} pairs, then [NP] g_z
   int32_t pad_;
+  int64_t vox0;        // first voxel of the group in mask order
+  int64_t yhat_off;    // its first row in the caller's y_hat
+};
+
+// One slice of a whole volume fitted in slabs: the groups and first slices of the slabs that hold it
+// (g1 = -1: one slab; g0 = -1: no masked voxel in any) and the later slab's weight.
+struct SliceDev {
+  int32_t g0, z0, g1, z1;
+  float w1;
 };
 
 // Kernel arguments shared by the iteration kernels (passed by value).

@@ -7,6 +7,7 @@
 #pragma once
 
 #include "prism_device.cuh"
+#include "prism_launch.h"
 
 namespace prism {
 
@@ -1677,22 +1678,26 @@ __global__ void k_fibers(const IterArgs a, const int32_t* __restrict__ slot_of_v
 
 // Slab stitching (Sec. 3 "Configuration": overlapping slabs stitched by weighted averaging;
 // the ramp weights and the fiber matching are this library's choice). Output voxel v takes
-// the estimate at handle voxel src0[v] and, where two slabs overlap, blends in the one at
-// src1[v] with weight w1[v] (src0's weight is 1 - w1). The later slab's fibers are matched to
+// the estimate of its slice's slab and, where two slabs overlap, blends in the later one's with the
+// slice's weight w1 (the earlier one's is 1 - w1). The later slab's fibers are matched to
 // the earlier slab's by the permutation maximising sum_k |d0_k . d1_pi(k)| (FP64 dot
 // products, first maximum in lexicographic order), each matched direction is flipped into
 // the same hemisphere, then S0, fractions, f_intra and the directions are averaged and the
 // directions renormalised.
 template <int K>
-__global__ void k_stitch(const IterArgs a, const int32_t* __restrict__ slot_of_vox, int64_t n_out,
-                         const int64_t* __restrict__ src0, const int64_t* __restrict__ src1,
-                         const float* __restrict__ w1, float* __restrict__ s0, float* __restrict__ fracs,
-                         float* __restrict__ fin, float* __restrict__ dirs) {
+__global__ void k_stitch(const IterArgs a, const StitchArgs sa) {
   const int64_t v = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (v >= n_out) return;
+  if (v >= sa.n) return;
+  const int gi = sa.grid_of_vox[v], z = gi % sa.nz, xy = gi / sa.nz;
+  const SliceDev sl = sa.slices[z];
+  float *s0 = sa.s0, *fracs = sa.fracs, *fin = sa.fin, *dirs = sa.dirs;
+  auto slot_in = [&](int g, int z0) {
+    const GroupDev gr = a.groups[g];
+    return sa.slot_of_grid[gr.grid_off + static_cast<int64_t>(xy) * gr.nz + (z - z0)];
+  };
   float th[4 * K + 5];
   Vox<K> A;
-  load_theta<K>(a.theta, a.Vpad, slot_of_vox[src0[v]], true, th);
+  load_theta<K>(a.theta, a.Vpad, slot_in(sl.g0, sl.z0), true, th);
   transform<K>(th, A);
   float S = A.S0, fi = A.fin, f[K + 3], d[K][3];
 #pragma unroll
@@ -1701,10 +1706,9 @@ __global__ void k_stitch(const IterArgs a, const int32_t* __restrict__ slot_of_v
   for (int k = 0; k < K; ++k)
 #pragma unroll
     for (int c = 0; c < 3; ++c) d[k][c] = A.d[k][c];
-  const int64_t b = src1[v];
-  if (b >= 0) {
+  if (sl.g1 >= 0) {
     Vox<K> B;
-    load_theta<K>(a.theta, a.Vpad, slot_of_vox[b], true, th);
+    load_theta<K>(a.theta, a.Vpad, slot_in(sl.g1, sl.z1), true, th);
     transform<K>(th, B);
     double ad[K][K];
 #pragma unroll
@@ -1739,7 +1743,7 @@ __global__ void k_stitch(const IterArgs a, const int32_t* __restrict__ slot_of_v
         p[r] = t;
       }
     }
-    const float wb = w1[v], wa = 1.f - wb;
+    const float wb = sl.w1, wa = 1.f - wb;
     S = wa * A.S0 + wb * B.S0;
     fi = wa * A.fin + wb * B.fin;
     f[0] = wa * A.f[0] + wb * B.f[0];
@@ -1821,8 +1825,7 @@ __global__ void __launch_bounds__(256) k_synth(const IterArgs a, const PlainArgs
 constexpr int kYhatC = 32;
 template <int K, bool CAL>
 __global__ void __launch_bounds__(256) k_yhat(const IterArgs a, const int32_t* __restrict__ vox_of_slot,
-                                             const int64_t* __restrict__ row_off, const int32_t* __restrict__ order,
-                                             float* __restrict__ out) {
+                                             const int32_t* __restrict__ order, float* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ float4 s_tab[kYhatC / 2][8];
   int64_t* s_row = reinterpret_cast<int64_t*>(smem);                 // [TV]
@@ -1834,7 +1837,7 @@ __global__ void __launch_bounds__(256) k_yhat(const IterArgs a, const int32_t* _
   const int TV = a.TV, lanes = static_cast<int>(blockDim.x) / TV;
   const int vl = threadIdx.x % TV, js = threadIdx.x / TV, slot = tl.slot0 + vl;
   const bool act = vl < tl.count;
-  if (js == 0 && act) s_row[vl] = row_off[vox_of_slot[slot]];
+  if (js == 0 && act) s_row[vl] = gr.yhat_off + (vox_of_slot[slot] - gr.vox0) * gr.N;
   float th[4 * K + 5];
   load_theta<K>(a.theta, a.Vpad, slot, act, th);
   Vox<K> P;

@@ -154,13 +154,12 @@ cudaError_t l_synth(const IterArgs& a, const PlainArgs& p, int cal, int tpv, int
   }
 }
 
-cudaError_t l_yhat(const IterArgs& a, int cal, const int32_t* vos, const int64_t* roff, const int32_t* order,
-                   float* out, cudaStream_t st) {
+cudaError_t l_yhat(const IterArgs& a, int cal, const int32_t* vos, const int32_t* order, float* out, cudaStream_t st) {
   if (a.ntiles <= 0) return cudaSuccess;
   const int nt = max(128, a.TV);   // TV: 8, 32, 128 or, on a plain handle with 256-thread CTAs, up to 256
   const size_t smem = static_cast<size_t>(a.TV) * ((kYhatC + 1) * sizeof(float) + sizeof(int64_t));   // at most 36 KB
-  if (cal) k_yhat<kK, true><<<a.ntiles, nt, smem, st>>>(a, vos, roff, order, out);
-  else k_yhat<kK, false><<<a.ntiles, nt, smem, st>>>(a, vos, roff, order, out);
+  if (cal) k_yhat<kK, true><<<a.ntiles, nt, smem, st>>>(a, vos, order, out);
+  else k_yhat<kK, false><<<a.ntiles, nt, smem, st>>>(a, vos, order, out);
   return cudaGetLastError();
 }
 
@@ -216,10 +215,9 @@ cudaError_t l_fibers(const IterArgs& a, const int32_t* sov, int64_t V, float rel
   k_fibers<kK><<<nblocks(V, 128), 128, 0, st>>>(a, sov, V, rel, dirs, fracs, peaks);
   return cudaGetLastError();
 }
-cudaError_t l_stitch(const IterArgs& a, const int32_t* sov, int64_t n_out, const int64_t* src0, const int64_t* src1,
-                     const float* w1, float* s0, float* fracs, float* fin, float* dirs, cudaStream_t st) {
-  if (n_out <= 0) return cudaSuccess;
-  k_stitch<kK><<<nblocks(n_out, 128), 128, 0, st>>>(a, sov, n_out, src0, src1, w1, s0, fracs, fin, dirs);
+cudaError_t l_stitch(const IterArgs& a, const StitchArgs& s, cudaStream_t st) {
+  if (s.n <= 0) return cudaSuccess;
+  k_stitch<kK><<<nblocks(s.n, 128), 128, 0, st>>>(a, s);
   return cudaGetLastError();
 }
 

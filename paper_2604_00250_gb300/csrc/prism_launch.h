@@ -28,6 +28,16 @@ cudaError_t launch_dep(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cud
   return cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
+// Stitching of a slab fit (k_stitch): the whole volume's voxels by grid position and its slices.
+struct StitchArgs {
+  const int32_t* grid_of_vox;
+  const SliceDev* slices;
+  const int32_t* slot_of_grid;
+  int64_t n;
+  int32_t ny, nz;
+  float *s0, *fracs, *fin, *dirs;
+};
+
 // Per-K launchers of the templated kernels (one translation unit per K).
 struct KernelSet {
   // shell = 1 or 2: the shell loop of one thread per voxel, MSE, no calibration (2: with padded odd
@@ -40,8 +50,8 @@ struct KernelSet {
   cudaError_t (*local_occupancy)(int loss, int tpv, size_t smem, int* blocks);
   cudaError_t (*transform)(const IterArgs& a, int tb, int te, cudaStream_t st);
   cudaError_t (*synth)(const IterArgs& a, const PlainArgs& p, int cal, int tpv, int nt, cudaStream_t st);
-  cudaError_t (*yhat)(const IterArgs& a, int cal, const int32_t* vox_of_slot, const int64_t* row_off,
-                      const int32_t* order, float* out, cudaStream_t st);
+  cudaError_t (*yhat)(const IterArgs& a, int cal, const int32_t* vox_of_slot, const int32_t* order, float* out,
+                      cudaStream_t st);
   cudaError_t (*adjoint)(const IterArgs& a, const PlainArgs& p, int cal, int tpv, int nt, size_t smem,
                          cudaStream_t st);
   cudaError_t (*prior_prep)(const IterArgs& a, int tb, int te, cudaStream_t st);
@@ -49,9 +59,7 @@ struct KernelSet {
   cudaError_t (*prior)(const IterArgs& a, const PlainArgs& p, cudaStream_t st);
   cudaError_t (*fibers)(const IterArgs& a, const int32_t* slot_of_vox, int64_t V, float rel, float* dirs,
                         float* fracs, uint8_t* peaks, cudaStream_t st);
-  cudaError_t (*stitch)(const IterArgs& a, const int32_t* slot_of_vox, int64_t n_out, const int64_t* src0,
-                        const int64_t* src1, const float* w1, float* s0, float* fracs, float* fin, float* dirs,
-                        cudaStream_t st);
+  cudaError_t (*stitch)(const IterArgs& a, const StitchArgs& s, cudaStream_t st);
 };
 
 const KernelSet& kernels_for_k(int K);
@@ -99,9 +107,24 @@ cudaError_t launch_sigma_init(const double* part, int nblocks, int64_t V, int nb
 cudaError_t launch_pack(const IterArgs& a, const float* sig, const int64_t* rows, const float* b0mean,
                         const int32_t* vox_of_slot, const int32_t* order, int64_t vox0, int tile_begin, int tile_end,
                         int N, int npos, float* ypack, int* bad, cudaStream_t st);
+// Slots of one volume's voxels (k_plan). `mask`, `line` (masked voxels before each (x, y) line) and
+// `ptile` (first tile of each patch, -1 for none) are the volume's; `stride` and `z0` as in a slab of a
+// larger mask, whose lines `wline` then counts and whose rows go to `rows`.
+struct PlanArgs {
+  const uint8_t* mask;
+  int32_t stride, z0;
+  const int32_t *line, *wline, *ptile;
+  int32_t g, P, TV;
+  int32_t *slot_of_grid, *slot_of_vox, *vox_of_slot;
+  uint32_t* vcoord;
+  int64_t* rows;
+};
+cudaError_t launch_plan(const PlanArgs& p, const GroupDev* groups, int npatch, cudaStream_t st);
+cudaError_t launch_grid_of_vox(const uint8_t* mask, const int32_t* line, int nx, int ny, int nz, int32_t* grid_of_vox,
+                               cudaStream_t st);
 cudaError_t launch_slot_data(const Tile* tiles, const GroupDev* groups, int G, const GroupDev* host_groups,
-                             const int32_t* slot_of_grid, const int32_t* slot_of_vox, int64_t V, int Vp, int TV, int nnb,
-                             int32_t* vox_of_slot, uint32_t* vcoord, uint32_t* vflag, int32_t* nbr, cudaStream_t st);
+                             const int32_t* slot_of_grid, int Vp, int TV, int nnb, uint32_t* vflag, int32_t* nbr,
+                             cudaStream_t st);
 cudaError_t launch_gather_rows(const float* src, const int64_t* rows, int64_t n, int len, float* dst,
                                cudaStream_t st);
 cudaError_t launch_table(const float* bvals, const float* bvecs, int N, MeasRow* rows, cudaStream_t st);

@@ -104,20 +104,22 @@ typedef struct prism_options {
   float rprop_step_min, rprop_step_max; /* Rprop step bounds, 1e-6 and 50 */
   int32_t fused;          /* 1: persistent fused iteration kernel; 0: plain unfused per-patch launches */
   int32_t use_graph;      /* 1: replay the fused iteration from a CUDA graph */
-  int32_t threads_per_voxel; /* 1, 4 or 16 (measurements split across lanes); 0 = automatic:
-                                16 below 2,048 voxels, 4 below 32,768, else 1 except where
-                                128-voxel tiles come to 0.75-1.25 waves of the fused kernel's
-                                resident CTAs (then 4); prism_get_shape reports the choice */
+  int32_t threads_per_voxel; /* 1, 4 or 16 (measurements split across lanes); 0 = automatic: 16 below
+                                2,048 voxels (1,400 without neighbour priors and calibration), 4 below
+                                32,768 (16,384 where one lane takes the shell loop with the MSE), else
+                                1 except just above one wave of 128-voxel tiles with the NLL or
+                                calibration (then 4); prism_get_shape reports the choice */
   int32_t cta_threads;    /* plain path: 128 or 256 threads per CTA; 0 = automatic (the fused kernel uses 128) */
   int32_t autotune;       /* 1: time the candidate launch shapes at init and keep the fastest: lanes
                              per voxel 1 / 4 / 16 (or the forced value) and, with one lane, the shell
                              loop or the per-measurement loop; above about 311k voxels on a bounded
                              sample of each volume's fullest patches */
   int32_t seed;           /* seed of the default initialisation (init == NULL) */
-  int32_t shells;         /* fused kernel, one thread per voxel, MSE, no calibration: 0 = take the shell
-                             loop (per b-value shell work done once; at most 16 shells in every
-                             volume, each of an even number of measurements below 32,768 voxels),
-                             -1 = never */
+  int32_t shells;         /* fused kernel, one or four lanes per voxel: 0 = take the shell loop (per
+                             b-value shell work done once) where every volume has at most 16 shells
+                             and, with one lane, the MSE, no calibration and fewer than 32,768
+                             voxels, every shell holds an even number of measurements; -1 = never.
+                             Small fits without neighbour priors and calibration never take it. */
   int32_t reserved[3];
 } prism_options;
 

@@ -105,6 +105,10 @@ struct prism_handle {
   std::vector<int64_t> pack_off;       // [G] first position of a group
   std::vector<int32_t> n_pos;          // [G]
   int32_t* d_pack_order = nullptr;
+  std::vector<int32_t> pos_of;         // [tab_rows] the caller's measurement -> its position
+  int32_t* d_pos_of = nullptr;
+  float* d_ctab = nullptr;             // shell loop with calibration: e^alpha_n, beta_n by position
+  int64_t ctab_len = 0;
   // slab fits (prism_fit_init_slabs): per voxel of the whole volume its grid position, and per slice
   // its slab or slabs
   bool slabbed = false;
@@ -296,6 +300,7 @@ void fill_args(prism_handle* h) {
   a.table2 = h->d_table2;
   a.gtab = h->d_gtab;
   a.runs = h->d_runs;
+  a.ctab = h->d_ctab;
   a.gparams = h->d_gparams;
   a.gU = h->d_gU;
   a.tile_ab = h->d_tile_ab;
@@ -358,6 +363,9 @@ void fill_args(prism_handle* h) {
   g.gparams = h->d_gparams;
   g.table = h->d_table;
   g.table2 = h->d_table2;
+  g.ctab = h->d_ctab;
+  g.pos_of = h->d_pos_of;
+  g.meas_of = h->d_pack_order;
   g.bscratch = h->d_bscratch;
   g.gdone = h->d_gdone;
   g.bs_off = h->d_bs_off;
@@ -450,7 +458,7 @@ int capture_graph(prism_handle* h, int iters, cudaGraphExec_t* out) {
 // caller's. Returns the number of leading pairs whose two measurements have b = 0.
 static int32_t meas_order(const prism_volume& v, bool cal, std::vector<int32_t>& order) {
   const int N = v.n_meas;
-  if (cal) {
+  if (cal) {   // table rows are indexed by measurement (alpha_n, beta_n); positions may be sorted (shell_runs)
     for (int n = 0; n < N; ++n) order.push_back(n);
     return 0;
   }
@@ -467,11 +475,12 @@ static int32_t meas_order(const prism_volume& v, bool cal, std::vector<int32_t>&
 // host-side constants.
 constexpr double kDpar = 1.7e-3, kDperp = 0.4e-3, kLog2e = 1.4426950408889634;
 
-// Shells of one group in table order `ord` (runs of equal b-value) with the constants of the shell
+// Shells of one group (runs of equal b-value in sorted order) with the constants of the shell
 // loop (ShellRun), each padded to an even count; `pos` receives the positions (-1: padding).
-static void shell_runs(const prism_volume& v, const int32_t* ord, std::vector<ShellRun>& runs,
-                       std::vector<int32_t>& pos) {
+static void shell_runs(const prism_volume& v, std::vector<ShellRun>& runs, std::vector<int32_t>& pos) {
   const int N = v.n_meas;
+  std::vector<int32_t> ord;
+  meas_order(v, false, ord);
   const size_t base = pos.size();
   for (int n = 0; n < N;) {
     const float b = v.bvals[ord[n]];
@@ -626,7 +635,7 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, const std:
     if (h->shell) {
       // shells and gradient rows of the group's positions (shell loop)
       gr.run_off = static_cast<int32_t>(h->runs.size());
-      shell_runs(v, ord, h->runs, h->pack_order);
+      shell_runs(v, h->runs, h->pack_order);
       gr.n_runs = static_cast<int32_t>(h->runs.size()) - gr.run_off;
       const int32_t* pos = h->pack_order.data() + h->pack_off[g];
       const int np = static_cast<int>(h->pack_order.size() - h->pack_off[g]), NPg = (np + 3) & ~3;
@@ -649,6 +658,13 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, const std:
     }
     const int npos = static_cast<int>(h->pack_order.size() - h->pack_off[g]);
     h->n_pos.push_back(npos);
+    gr.npos = npos;
+    gr.pos_off = static_cast<int32_t>(h->pack_off[g]);
+    h->pos_of.resize(tab + v.n_meas);
+    for (int i = 0; i < npos; ++i)
+      if (h->pack_order[h->pack_off[g] + i] >= 0) h->pos_of[tab + h->pack_order[h->pack_off[g] + i]] = i;
+    gr.ctab_off = static_cast<int32_t>(h->ctab_len);
+    if (h->shell && h->cal) h->ctab_len += 2 * static_cast<int64_t>((npos + 3) & ~3);
     tab += v.n_meas;
     gr.table2_off = static_cast<int32_t>(h->tab2_pairs);
     h->tab2_pairs += ((v.n_meas + 3) & ~3) / 2;
@@ -682,7 +698,7 @@ int build_plan(prism_handle* h, const prism_volume* vols, int n_vols, const std:
         t.ab_off = static_cast<int32_t>(aboff);
         t.n_meas = npos;
         yoff += static_cast<int64_t>((npos + 3) & ~3) * TV;
-        aboff += 2 * v.n_meas;
+        aboff += 2 * npos;
         h->tiles.push_back(t);
       }
       h->patches.push_back({tb, static_cast<int>(h->tiles.size())});
@@ -718,15 +734,17 @@ int upload(T* dst, const std::vector<T, A>& src, cudaStream_t st) {
     if (r_ != PRISM_OK) return r_; \
   } while (0)
 
-// The form of the shell loop that the fused kernel would take with one thread per voxel, 0 for none:
-// MSE without calibration, shells not switched off, and in every volume at most kMaxRuns b-value
-// shells (runs of equal b in sorted order). Shells of even length throughout: 1. With odd ones, padded:
-// 2, from kPadVoxels voxels on, where one thread per voxel is the automatic shape (four 56 x 61 x 47 and
-// smaller ellipsoids at N = 271, shells of 86, K = 3: fused kernel 152 -> 129 us; 48^3 at N = 271 with four
-// fibers 196 -> 119 us an iteration; below, a forced one-lane fit is bound by latency, not by its operations).
+// The form of the shell loop that the fused kernel takes (k_iter_fused's SHELL), 0 for none: shells not
+// switched off, in every volume at most kMaxRuns b-value shells (runs of equal b in sorted order), and
+// one or four lanes per voxel (sixteen: one pair per lane and chunk, nothing to share). With one lane,
+// MSE and no calibration the segmented forms: shells of even length throughout 1; with odd ones,
+// padded, 2, from kPadVoxels voxels on, where one thread per voxel is the automatic shape (four 56 x 61 x 47
+// and smaller ellipsoids at N = 271, shells of 86, K = 3: fused kernel 152 -> 129 us; 48^3 at N = 271 with
+// four fibers 196 -> 119 us an iteration; below, a forced one-lane fit is bound by latency, not by its
+// operations). Otherwise the general form, 3.
 constexpr int64_t kPadVoxels = 32768;
-int shells_apply(const prism_volume* vols, int n, const prism_options& o, int64_t V) {
-  if (!o.fused || o.loss != PRISM_LOSS_MSE || o.calibration || o.shells != 0) return 0;
+int shell_form(const prism_volume* vols, int n, const prism_options& o, int64_t V, int tpv) {
+  if (!o.fused || o.shells != 0 || tpv == 16) return 0;
   bool even = true;
   for (int g = 0; g < n; ++g) {
     std::vector<float> b(vols[g].bvals, vols[g].bvals + vols[g].n_meas);
@@ -741,7 +759,14 @@ int shells_apply(const prism_volume* vols, int n, const prism_options& o, int64_
     }
     if (runs > kMaxRuns) return 0;
   }
+  if (tpv != 1 || o.loss != PRISM_LOSS_MSE || o.calibration) return 3;
   return even ? 1 : (V >= kPadVoxels ? 2 : 0);
+}
+
+// Whether one thread per voxel would run the segmented shell loop (choose_shape).
+bool shells_apply(const prism_volume* vols, int n, const prism_options& o, int64_t V) {
+  const int f = shell_form(vols, n, o, V, 1);
+  return f == 1 || f == 2;
 }
 
 // Slabs of one whole volume (prism_fit_init_slabs): the volumes are slices [z0[g], z0[g] + nz) of its
@@ -765,7 +790,27 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   h->TV = h->NT / h->TPV;
   int64_t Vsum = 0;
   for (const MaskIndex& ix : idx) Vsum += ix.count;
-  h->shell = (h->TPV == 1) ? shells_apply(vols, n_vols, o, Vsum) : 0;
+  int dev = 0, sms = 0;
+  if (o.fused && (cudaGetDevice(&dev) != cudaSuccess ||
+                  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
+    cudaGetLastError();   // no usable device: the first allocation reports it, after the plan's own checks
+  // The local kernel (prism_local.cuh): several lanes per voxel, no neighbour priors, no calibration; with
+  // the Rician NLL, whose CTAs exchange sums, only where all tiles are resident at once. It takes the
+  // per-measurement step: its iterations are bound by latency, to which the shell loop's look-ups add
+  // (3,400 voxels at N = 193, K = 2: 87 us per 16 iterations, 108 with it).
+  if (o.fused && !h->cal && !h->nb && h->TPV > 1 && sms > 0) {
+    int64_t tiles = 0;
+    int nmax = 0, bps = 0;
+    for (int g = 0; g < n_vols; ++g) {
+      for (int32_t c : idx[g].pcount) tiles += (c + h->TV - 1) / h->TV;
+      nmax = std::max(nmax, (vols[g].n_meas + 3) & ~3);
+    }
+    h->local_smem = local_smem(h->K, h->TPV, nmax);
+    CK(h->ks->local_occupancy(o.loss, h->TPV, h->local_smem, &bps));
+    h->local_grid = static_cast<int>(std::min<int64_t>(tiles, static_cast<int64_t>(sms) * bps));
+    h->local = bps > 0 && (o.loss == PRISM_LOSS_MSE || h->local_grid == tiles);
+  }
+  h->shell = h->local ? 0 : shell_form(vols, n_vols, o, Vsum, h->TPV);
   // Host signals start their copy to the device before the plan is built: a copy needs only the
   // voxel count, and the DMA then runs while the host builds the plan. All copies start at once
   // when together they take at most a quarter of the free device memory; otherwise each volume
@@ -787,11 +832,6 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   }
   Plan pl;
   RC(build_plan(h, vols, n_vols, idx, pl));
-  int dev = 0, sms = 0;
-  if (o.fused) {
-    CK(cudaGetDevice(&dev));
-    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
   const int Vp = h->Vpad, Q = h->Q, G = h->G;
   // group reduction geometry
   h->max_e = 3 + (h->cal ? 2 * h->Nmax : 0);
@@ -805,15 +845,6 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
     h->max_split = std::max(h->max_split, ns);
   }
   const int nce = (h->max_e + kRedE - 1) / kRedE;
-  // The local kernel (prism_local.cuh): several lanes per voxel, no neighbour priors, no calibration;
-  // with the Rician NLL, whose CTAs exchange sums, only where all tiles are resident at once.
-  if (o.fused && !h->cal && !h->nb && h->TPV > 1) {
-    int bps = 0;
-    h->local_smem = local_smem(h->K, h->TPV, h->Nmax);
-    CK(h->ks->local_occupancy(o.loss, h->TPV, h->local_smem, &bps));
-    h->local_grid = std::min(h->ntiles, sms * bps);
-    h->local = bps > 0 && (o.loss == PRISM_LOSS_MSE || h->local_grid == h->ntiles);
-  }
   // allocations
   RC(h->alloc(&h->d_tiles, h->ntiles));
   RC(h->alloc(&h->d_tile_order, h->ntiles));
@@ -857,6 +888,8 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   RC(h->alloc(&h->d_slot_of_grid, pl.grid_tot));
   RC(h->alloc(&h->d_order, std::max<int64_t>(h->tab_rows, 1)));
   RC(h->alloc(&h->d_pack_order, h->pack_order.size()));
+  RC(h->alloc(&h->d_pos_of, h->pos_of.size()));
+  if (h->ctab_len) RC(h->alloc(&h->d_ctab, h->ctab_len));
   RC(h->alloc(&h->d_split_off, G));
   RC(h->alloc(&h->d_part2, static_cast<size_t>(tot_split) * h->max_e));
   RC(h->alloc(&h->d_counters, static_cast<size_t>(G) * nce));
@@ -965,6 +998,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
                       h->opt.connectivity, h->d_vflag, h->d_nbr, st));
   RC(upload(h->d_order, h->order, st));
   RC(upload(h->d_pack_order, h->pack_order, st));
+  RC(upload(h->d_pos_of, h->pos_of, st));
   RC(upload(h->d_gtab, h->gtab, st));
   RC(upload(h->d_runs, h->runs, st));
   RC(upload(h->d_split_off, split_off, st));
@@ -1045,12 +1079,17 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
     return fail(PRISM_E_NONFINITE, std::to_string(bad) + " voxel(s) with a non-finite signal or a non-positive b0 mean");
   CK(h->ks->transform(h->ia, 0, h->ntiles, st));
   CK(launch_adam_constants(h->ia, st));
+  if (h->d_ctab) {   // the identity calibration by position; padding stays 0
+    CK(cudaMemsetAsync(h->d_ctab, 0, sizeof(float) * h->ctab_len, st));
+    CK(launch_table_refresh(h->ga, h->ia, st));
+  }
   // launch geometry of the fused kernel
   const int NW = h->NT / 32;
   const size_t ring = static_cast<size_t>(kStages) * kChunk * (kFusedThreads / h->TPV) * sizeof(float);
   if (h->shell) {
     h->fused_smem = 3 * static_cast<size_t>(h->Nmax) * sizeof(float) + kMaxRuns * sizeof(ShellRun) +
-                    static_cast<size_t>(kShellCols) * kFusedThreads * sizeof(float) + ring;
+                    static_cast<size_t>(kShellCols) * kFusedThreads * sizeof(float) + ring +
+                    (h->cal ? (2 * static_cast<size_t>(h->Nmax) + kNGrid + static_cast<size_t>(NW) * 2 * h->Nmax) * sizeof(float) : 0);
   } else {
     h->fused_smem = static_cast<size_t>(h->Nmax) * sizeof(MeasRow) + ring +
                     (h->cal ? kNGrid * sizeof(float) + static_cast<size_t>(NW) * 2 * h->Nmax * sizeof(float) : 0);
@@ -1066,35 +1105,40 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   return PRISM_OK;
 }
 
+// Lanes per voxel of a fit, by measurement on GB300 (cubes of bundle and crossing phantoms, N = 96-364,
+// K = 3 and 5; us an iteration). `shell`: one thread per voxel would run the segmented shell loop.
 int choose_shape(const prism_options& o, int64_t V, bool shell, int* tpv, int* nt) {
-  // Measured on GB300 (bundle phantoms, K = 3 and 5, MSE and NLL): sixteen lanes per voxel
-  // below 2,048 voxels, four below 32,768 (1.1-1.9x faster than one). Above, one thread per
-  // voxel, except where its 128-voxel tiles come to about one wave of the SMs' resident CTAs
-  // (0.75-1.25 waves: the last tiles then run nearly alone); four lanes then balance the SMs
-  // better (40^3: 7-19 % faster; calibrated, 14-19 %). Where the shell loop applies (`shell`:
-  // it needs one thread per voxel) four lanes pay only above one wave: 40^3 (0.82 waves) 20 %
-  // slower than the shell loop, 45^3 (1.17 waves) 2 % faster, 47^3 (1.33 waves) 4 % slower.
+  // No neighbour priors and no calibration: the local kernel with four or sixteen lanes. Sixteen below
+  // 1,400 voxels (10^3 at N = 96: 3.75 against 3.88 with four, 12^3 4.8 and 4.2; NLL 8.7 and 8.4, 10.7 and
+  // 9.3), one from 32,768 on (28^3 at N = 96: 15.1 with four, 20.4 with one; 32^3 23.0 and 21.0).
   const bool local = o.fused && !o.calibration && !(o.lam_sp > 0.f) && !(o.lam_dir > 0.f);
   if (o.threads_per_voxel) {
     *tpv = o.threads_per_voxel;
   } else if (V < (local ? 1400 : 2048)) {
-    // (without neighbour priors and calibration the local kernel runs: 10^3 voxels at N = 96 3.75 us
-    // an iteration with sixteen lanes, 3.88 with four, 12^3 4.8 and 4.2; NLL 8.7 and 8.4, 10.7 and 9.3)
     *tpv = 16;
-  } else if (V < 32768) {
+  } else if (V < ((shell && !local) ? 16384 : 32768)) {
+    // the segmented shell loop with one lane is ahead from 16,384 voxels on (N = 288: 24^3 36.2 against 35.0
+    // with four, 26^3 36.7 and 38.7, 28^3 43.9 and 60.4; five fibers 28^3 60 and 69), the other forms are
+    // level with four lanes up to 32^3 (NLL, N = 288: 28^3 62.5 and 60.6, 32^3 62.8 and 71.3)
     *tpv = 4;
   } else {
+    // One lane, except just above a whole wave of its 128-voxel tiles, whose second wave is then nearly
+    // empty: four lanes up to 1.45 waves of the NLL and calibrated kernels (NLL at N = 288, three CTAs per SM:
+    // 0.94 waves 102 with four against 81 with one, 1.10 119 and 142, 1.27 133 and 146, 1.46 150 and
+    // 148; five fibers 1.10 190 and 245, 1.46 239 and 249). The segmented shell loop gains too much from
+    // one lane (44^3, 1.09 waves, 120 and 118). The MSE without it (more than 16 b-values): 0.75 to 1.25.
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
       cudaGetLastError();
       sms = 152;
     }
-    // CTAs per SM of the one-thread-per-voxel kernel (3 for five fibers, NLL or calibration)
-    const int occ = (o.K >= 5 || o.loss == PRISM_LOSS_NLL || o.calibration) ? 3 : 4;
+    const bool heavy = o.loss == PRISM_LOSS_NLL || o.calibration;
+    const int occ = (o.K >= 5 || heavy) ? 3 : 4;   // CTAs per SM of the one-lane kernel
     const double waves = static_cast<double>(V) / 128.0 / (static_cast<double>(sms) * occ);
-    *tpv = (waves > (shell ? 1.0 : 0.75) && waves <= 1.25) ? 4 : 1;
+    const bool four = heavy ? (waves > 1.0 && waves <= 1.45) : (!shell && waves > 0.75 && waves <= 1.25);
+    *tpv = four ? 4 : 1;
   }
-  // the fused kernel is compiled for 128-thread CTAs (4 resident per SM)
+  // the fused kernel is compiled for 128-thread CTAs
   *nt = o.fused ? 128 : (o.cta_threads ? o.cta_threads : 128);
   return PRISM_OK;
 }
@@ -1311,7 +1355,7 @@ int fit_init(const prism_volume* vols, int n_vols, const prism_options* opt, con
     V += idx.back().count;
   }
   int tpv = 1, nt = 128;
-  choose_shape(o, V, shells_apply(vols, n_vols, o, V) != 0, &tpv, &nt);
+  choose_shape(o, V, shells_apply(vols, n_vols, o, V), &tpv, &nt);
   if (o.autotune && o.fused && !slabs) {
     int shells = o.shells;
     autotune_shape(vols, n_vols, idx, o, st, &tpv, &shells);
@@ -1788,7 +1832,7 @@ extern "C" int prism_fit_init_slabs(const prism_volume* vol, int32_t slab, int32
     w.init = init;
     const std::vector<MaskIndex> wi{src.index};
     int tpv = 1, nt = 128, shells = o.shells;
-    choose_shape(o, V, shells_apply(&w, 1, o, V) != 0, &tpv, &nt);
+    choose_shape(o, V, shells_apply(&w, 1, o, V), &tpv, &nt);
     autotune_shape(&w, 1, wi, o, st, &tpv, &shells);
     o.threads_per_voxel = tpv;
     o.shells = shells;

@@ -465,7 +465,7 @@ __device__ __forceinline__ void group_reduce_block(const IterArgs& a, const Grou
   const GroupDev gr = a.groups[gi];
   const int nsplit = (gr.ntiles + g.split_tiles - 1) / g.split_tiles;
   if (s >= nsplit) return;
-  const int E = 3 + ((gr.calib && (what & 2)) ? 2 * gr.N : 0);
+  const int E = 3 + ((gr.calib && (what & 2)) ? 2 * gr.npos : 0);
   if (ce * kRedE >= E) return;
   const int el = threadIdx.x % kRedE, sub = threadIdx.x / kRedE, e = ce * kRedE + el;
   const int per = (g.split_tiles + 3) / 4, first = s * g.split_tiles + sub * per;
@@ -481,7 +481,7 @@ __device__ __forceinline__ void group_reduce_block(const IterArgs& a, const Grou
       const float* src = a.tile_ab + a.tiles[t0].ab_off + (e - 3);   // a group's tiles follow one another
       float hi = 0.f, lo = 0.f;
 #pragma unroll 8
-      for (int t = 0; t < n; ++t) two_sum(hi, lo, src[static_cast<size_t>(t) * 2 * gr.N]);
+      for (int t = 0; t < n; ++t) two_sum(hi, lo, src[static_cast<size_t>(t) * 2 * gr.npos]);
       acc = static_cast<double>(hi) + static_cast<double>(lo);
     }
   }
@@ -516,8 +516,11 @@ __device__ __forceinline__ void group_reduce_block(const IterArgs& a, const Grou
     } else if (e == 2) {
       if (what & 1) g.gprior[gi] = tot;
     }
-    else if (e < 3 + gr.N) g.gred[gr.gp_off + 4 + (e - 3)] = tot;
-    else g.gred[gr.gp_off + 4 + gr.N4 + (e - 3 - gr.N)] = tot;
+    else {   // the partials run over positions, the gradients over the caller's measurements
+      const bool beta = e >= 3 + gr.npos;
+      const int n = g.meas_of[gr.pos_off + e - 3 - (beta ? gr.npos : 0)];
+      if (n >= 0) g.gred[gr.gp_off + 4 + (beta ? gr.N4 : 0) + n] = tot;
+    }
   }
   if (threadIdx.x == 0) g.counters[gi * nce + ce] = 0;
 }
@@ -715,12 +718,16 @@ __global__ void __launch_bounds__(kGroupThreads) k_group_adam(const IterArgs a, 
           const int n = (i < 4 + N4) ? i - 4 : i - 4 - N4;
           MeasRow* row = g.table + gr.table_off + n;
           float* pr = reinterpret_cast<float*>(g.table2 + gr.table2_off + n / 2) + (n & 1);
+          const int pos = g.pos_of[gr.table_off + n];
+          float* pc = g.ctab + gr.ctab_off + pos / 2 * 4 + (pos & 1);
           if (i < 4 + N4) {
             row->A = expf(xn);
             pr[2 * kPairFieldA] = row->A;
+            if (g.ctab) pc[0] = row->A;
           } else {
             row->beta = xn;
             pr[2 * kPairFieldBeta] = xn;
+            if (g.ctab) pc[2] = xn;
           }
         }
       }
@@ -762,6 +769,12 @@ __global__ void k_table_refresh(const GroupArgs g, const IterArgs a) {
     float* pr = reinterpret_cast<float*>(g.table2 + gr.table2_off + n / 2) + (n & 1);
     pr[2 * kPairFieldA] = row->A;
     pr[2 * kPairFieldBeta] = row->beta;
+    if (g.ctab) {
+      const int pos = g.pos_of[gr.table_off + n];
+      float* pc = g.ctab + gr.ctab_off + pos / 2 * 4 + (pos & 1);
+      pc[0] = row->A;
+      pc[2] = row->beta;
+    }
   }
 }
 

@@ -90,7 +90,9 @@ struct GroupDev {
   int32_t run_off;     // first ShellRun of the group (shell loop)
   int32_t n_runs;      // its shells
   int32_t gtab_off;    // float offset of the group's gradient table: [NP / 2][4] {g_x, g_y} pairs, then [NP] g_z
-  int32_t pad_;
+  int32_t npos;        // positions of the packed signal (Tile::n_meas)
+  int32_t pos_off;     // first of them in the position -> measurement table
+  int32_t ctab_off;    // float offset of the group's calibration table: per pair {A, A, beta, beta} (shell loop)
   int64_t vox0;        // first voxel of the group in mask order
   int64_t yhat_off;    // its first row in the caller's y_hat
 };
@@ -124,6 +126,7 @@ struct IterArgs {
   const MeasPair* table2;  // the same, paired (see MeasPair)
   const float* gtab;       // per group gradient directions in table order (shell loop; see GroupDev)
   const ShellRun* runs;    // per group shells in table order (shell loop)
+  const float* ctab;       // per group e^alpha_n and beta_n by position (shell loop with calibration)
   const float* gparams;    // packed group parameters
   float* gU;               // [Vpad] dJ/dU(x)
   float* tile_ab;          // per-tile [2][N] alpha / beta gradient partials

@@ -932,6 +932,135 @@ __device__ __forceinline__ void data_grad_shell(const Vox<K>& P, const Acc<K>& A
   gu = gin * sS;
 }
 
+// The shell loop's general form (MSE or Rician NLL, with or without calibration, any lanes per voxel): the
+// pairs are taken one after the other (a lane its own share of them), the shell of a pair looked up as
+// it changes, b = 0 treated as any other b (c' = 0 gives f_in e1 = f_in and (1 - f_in) p = 1 - f_in),
+// and the second measurement of an odd shell's last pair masked. With calibration (Eq. 6) the
+// prediction is beta_n - (A_n B) s with s = -S, and the accumulators take q = -r A_n B (the other sign
+// than without: shell_sums). Against the per-measurement step (step2) it saves a third of the packed operations
+// and two thirds of the table's bytes: XXSHELL3XX.
+struct ShellExtra {
+  float l2, l3;   // Rician NLL: sum y |y_hat| Q, sum L
+  float2 u;       // calibration: sum of q s (dJ/dU unscaled, negated)
+  int podd;       // the pair whose second measurement is padding (-1: none in this shell)
+};
+
+template <int K>
+__device__ __forceinline__ void shell_close_any(ShellState<K>& S, const ShellRun& R, float* col) {
+  using SR = ShellRows<K>;
+  constexpr int C = kFusedThreadsShell;
+  const float q = S.Qs.x + S.Qs.y;
+  col[SR::gcsf * C] = fmaf(R.ecsf, q, col[SR::gcsf * C]);
+  col[SR::ggm * C] = fmaf(R.egm, q, col[SR::ggm * C]);
+  col[SR::gres * C] = fmaf(R.eres, q, col[SR::gres * C]);
+  S.Qs = make_float2(0.f, 0.f);
+}
+
+template <int K>
+__device__ __forceinline__ void shell_advance(ShellState<K>& S, ShellExtra& X, const ShellRun* runs, int n_runs, int p,
+                                              float* col) {
+  using SR = ShellRows<K>;
+  constexpr int C = kFusedThreadsShell;
+  while (p >= S.pend && S.ri + 1 < n_runs) {
+    if (S.ri >= 0) shell_close_any(S, runs[S.ri], col);
+    const ShellRun R = runs[++S.ri];
+    S.pend = R.p1;
+    X.podd = R.odd ? R.p1 - 1 : -1;
+    const float T0 = fmaf(col[SR::fcsf * C], R.ecsf, fmaf(col[SR::fgm * C], R.egm, col[SR::fres * C] * R.eres));
+    S.c0 = dup2(-col[SR::s0 * C] * T0);
+    S.Kp = dup2(col[SR::c0 * C] + R.nbperp);
+  }
+}
+
+// One pair p at table row {gx, gy}, {gz}; `ab` = {A, A, beta, beta} of the pair (calibration), nB2 = -B.
+template <int K, int LOSS, bool CAL>
+__device__ __forceinline__ void shell_step_any(ShellState<K>& S, ShellExtra& X, const ShellRun* runs, int n_runs, int p,
+                                               float* col, float4 gxy, float2 gz, float2 y, float4 ab, float2 nB2,
+                                               float inv_s2, const float4* bess, float2* uo, float2* ro) {
+  if (p >= S.pend) shell_advance(S, X, runs, n_runs, p, col);
+  const float2 nrho = make_float2(-kRho, -kRho), rho = make_float2(kRho, kRho);
+  const float2 gx = lo2(gxy), gy = hi2(gxy);
+  float2 cp[K], e1[K], pp[K];
+  float2 s = S.c0;   // -S
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    cp[k] = __ffma2_rn(S.dp[k][0], gx, __ffma2_rn(S.dp[k][1], gy, __fmul2_rn(S.dp[k][2], gz)));
+    const float2 m = __ffma2_rn(cp[k], cp[k], S.nlfin);
+    e1[k] = make_float2(ex2f_(-m.x), ex2f_(-m.y));
+    pp[k] = ex2_2(__ffma2_rn(nrho, m, S.Kp));
+    s = __ffma2_rn(S.nf[k], __fadd2_rn(e1[k], pp[k]), s);
+  }
+  const float my = (p == X.podd) ? 0.f : 1.f;
+  float2 r, q;   // r = -dL/dy_hat (MSE: y - y_hat)
+  float2 ABn = make_float2(1.f, 1.f);
+  if constexpr (CAL) ABn = __fmul2_rn(lo2(ab), nB2);
+  if constexpr (LOSS == kLossMSE) {
+    r = CAL ? __ffma2_rn(make_float2(-1.f, -1.f), __ffma2_rn(ABn, s, hi2(ab)), y) : __fadd2_rn(y, s);
+    r.y *= my;
+    S.l1 = __ffma2_rn(r, r, S.l1);
+  } else {
+    const float2 yh = CAL ? __ffma2_rn(ABn, s, hi2(ab)) : make_float2(-s.x, -s.y);
+    r.x = -nll_lane(yh.x, y.x, inv_s2, 1.f, S.l1.x, X.l2, X.l3, bess);
+    r.y = -nll_lane(yh.y, y.y, inv_s2, my, S.l1.y, X.l2, X.l3, bess);
+  }
+  if constexpr (CAL) {
+    q = __fmul2_rn(r, ABn);
+    const float2 u = __fmul2_rn(make_float2(-q.x, -q.y), make_float2(-s.x, -s.y));
+    X.u = __fadd2_rn(X.u, u);
+    *uo = u;
+    *ro = r;
+  } else {
+    q = r;
+  }
+  S.Qs = __fadd2_rn(S.Qs, q);
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    S.ga[k] = __ffma2_rn(q, e1[k], S.ga[k]);
+    S.gb[k] = __ffma2_rn(q, pp[k], S.gb[k]);
+    const float2 inner = __ffma2_rn(rho, pp[k], e1[k]);
+    const float2 w = __fmul2_rn(__fmul2_rn(q, cp[k]), inner);
+    S.gd[k][0] = __ffma2_rn(w, gx, S.gd[k][0]);
+    S.gd[k][1] = __ffma2_rn(w, gy, S.gd[k][1]);
+    S.gd[k][2] = __ffma2_rn(w, gz, S.gd[k][2]);
+  }
+}
+
+// The lane's sums as (unscaled) accumulators of q = dJ/dS, in the shell loop's scaled forms (shell_fold).
+template <int K, int LOSS, bool CAL>
+__device__ __forceinline__ void shell_sums(ShellState<K>& S, const ShellExtra& X, const ShellRun* runs, float* col,
+                                           Acc<K>& A) {
+  using SR = ShellRows<K>;
+  constexpr int C = kFusedThreadsShell;
+  constexpr float sg = CAL ? 1.f : -1.f;
+  if (S.ri >= 0) shell_close_any(S, runs[S.ri], col);
+  A.gS0 = 0.f;
+  A.gcsf = sg * col[SR::gcsf * C];
+  A.ggm = sg * col[SR::ggm * C];
+  A.gres = sg * col[SR::gres * C];
+  A.l1 = S.l1.x + S.l1.y;
+  if constexpr (LOSS == kLossNLL) {
+    A.l2 = X.l2;
+    A.l3 = X.l3;
+  }
+  if constexpr (CAL) A.u = -(X.u.x + X.u.y);
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    A.gwa[k] = sg * (S.ga[k].x + S.ga[k].y);
+    A.gwb[k] = sg * (S.gb[k].x + S.gb[k].y);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) A.gd[k][c] = -sg * kTwoLn2 * (S.gd[k][c].x + S.gd[k][c].y);
+  }
+}
+
+// sum_n q_n T_n from the shell loop's sums (dJ/dS0).
+template <int K>
+__device__ __forceinline__ float shell_gS0(const Vox<K>& P, const Acc<K>& A) {
+  float g = P.f[0] * A.gcsf + P.f[1] * A.ggm + P.f[K + 2] * A.gres;
+#pragma unroll
+  for (int k = 0; k < K; ++k) g = fmaf(P.f[2 + k], A.gwa[k] + A.gwb[k], g);
+  return g;
+}
+
 // ===========================================================================
 // Fused iteration: one persistent kernel over the tile queue does synthesis,
 // calibration, data term, adjoint, priors, chain rule and the voxel Adam update.
@@ -1076,10 +1205,11 @@ constexpr int fused_min_blocks() {
   return ((K >= 5 || (K == 4 && SHELL)) || (fused_packed<K, TPV, LOSS, CAL>() && (CAL || LOSS == kLossNLL))) ? 3 : 4;
 }
 
-// SHELL: the shell loop (see ShellState) instead of the packed pairs; only for one thread per
-// voxel, the MSE and no calibration. 1: every group's shells have even length; 2: odd shells are
-// padded to even ones and their last pair takes its first measurement only (a kernel of its own:
-// the extra step costs the even case registers it needs).
+// SHELL: the shell loop (see ShellState) instead of the packed pairs. 1 and 2: one thread per voxel, the
+// MSE, no calibration, segments inside one shell; 1 with every group's shells of even length, 2 with odd
+// ones padded, whose last pair takes its first measurement only (a kernel of its own: the extra step
+// costs the even case registers it needs). 3: the general form (shell_step_any), for one or four lanes
+// per voxel and every data term.
 // GRAD: the gradient form behind prism_forward / prism_backward: the same pass over the signal, its
 // epilogue writes the raw-parameter gradient instead of updating, and no state advances.
 template <int K, int TPV, int LOSS, bool CAL, int SHELL = 0, bool GRAD = false>
@@ -1089,7 +1219,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
   constexpr int VW = 32 / TPV;              // voxels per warp
   constexpr bool PACKED = fused_packed<K, TPV, LOSS, CAL>();
   constexpr bool HOIST = PACKED && TPV == 1 && K <= 3 && LOSS == kLossMSE && !CAL;
-  static_assert(!SHELL || (TPV == 1 && LOSS == kLossMSE && !CAL), "the shell loop covers one thread per voxel, MSE, no calibration");
+  static_assert(SHELL == 0 || SHELL == 3 || (TPV == 1 && LOSS == kLossMSE && !CAL), "forms 1 and 2: one thread per voxel, MSE, no calibration");
   using SR = ShellRows<K>;
   // ring stages per warp (kStages; a ring as deep in bytes for four or sixteen lanes per voxel,
   // kStages * TPV, measured 0-25 % slower)
@@ -1100,7 +1230,8 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
   MeasRow* s_tab = reinterpret_cast<MeasRow*>(smem);
   // shell loop: [3][Nmax] gradient rows, kMaxRuns shells, the threads' columns, then the ring
   float* s_g = reinterpret_cast<float*>(smem);
-  ShellRun* s_runs = reinterpret_cast<ShellRun*>(s_g + 3 * a.Nmax);
+  float* s_cal = s_g + 3 * a.Nmax;           // calibration: [Nmax / 2] {A, A, beta, beta}
+  ShellRun* s_runs = reinterpret_cast<ShellRun*>(s_cal + (CAL ? 2 * a.Nmax : 0));
   float* s_col = reinterpret_cast<float*>(s_runs + kMaxRuns);
   float* s_ring = SHELL ? s_col + SR::count * kFusedThreads
                         : reinterpret_cast<float*>(s_tab + a.Nmax);       // [NW][NS][kChunk][VW]
@@ -1185,9 +1316,14 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         if (SHELL) {
           const uint32_t gb = 3u * static_cast<uint32_t>(NP) * 4u;
           const uint32_t rb = static_cast<uint32_t>(gr.n_runs) * static_cast<uint32_t>(sizeof(ShellRun));
-          mbar_expect_tx(&s_bar, gb + rb);
+          const uint32_t cb = CAL ? 2u * static_cast<uint32_t>(NP) * 4u : 0u;
+          mbar_expect_tx(&s_bar, gb + rb + cb + (CAL ? kNGrid * 4u : 0u));
           tma_bulk_g2s(s_g, a.gtab + gr.gtab_off, gb, &s_bar);
           tma_bulk_g2s(s_runs, a.runs + gr.run_off, rb, &s_bar);
+          if (CAL) {
+            tma_bulk_g2s(s_cal, a.ctab + gr.ctab_off, cb, &s_bar);
+            tma_bulk_g2s(s_blr, a.gparams + gr.gp_off + 4 + 2 * gr.N4, kNGrid * 4u, &s_bar);
+          }
         } else if (PACKED) {
           const uint32_t tb = static_cast<uint32_t>(NP / 2 * sizeof(MeasPair));
           mbar_expect_tx(&s_bar, tb + (CAL ? kNGrid * 4u : 0u));
@@ -1258,9 +1394,13 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
     VoxP<K> DP;
     AccP<K> AP;
     ShellState<K> SS;
+    ShellExtra SX;
     float* col = s_col + tid;
     if constexpr (SHELL) {
       shell_begin(SS, P, col);
+      SX.l2 = SX.l3 = 0.f;
+      SX.u = make_float2(0.f, 0.f);
+      SX.podd = -1;
     } else if constexpr (PACKED) {
       voxp_init<K>(P, DP, AP);
     }
@@ -1281,7 +1421,54 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         failed = true;
       }
       const int cnt = min(kChunk, N - j * kChunk);
-      if constexpr (SHELL) {
+      if constexpr (SHELL == 3) {
+        const float2* __restrict__ yc2 = reinterpret_cast<const float2*>(ring + s * (kChunk * VW)) + lv;
+        const float4* __restrict__ gxy = reinterpret_cast<const float4*>(s_g);
+        const float2* __restrict__ gz2 = reinterpret_cast<const float2*>(s_g + 2 * NP);
+        const float4* __restrict__ cal4 = reinterpret_cast<const float4*>(s_cal);
+        const int pc0 = j * (kChunk / 2), npc = min(kChunk / 2, N / 2 - pc0);   // this chunk's pairs
+        const float2 nB2 = make_float2(-B, -B);
+        if constexpr (CAL) {
+          // two steps (four measurements) of each lane per reduce-scatter of the alpha / beta partials
+          // over the VW lanes that share js; the sums hold the negated values, so the stores negate
+          constexpr int LVW = (VW == 8) ? 3 : (VW == 16) ? 4 : 5;
+#pragma unroll 1
+          for (int i = 0; i < kChunk / 2 / TPV; i += 2) {
+            float uu[4], rv[4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int pi = (i + h) * TPV + js, p = pc0 + pi;
+              float2 u = make_float2(0.f, 0.f), r = make_float2(0.f, 0.f);
+              if (act && pi < npc)
+                shell_step_any<K, LOSS, true>(SS, SX, s_runs, gr.n_runs, p, col, gxy[p], gz2[p], yc2[pi * VW], cal4[p],
+                                              nB2, inv_s2, s_bess, &u, &r);
+              uu[2 * h] = u.x;
+              uu[2 * h + 1] = u.y;
+              rv[2 * h] = r.x;
+              rv[2 * h + 1] = r.y;
+            }
+            const float su = warp_scatter_sum<4, VW>(uu);
+            const float sr = warp_scatter_sum<4, VW>(rv);
+            const int q = lv >> (LVW - 2);
+            const int n = 2 * ((i + (q >> 1)) * TPV + js) + (q & 1);
+            if ((lv & ((VW >> 2) - 1)) == 0 && n < 2 * npc) {
+              s_ab[(warp * 2) * a.Nmax + j * kChunk + n] = -su;
+              s_ab[(warp * 2 + 1) * a.Nmax + j * kChunk + n] = -sr;
+            }
+          }
+        } else if (act) {
+#pragma unroll ((K >= 4 || LOSS == kLossNLL) ? 1 : 2)
+          for (int pi = js; pi < npc; pi += TPV) {
+            const int p = pc0 + pi;
+            shell_step_any<K, LOSS, false>(SS, SX, s_runs, gr.n_runs, p, col, gxy[p], gz2[p], yc2[pi * VW],
+                                           make_float4(1.f, 1.f, 0.f, 0.f), nB2, inv_s2, s_bess, nullptr, nullptr);
+          }
+        }
+        __syncwarp();
+        ++g;
+        continue;
+      }
+      if constexpr (SHELL == 1 || SHELL == 2) {
         // pairs of this chunk, in segments that stay inside one shell (shells have even lengths)
         const float2* __restrict__ yc2 = reinterpret_cast<const float2*>(ring + s * (kChunk * VW)) + lv;
         // gradient rows: {g_x, g_y} of a pair as one float4, then the g_z pairs
@@ -1485,13 +1672,14 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
       ++g;
     }
     base += nch;
-    if constexpr (SHELL) {
+    if constexpr (SHELL == 1 || SHELL == 2) {
       if (act && SS.ri >= 0) shell_close(SS, s_runs[SS.ri], col);
     }
+    if constexpr (SHELL == 3) shell_sums<K, LOSS, CAL>(SS, SX, s_runs, col, A);
     if constexpr (TPV > 1) {
       // sum each voxel's lanes and hand the sums to one epilogue thread: voxel v of the tile
       // goes to thread v, so that a warp's epilogue serves 32 voxels, as with one thread per voxel
-      if constexpr (PACKED) accp_sums<K, LOSS, CAL>(AP, A);
+      if constexpr (PACKED && !SHELL) accp_sums<K, LOSS, CAL>(AP, A);
       acc_reduce_tpv<K, TPV, VW>(A);
       if (js == 0) acc_put<K>(A, s_acc, TV, vl);
       __syncthreads();
@@ -1516,14 +1704,17 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
       if constexpr (HOIST && !GRAD) load_moments<Q>(a, eslot, writer, mq, vq);
       transform<K>(th, P);
       if constexpr (TPV == 1) {
-        if constexpr (SHELL) {
+        if constexpr (SHELL == 3) {
+          A.gS0 = shell_gS0<K>(P, A);
+        } else if constexpr (SHELL) {
           shell_fold(P, SS, col, A);
         } else if constexpr (PACKED) {
           accp_fold<K, LOSS, CAL>(P, AP, A);
         }
       } else {
         acc_get<K>(A, s_acc, TV, tid);
-        if constexpr (PACKED) A.gS0 = acc_gS0<K>(P, A);
+        if constexpr (SHELL) A.gS0 = shell_gS0<K>(P, A);
+        else if constexpr (PACKED) A.gS0 = acc_gS0<K>(P, A);
         if constexpr (CAL) {
           unpack_coord(eact ? a.vcoord[eslot] : 0u, cx, cy, cz);
           B = expf(tri_eval(s_blr, tri_weights(cx, cy, cz, gr.nx, gr.ny, gr.nz)));
@@ -1540,8 +1731,9 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
       if (LOSS == kLossMSE) {
         dloss = A.l1 * gr.inv_M;
       } else {
-        dloss = 2.f * slog * N + 0.5f * inv_s2 * A.l1 - A.l3;
-        dsig = 2.f * N - inv_s2 * (A.l1 + 2.f * A.l2);
+        // (the measurements proper: N counts an odd shell's padding)
+        dloss = 2.f * slog * gr.N + 0.5f * inv_s2 * A.l1 - A.l3;
+        dsig = 2.f * gr.N - inv_s2 * (A.l1 + 2.f * A.l2);
       }
       // ---- priors
       ploss = priors<K, true>(a, P, eslot, gr.inv_M, xf_cur, gS0, gf, gd);

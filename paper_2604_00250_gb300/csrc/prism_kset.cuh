@@ -35,6 +35,25 @@ cudaError_t fused_occ(int nt, size_t smem, int* blocks) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, fn, nt, smem);
 }
 
+// The kernels of the shell loop's general form: four lanes per voxel, and one where forms 1 and 2 do
+// not apply.
+template <int TPV, int LOSS, bool CAL>
+struct Shell3 {
+  template <bool GRAD>
+  cudaError_t launch(const IterArgs& a, int grid, int nt, size_t smem, cudaStream_t st) const {
+    return fused_one<TPV, LOSS, CAL, 3, GRAD>(a, grid, nt, smem, st);
+  }
+  cudaError_t occupancy(int nt, size_t smem, int* blocks) const { return fused_occ<TPV, LOSS, CAL, 3>(nt, smem, blocks); }
+};
+template <typename F>
+cudaError_t shell3(int loss, int cal, int tpv, F go) {
+  if (tpv == 1 && loss == kLossMSE && cal) return go(Shell3<1, kLossMSE, true>{});
+  if (tpv == 1 && loss == kLossNLL) return cal ? go(Shell3<1, kLossNLL, true>{}) : go(Shell3<1, kLossNLL, false>{});
+  if (tpv == 4 && loss == kLossMSE) return cal ? go(Shell3<4, kLossMSE, true>{}) : go(Shell3<4, kLossMSE, false>{});
+  if (tpv == 4) return cal ? go(Shell3<4, kLossNLL, true>{}) : go(Shell3<4, kLossNLL, false>{});
+  return cudaErrorInvalidValue;
+}
+
 template <int TPV, bool GRAD>
 cudaError_t fused_tpv(const IterArgs& a, int loss, int cal, int grid, int nt, size_t smem, cudaStream_t st) {
   if (loss == kLossMSE) {
@@ -56,6 +75,7 @@ cudaError_t occ_tpv(int loss, int cal, int nt, size_t smem, int* blocks) {
 template <bool GRAD>
 cudaError_t fused_any(const IterArgs& a, int loss, int cal, int tpv, int shell, int grid, int nt, size_t smem,
                       cudaStream_t st) {
+  if (shell == 3) return shell3(loss, cal, tpv, [&](auto f) { return f.template launch<GRAD>(a, grid, nt, smem, st); });
   if (shell) {
     if (tpv != 1 || loss != kLossMSE || cal) return cudaErrorInvalidValue;
     return shell == 2 ? fused_one<1, kLossMSE, false, 2, GRAD>(a, grid, nt, smem, st)
@@ -76,6 +96,7 @@ cudaError_t l_fused(const IterArgs& a, int loss, int cal, int tpv, int shell, in
 }
 
 cudaError_t l_fused_occupancy(int loss, int cal, int tpv, int shell, int nt, size_t smem, int* blocks) {
+  if (shell == 3) return shell3(loss, cal, tpv, [&](auto f) { return f.occupancy(nt, smem, blocks); });
   if (shell) {
     if (tpv != 1 || loss != kLossMSE || cal) return cudaErrorInvalidValue;
     return shell == 2 ? fused_occ<1, kLossMSE, false, 2>(nt, smem, blocks)

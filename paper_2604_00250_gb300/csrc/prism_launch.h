@@ -40,8 +40,7 @@ struct StitchArgs {
 
 // Per-K launchers of the templated kernels (one translation unit per K).
 struct KernelSet {
-  // shell = 1 or 2: the shell loop of one thread per voxel, MSE, no calibration (2: with padded odd
-  // shells); grad = 1: the gradient form (no update)
+  // shell = 1..3: the shell loop (see k_iter_fused); grad = 1: the gradient form (no update)
   cudaError_t (*fused)(const IterArgs& a, int loss, int cal, int tpv, int shell, int grad, int grid, int nt,
                        size_t smem, cudaStream_t st);
   cudaError_t (*fused_occupancy)(int loss, int cal, int tpv, int shell, int nt, size_t smem, int* blocks);
@@ -79,6 +78,9 @@ struct GroupArgs {
   float* gparams;
   MeasRow* table;
   MeasPair* table2;   // the paired copy (its e^alpha_n and beta_n follow the rows)
+  float* ctab;                // the same by position (GroupDev::ctab_off), or null
+  const int32_t* pos_of;      // measurement -> position, rows as in `table`
+  const int32_t* meas_of;     // position -> measurement or -1 (GroupDev::pos_off)
   const int32_t* slot_of_grid;
   double* hist;               // [H][G] loss history
   int32_t hist_len;

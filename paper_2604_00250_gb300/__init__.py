@@ -53,12 +53,25 @@ def options(**kw):
 def _stream_ptr(stream):
     torch = _torch()
     if stream is None:
-        if torch.cuda.is_available():
-            return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-        return ctypes.c_void_p(0)
+        if not torch.cuda.is_initialized():
+            if not torch.cuda.is_available():
+                return ctypes.c_void_p(0)
+            torch.cuda.init()
+        # the current stream's handle without a Stream object (a few microseconds of every call)
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     if isinstance(stream, int):
         return ctypes.c_void_p(stream)
     return ctypes.c_void_p(stream.cuda_stream)
+
+
+def _f32(t):
+    """A contiguous float32 view of tensor `t` off the autograd graph, itself where it is one already."""
+    torch = _torch()
+    if t.requires_grad:
+        t = t.detach()
+    if t.dtype != torch.float32:
+        t = t.to(torch.float32)
+    return t if t.is_contiguous() else t.contiguous()
 
 
 def _host_f32(a, shape=None):
@@ -292,12 +305,12 @@ class Fitter:
         loss = torch.empty(self.n_groups, dtype=torch.float64, device="cuda")
         tp = gp = None
         if theta is not None:
-            theta = theta.detach().to(torch.float32).contiguous()
+            theta = _f32(theta)
             if not theta.is_cuda or tuple(theta.shape) != (self.n_vox, self.Q):
                 raise ValueError(f"theta must be a CUDA tensor [V={self.n_vox}, Q={self.Q}]")
             tp = ctypes.c_void_p(theta.data_ptr())
         if groups is not None:
-            groups = groups.detach().to(torch.float32).contiguous()
+            groups = _f32(groups)
             if not groups.is_cuda or tuple(groups.shape) != (self.n_group_params,):
                 raise ValueError(f"groups must be a CUDA tensor [{self.n_group_params}]")
             gp = ctypes.c_void_p(groups.data_ptr())
@@ -412,8 +425,8 @@ def _make_autograd():
 
         @staticmethod
         def forward(ctx, theta, groups, fitter):
-            th = theta.detach().to(torch.float32).contiguous()
-            gp = groups.detach().to(torch.float32).contiguous() if groups is not None else fitter.groups_device()
+            th = _f32(theta)
+            gp = _f32(groups) if groups is not None else fitter.groups_device()
             loss, _ = fitter.forward(th, gp)
             ctx.fitter = fitter
             ctx.token = fitter._fwd_token
@@ -428,9 +441,12 @@ def _make_autograd():
                 f.forward(*ctx.point)
                 ctx.token = f._fwd_token
             gth, gg = f.backward()
-            s = gout.to(torch.float32)
-            g_theta = (gth * s).to(ctx.dtypes[0]) if ctx.needs_input_grad[0] else None
-            g_groups = (gg * s).to(ctx.dtypes[1]) if ctx.needs_input_grad[1] else None
+            if gout.requires_grad:   # a graph through the factor (create_graph): out of place
+                gth, gg = gth * gout, gg * gout
+            else:                    # in place on the fresh gradients; the 0-dim factor takes their type
+                gth, gg = gth.mul_(gout), gg.mul_(gout)
+            g_theta = gth.to(ctx.dtypes[0]) if ctx.needs_input_grad[0] else None
+            g_groups = gg.to(ctx.dtypes[1]) if ctx.needs_input_grad[1] else None
             return g_theta, g_groups, None
 
     return PrismLoss

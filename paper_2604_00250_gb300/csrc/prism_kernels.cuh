@@ -938,7 +938,8 @@ __device__ __forceinline__ void data_grad_shell(const Vox<K>& P, const Acc<K>& A
 // and the second measurement of an odd shell's last pair masked. With calibration (Eq. 6) the
 // prediction is beta_n - (A_n B) s with s = -S, and the accumulators take q = -r A_n B (the other sign
 // than without: shell_sums). Against the per-measurement step (step2) it saves a third of the packed operations
-// and two thirds of the table's bytes: XXSHELL3XX.
+// and two thirds of the table's bytes: calibrated NLL phantom 537 -> 507 us, DiSCo1-shaped (five fibers, four
+// lanes) 206 -> 186.
 struct ShellExtra {
   float l2, l3;   // Rician NLL: sum y |y_hat| Q, sum L
   float2 u;       // calibration: sum of q s (dJ/dU unscaled, negated)

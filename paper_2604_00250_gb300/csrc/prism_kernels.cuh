@@ -722,6 +722,29 @@ __device__ __forceinline__ void data_grad(const Vox<K>& P, const Acc<K>& A, floa
   gfin = gin * sS;
 }
 
+// Block sums of v0 and, with TWO, v1 in a fixed order into out[0], out[1] (thread 0). FP64 adds are slow
+// on GB300 (about 16 cycles of the SM per warp), so the fused kernel reduces no more than it needs: the
+// whole objective as one value, dJ/dsigma for the Rician NLL only.
+template <bool TWO>
+__device__ __forceinline__ void block_reduce(double v0, double v1, double (*s_red)[3], double* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  v0 = warp_sum_d(v0);
+  if (TWO) v1 = warp_sum_d(v1);
+  if (lane == 0) {
+    s_red[warp][0] = v0;
+    if (TWO) s_red[warp][1] = v1;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < static_cast<int>(blockDim.x >> 5); ++w) {
+      v0 += s_red[w][0];
+      if (TWO) v1 += s_red[w][1];
+    }
+    out[0] = v0;
+    if (TWO) out[1] = v1;
+  }
+}
+
 __device__ __forceinline__ void block_reduce3(double v0, double v1, double v2, double (*s_red)[3],
                                               double* out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1103,28 +1126,25 @@ __device__ __forceinline__ void load_moments(const IterArgs& a, int slot, bool w
 template <bool GRAD>
 __device__ __forceinline__ void finalize_groups(const IterArgs& a) {
   constexpr int NW = kFusedThreads / 32;
-  __shared__ double s_part[NW][3];
+  __shared__ double s_part[NW][2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int step = *a.step;
   const float stepsz = a.adamc[0], isbc2 = a.adamc[1];
   const bool nll = a.loss_mode == kLossNLL;
   const bool by_warp = a.G >= NW;
   bool bad = false;
-  auto sums = [&](const GroupDev& gr, int first, int stride, double& l, double& sg, double& pr) {
-    l = sg = pr = 0.0;
+  auto sums = [&](const GroupDev& gr, int first, int stride, double& l, double& sg) {
+    l = sg = 0.0;
 #pragma unroll 8
     for (int t = gr.tile0 + first; t < gr.tile0 + gr.ntiles; t += stride) {
       const double* tr = a.tile_red + 4 * static_cast<size_t>(t);
       l += __ldcg(tr);
       if (nll) sg += __ldcg(tr + 1);
-      pr += __ldcg(tr + 2);
     }
     l = warp_sum_d(l);
     if (nll) sg = warp_sum_d(sg);
-    pr = warp_sum_d(pr);
   };
-  auto finish = [&](int gi, const GroupDev& gr, double l, double sg, double pr) {
-    const double J = l + pr;
+  auto finish = [&](int gi, const GroupDev& gr, double J, double sg) {
     a.gloss[gi] = J;
     if (!isfinite(J)) bad = true;
     if constexpr (GRAD) {
@@ -1153,28 +1173,26 @@ __device__ __forceinline__ void finalize_groups(const IterArgs& a) {
   if (by_warp) {
     for (int gi = warp; gi < a.G; gi += NW) {
       const GroupDev gr = a.groups[gi];
-      double l, sg, pr;
-      sums(gr, lane, 32, l, sg, pr);
-      if (lane == 0) finish(gi, gr, l, sg, pr);
+      double l, sg;
+      sums(gr, lane, 32, l, sg);
+      if (lane == 0) finish(gi, gr, l, sg);
     }
   } else {
     for (int gi = 0; gi < a.G; ++gi) {
       const GroupDev gr = a.groups[gi];
-      double l, sg, pr;
-      sums(gr, tid, kFusedThreads, l, sg, pr);
+      double l, sg;
+      sums(gr, tid, kFusedThreads, l, sg);
       if (lane == 0) {
         s_part[warp][0] = l;
         s_part[warp][1] = sg;
-        s_part[warp][2] = pr;
       }
       __syncthreads();
       if (tid == 0) {
         for (int w = 1; w < NW; ++w) {
           l += s_part[w][0];
           sg += s_part[w][1];
-          pr += s_part[w][2];
         }
-        finish(gi, gr, l, sg, pr);
+        finish(gi, gr, l, sg);
       }
       __syncthreads();
     }
@@ -1784,8 +1802,10 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
       if (CAL && writer) a.gU[eslot] = gUv;
     }
     // ---- tile partials (fixed-order reductions)
-    block_reduce3(writer ? static_cast<double>(dloss) : 0.0, writer ? static_cast<double>(dsig) : 0.0,
-                  writer ? static_cast<double>(ploss) : 0.0, s_red, a.tile_red + 4 * static_cast<size_t>(t));
+    // (the separate prior field, tile_red[2], stays zero)
+    block_reduce<LOSS == kLossNLL>(writer ? static_cast<double>(dloss) + static_cast<double>(ploss) : 0.0,
+                                   writer ? static_cast<double>(dsig) : 0.0, s_red,
+                                   a.tile_red + 4 * static_cast<size_t>(t));
     if (CAL) {
       for (int e = tid; e < 2 * N; e += kFusedThreads) {
         const int w2 = (e < N) ? 0 : 1;

@@ -105,7 +105,8 @@ typedef struct prism_options {
   int32_t fused;          /* 1: persistent fused iteration kernel; 0: plain unfused per-patch launches */
   int32_t use_graph;      /* 1: replay the fused iteration from a CUDA graph */
   int32_t threads_per_voxel; /* 1, 4 or 16 (measurements split across lanes); 0 = automatic: 16 below
-                                2,048 voxels (1,400 without neighbour priors and calibration), 4 below
+                                2,048 voxels (without neighbour priors and calibration: 1,400 with
+                                the MSE, 4,200 with the NLL), 4 below
                                 32,768 (16,384 where one lane takes the shell loop with the MSE), else
                                 1 except just above one wave of 128-voxel tiles with the NLL or
                                 calibration (then 4); prism_get_shape reports the choice */

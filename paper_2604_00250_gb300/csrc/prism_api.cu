@@ -1109,12 +1109,14 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
 // K = 3 and 5; us an iteration). `shell`: one thread per voxel would run the segmented shell loop.
 int choose_shape(const prism_options& o, int64_t V, bool shell, int* tpv, int* nt) {
   // No neighbour priors and no calibration: the local kernel with four or sixteen lanes. Sixteen below
-  // 1,400 voxels (10^3 at N = 96: 3.75 against 3.88 with four, 12^3 4.8 and 4.2; NLL 8.7 and 8.4, 10.7 and
-  // 9.3), one from 32,768 on (28^3 at N = 96: 15.1 with four, 20.4 with one; 32^3 23.0 and 21.0).
+  // 1,400 voxels with the MSE (10^3 at N = 96: 2.8 against 3.2 with four, 12^3 4.1 and 3.5; N = 288 3.4 and
+  // 5.5, 4.9 and 5.7) and below 4,200 with the NLL, whose measurements cost more (N = 96: 12^3 6.0 and 8.0,
+  // 16^3 8.1 and 7.5; N = 288 16^3 11.4 and 14.5; 20^3 no longer fits the chip at once); one from
+  // 32,768 on (28^3 at N = 96: 13.7 with four, 19.6 with one; 32^3 21.3 and 19.8).
   const bool local = o.fused && !o.calibration && !(o.lam_sp > 0.f) && !(o.lam_dir > 0.f);
   if (o.threads_per_voxel) {
     *tpv = o.threads_per_voxel;
-  } else if (V < (local ? 1400 : 2048)) {
+  } else if (V < (!local ? 2048 : o.loss == PRISM_LOSS_NLL ? 4200 : 1400)) {
     *tpv = 16;
   } else if (V < ((shell && !local) ? 16384 : 32768)) {
     // the segmented shell loop with one lane is ahead from 16,384 voxels on (N = 288: 24^3 36.2 against 35.0

@@ -5,17 +5,17 @@
 // shared memory and runs up to kMaxIters iterations on it. An iteration of the general fused kernel
 // at these sizes is a chain of latencies (launch, queue, tile and group records, staging, three
 // transforms, block-wide FP64 sums, the last CTA's tail): 13.8 us for an 8^3 patch, of which the
-// arithmetic is under 1 us. Here a voxel's lanes sit in one warp and all of them carry out the
-// voxel's chain rule and update on the summed accumulators, so that an iteration has no block
-// barrier and no hand-over at all; the redundant arithmetic uses issue slots that a small fit leaves
-// idle. Measured per iteration (GB300, MSE, K = 3, N = 96): 8^3 voxels 3.2 us (general kernel 13.8),
-// 16^3 4.7 us, 24^3 9.7 us (general kernel with one thread per voxel 17.5 and 18.1).
+// arithmetic is under 1 us. Here a voxel's lanes sit in one warp: all of them carry out the voxel's
+// chain rule on the summed accumulators (issue slots that a small fit leaves idle) and share its update,
+// so that an iteration of the MSE has no block barrier. Measured per iteration (GB300, MSE, K = 3, N = 96):
+// 8^3 voxels 2.3 us (general kernel 13.8), 16^3 4.1 and 24^3 8.9 us (general kernel with one thread per
+// voxel 17.5 and 18.1).
 //
-// Rician NLL: dJ/dsigma is a sum over the volume in each iteration. The warps of a volume's tiles
+// Rician NLL: dJ/dsigma is a sum over the volume in each iteration. The tiles of a volume
 // write their FP64 partials, count themselves in on a per-volume counter and wait for the count of
-// the iteration; then every warp takes the same fixed-order sum and updates its own copy of sigma.
+// the iteration; then every tile takes the same fixed-order sum and updates its own copy of sigma.
 // The launch is cooperative (every CTA resident, one tile each) and every wait has a limit. 16
-// volumes of 10^3 voxels: 75 -> 17 us an iteration (N = 96).
+// volumes of 10^3 voxels: 75 -> 12.8 us an iteration (N = 96).
 #pragma once
 
 #include "prism_kernels.cuh"
@@ -26,12 +26,16 @@ constexpr int kMaxIters = 32;      // iterations per launch (Adam's constants of
 constexpr int kLocalRow = 7;       // float4 per measurement pair in shared memory: the six that the
                                    // uncalibrated step reads and one of padding, so that eight lanes
                                    // reading eight neighbouring rows hit different banks
-constexpr int kLocalRed = 2 * (kFusedThreads / 32);   // partials per tile and iteration: {J, dJ/dsigma} per warp
+// partials per tile and iteration: J of every warp (MSE), or J and dJ/dsigma of the tile (NLL)
+constexpr int kLocalRed = kFusedThreads / 32;
+// Floats per voxel of a state array in shared memory: 4K + 5 rounded up to an odd multiple of 4, so that
+// eight voxels' rows fall into different banks, whether a lane reads a float or four.
+__host__ __device__ constexpr int local_stride(int K) { return K <= 1 ? 12 : K <= 3 ? 20 : 28; }
 
 __host__ __device__ inline size_t local_smem(int K, int tpv, int NP) {
   const size_t tv = kFusedThreads / tpv;
   return static_cast<size_t>(NP / 2) * kLocalRow * sizeof(float4) + static_cast<size_t>(NP) * tv * sizeof(float) +
-         3 * static_cast<size_t>(4 * K + 5) * tv * sizeof(float);
+         4 * static_cast<size_t>(local_stride(K)) * tv * sizeof(float);
 }
 
 __device__ __forceinline__ int ld_acquire(const int32_t* p) {
@@ -40,28 +44,32 @@ __device__ __forceinline__ int ld_acquire(const int32_t* p) {
   return v;
 }
 
-// Sum over a group's partials of one iteration (field 0: J, 1: dJ/dsigma_log), fixed order: strided
+// Sum over a group's partials of one iteration, fixed order: every NF-th value from `field` on, strided
 // over the warp's lanes, then a butterfly; every lane ends with it.
+template <int NF>
 __device__ __forceinline__ double local_group_sum(const IterArgs& a, const GroupDev& gr, int it, int field) {
   const double* red = a.tile_red + (static_cast<size_t>(it) * a.ntiles + gr.tile0) * kLocalRed + field;
   double s = 0.0;
 #pragma unroll 4
-  for (int i = threadIdx.x & 31; i < gr.ntiles * (kLocalRed / 2); i += 32) s += __ldcg(red + 2 * i);
+  for (int i = threadIdx.x & 31; i < gr.ntiles * (kLocalRed / NF); i += 32) s += __ldcg(red + NF * i);
   return warp_sum_d(s);
 }
 
 template <int K, int TPV, int LOSS>
 __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(const IterArgs a) {
-  constexpr int NF = K + 3, Q = 4 * K + 5, VW = 32 / TPV, TV = kFusedThreads / TPV, NW = kFusedThreads / 32;
+  constexpr int NF = K + 3, Q = 4 * K + 5, QS = local_stride(K), VW = 32 / TPV, TV = kFusedThreads / TPV, NW = kFusedThreads / 32;
   static_assert(TPV > 1, "one warp holds a voxel's lanes and several voxels");
   extern __shared__ __align__(16) unsigned char smem[];
   const int NPmax = a.Nmax;
   float4* s_tab = reinterpret_cast<float4*>(smem);                      // [NPmax / 2][kLocalRow]
   float* s_y = reinterpret_cast<float*>(s_tab + NPmax / 2 * kLocalRow);  // [NP][TV], packed as in HBM
-  float* s_st = s_y + static_cast<size_t>(NPmax) * TV;                   // [3][Q][TV]: theta, m, v
+  // [4][TV][QS]: theta, m, v and the gradient
+  float* s_st = s_y + static_cast<size_t>(NPmax) * TV;
   __shared__ uint64_t s_bar;
   __shared__ float s_ac[2 * kMaxIters];
   __shared__ int s_last;
+  __shared__ double s_ex[NW][2];   // NLL: the warps' partials, and the volume's sigma_log of the next iteration
+  __shared__ float s_sig;
   __shared__ float4 s_bess[(LOSS == kLossNLL) ? kBesselTab : 1];
   if constexpr (LOSS == kLossNLL) bessel_stage(s_bess);   // visible after the first tile's barriers
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -98,9 +106,10 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
     }
     for (int e = tid; e < Q * TV; e += kFusedThreads) {
       const size_t ix = static_cast<size_t>(e / TV) * Vp + tl.slot0 + e % TV;
-      s_st[e] = a.theta[ix];
-      s_st[Q * TV + e] = a.m[ix];
-      s_st[2 * Q * TV + e] = a.v[ix];
+      const int at = e % TV * QS + e / TV;
+      s_st[at] = a.theta[ix];
+      s_st[TV * QS + at] = a.m[ix];
+      s_st[2 * TV * QS + at] = a.v[ix];
     }
     if (!failed && !mbar_wait(&s_bar, phase)) {
       atomicOr(a.status, kStTimeout);
@@ -109,10 +118,10 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
     phase ^= 1;
     failed = __syncthreads_or(failed);
     const bool act = vl < tl.count;
-    float* st = s_st + vl;
+    float* st = s_st + vl * QS;
     float th[Q];
 #pragma unroll
-    for (int q = 0; q < Q; ++q) th[q] = st[q * TV];
+    for (int q = 0; q < Q; ++q) th[q] = st[q];
     Vox<K> P;
     transform<K>(th, P);
     float slog = 0.f, sgm = 0.f, sgv = 0.f;   // the volume's noise level and its moments (NLL)
@@ -160,30 +169,34 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
       float g[Q];
       chain_raw<K>(P, gS0, gf, gd, gfin, g);
       const float stepsz = s_ac[2 * it], isbc2 = s_ac[2 * it + 1];
-      float m[Q], v[Q];
+      // The voxel's lanes share the update, lane js taking parameters js, js + TPV, ...: every lane holds
+      // the whole gradient, but the update's 17 instructions per parameter are a quarter of an iteration.
+      if (js == 0) {
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        th[q] = st[q * TV];
-        m[q] = st[(Q + q) * TV];
-        v[q] = st[(2 * Q + q) * TV];
+        for (int q = 0; q < Q; ++q) st[3 * TV * QS + q] = g[q];
       }
-      __syncwarp();   // every lane of the voxel has read its state
+      __syncwarp();
 #pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        if (a.optimizer == 0) {
-          m[q] = fmaf(a.beta1, m[q], (1.f - a.beta1) * g[q]);
-          v[q] = fmaf(a.beta2, v[q], (1.f - a.beta2) * g[q] * g[q]);
-          th[q] -= stepsz * m[q] * frcp(fmaf(fsqrt(v[q]), isbc2, a.eps));
-        } else {
-          rprop_update(th[q], m[q], v[q], g[q], a.lr, a.eta_minus, a.eta_plus, a.step_min, a.step_max);
-        }
-        if (js == 0) {
-          st[q * TV] = th[q];
-          st[(Q + q) * TV] = m[q];
-          st[(2 * Q + q) * TV] = v[q];
+      for (int i = 0; i < (Q + TPV - 1) / TPV; ++i) {
+        float* p = st + js + TPV * i;
+        if (js + TPV * i < Q) {
+          float x = p[0], m = p[TV * QS], v = p[2 * TV * QS];
+          const float gq = p[3 * TV * QS];
+          if (a.optimizer == 0) {
+            m = fmaf(a.beta1, m, (1.f - a.beta1) * gq);
+            v = fmaf(a.beta2, v, (1.f - a.beta2) * gq * gq);
+            x -= stepsz * m * frcp(fmaf(fsqrt(v), isbc2, a.eps));
+          } else {
+            rprop_update(x, m, v, gq, a.lr, a.eta_minus, a.eta_plus, a.step_min, a.step_max);
+          }
+          p[0] = x;
+          p[TV * QS] = m;
+          p[2 * TV * QS] = v;
         }
       }
       __syncwarp();
+#pragma unroll
+      for (int q = 0; q < Q; ++q) th[q] = st[q];
       transform<K>(th, P);
       // the warp's partials of the objective and dJ/dsigma: lanes 0 .. VW - 1 hold its voxels
       double J = act ? static_cast<double>(dloss) + static_cast<double>(ploss) : 0.0;
@@ -193,52 +206,69 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
         J += __shfl_xor_sync(0xffffffffu, J, o);
         if (LOSS == kLossNLL) dS += __shfl_xor_sync(0xffffffffu, dS, o);
       }
-      double* red = a.tile_red + (static_cast<size_t>(it) * a.ntiles + t) * kLocalRed + 2 * warp;
-      if (lane == 0) {
-        red[0] = J;
-        if (LOSS == kLossNLL) red[1] = dS;
-      }
-      if (LOSS == kLossNLL) {
-        const bool leader = t == gr.tile0 && warp == 0;
-        int32_t* bar = a.gbar + tl.group;
+      double* red = a.tile_red + (static_cast<size_t>(it) * a.ntiles + t) * kLocalRed;
+      if (LOSS == kLossMSE) {
+        if (lane == 0) red[warp] = J;
+      } else {
+        // the tile's sums by its first warp, which alone counts the tile in, waits and takes the volume's
+        // sum (with every warp doing so, a third of the iteration went into the exchange)
         if (lane == 0) {
-          __threadfence();
-          atomicAdd(bar, 1);
+          s_ex[warp][0] = J;
+          s_ex[warp][1] = dS;
         }
-        if (it + 1 < n_it || leader) {
-          const int want = gr.ntiles * NW * (it + 1);
-          if (!failed) {
-            bool ok = true;
-            if (lane == 0) {
-              int polls = 0;
-              while (ld_acquire(bar) < want && polls < (1 << 21)) ++polls;
-              ok = polls < (1 << 21);
-              if (!ok) atomicOr(a.status, kStTimeout);
+        __syncthreads();
+        if (warp == 0) {
+          const bool leader = t == gr.tile0;
+          int32_t* bar = a.gbar + tl.group;
+          if (lane == 0) {
+            double sj = s_ex[0][0], ss = s_ex[0][1];
+            for (int w = 1; w < NW; ++w) {
+              sj += s_ex[w][0];
+              ss += s_ex[w][1];
             }
-            failed = __any_sync(0xffffffffu, !ok);
+            red[0] = sj;
+            red[1] = ss;
+            __threadfence();
+            atomicAdd(bar, 1);
           }
-          const float gsig = static_cast<float>(local_group_sum(a, gr, it, 1));
-          if (a.optimizer == 0) {
-            sgm = fmaf(a.beta1, sgm, (1.f - a.beta1) * gsig);
-            sgv = fmaf(a.beta2, sgv, (1.f - a.beta2) * gsig * gsig);
-            slog -= stepsz * sgm / fmaf(sqrtf(sgv), isbc2, a.eps);
-          } else {
-            rprop_update(slog, sgm, sgv, gsig, a.lr, a.eta_minus, a.eta_plus, a.step_min, a.step_max);
-          }
-          if (leader) {
-            const double tot = local_group_sum(a, gr, it, 0);
-            if (lane == 0) {
-              if (!isfinite(tot)) atomicOr(a.status, kStNonfinite);
-              a.hist[static_cast<size_t>((step + it) % a.hist_len) * a.G + tl.group] = tot;
-              if (it == n_it - 1) {
-                a.gloss[tl.group] = tot;
-                a.gparams_rw[gr.gp_off] = slog;
-                a.gm[gr.gp_off] = sgm;
-                a.gv[gr.gp_off] = sgv;
+          if (it + 1 < n_it || leader) {
+            const int want = gr.ntiles * (it + 1);
+            if (!failed) {
+              bool ok = true;
+              if (lane == 0) {
+                int polls = 0;
+                while (ld_acquire(bar) < want && polls < (1 << 21)) ++polls;
+                ok = polls < (1 << 21);
+                if (!ok) atomicOr(a.status, kStTimeout);
+              }
+              failed = __any_sync(0xffffffffu, !ok);
+            }
+            const float gsig = static_cast<float>(local_group_sum<kLocalRed>(a, gr, it, 1));
+            if (a.optimizer == 0) {
+              sgm = fmaf(a.beta1, sgm, (1.f - a.beta1) * gsig);
+              sgv = fmaf(a.beta2, sgv, (1.f - a.beta2) * gsig * gsig);
+              slog -= stepsz * sgm / fmaf(sqrtf(sgv), isbc2, a.eps);
+            } else {
+              rprop_update(slog, sgm, sgv, gsig, a.lr, a.eta_minus, a.eta_plus, a.step_min, a.step_max);
+            }
+            if (leader) {
+              const double tot = local_group_sum<kLocalRed>(a, gr, it, 0);
+              if (lane == 0) {
+                if (!isfinite(tot)) atomicOr(a.status, kStNonfinite);
+                a.hist[static_cast<size_t>((step + it) % a.hist_len) * a.G + tl.group] = tot;
+                if (it == n_it - 1) {
+                  a.gloss[tl.group] = tot;
+                  a.gparams_rw[gr.gp_off] = slog;
+                  a.gm[gr.gp_off] = sgm;
+                  a.gv[gr.gp_off] = sgv;
+                }
               }
             }
+            if (lane == 0) s_sig = slog;
           }
         }
+        __syncthreads();
+        if (it + 1 < n_it) slog = s_sig;
       }
     }
     __syncthreads();
@@ -246,9 +276,10 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
       const int v = e % TV;
       if (v >= tl.count) continue;
       const size_t ix = static_cast<size_t>(e / TV) * Vp + tl.slot0 + v;
-      a.theta[ix] = s_st[e];
-      a.m[ix] = s_st[Q * TV + e];
-      a.v[ix] = s_st[2 * Q * TV + e];
+      const int at = v * QS + e / TV;
+      a.theta[ix] = s_st[at];
+      a.m[ix] = s_st[TV * QS + at];
+      a.v[ix] = s_st[2 * TV * QS + at];
     }
   }
   // the last CTA: objective and history (MSE), step counter, the next constants, counters
@@ -262,7 +293,7 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
   if (LOSS == kLossMSE) {
     for (int i = warp; i < n_it * a.G; i += NW) {
       const int it = i / a.G, gi = i - it * a.G;
-      const double J = local_group_sum(a, a.groups[gi], it, 0);
+      const double J = local_group_sum<1>(a, a.groups[gi], it, 0);
       if (lane == 0) {
         if (!isfinite(J)) atomicOr(a.status, kStNonfinite);
         if (it == n_it - 1) a.gloss[gi] = J;

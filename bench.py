@@ -56,9 +56,9 @@ FLOPS_PER_B0_PAIR_SHELL = 4
 # scaled brain (traffic grows in proportion to the voxels), valid only for the kernel sources
 # whose SHA-256 (comments and blank lines left out, fused_sources_sha256) is
 # TRAFFIC_SOURCES_SHA256: any other hash reports the traffic as null.
-# 212,900 voxels: 384.4 and 384.1 MB in two launches (profiles/k_iter_fused_hcp_brain_dram_traffic.md).
-TRAFFIC_BYTES_PER_VOXEL_ITER = 1804.7
-TRAFFIC_SOURCES_SHA256 = "da28403d796e239c782cce8c6b9ec39009e819adfb07ce51d095c30ec0152732"
+# 212,900 voxels: 349.7 MB read and 36.1 MB written in one launch (profiles/k_iter_fused_hcp_brain_dram_traffic.md).
+TRAFFIC_BYTES_PER_VOXEL_ITER = 1812.3
+TRAFFIC_SOURCES_SHA256 = "2df9cd9177fa98b426c0f1b2a728cec677eb47acfd420da9526b4929cc20847d"
 FUSED_SOURCES = ("prism_kernels.cuh", "prism_device.cuh", "prism_kset.cuh", "bessel_fit.h", "prism_k3.cu")
 # FP32 lanes per SM on GB300 (4 sub-partitions x 32); the peak multiplies them by the device's
 # SM count, 2 flops per fused multiply-add and the maximum SM clock seen by nvidia-smi.
@@ -75,9 +75,14 @@ def flops_per_measurement(loss, cal, K, shell):
     y_hat = S0 T (1) and the NLL terms (71: z = y |y_hat| / sigma^2 2; Q(z) and L(z) from the
     fitted functions of 4/z, 55 -- two degree-12 Horner chains 48, the argument and scale 3,
     log terms 4; (y - |y_hat|)^2, y |y_hat| Q and L sums 9; dL/dy_hat 4; the rest 1) -- 85 + 28 K;
-    with calibration 94 + 28 K. Shell loop: 4 + 26 K (see FLOPS_PER_PAIR_SHELL)."""
+    with calibration 94 + 28 K; the count keeps the two degree-12 chains of the earlier two-branch
+    evaluation (the segment tables' degree-7 chains take 20 fewer). Shell loop: 4 + 26 K (see
+    FLOPS_PER_PAIR_SHELL); with the Rician NLL the residual and its square (3) give way to the NLL
+    terms (50: z 2, segment and argument 4, the degree-7 chains 28, Q and L 3, (y - |y_hat|)^2, y |y_hat| Q
+    and L sums 9, dL/dy_hat 4); calibration adds e^alpha_n B 1, y_hat 2, q 1, u and its sum 2, the partials'
+    reduce-scatter 1, and the residual's 1 with the MSE."""
     if shell:
-        return 4 + 26 * K
+        return 4 + 26 * K + (47 if loss == "nll" else 0) + (0 if not cal else 7 if loss == "nll" else 8)
     if loss == "mse":
         return (28 + 28 * K) if cal else (17 + 28 * K)
     return (94 + 28 * K) if cal else (85 + 28 * K)

@@ -416,7 +416,8 @@ def _make_autograd():
         theta ([V, Q] CUDA) and the packed group parameters (CUDA, or None for the handle's
         current ones, which then get no gradient). Forward: prism_forward (synthesis,
         calibration, data term, priors). Backward: prism_backward, the hand-written adjoint,
-        which recomputes the compartment exponentials instead of storing them (Sec. 2.1: every
+        which stores no compartment exponentials (a fused handle forms the gradient in the
+        forward's own pass, a plain one recomputes them; Sec. 2.1: every
         component is differentiable, so tissue and calibration parameters can be updated
         jointly). Each node keeps its own evaluation point; when the handle has evaluated
         another point since (a second node on the same Fitter, a step), backward first repeats

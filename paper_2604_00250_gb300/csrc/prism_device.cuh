@@ -151,7 +151,7 @@ struct IterArgs {
   // griddepcontrol, before it reads what the predecessor writes).
   int32_t pdl;
   int32_t n_it;            // iterations of this launch (k_iter_local; else 1)
-  int32_t* gbar;           // [G] arrivals of the current launch (k_iter_local, Rician NLL)
+  int32_t* gbar;           // [G] tiles counted in by the current launch (k_iter_local)
   float* gparams_rw;       // same array as gparams
   float* gm;               // group Adam moments (packed like gparams)
   float* gv;

@@ -55,6 +55,39 @@ __device__ __forceinline__ double local_group_sum(const IterArgs& a, const Group
   return warp_sum_d(s);
 }
 
+// A volume's objective of every iteration of the launch (MSE), by the CTA that finished the volume's last
+// tile: a warp takes kSums iterations at a time, so that their loads and butterflies overlap (one after the
+// other they are chains of about half a microsecond each). With the launch's last CTA doing all volumes' sums
+// one by one, 16 volumes of 10^3 voxels took 13.6 us an iteration instead of 7.0 and the 8^3 patch 48 instead of
+// 43 us a call of 16.
+constexpr int kSums = 4;
+__device__ __forceinline__ void local_objectives(const IterArgs& a, const GroupDev& gr, int group, int step) {
+  constexpr int NW = kFusedThreads / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = gr.ntiles * kLocalRed;
+  const size_t row = static_cast<size_t>(a.ntiles) * kLocalRed;
+  for (int i0 = warp; i0 < a.n_it; i0 += kSums * NW) {
+    const double* red = a.tile_red + i0 * row + static_cast<size_t>(gr.tile0) * kLocalRed;
+    double J[kSums];
+#pragma unroll
+    for (int u = 0; u < kSums; ++u) J[u] = 0.0;
+    for (int i = lane; i < n; i += 32) {
+#pragma unroll
+      for (int u = 0; u < kSums; ++u)
+        if (i0 + u * NW < a.n_it) J[u] += __ldcg(red + u * NW * row + i);
+    }
+#pragma unroll
+    for (int u = 0; u < kSums; ++u) J[u] = warp_sum_d(J[u]);
+#pragma unroll
+    for (int u = 0; u < kSums; ++u) {
+      const int it = i0 + u * NW;
+      if (lane != 0 || it >= a.n_it) continue;
+      if (!isfinite(J[u])) atomicOr(a.status, kStNonfinite);
+      if (it == a.n_it - 1) a.gloss[group] = J[u];
+      a.hist[static_cast<size_t>((step + it) % a.hist_len) * a.G + group] = J[u];
+    }
+  }
+}
+
 template <int K, int TPV, int LOSS>
 __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(const IterArgs a) {
   constexpr int NF = K + 3, Q = 4 * K + 5, QS = local_stride(K), VW = 32 / TPV, TV = kFusedThreads / TPV, NW = kFusedThreads / 32;
@@ -67,7 +100,7 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
   float* s_st = s_y + static_cast<size_t>(NPmax) * TV;
   __shared__ uint64_t s_bar;
   __shared__ float s_ac[2 * kMaxIters];
-  __shared__ int s_last;
+  __shared__ int s_last[2];   // this CTA counted in last: of the tile's volume (MSE), of the launch
   __shared__ double s_ex[NW][2];   // NLL: the warps' partials, and the volume's sigma_log of the next iteration
   __shared__ float s_sig;
   __shared__ float4 s_bess[(LOSS == kLossNLL) ? kBesselTab : 1];
@@ -272,6 +305,14 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
       }
     }
     __syncthreads();
+    if (tid == 0) {   // both counts in flight at once, under the stores below
+      __threadfence();
+      int left = 1, left_all = 1;
+      if (LOSS == kLossMSE) left = gr.ntiles - 1 - atomicAdd(a.gbar + tl.group, 1);
+      if (ti + static_cast<int>(gridDim.x) >= a.ntiles) left_all = static_cast<int>(gridDim.x) - 1 - atomicAdd(a.done, 1);
+      s_last[0] = left == 0;
+      s_last[1] = left_all == 0;
+    }
     for (int e = tid; e < Q * TV; e += kFusedThreads) {
       const int v = e % TV;
       if (v >= tl.count) continue;
@@ -281,28 +322,20 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
       a.m[ix] = s_st[TV * QS + at];
       a.v[ix] = s_st[2 * TV * QS + at];
     }
-  }
-  // the last CTA: objective and history (MSE), step counter, the next constants, counters
-  if (tid == 0) {
-    __threadfence();
-    s_last = (atomicAdd(a.done, 1) == static_cast<int>(gridDim.x) - 1);
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (LOSS == kLossMSE) {
-    for (int i = warp; i < n_it * a.G; i += NW) {
-      const int it = i / a.G, gi = i - it * a.G;
-      const double J = local_group_sum<1>(a, a.groups[gi], it, 0);
-      if (lane == 0) {
-        if (!isfinite(J)) atomicOr(a.status, kStNonfinite);
-        if (it == n_it - 1) a.gloss[gi] = J;
-        a.hist[static_cast<size_t>((step + it) % a.hist_len) * a.G + gi] = J;
+    if (LOSS == kLossMSE) {
+      __syncthreads();
+      if (s_last[0]) {
+        __threadfence();
+        local_objectives(a, gr, tl.group, step);
+        if (tid == 0) a.gbar[tl.group] = 0;
       }
     }
-  } else {
-    for (int i = tid; i < a.G; i += kFusedThreads) a.gbar[i] = 0;
   }
+  // the last CTA: step counter, the next constants, counters
+  __syncthreads();
+  if (!s_last[1]) return;
+  if (LOSS == kLossNLL)
+    for (int i = tid; i < a.G; i += kFusedThreads) a.gbar[i] = 0;
   if (tid < 2)
     const_cast<float*>(a.adamc)[tid] = adam_constant(tid, a.lr, a.beta1, a.beta2, static_cast<int64_t>(step) + n_it + 1);
   if (tid == 0) {

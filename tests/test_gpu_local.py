@@ -70,3 +70,28 @@ def test_gradient_against_the_oracle(lanes, K, N, loss):
     for name, sl in block_slices(K).items():
         assert normwise(g[:, sl], gr.numpy()[:, sl]) <= TOL_GRAD, name
 
+
+
+@pytest.mark.parametrize("n_vols", [3, 700])
+def test_objectives_of_many_volumes(n_vols):
+    """Each volume's objectives are summed by the CTA that finishes its last tile; 700 one-tile volumes are
+    more tiles than CTAs. A volume's history is that of its lone fit, bit for bit (same tiles, same sums)."""
+    import paper_2604_00250_gb300 as prism
+    from phantoms import schemes
+    sch = schemes.scheme_96(3)
+    vols = [P.random_volume((2, 2, 1 + i % 2), scheme=sch, seed=900 + i, mask_density=1.0) for i in range(n_vols)]
+    for i, v in enumerate(vols):
+        v.init = P.default_init(v.n_vox, 2, i).astype(np.float32)
+    kw = dict(K=2, loss="mse", patch_dim=4, threads_per_voxel=16)
+    at = np.cumsum([0] + [v.n_vox for v in vols])
+    with prism.Fitter(vols, prism.options(**kw)) as f:
+        f.step(37)
+        f.step(2)
+        h, J, th = f.loss_history(), f.loss(), f.params_host()
+    assert h.shape == (39, n_vols)
+    for i in (0, 1, n_vols // 2, n_vols - 1):
+        with prism.Fitter([vols[i]], prism.options(**kw)) as f:
+            f.step(39)
+            assert np.array_equal(f.loss_history()[:, 0], h[:, i])
+            assert f.loss()[0] == J[i]
+            assert np.array_equal(f.params_host(), th[at[i]:at[i + 1]])

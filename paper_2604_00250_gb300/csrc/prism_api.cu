@@ -861,7 +861,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   CK(cudaMemsetAsync(h->d_pg, 0, sizeof(float) * pg_len, st));
   RC(h->alloc(&h->d_gU, Vp));
   RC(h->alloc(&h->d_tile_ab, h->ab_len));
-  const size_t red_len = static_cast<size_t>(h->ntiles) * (h->local ? kMaxIters * kLocalRed : 4);
+  const size_t red_len = static_cast<size_t>(h->ntiles) * (h->local ? kMaxIters * (kLocalRed + 1) : 4);
   RC(h->alloc(&h->d_tile_red, red_len));
   RC(h->alloc(&h->d_nbr, static_cast<size_t>(o.connectivity) * Vp));
   RC(h->alloc(&h->d_vcoord, Vp));
@@ -894,8 +894,8 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   RC(h->alloc(&h->d_part2, static_cast<size_t>(tot_split) * h->max_e));
   RC(h->alloc(&h->d_counters, static_cast<size_t>(G) * nce));
   RC(h->alloc(&h->d_gdone, 1));
-  RC(h->alloc(&h->d_gbar, G));
-  CK(cudaMemsetAsync(h->d_gbar, 0, sizeof(int32_t) * G, st));
+  RC(h->alloc(&h->d_gbar, 2 * G));
+  CK(cudaMemsetAsync(h->d_gbar, 0, sizeof(int32_t) * 2 * G, st));
   CK(cudaMemsetAsync(h->d_gdone, 0, sizeof(int32_t), st));
   if (h->cal) {
     // per group [nx][ny][8] doubles for the separable bias-field adjoint

@@ -151,7 +151,7 @@ struct IterArgs {
   // griddepcontrol, before it reads what the predecessor writes).
   int32_t pdl;
   int32_t n_it;            // iterations of this launch (k_iter_local; else 1)
-  int32_t* gbar;           // [G] tiles counted in by the current launch (k_iter_local)
+  int32_t* gbar;           // [2][G] tiles counted in by the current launch (k_iter_local): per iteration (Rician NLL), at the end
   float* gparams_rw;       // same array as gparams
   float* gm;               // group Adam moments (packed like gparams)
   float* gv;

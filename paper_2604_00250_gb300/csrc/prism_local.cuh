@@ -12,10 +12,11 @@
 // voxel 17.5 and 18.1).
 //
 // Rician NLL: dJ/dsigma is a sum over the volume in each iteration. The tiles of a volume
-// write their FP64 partials, count themselves in on a per-volume counter and wait for the count of
-// the iteration; then every tile takes the same fixed-order sum and updates its own copy of sigma.
+// write their FP64 partials and count themselves in on a per-volume counter, before the chain rule and the
+// update; after these they wait for the count of the iteration; then every tile takes the same
+// fixed-order sum and updates its own copy of sigma.
 // The launch is cooperative (every CTA resident, one tile each) and every wait has a limit. 16
-// volumes of 10^3 voxels: 75 -> 12.8 us an iteration (N = 96).
+// volumes of 10^3 voxels: 75 -> 11.6 us an iteration (N = 96; 12.2 with the partials written after the update).
 #pragma once
 
 #include "prism_kernels.cuh"
@@ -26,8 +27,7 @@ constexpr int kMaxIters = 32;      // iterations per launch (Adam's constants of
 constexpr int kLocalRow = 7;       // float4 per measurement pair in shared memory: the six that the
                                    // uncalibrated step reads and one of padding, so that eight lanes
                                    // reading eight neighbouring rows hit different banks
-// partials per tile and iteration: J of every warp (MSE), or J and dJ/dsigma of the tile (NLL)
-constexpr int kLocalRed = kFusedThreads / 32;
+constexpr int kLocalRed = kFusedThreads / 32;   // partials of J per tile and iteration: one per warp
 // Floats per voxel of a state array in shared memory: 4K + 5 rounded up to an odd multiple of 4, so that
 // eight voxels' rows fall into different banks, whether a lane reads a float or four.
 __host__ __device__ constexpr int local_stride(int K) { return K <= 1 ? 12 : K <= 3 ? 20 : 28; }
@@ -44,18 +44,22 @@ __device__ __forceinline__ int ld_acquire(const int32_t* p) {
   return v;
 }
 
-// Sum over a group's partials of one iteration, fixed order: every NF-th value from `field` on, strided
-// over the warp's lanes, then a butterfly; every lane ends with it.
-template <int NF>
-__device__ __forceinline__ double local_group_sum(const IterArgs& a, const GroupDev& gr, int it, int field) {
-  const double* red = a.tile_red + (static_cast<size_t>(it) * a.ntiles + gr.tile0) * kLocalRed + field;
+// dJ/dsigma of a tile (Rician NLL), behind the objective's partials: [kMaxIters][ntiles].
+__device__ __forceinline__ double* local_dsig(const IterArgs& a, int it, int tile) {
+  return a.tile_red + static_cast<size_t>(kMaxIters) * a.ntiles * kLocalRed + static_cast<size_t>(it) * a.ntiles + tile;
+}
+
+// Sum of a volume's dJ/dsigma of one iteration, fixed order: strided over the warp's lanes, then a
+// butterfly; every lane ends with it.
+__device__ __forceinline__ double local_dsig_sum(const IterArgs& a, const GroupDev& gr, int it) {
+  const double* d = local_dsig(a, it, gr.tile0);
   double s = 0.0;
 #pragma unroll 4
-  for (int i = threadIdx.x & 31; i < gr.ntiles * (kLocalRed / NF); i += 32) s += __ldcg(red + NF * i);
+  for (int i = threadIdx.x & 31; i < gr.ntiles; i += 32) s += __ldcg(d + i);
   return warp_sum_d(s);
 }
 
-// A volume's objective of every iteration of the launch (MSE), by the CTA that finished the volume's last
+// A volume's objective of every iteration of the launch, by the CTA that finished the volume's last
 // tile: a warp takes kSums iterations at a time, so that their loads and butterflies overlap (one after the
 // other they are chains of about half a microsecond each). With the launch's last CTA doing all volumes' sums
 // one by one, 16 volumes of 10^3 voxels took 13.6 us an iteration instead of 7.0 and the 8^3 patch 48 instead of
@@ -100,8 +104,8 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
   float* s_st = s_y + static_cast<size_t>(NPmax) * TV;
   __shared__ uint64_t s_bar;
   __shared__ float s_ac[2 * kMaxIters];
-  __shared__ int s_last[2];   // this CTA counted in last: of the tile's volume (MSE), of the launch
-  __shared__ double s_ex[NW][2];   // NLL: the warps' partials, and the volume's sigma_log of the next iteration
+  __shared__ int s_last[2];   // this CTA counted in last: of the tile's volume, of the launch
+  __shared__ double s_ex[NW];   // NLL: the warps' dJ/dsigma, and the volume's sigma_log of the next iteration
   __shared__ float s_sig;
   __shared__ float4 s_bess[(LOSS == kLossNLL) ? kBesselTab : 1];
   if constexpr (LOSS == kLossNLL) bessel_stage(s_bess);   // visible after the first tile's barriers
@@ -191,12 +195,26 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
       A.gS0 = acc_gS0<K>(P, A);
       float gS0, gf[NF], gd[K][3], gfin;
       data_grad<K>(P, A, scale, gS0, gf, gd, gfin);
-      float dloss, dsig = 0.f;
+      float dloss;
       if (LOSS == kLossMSE) {
         dloss = A.l1 * gr.inv_M;
       } else {
         dloss = 2.f * slog * N + 0.5f * inv_s2 * A.l1 - A.l3;
-        dsig = 2.f * N - inv_s2 * (A.l1 + 2.f * A.l2);
+        const float dsig = 2.f * N - inv_s2 * (A.l1 + 2.f * A.l2);
+        // the tile's part of dJ/dsigma leaves first (its last warp counts the tile in): the chain rule and the
+        // update below run while the volume's other tiles arrive
+        double dS = act ? static_cast<double>(dsig) : 0.0;
+#pragma unroll
+        for (int o = 1; o < VW; o <<= 1) dS += __shfl_xor_sync(0xffffffffu, dS, o);
+        if (lane == 0) s_ex[warp] = dS;
+        __syncthreads();
+        if (tid == kFusedThreads - 32) {
+          double ss = s_ex[0];
+          for (int w = 1; w < NW; ++w) ss += s_ex[w];
+          *local_dsig(a, it, t) = ss;
+          __threadfence();
+          atomicAdd(a.gbar + tl.group, 1);
+        }
       }
       const float ploss = priors<K, true>(a, P, 0, gr.inv_M, nullptr, gS0, gf, gd);
       float g[Q];
@@ -231,73 +249,40 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
 #pragma unroll
       for (int q = 0; q < Q; ++q) th[q] = st[q];
       transform<K>(th, P);
-      // the warp's partials of the objective and dJ/dsigma: lanes 0 .. VW - 1 hold its voxels
+      // the warp's partial of the objective: lanes 0 .. VW - 1 hold its voxels
       double J = act ? static_cast<double>(dloss) + static_cast<double>(ploss) : 0.0;
-      double dS = (LOSS == kLossNLL && act) ? static_cast<double>(dsig) : 0.0;
 #pragma unroll
-      for (int o = 1; o < VW; o <<= 1) {
-        J += __shfl_xor_sync(0xffffffffu, J, o);
-        if (LOSS == kLossNLL) dS += __shfl_xor_sync(0xffffffffu, dS, o);
-      }
-      double* red = a.tile_red + (static_cast<size_t>(it) * a.ntiles + t) * kLocalRed;
-      if (LOSS == kLossMSE) {
-        if (lane == 0) red[warp] = J;
-      } else {
-        // the tile's sums by its first warp, which alone counts the tile in, waits and takes the volume's
-        // sum (with every warp doing so, a third of the iteration went into the exchange)
-        if (lane == 0) {
-          s_ex[warp][0] = J;
-          s_ex[warp][1] = dS;
-        }
-        __syncthreads();
-        if (warp == 0) {
-          const bool leader = t == gr.tile0;
-          int32_t* bar = a.gbar + tl.group;
-          if (lane == 0) {
-            double sj = s_ex[0][0], ss = s_ex[0][1];
-            for (int w = 1; w < NW; ++w) {
-              sj += s_ex[w][0];
-              ss += s_ex[w][1];
+      for (int o = 1; o < VW; o <<= 1) J += __shfl_xor_sync(0xffffffffu, J, o);
+      if (lane == 0) a.tile_red[(static_cast<size_t>(it) * a.ntiles + t) * kLocalRed + warp] = J;
+      if (LOSS == kLossNLL) {
+        // the first warp alone waits for the volume's tiles and takes its sum (with every warp doing so, a
+        // third of the iteration went into the exchange)
+        const bool leader = t == gr.tile0;
+        if (warp == 0 && (it + 1 < n_it || leader)) {
+          const int want = gr.ntiles * (it + 1);
+          if (!failed) {
+            bool ok = true;
+            if (lane == 0) {
+              int polls = 0;
+              while (ld_acquire(a.gbar + tl.group) < want && polls < (1 << 21)) ++polls;
+              ok = polls < (1 << 21);
+              if (!ok) atomicOr(a.status, kStTimeout);
             }
-            red[0] = sj;
-            red[1] = ss;
-            __threadfence();
-            atomicAdd(bar, 1);
+            failed = __any_sync(0xffffffffu, !ok);
           }
-          if (it + 1 < n_it || leader) {
-            const int want = gr.ntiles * (it + 1);
-            if (!failed) {
-              bool ok = true;
-              if (lane == 0) {
-                int polls = 0;
-                while (ld_acquire(bar) < want && polls < (1 << 21)) ++polls;
-                ok = polls < (1 << 21);
-                if (!ok) atomicOr(a.status, kStTimeout);
-              }
-              failed = __any_sync(0xffffffffu, !ok);
-            }
-            const float gsig = static_cast<float>(local_group_sum<kLocalRed>(a, gr, it, 1));
-            if (a.optimizer == 0) {
-              sgm = fmaf(a.beta1, sgm, (1.f - a.beta1) * gsig);
-              sgv = fmaf(a.beta2, sgv, (1.f - a.beta2) * gsig * gsig);
-              slog -= stepsz * sgm / fmaf(sqrtf(sgv), isbc2, a.eps);
-            } else {
-              rprop_update(slog, sgm, sgv, gsig, a.lr, a.eta_minus, a.eta_plus, a.step_min, a.step_max);
-            }
-            if (leader) {
-              const double tot = local_group_sum<kLocalRed>(a, gr, it, 0);
-              if (lane == 0) {
-                if (!isfinite(tot)) atomicOr(a.status, kStNonfinite);
-                a.hist[static_cast<size_t>((step + it) % a.hist_len) * a.G + tl.group] = tot;
-                if (it == n_it - 1) {
-                  a.gloss[tl.group] = tot;
-                  a.gparams_rw[gr.gp_off] = slog;
-                  a.gm[gr.gp_off] = sgm;
-                  a.gv[gr.gp_off] = sgv;
-                }
-              }
-            }
-            if (lane == 0) s_sig = slog;
+          const float gsig = static_cast<float>(local_dsig_sum(a, gr, it));
+          if (a.optimizer == 0) {
+            sgm = fmaf(a.beta1, sgm, (1.f - a.beta1) * gsig);
+            sgv = fmaf(a.beta2, sgv, (1.f - a.beta2) * gsig * gsig);
+            slog -= stepsz * sgm / fmaf(sqrtf(sgv), isbc2, a.eps);
+          } else {
+            rprop_update(slog, sgm, sgv, gsig, a.lr, a.eta_minus, a.eta_plus, a.step_min, a.step_max);
+          }
+          if (lane == 0) s_sig = slog;
+          if (lane == 0 && leader && it == n_it - 1) {
+            a.gparams_rw[gr.gp_off] = slog;
+            a.gm[gr.gp_off] = sgm;
+            a.gv[gr.gp_off] = sgv;
           }
         }
         __syncthreads();
@@ -307,8 +292,8 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
     __syncthreads();
     if (tid == 0) {   // both counts in flight at once, under the stores below
       __threadfence();
-      int left = 1, left_all = 1;
-      if (LOSS == kLossMSE) left = gr.ntiles - 1 - atomicAdd(a.gbar + tl.group, 1);
+      const int left = gr.ntiles - 1 - atomicAdd(a.gbar + a.G + tl.group, 1);
+      int left_all = 1;
       if (ti + static_cast<int>(gridDim.x) >= a.ntiles) left_all = static_cast<int>(gridDim.x) - 1 - atomicAdd(a.done, 1);
       s_last[0] = left == 0;
       s_last[1] = left_all == 0;
@@ -322,17 +307,14 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
       a.m[ix] = s_st[TV * QS + at];
       a.v[ix] = s_st[2 * TV * QS + at];
     }
-    if (LOSS == kLossMSE) {
-      __syncthreads();
-      if (s_last[0]) {
-        __threadfence();
-        local_objectives(a, gr, tl.group, step);
-        if (tid == 0) a.gbar[tl.group] = 0;
-      }
+    __syncthreads();
+    if (s_last[0]) {
+      __threadfence();
+      local_objectives(a, gr, tl.group, step);
+      if (tid == 0) a.gbar[a.G + tl.group] = 0;
     }
   }
   // the last CTA: step counter, the next constants, counters
-  __syncthreads();
   if (!s_last[1]) return;
   if (LOSS == kLossNLL)
     for (int i = tid; i < a.G; i += kFusedThreads) a.gbar[i] = 0;

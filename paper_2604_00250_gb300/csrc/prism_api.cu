@@ -1098,6 +1098,19 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   if (o.fused) {
     int bps = 0;
     CK(h->ks->fused_occupancy(o.loss, h->cal ? 1 : 0, h->TPV, h->shell, h->NT, h->fused_smem, &bps));
+    h->ia.cal_stage = 0;
+    if (h->shell && h->cal) {   // the partials' staging rows, where they cost no CTA (cal_flush)
+      const size_t smem = h->fused_smem + static_cast<size_t>(NW) * kAbSteps * kAbRow * sizeof(float4);
+      int staged = 0;
+      if (h->ks->fused_occupancy(o.loss, 1, h->TPV, h->shell, h->NT, smem, &staged) != cudaSuccess) {
+        cudaGetLastError();   // more than a CTA can have
+        staged = 0;
+      }
+      if (bps > 0 && staged >= bps) {
+        h->fused_smem = smem;
+        h->ia.cal_stage = 1;
+      }
+    }
     if (bps < 1) return fail(PRISM_E_CUDA, "fused kernel does not fit on an SM");
     h->fused_grid = std::max(1, std::min(h->ntiles, sms * bps));
   }

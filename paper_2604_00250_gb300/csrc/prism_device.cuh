@@ -152,6 +152,7 @@ struct IterArgs {
   int32_t pdl;
   int32_t n_it;            // iterations of this launch (k_iter_local; else 1)
   int32_t* gbar;           // [2][G] tiles counted in by the current launch (k_iter_local): per iteration (Rician NLL), at the end
+  int32_t cal_stage;       // calibrated shell loop: partials through shared memory (see cal_flush)
   float* gparams_rw;       // same array as gparams
   float* gm;               // group Adam moments (packed like gparams)
   float* gv;

@@ -961,8 +961,8 @@ __device__ __forceinline__ void data_grad_shell(const Vox<K>& P, const Acc<K>& A
 // and the second measurement of an odd shell's last pair masked. With calibration (Eq. 6) the
 // prediction is beta_n - (A_n B) s with s = -S, and the accumulators take q = -r A_n B (the other sign
 // than without: shell_sums). Against the per-measurement step (step2) it saves a third of the packed operations
-// and two thirds of the table's bytes: calibrated NLL phantom 537 -> 507 us, DiSCo1-shaped (five fibers, four
-// lanes) 206 -> 186.
+// and two thirds of the table's bytes: calibrated NLL phantom 537 -> 507 us (482 with the alpha / beta partials
+// through shared memory), DiSCo1-shaped (five fibers, four lanes) 206 -> 186.
 struct ShellExtra {
   float l2, l3;   // Rician NLL: sum y |y_hat| Q, sum L
   float2 u;       // calibration: sum of q s (dJ/dU unscaled, negated)
@@ -1047,6 +1047,36 @@ __device__ __forceinline__ void shell_step_any(ShellState<K>& S, ShellExtra& X, 
     S.gd[k][1] = __ffma2_rn(w, gy, S.gd[k][1]);
     S.gd[k][2] = __ffma2_rn(w, gz, S.gd[k][2]);
   }
+}
+
+// The alpha / beta partials of the calibrated shell loop: a lane's {u, r} of kAbSteps pairs are staged as rows
+// of the warp's lanes, and a flush sums them over the voxels: lane L takes u (even L) or r of step (L & 7) / 2 over
+// the eight lanes of its group L / 8, which with four lanes per voxel are the voxels of one pair; with one
+// lane the four groups then add up. The rows' stride and the rotated order keep the 8-byte reads free of bank
+// conflicts. Against a butterfly of shuffles per two pairs (18 instructions a pair, 6 here): calibrated NLL phantom,
+// N = 360, fused kernel 508 -> 482 us. Its 8.7 KB per CTA are taken only where they leave as many CTAs on an SM
+// (a.cal_stage; 128-voxel tiles: up to about 490 measurements): with two instead of three CTAs N = 520 took
+// 800 us against 715 by the butterfly, which stays there.
+constexpr int kAbSteps = 4, kAbRow = 34;
+
+template <int TPV>
+__device__ __forceinline__ float2 cal_flush(const float4* stage) {
+  static_assert(TPV == 1 || TPV == 4, "a group of eight lanes holds one pair's voxels, or a quarter of them");
+  const int lane = threadIdx.x & 31, gi = lane >> 3;
+  const float2* row = reinterpret_cast<const float2*>(stage + ((lane & 7) >> 1) * kAbRow + 8 * gi) + (lane & 1);
+  float2 v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = row[2 * ((k + gi) & 7)];
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+    for (int k = 0; k < 8; k += 2 * o) v[k] = __fadd2_rn(v[k], v[k + o]);
+  if (TPV == 1) {
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1)
+      v[0] = __fadd2_rn(v[0], make_float2(__shfl_xor_sync(0xffffffffu, v[0].x, o), __shfl_xor_sync(0xffffffffu, v[0].y, o)));
+  }
+  return v[0];
 }
 
 // The lane's sums as (unscaled) accumulators of q = dJ/dS, in the shell loop's scaled forms (shell_fold).
@@ -1256,6 +1286,8 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
                         : reinterpret_cast<float*>(s_tab + a.Nmax);       // [NW][NS][kChunk][VW]
   float* s_blr = s_ring + NW * NS * kChunk * VW;                       // [512] (calibration)
   float* s_ab = s_blr + (CAL ? kNGrid : 0);                                 // [NW][2][Nmax] (calibration)
+  // [NW][kAbSteps][kAbRow] (calibration, shell loop)
+  float4* s_stage = reinterpret_cast<float4*>(s_ab + (CAL ? NW * 2 * a.Nmax : 0));
   __shared__ uint64_t s_bar;                 // table / bias grid
   __shared__ uint64_t s_full[NW][NS];
   __shared__ int s_first, s_next;
@@ -1448,31 +1480,55 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         const int pc0 = j * (kChunk / 2), npc = min(kChunk / 2, N / 2 - pc0);   // this chunk's pairs
         const float2 nB2 = make_float2(-B, -B);
         if constexpr (CAL) {
-          // two steps (four measurements) of each lane per reduce-scatter of the alpha / beta partials
-          // over the VW lanes that share js; the sums hold the negated values, so the stores negate
-          constexpr int LVW = (VW == 8) ? 3 : (VW == 16) ? 4 : 5;
+          if (a.cal_stage) {
+            // The alpha / beta partials go through shared memory, kAbSteps steps of a lane at a time (cal_flush).
+            float4* __restrict__ stage = s_stage + warp * (kAbSteps * kAbRow);
 #pragma unroll 1
-          for (int i = 0; i < kChunk / 2 / TPV; i += 2) {
-            float uu[4], rv[4];
+            for (int i = 0; i * TPV < npc; i += kAbSteps) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int pi = (i + h) * TPV + js, p = pc0 + pi;
-              float2 u = make_float2(0.f, 0.f), r = make_float2(0.f, 0.f);
-              if (act && pi < npc)
-                shell_step_any<K, LOSS, true>(SS, SX, s_runs, gr.n_runs, p, col, gxy[p], gz2[p], yc2[pi * VW], cal4[p],
-                                              nB2, inv_s2, s_bess, &u, &r);
-              uu[2 * h] = u.x;
-              uu[2 * h + 1] = u.y;
-              rv[2 * h] = r.x;
-              rv[2 * h + 1] = r.y;
+              for (int h = 0; h < kAbSteps; ++h) {
+                const int pi = (i + h) * TPV + js, p = pc0 + pi;
+                float2 u = make_float2(0.f, 0.f), r = make_float2(0.f, 0.f);
+                if (act && pi < npc)
+                  shell_step_any<K, LOSS, true>(SS, SX, s_runs, gr.n_runs, p, col, gxy[p], gz2[p], yc2[pi * VW], cal4[p],
+                                                nB2, inv_s2, s_bess, &u, &r);
+                stage[h * kAbRow + lane] = make_float4(u.x, u.y, r.x, r.y);
+              }
+              __syncwarp();
+              const float2 sum = cal_flush<TPV>(stage);
+              const int pi = (i + ((lane & 7) >> 1)) * TPV + ((TPV == 1) ? 0 : lane >> 3);
+              if ((TPV > 1 || lane < 8) && pi < npc)
+                *reinterpret_cast<float2*>(s_ab + (warp * 2 + (lane & 1)) * a.Nmax + j * kChunk + 2 * pi) =
+                    make_float2(-sum.x, -sum.y);
+              __syncwarp();
             }
-            const float su = warp_scatter_sum<4, VW>(uu);
-            const float sr = warp_scatter_sum<4, VW>(rv);
-            const int q = lv >> (LVW - 2);
-            const int n = 2 * ((i + (q >> 1)) * TPV + js) + (q & 1);
-            if ((lv & ((VW >> 2) - 1)) == 0 && n < 2 * npc) {
-              s_ab[(warp * 2) * a.Nmax + j * kChunk + n] = -su;
-              s_ab[(warp * 2 + 1) * a.Nmax + j * kChunk + n] = -sr;
+          } else {
+            // two steps (four measurements) of each lane per reduce-scatter of the alpha / beta partials
+            // over the VW lanes that share js; the sums hold the negated values, so the stores negate
+            constexpr int LVW = (VW == 8) ? 3 : (VW == 16) ? 4 : 5;
+#pragma unroll 1
+            for (int i = 0; i < kChunk / 2 / TPV; i += 2) {
+              float uu[4], rv[4];
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const int pi = (i + h) * TPV + js, p = pc0 + pi;
+                float2 u = make_float2(0.f, 0.f), r = make_float2(0.f, 0.f);
+                if (act && pi < npc)
+                  shell_step_any<K, LOSS, true>(SS, SX, s_runs, gr.n_runs, p, col, gxy[p], gz2[p], yc2[pi * VW], cal4[p],
+                                                nB2, inv_s2, s_bess, &u, &r);
+                uu[2 * h] = u.x;
+                uu[2 * h + 1] = u.y;
+                rv[2 * h] = r.x;
+                rv[2 * h + 1] = r.y;
+              }
+              const float su = warp_scatter_sum<4, VW>(uu);
+              const float sr = warp_scatter_sum<4, VW>(rv);
+              const int q = lv >> (LVW - 2);
+              const int n = 2 * ((i + (q >> 1)) * TPV + js) + (q & 1);
+              if ((lv & ((VW >> 2) - 1)) == 0 && n < 2 * npc) {
+                s_ab[(warp * 2) * a.Nmax + j * kChunk + n] = -su;
+                s_ab[(warp * 2 + 1) * a.Nmax + j * kChunk + n] = -sr;
+              }
             }
           }
         } else if (act) {

@@ -103,7 +103,8 @@ typedef struct prism_options {
   float rprop_eta_plus;   /* Rprop step factor while the sign holds, 1.2 */
   float rprop_step_min, rprop_step_max; /* Rprop step bounds, 1e-6 and 50 */
   int32_t fused;          /* 1: persistent fused iteration kernel; 0: plain unfused per-patch launches */
-  int32_t use_graph;      /* 1: replay the fused iteration from a CUDA graph */
+  int32_t use_graph;      /* 1: replay the fused iteration from a CUDA graph (small fits run up to 32
+                             iterations per launch instead and need none) */
   int32_t threads_per_voxel; /* 1, 4 or 16 (measurements split across lanes); 0 = automatic: 16 below
                                 2,048 voxels (without neighbour priors and calibration: 1,400 with
                                 the MSE, 4,200 with the NLL), 4 below
@@ -193,8 +194,8 @@ int prism_get_fibers(prism_handle* h, float* dirs, float* fracs, uint8_t* peaks,
  * along its last axis into slabs of `slab` slices advancing by slab - overlap, the last one
  * reaching the last slice; every non-empty slab becomes one volume of a handle initialised as
  * by prism_fit_init (its own sigma and calibration; neighbour priors stay inside the slab).
- * The slab signals (and `init` rows) are gathered on the device from vol->signal in `vol->mem`
- * memory; the caller's buffers are not kept. Step the handle as usual, then read the
+ * Each slab's rows are read on the device from the volume's own signal (and `init`), which in
+ * `vol->mem` memory is uploaded or read once; the caller's buffers are not kept. Step the handle as usual, then read the
  * whole-volume maps with prism_stitch_slabs. E_INVALID_ARG for slab < 1, overlap < 0 or
  * 2 * overlap > slab, E_SHAPE for an empty mask, plus every error of prism_fit_init.
  */
@@ -239,16 +240,16 @@ int prism_get_loss(prism_handle* h, double* loss, double* hist, int32_t max_iter
  * data term, plus the prior values. A given theta / groups becomes the handle's
  * current parameters (as by prism_set_params / prism_set_groups). Writes y_hat (DEVICE, NULL to skip; group g
  * at offset sum_{g'<g} V_g' N_g', rows [V_g][N_g] in mask order) and J_g
- * (DEVICE double [G]). Keeps the residual derivative dL/dy_hat (V x N, not the
- * V x N x K compartment terms) for prism_backward.
+ * (DEVICE double [G]). A fused handle's pass also leaves the gradient for prism_backward; a
+ * plain one keeps the residual derivative dL/dy_hat (V x N, not the V x N x K compartment terms).
  */
 int prism_forward(prism_handle* h, const float* theta, const float* groups, float* yhat,
                   double* loss, void* stream);
 
 /*
- * Gradient of the objective at the point of the last prism_forward: recomputes
- * the compartment exponentials, then the adjoint of synthesis, calibration,
- * data term and priors. grad_theta DEVICE [V][Q]; grad_groups DEVICE packed
+ * Gradient of the objective at the point of the last prism_forward (adjoint of synthesis,
+ * calibration, data term and priors). A fused handle hands out what the forward's pass left; a
+ * plain one runs the adjoint here, recomputing the compartment exponentials. grad_theta DEVICE [V][Q]; grad_groups DEVICE packed
  * (NULL to skip). E_STATE without a preceding forward.
  */
 int prism_backward(prism_handle* h, float* grad_theta, float* grad_groups, void* stream);

@@ -56,7 +56,7 @@ FLOPS_PER_B0_PAIR_SHELL = 4
 # scaled brain (traffic grows in proportion to the voxels), valid only for the kernel sources
 # whose SHA-256 (comments and blank lines left out, fused_sources_sha256) is
 # TRAFFIC_SOURCES_SHA256: any other hash reports the traffic as null.
-# 212,900 voxels: 349.7 MB read and 36.1 MB written in one launch (profiles/k_iter_fused_hcp_brain_dram_traffic.md).
+# 212,900 voxels: 350.2 MB read and 35.2 MB written in one launch (profiles/k_iter_fused_hcp_brain_dram_traffic.md).
 TRAFFIC_BYTES_PER_VOXEL_ITER = 1810.0
 TRAFFIC_SOURCES_SHA256 = "4690d88d01b46a6c1f647a85768af13f5f41b04cc38e3393abcc26d1f90479af"
 FUSED_SOURCES = ("prism_kernels.cuh", "prism_device.cuh", "prism_kset.cuh", "bessel_fit.h", "prism_k3.cu")

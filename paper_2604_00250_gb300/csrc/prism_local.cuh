@@ -270,6 +270,9 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
             }
             failed = __any_sync(0xffffffffu, !ok);
           }
+          // lane 0's acquire orders the other lanes' reads of the partials only through a warp barrier (a vote
+          // orders no memory accesses)
+          __syncwarp();
           const float gsig = static_cast<float>(local_dsig_sum(a, gr, it));
           if (a.optimizer == 0) {
             sgm = fmaf(a.beta1, sgm, (1.f - a.beta1) * gsig);

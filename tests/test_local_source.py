@@ -1,0 +1,21 @@
+"""CPU checks of the order of waits and memory accesses in the many-iteration kernel's source (k_iter_local):
+what must hold there shows in no result on the hardware at hand, so it is read off the code."""
+import os
+
+import bench
+
+SRC = os.path.join(bench.ROOT, "paper_2604_00250_gb300", "csrc", "prism_local.cuh")
+
+
+def kernel():
+    src = bench.strip_c_comments(open(SRC).read())
+    return src[src.index("k_iter_local(const IterArgs a)"):]
+
+
+def test_partials_are_read_after_a_warp_barrier():
+    """One lane acquires the volume's count; the others read the tiles' partials after a warp barrier (a
+    vote would order no memory accesses)."""
+    k = kernel()
+    wait = k.index("ld_acquire(")
+    read = k.index("local_dsig_sum(", wait)
+    assert "__syncwarp();" in k[wait:read]

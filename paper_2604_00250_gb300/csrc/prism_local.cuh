@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
     const GroupDev gr = a.groups[tl.group];
     const int N = tl.n_meas, NP = (N + 3) & ~3;
     __syncthreads();   // the previous tile's shared data are no longer read (and s_bar is set up)
-    if (tid == 0) {
+    if (tid == 0 && !failed) {
       const uint32_t bytes = static_cast<uint32_t>(NP) * TV * 4u;   // multiple of 16: NP % 4 == 0
       fence_proxy_async_smem();
       mbar_expect_tx(&s_bar, bytes);
@@ -150,10 +150,14 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
     }
     if (!failed && !mbar_wait(&s_bar, phase)) {
       atomicOr(a.status, kStTimeout);
+      mbar_wait(&s_bar, phase);   // let the copy land before its shared memory is released
       failed = true;
     }
     phase ^= 1;
     failed = __syncthreads_or(failed);
+    // without its signal the tile keeps its state, as the CTA's later ones do, and is counted in for every
+    // iteration, so that no other tile waits for it (the handle's status says that the launch failed)
+    if (LOSS == kLossNLL && tid == 0 && failed) atomicAdd(a.gbar + tl.group, n_it);
     const bool act = vl < tl.count;
     float* st = s_st + vl * QS;
     float th[Q];
@@ -168,7 +172,7 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
       sgv = a.gv[gr.gp_off];
     }
     const float2* yc2 = reinterpret_cast<const float2*>(s_y + static_cast<size_t>(warp) * NP * VW) + lv;
-    for (int it = 0; it < n_it; ++it) {
+    for (int it = failed ? n_it : 0; it < n_it; ++it) {
       const float inv_s2 = (LOSS == kLossNLL) ? expf(-2.f * slog) : 0.f;
       const float scale = (LOSS == kLossMSE) ? 2.f * gr.inv_M : inv_s2;
       Acc<K> A;
@@ -301,7 +305,7 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
       s_last[0] = left == 0;
       s_last[1] = left_all == 0;
     }
-    for (int e = tid; e < Q * TV; e += kFusedThreads) {
+    for (int e = tid; e < Q * TV && !failed; e += kFusedThreads) {
       const int v = e % TV;
       if (v >= tl.count) continue;
       const size_t ix = static_cast<size_t>(e / TV) * Vp + tl.slot0 + v;

@@ -442,12 +442,10 @@ def _make_autograd():
                 f.forward(*ctx.point)
                 ctx.token = f._fwd_token
             gth, gg = f.backward()
-            if gout.requires_grad:   # a graph through the factor (create_graph): out of place
-                gth, gg = gth * gout, gg * gout
-            else:                    # in place on the fresh gradients; the 0-dim factor takes their type
-                gth, gg = gth.mul_(gout), gg.mul_(gout)
-            g_theta = gth.to(ctx.dtypes[0]) if ctx.needs_input_grad[0] else None
-            g_groups = gg.to(ctx.dtypes[1]) if ctx.needs_input_grad[1] else None
+            # Out of place: the factor may be part of a graph (create_graph) or a batch of factors
+            # (is_grads_batched, a vectorised Jacobian). 0-dim, it takes the gradients' type.
+            g_theta = (gth * gout).to(ctx.dtypes[0]) if ctx.needs_input_grad[0] else None
+            g_groups = (gg * gout).to(ctx.dtypes[1]) if ctx.needs_input_grad[1] else None
             return g_theta, g_groups, None
 
     return PrismLoss

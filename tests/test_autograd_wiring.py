@@ -84,3 +84,30 @@ def test_same_point_is_not_recomputed():
     th = torch.randn(3, 4, requires_grad=True)
     prism.PrismLoss.apply(th, None, f).backward()
     assert f.forward_calls == 1
+
+
+def test_batched_upstream_factors():
+    """A batch of factors (is_grads_batched) and a vectorised Jacobian: one gradient per factor, in the
+    inputs' types."""
+    f = FakeHandle()
+    th = torch.randn(3, 4, requires_grad=True)
+    g = torch.randn(5, dtype=torch.float64, requires_grad=True)
+    J = prism.PrismLoss.apply(th, g, f)
+    s = torch.tensor([1.0, -2.0, 0.5], dtype=J.dtype)
+    gth, gg = torch.autograd.grad(J, (th, g), s, is_grads_batched=True)
+    g0 = g.detach().float()   # the handle works in float32
+    assert gth.dtype == th.dtype and gg.dtype == g.dtype
+    torch.testing.assert_close(gth, s.float().reshape(3, 1, 1) * (2 * f.w * th.detach()))
+    torch.testing.assert_close(gg.float(), s.float().reshape(3, 1) * (2 * f.c * g0))
+    jac = torch.autograd.functional.jacobian(lambda t: 3.0 * prism.PrismLoss.apply(t, None, f), th, vectorize=True)
+    torch.testing.assert_close(jac, 3.0 * 2 * f.w * th.detach())
+
+
+def test_factor_in_a_graph():
+    """create_graph: the gradient of the gradient's norm w.r.t. the factor."""
+    f = FakeHandle()
+    th = torch.randn(3, 4, requires_grad=True)
+    s = torch.tensor(2.0, dtype=torch.float64, requires_grad=True)
+    (gth,) = torch.autograd.grad(s * prism.PrismLoss.apply(th, None, f), th, create_graph=True)
+    (gs,) = torch.autograd.grad(gth.sum(), s)
+    torch.testing.assert_close(gs.float(), (2 * f.w * th.detach()).sum())

@@ -454,11 +454,6 @@ __global__ void k_adam_voxel(const IterArgs a, const PlainArgs pa) {
 // only the few sums of sums in FP64; a split's tiles lie at one stride, so their loads go out together.
 // (One FP64 chain of 64 tiles per thread, offsets looked up: 34 us for 2,048 tiles at N = 360; 17.5 us now, the adjoint's z pass, 7.4 us before, included.)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
-  const float s = hi + x, bb = s - hi;
-  lo += (hi - (s - bb)) + (x - bb);
-  hi = s;
-}
 __device__ __forceinline__ void group_reduce_block(const IterArgs& a, const GroupArgs& g, int gi, int s, int ce, int what) {
   __shared__ int s_last;
   __shared__ double s_q[4][kRedE];

@@ -416,6 +416,18 @@ __device__ __forceinline__ float adam_constant(int lane, float lr, float beta1, 
   return static_cast<float>((odd ? 1.0 : static_cast<double>(lr)) / q);
 }
 
+// hi + lo += x without the rounding of the sum (Knuth's two-sum; lo collects the rounded-off parts). The
+// intrinsics keep a product in x from being contracted into the additions.
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x), bb = __fsub_rn(s, hi);
+  lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb));
+  hi = s;
+}
+// hi + lo in FP64; an infinite hi, which leaves a NaN in lo, stays infinite.
+__device__ __forceinline__ double two_float(float hi, float lo) {
+  return static_cast<double>(hi) + static_cast<double>(isfinite(hi) ? lo : 0.f);
+}
+
 __device__ __forceinline__ double warp_sum_d(double x) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);

@@ -701,6 +701,35 @@ __device__ __forceinline__ void acc_get(Acc<K>& A, const float* s, int TV, int v
   }
 }
 
+// The data term's sums of a voxel in the gradient form: [0] the objective's (MSE: sum r^2; NLL: without the 2 N log
+// sigma), [1] the NLL's l1 + 2 l2 of dJ/dsigma. They take the FP32 sums of one ring stage after the other and are
+// combined in two-float arithmetic (two_sum), so that the
+// objective keeps the accuracy of an FP64 sum over the elements, which a caller of prism_forward compares
+// between points: in FP32 to the end, like terms (a voxel's 1,024 b = 0 measurements) drifted by up to 7e-6, and 2 N log
+// sigma rounded alike for all voxels.
+struct DataSums {
+  float hi[2], lo[2];
+};
+__device__ __forceinline__ void data_sum_add(DataSums& D, int i, float x) { two_sum(D.hi[i], D.lo[i], x); }
+// Sum over a voxel's TPV lanes, STRIDE apart (every lane ends with it).
+template <int NS, int TPV, int STRIDE>
+__device__ __forceinline__ void data_sums_reduce(DataSums& D) {
+#pragma unroll
+  for (int o = STRIDE; o < STRIDE * TPV; o <<= 1)
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      const float h = __shfl_xor_sync(0xffffffffu, D.hi[i], o), l = __shfl_xor_sync(0xffffffffu, D.lo[i], o);
+      D.lo[i] += l;
+      two_sum(D.hi[i], D.lo[i], h);
+    }
+}
+// hi + lo += a (sum i of D).
+__device__ __forceinline__ void data_sum_scaled(float& hi, float& lo, float a, const DataSums& D, int i) {
+  const float p = __fmul_rn(a, D.hi[i]);
+  lo += fmaf(a, D.lo[i], fmaf(a, D.hi[i], -p));
+  two_sum(hi, lo, p);
+}
+
 // Scaled data-term gradient w.r.t. transformed parameters.
 template <int K>
 __device__ __forceinline__ void data_grad(const Vox<K>& P, const Acc<K>& A, float scale, float& gS0,
@@ -1294,7 +1323,8 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
   __shared__ double s_red[8][3];
   // several lanes per voxel: the tile's reduced accumulators, handed to the epilogue threads
   constexpr int TV = kFusedThreads / TPV;
-  __shared__ float s_acc[(TPV > 1) ? (8 + 5 * K) * TV : 1];
+  constexpr int kAccRows = 8 + 5 * K;
+  __shared__ float s_acc[(TPV > 1) ? (kAccRows + (GRAD ? 4 : 0)) * TV : 1];   // gradient form: DataSums behind them
 
   __shared__ float4 s_bess[(LOSS == kLossNLL) ? kBesselTab : 1];
   if constexpr (LOSS == kLossNLL) bessel_stage(s_bess);   // visible after the block barrier below
@@ -1455,6 +1485,28 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
     } else if constexpr (PACKED) {
       voxp_init<K>(P, DP, AP);
     }
+    constexpr int kSumsD = (LOSS == kLossNLL) ? 2 : 1;
+    DataSums DS{};
+    // gradient form: the stage's FP32 sums of the data term move to DS
+    auto stage_sums = [&]() {
+      if constexpr (GRAD) {
+        float2 l1 = make_float2(A.l1, 0.f);
+        float l2 = A.l2, l3 = A.l3;
+        A.l1 = A.l2 = A.l3 = 0.f;
+        if constexpr (SHELL) {
+          l1 = SS.l1, l2 = SX.l2, l3 = SX.l3;
+          SS.l1 = make_float2(0.f, 0.f), SX.l2 = SX.l3 = 0.f;
+        } else if constexpr (PACKED) {
+          l1 = AP.l1, l2 = AP.l2, l3 = AP.l3;
+          AP.l1 = make_float2(0.f, 0.f), AP.l2 = AP.l3 = 0.f;
+        }
+        const float q1 = l1.x + l1.y;
+        data_sum_add(DS, 0, (LOSS == kLossNLL) ? fmaf(0.5f * inv_s2, q1, -l3) : q1);
+        if (LOSS == kLossNLL) data_sum_add(DS, 1, fmaf(2.f, l2, q1));
+      }
+      __syncwarp();
+      ++g;
+    };
     for (int j = 0; j < nch; ++j) {
       if (lane == 0) {
         // keep NS chunks of this warp's stream in flight (this tile, then the next)
@@ -1539,8 +1591,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
                                            make_float4(1.f, 1.f, 0.f, 0.f), nB2, inv_s2, s_bess, nullptr, nullptr);
           }
         }
-        __syncwarp();
-        ++g;
+        stage_sums();
         continue;
       }
       if constexpr (SHELL == 1 || SHELL == 2) {
@@ -1597,8 +1648,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
             }
           }
         }
-        __syncwarp();
-        ++g;
+        stage_sums();
         continue;
       }
       if constexpr (PACKED) {
@@ -1686,8 +1736,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
             step2<K, true, LOSS>(DP, tab2[pi], yc2[pi * VW], make_float2(1.f, (2 * pi + 1 < cnt) ? 1.f : 0.f), AP,
                                  inv_s2, s_bess);
         }
-        __syncwarp();
-        ++g;
+        stage_sums();
         continue;
       }
       // pair-interleaved slice: chunk-relative measurement nl of voxel lv
@@ -1743,8 +1792,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
           }
         }
       }
-      __syncwarp();
-      ++g;
+      stage_sums();
     }
     base += nch;
     if constexpr (SHELL == 1 || SHELL == 2) {
@@ -1757,6 +1805,16 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
       if constexpr (PACKED && !SHELL) accp_sums<K, LOSS, CAL>(AP, A);
       acc_reduce_tpv<K, TPV, VW>(A);
       if (js == 0) acc_put<K>(A, s_acc, TV, vl);
+      if constexpr (GRAD) {
+        data_sums_reduce<kSumsD, TPV, VW>(DS);
+        if (js == 0) {
+#pragma unroll
+          for (int i = 0; i < kSumsD; ++i) {
+            s_acc[(kAccRows + i) * TV + vl] = DS.hi[i];
+            s_acc[(kAccRows + 2 + i) * TV + vl] = DS.lo[i];
+          }
+        }
+      }
       __syncthreads();
     }
     if (!dep_done) {
@@ -1770,6 +1828,7 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
     const bool eact = (TPV == 1) ? act : (tid < tl.count);
     const bool writer = eact && (js == 0 || TPV > 1);
     float dloss = 0.f, dsig = 0.f, ploss = 0.f;
+    float dloss_lo = 0.f, dsig_lo = 0.f;   // gradient form: what the rounding of dloss and dsig left
     if (epi) {
       // voxel transforms again (not kept live across the loop). Where registers allow (HOIST),
       // the raw parameters and the moments are read here, once, so that their latency overlaps
@@ -1788,6 +1847,13 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         }
       } else {
         acc_get<K>(A, s_acc, TV, tid);
+        if constexpr (GRAD) {
+#pragma unroll
+          for (int i = 0; i < kSumsD; ++i) {
+            DS.hi[i] = s_acc[(kAccRows + i) * TV + tid];
+            DS.lo[i] = s_acc[(kAccRows + 2 + i) * TV + tid];
+          }
+        }
         if constexpr (SHELL) A.gS0 = shell_gS0<K>(P, A);
         else if constexpr (PACKED) A.gS0 = acc_gS0<K>(P, A);
         if constexpr (CAL) {
@@ -1803,10 +1869,21 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
       } else {
         data_grad<K>(P, A, scale, gS0, gf, gd, gfin);
       }
-      if (LOSS == kLossMSE) {
+      // (the NLL over the measurements proper: N counts an odd shell's padding)
+      if constexpr (GRAD) {
+        if (LOSS == kLossMSE) {
+          data_sum_scaled(dloss, dloss_lo, gr.inv_M, DS, 0);
+        } else {
+          const float n = gr.N;
+          dloss = __fmul_rn(2.f * slog, n);
+          dloss_lo = fmaf(2.f * slog, n, -dloss);
+          data_sum_scaled(dloss, dloss_lo, 1.f, DS, 0);
+          dsig = 2.f * n;
+          data_sum_scaled(dsig, dsig_lo, -inv_s2, DS, 1);
+        }
+      } else if (LOSS == kLossMSE) {
         dloss = A.l1 * gr.inv_M;
       } else {
-        // (the measurements proper: N counts an odd shell's padding)
         dloss = 2.f * slog * gr.N + 0.5f * inv_s2 * A.l1 - A.l3;
         dsig = 2.f * gr.N - inv_s2 * (A.l1 + 2.f * A.l2);
       }
@@ -1859,8 +1936,13 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
     }
     // ---- tile partials (fixed-order reductions)
     // (the separate prior field, tile_red[2], stays zero)
-    block_reduce<LOSS == kLossNLL>(writer ? static_cast<double>(dloss) + static_cast<double>(ploss) : 0.0,
-                                   writer ? static_cast<double>(dsig) : 0.0, s_red,
+    double val = static_cast<double>(dloss) + static_cast<double>(ploss), val_sig = static_cast<double>(dsig);
+    if constexpr (GRAD) {
+      two_sum(dloss, dloss_lo, ploss);
+      val = two_float(dloss, dloss_lo);
+      val_sig = two_float(dsig, dsig_lo);
+    }
+    block_reduce<LOSS == kLossNLL>(writer ? val : 0.0, writer ? val_sig : 0.0, s_red,
                                    a.tile_red + 4 * static_cast<size_t>(t));
     if (CAL) {
       for (int e = tid; e < 2 * N; e += kFusedThreads) {

@@ -477,7 +477,7 @@ __device__ __forceinline__ void group_reduce_block(const IterArgs& a, const Grou
       float hi = 0.f, lo = 0.f;
 #pragma unroll 8
       for (int t = 0; t < n; ++t) two_sum(hi, lo, src[static_cast<size_t>(t) * 2 * gr.npos]);
-      acc = static_cast<double>(hi) + static_cast<double>(lo);
+      acc = two_float(hi, lo);
     }
   }
   s_q[sub][el] = acc;

@@ -107,7 +107,8 @@ typedef struct prism_options {
                              iterations per launch instead and need none) */
   int32_t threads_per_voxel; /* 1, 4 or 16 (measurements split across lanes); 0 = automatic: 16 below
                                 2,048 voxels (without neighbour priors and calibration: 1,400 with
-                                the MSE, 4,200 with the NLL), 4 below
+                                the MSE, 4,200 with the NLL where all tiles of 8 voxels are
+                                resident at once), 4 below
                                 32,768 (16,384 where one lane takes the shell loop with the MSE), else
                                 1 except just above one wave of 128-voxel tiles with the NLL or
                                 calibration (then 4); prism_get_shape reports the choice */

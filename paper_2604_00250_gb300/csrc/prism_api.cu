@@ -126,7 +126,7 @@ struct prism_handle {
   int shell = 0;                       // the fused kernel takes the shell loop (2: with padded odd shells)
   bool local = false;                  // iterations run in k_iter_local, many per launch
   int local_grid = 0;
-  size_t local_smem = 0;
+  size_t local_bytes = 0;
   float* d_gtab = nullptr;
   ShellRun* d_runs = nullptr;
   double *d_tile_red = nullptr, *d_part2 = nullptr, *d_gred = nullptr, *d_gloss = nullptr;
@@ -407,7 +407,7 @@ int enqueue_fused_iters(prism_handle* h, int n, cudaStream_t st) {
   IterArgs a = h->ia;
   for (; n > 0; n -= a.n_it) {
     a.n_it = std::min(n, kMaxIters);
-    CK(h->ks->local(a, h->opt.loss, h->TPV, h->local_grid, h->local_smem, st));
+    CK(h->ks->local(a, h->opt.loss, h->TPV, h->local_grid, h->local_bytes, st));
   }
   return PRISM_OK;
 }
@@ -769,6 +769,35 @@ bool shells_apply(const prism_volume* vols, int n, const prism_options& o, int64
   return f == 1 || f == 2;
 }
 
+// The local kernel (prism_local.cuh) with `tpv` lanes per voxel: whether the fit can take it (several lanes, no
+// neighbour priors, no calibration; with the Rician NLL, whose CTAs exchange sums, only where all tiles are
+// resident at once), its CTAs and their shared memory.
+struct LocalShape {
+  bool ok = false;
+  int grid = 0;
+  size_t bytes = 0;
+};
+LocalShape local_shape(const prism_volume* vols, int n, const std::vector<MaskIndex>& idx, const prism_options& o, int tpv) {
+  LocalShape L;
+  if (!o.fused || o.calibration || o.lam_sp > 0.f || o.lam_dir > 0.f || tpv <= 1) return L;
+  int dev = 0, sms = 0, bps = 0, nmax = 0;
+  int64_t tiles = 0;
+  const int TV = kFusedThreads / tpv;
+  for (int g = 0; g < n; ++g) {
+    for (int32_t c : idx[g].pcount) tiles += (c + TV - 1) / TV;
+    nmax = std::max(nmax, (vols[g].n_meas + 3) & ~3);
+  }
+  L.bytes = local_smem(o.K, tpv, nmax);
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      kernels_for_k(o.K).local_occupancy(o.loss, tpv, L.bytes, &bps) != cudaSuccess) {
+    cudaGetLastError();   // no usable device: the first allocation reports it
+    return L;
+  }
+  L.grid = static_cast<int>(std::min<int64_t>(tiles, static_cast<int64_t>(sms) * bps));
+  L.ok = bps > 0 && (o.loss == PRISM_LOSS_MSE || L.grid == tiles);
+  return L;
+}
+
 // Slabs of one whole volume (prism_fit_init_slabs): the volumes are slices [z0[g], z0[g] + nz) of its
 // mask, and their signal and init rows are those of the whole volume (whole-volume pointers in vols[g]).
 struct SlabSrc {
@@ -794,22 +823,12 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   if (o.fused && (cudaGetDevice(&dev) != cudaSuccess ||
                   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess))
     cudaGetLastError();   // no usable device: the first allocation reports it, after the plan's own checks
-  // The local kernel (prism_local.cuh): several lanes per voxel, no neighbour priors, no calibration; with
-  // the Rician NLL, whose CTAs exchange sums, only where all tiles are resident at once. It takes the
-  // per-measurement step: its iterations are bound by latency, to which the shell loop's look-ups add
-  // (3,400 voxels at N = 193, K = 2: 87 us per 16 iterations, 108 with it).
-  if (o.fused && !h->cal && !h->nb && h->TPV > 1 && sms > 0) {
-    int64_t tiles = 0;
-    int nmax = 0, bps = 0;
-    for (int g = 0; g < n_vols; ++g) {
-      for (int32_t c : idx[g].pcount) tiles += (c + h->TV - 1) / h->TV;
-      nmax = std::max(nmax, (vols[g].n_meas + 3) & ~3);
-    }
-    h->local_smem = local_smem(h->K, h->TPV, nmax);
-    CK(h->ks->local_occupancy(o.loss, h->TPV, h->local_smem, &bps));
-    h->local_grid = static_cast<int>(std::min<int64_t>(tiles, static_cast<int64_t>(sms) * bps));
-    h->local = bps > 0 && (o.loss == PRISM_LOSS_MSE || h->local_grid == tiles);
-  }
+  // The local kernel takes the per-measurement step: its iterations are bound by latency, to which the shell
+  // loop's look-ups add (3,400 voxels at N = 193, K = 2: 87 us per 16 iterations, 108 with it).
+  const LocalShape L = local_shape(vols, n_vols, idx, o, h->TPV);
+  h->local = L.ok;
+  h->local_grid = L.grid;
+  h->local_bytes = L.bytes;
   h->shell = h->local ? 0 : shell_form(vols, n_vols, o, Vsum, h->TPV);
   // Host signals start their copy to the device before the plan is built: a copy needs only the
   // voxel count, and the DMA then runs while the host builds the plan. All copies start at once
@@ -1120,18 +1139,29 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
 
 // Lanes per voxel of a fit, by measurement on GB300 (cubes of bundle and crossing phantoms, N = 96-364,
 // K = 3 and 5; us an iteration). `shell`: one thread per voxel would run the segmented shell loop.
-int choose_shape(const prism_options& o, int64_t V, bool shell, int* tpv, int* nt) {
+int choose_shape(const prism_options& o, const prism_volume* vols, int n, const std::vector<MaskIndex>& idx, int64_t V,
+                 bool shell, int* tpv, int* nt) {
   // No neighbour priors and no calibration: the local kernel with four or sixteen lanes. Sixteen below
   // 1,400 voxels with the MSE (10^3 at N = 96: 2.8 against 3.2 with four, 12^3 4.1 and 3.5; N = 288 3.4 and
   // 5.5, 4.9 and 5.7) and below 4,200 with the NLL, whose measurements cost more (N = 96: 12^3 6.0 and 8.0,
-  // 16^3 8.1 and 7.5; N = 288 16^3 11.4 and 14.5; 20^3 no longer fits the chip at once); one from
-  // 32,768 on (28^3 at N = 96: 13.7 with four, 19.6 with one; 32^3 21.3 and 19.8).
-  const bool local = o.fused && !o.calibration && !(o.lam_sp > 0.f) && !(o.lam_dir > 0.f);
+  // 16^3 8.1 and 7.5; N = 288 16^3 11.4 and 14.5); one from 32,768 on (28^3 at N = 96: 13.7 with four, 19.6 with
+  // one; 32^3 21.3 and 19.8). The NLL's tiles must fit the chip at once: where those of eight voxels do not
+  // (large N, K >= 4, many part-filled tiles), four lanes, whose tiles hold 32 (16^3, K = 5, N = 96: general kernel
+  // with sixteen lanes 25.6, local with four 8.3; K = 3, N = 1,000: 68 and 40); where neither does, the general
+  // kernel's lines.
+  int local = 0;
+  if (!o.threads_per_voxel && V < 32768) {
+    const int first = V < (o.loss == PRISM_LOSS_NLL ? 4200 : 1400) ? 16 : 4;
+    if (local_shape(vols, n, idx, o, first).ok) local = first;
+    else if (first != 4 && local_shape(vols, n, idx, o, 4).ok) local = 4;
+  }
   if (o.threads_per_voxel) {
     *tpv = o.threads_per_voxel;
-  } else if (V < (!local ? 2048 : o.loss == PRISM_LOSS_NLL ? 4200 : 1400)) {
+  } else if (local) {
+    *tpv = local;
+  } else if (V < 2048) {
     *tpv = 16;
-  } else if (V < ((shell && !local) ? 16384 : 32768)) {
+  } else if (V < (shell ? 16384 : 32768)) {
     // the segmented shell loop with one lane is ahead from 16,384 voxels on (N = 288: 24^3 36.2 against 35.0
     // with four, 26^3 36.7 and 38.7, 28^3 43.9 and 60.4; five fibers 28^3 60 and 69), the other forms are
     // level with four lanes up to 32^3 (NLL, N = 288: 28^3 62.5 and 60.6, 32^3 62.8 and 71.3)
@@ -1370,7 +1400,7 @@ int fit_init(const prism_volume* vols, int n_vols, const prism_options* opt, con
     V += idx.back().count;
   }
   int tpv = 1, nt = 128;
-  choose_shape(o, V, shells_apply(vols, n_vols, o, V), &tpv, &nt);
+  choose_shape(o, vols, n_vols, idx, V, shells_apply(vols, n_vols, o, V), &tpv, &nt);
   if (o.autotune && o.fused && !slabs) {
     int shells = o.shells;
     autotune_shape(vols, n_vols, idx, o, st, &tpv, &shells);
@@ -1847,7 +1877,7 @@ extern "C" int prism_fit_init_slabs(const prism_volume* vol, int32_t slab, int32
     w.init = init;
     const std::vector<MaskIndex> wi{src.index};
     int tpv = 1, nt = 128, shells = o.shells;
-    choose_shape(o, V, shells_apply(&w, 1, o, V), &tpv, &nt);
+    choose_shape(o, &w, 1, wi, V, shells_apply(&w, 1, o, V), &tpv, &nt);
     autotune_shape(&w, 1, wi, o, st, &tpv, &shells);
     o.threads_per_voxel = tpv;
     o.shells = shells;

@@ -117,9 +117,14 @@ def fp32_peak_tflops(device_index=0):
     return n_sm * FP32_LANES_PER_SM * 2 * mhz * 1e6 / 1e12, f"{n_sm} SMs x {FP32_LANES_PER_SM} x 2 x {mhz:.0f} MHz"
 
 
+def kernel_name(shape):
+    """The iteration kernel of a Fitter with this shape()."""
+    return "k_iter_local" if shape["iterations_per_launch"] > 1 else "k_iter_fused"
+
+
 def speed_leg(vols, kw, steps, warmup, unfused_steps=2):
-    """Fused iterations (graph replay, CUDA events), the fused kernel's roofline fraction from the
-    per-kernel timing pass, and the plain per-patch path on the same volumes. `vols` hold device
+    """Fused iterations (as step() runs them, CUDA events), the iteration kernel's roofline fraction from
+    the timing pass of profile(), and the plain per-patch path on the same volumes. `vols` hold device
     signals."""
     import torch
     import paper_2604_00250_gb300 as prism
@@ -144,7 +149,7 @@ def speed_leg(vols, kw, steps, warmup, unfused_steps=2):
     f.close()
     out = {"value": V / (ms / 1e3), "ms_per_step": ms, "steps": steps, "profile_ms": prof, "launch": shape,
            "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                        "kernel": "k_iter_fused", "flops_per_launch": flops, "peak_source": "derived: " + peak_src}}
+                        "kernel": kernel_name(shape), "flops_per_iteration": flops, "peak_source": "derived: " + peak_src}}
     if unfused_steps:
         fu = prism.Fitter(vols, prism.options(**dict(kw, fused=0, use_graph=0)))
         fu.step(1)
@@ -766,7 +771,7 @@ def run_crossing(args):
             flops = f.n_vox * flops_per_voxel_iteration(vol.bvals, loss, False, CROSS_OPTS["K"], shape["shell_loop"])
             peak, _ = fp32_peak_tflops()
             roof = {"bound": "alu", "achieved": flops / (prof["fused_ms"] / 1e3) / 1e12, "peak": peak,
-                    "unit": "TFLOP/s", "kernel": "k_iter_fused"}
+                    "unit": "TFLOP/s", "kernel": kernel_name(shape)}
             roof["frac"] = roof["achieved"] / peak
             fu = prism.Fitter(vol, prism.options(loss=loss, fused=0, use_graph=0, **CROSS_OPTS))
             fu.step(1)

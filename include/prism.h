@@ -167,13 +167,17 @@ int prism_info(const prism_handle* h, int64_t* n_vox, int32_t* n_groups, int32_t
 /*
  * Launch shape the handle runs with: lanes per voxel (1, 4 or 16; chosen at init from the
  * voxel count unless prism_options.threads_per_voxel forces one), voxels per tile, CTAs of
- * the persistent fused kernel (0 for a plain handle) and whether the fused kernel takes the
+ * the persistent kernel that prism_step launches (0 for a plain handle) and whether it takes the
  * shell loop (1) or the per-measurement loop (0). Any output pointer may be NULL. The paper
  * has no counterpart: the shape is this implementation's. Errors: PRISM_E_INVALID_ARG for a
  * NULL handle.
  */
 int prism_get_shape(const prism_handle* h, int32_t* threads_per_voxel, int32_t* tile_voxels, int32_t* fused_grid,
                     int32_t* shell_loop);
+
+/* Iterations that one launch of prism_step holds at most: 32 where a small fit takes the many-iteration
+ * kernel (k_iter_local), else 1. E_INVALID_ARG for a NULL argument. */
+int prism_launch_iterations(const prism_handle* h, int32_t* iterations);
 
 /* Raw parameters [V][Q] in mask order, to/from host or device memory (per `mem`). */
 int prism_get_params(prism_handle* h, float* out, int32_t mem, void* stream);
@@ -261,8 +265,9 @@ int prism_backward(prism_handle* h, float* grad_theta, float* grad_groups, void*
  * milliseconds per iteration to ms_out (HOST float[4]): [0] the fused iteration kernel,
  * [1] the neighbour-prior preparation kernel, [2] the group kernels (bias gradient,
  * reductions, group Adam; launched only with calibration -- otherwise the fused kernel's
- * last CTA finalises the groups and [2] is 0), [3] the whole iteration. The iterations are
- * real updates.
+ * last CTA finalises the groups and [2] is 0), [3] the whole iteration. Where one launch holds
+ * many iterations (prism_launch_iterations), n_iters of them are enqueued as by prism_step and timed
+ * as a whole: [0] and [3] are their average, [1] and [2] 0. The iterations are real updates.
  * E_STATE on a handle created with fused = 0.
  */
 int prism_profile(prism_handle* h, int32_t n_iters, void* stream, float* ms_out);

@@ -334,14 +334,18 @@ class Fitter:
         return gth, gg
 
     def shape(self):
-        """Launch shape: lanes per voxel, voxels per tile, CTAs of the fused kernel, shell loop."""
-        tpv, tv, grid, sh = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
+        """Launch shape: lanes per voxel, voxels per tile, CTAs of the kernel that step() launches, shell loop,
+        iterations that one launch holds at most."""
+        tpv, tv, grid, sh, it = (ctypes.c_int32() for _ in range(5))
         _lib.check(self._lib.prism_get_shape(self._h, ctypes.byref(tpv), ctypes.byref(tv), ctypes.byref(grid),
                                              ctypes.byref(sh)))
-        return dict(threads_per_voxel=tpv.value, tile_voxels=tv.value, fused_grid=grid.value, shell_loop=sh.value)
+        _lib.check(self._lib.prism_launch_iterations(self._h, ctypes.byref(it)))
+        return dict(threads_per_voxel=tpv.value, tile_voxels=tv.value, fused_grid=grid.value, shell_loop=sh.value,
+                    iterations_per_launch=it.value)
 
     def profile(self, n_iters=10, stream=None):
-        """Average ms per iteration: fused kernel, prior preparation, group kernels, total."""
+        """Average ms per iteration: fused kernel, prior preparation, group kernels, total. (A small fit's many
+        iterations per launch are timed as a whole.)"""
         ms = (ctypes.c_float * 4)()
         self._fwd_token = None
         _lib.check(self._lib.prism_profile(self._h, int(n_iters), _stream_ptr(stream), ms))

@@ -19,6 +19,7 @@ EXPORTS = [
     "prism_get_state", "prism_set_state", "prism_fit", "prism_fit_destroy", "prism_last_error",
     "prism_profile", "prism_grad_noalloc", "prism_microbench", "prism_get_fibers",
     "prism_fit_init_slabs", "prism_stitch_slabs", "prism_get_shape", "prism_wait_probe",
+    "prism_launch_iterations",
 ]
 
 
@@ -80,6 +81,7 @@ def load():
         "prism_wait_probe": (ctypes.c_int, [vp, i32, vp]),
         "prism_info": (ctypes.c_int, [vp, P(i64), P(i32), P(i32), P(i64), P(i64)]),
         "prism_get_shape": (ctypes.c_int, [vp, P(i32), P(i32), P(i32), P(i32)]),
+        "prism_launch_iterations": (ctypes.c_int, [vp, P(i32)]),
         "prism_get_params": (ctypes.c_int, [vp, vp, i32, vp]),
         "prism_set_params": (ctypes.c_int, [vp, vp, i32, vp]),
         "prism_group_layout": (ctypes.c_int, [vp, vp]),

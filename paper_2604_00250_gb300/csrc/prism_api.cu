@@ -1475,8 +1475,14 @@ extern "C" int prism_get_shape(const prism_handle* h, int32_t* threads_per_voxel
   if (!h) return fail(PRISM_E_INVALID_ARG, "handle is NULL");
   if (threads_per_voxel) *threads_per_voxel = h->TPV;
   if (tile_voxels) *tile_voxels = h->TV;
-  if (fused_grid) *fused_grid = h->opt.fused ? h->fused_grid : 0;
+  if (fused_grid) *fused_grid = !h->opt.fused ? 0 : h->local ? h->local_grid : h->fused_grid;
   if (shell_loop) *shell_loop = h->shell ? 1 : 0;   // either form
+  return PRISM_OK;
+}
+
+extern "C" int prism_launch_iterations(const prism_handle* h, int32_t* iterations) {
+  if (!h || !iterations) return fail(PRISM_E_INVALID_ARG, "NULL argument");
+  *iterations = h->local ? kMaxIters : 1;
   return PRISM_OK;
 }
 
@@ -1668,7 +1674,18 @@ extern "C" int prism_profile(prism_handle* h, int32_t n_iters, void* stream, flo
   for (auto& e : ev) CK(cudaEventCreate(&e));
   double acc[4] = {0, 0, 0, 0};
   int rc = PRISM_OK;
-  for (int i = 0; i < n_iters && rc == PRISM_OK; ++i) {
+  if (h->local) {   // its launches hold many iterations: the whole run is timed, as prism_step enqueues it
+    cudaError_t e = cudaEventRecord(ev[0], st);
+    if (e == cudaSuccess) rc = enqueue_fused_iters(h, n_iters, st);
+    if (e == cudaSuccess && rc == PRISM_OK) e = cudaEventRecord(ev[3], st);
+    if (e == cudaSuccess && rc == PRISM_OK) e = cudaEventSynchronize(ev[3]);
+    float t = 0.f;
+    if (e == cudaSuccess && rc == PRISM_OK) e = cudaEventElapsedTime(&t, ev[0], ev[3]);
+    if (e != cudaSuccess) rc = cuda_fail(e, "prism_profile");
+    acc[0] = acc[3] = t;
+    if (rc == PRISM_OK) h->iters += n_iters;
+  }
+  for (int i = 0; i < n_iters && rc == PRISM_OK && !h->local; ++i) {
     cudaError_t e = cudaEventRecord(ev[0], st);
     if (e == cudaSuccess && h->opt.lam_sp > 0.f) e = h->ks->prior_prep(a, 0, h->ntiles, st);
     if (e == cudaSuccess && h->nb) e = h->ks->prior_grad(a, 0, h->ntiles, st);

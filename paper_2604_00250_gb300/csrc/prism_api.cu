@@ -880,7 +880,7 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
   CK(cudaMemsetAsync(h->d_pg, 0, sizeof(float) * pg_len, st));
   RC(h->alloc(&h->d_gU, Vp));
   RC(h->alloc(&h->d_tile_ab, h->ab_len));
-  const size_t red_len = static_cast<size_t>(h->ntiles) * (h->local ? kMaxIters * (kLocalRed + 1) : 4);
+  const size_t red_len = static_cast<size_t>(h->ntiles) * (h->local ? 2 * kMaxIters : 4);
   RC(h->alloc(&h->d_tile_red, red_len));
   RC(h->alloc(&h->d_nbr, static_cast<size_t>(o.connectivity) * Vp));
   RC(h->alloc(&h->d_vcoord, Vp));

@@ -27,7 +27,6 @@ constexpr int kMaxIters = 32;      // iterations per launch (Adam's constants of
 constexpr int kLocalRow = 7;       // float4 per measurement pair in shared memory: the six that the
                                    // uncalibrated step reads and one of padding, so that eight lanes
                                    // reading eight neighbouring rows hit different banks
-constexpr int kLocalRed = kFusedThreads / 32;   // partials of J per tile and iteration: one per warp
 // Floats per voxel of a state array in shared memory: 4K + 5 rounded up to an odd multiple of 4, so that
 // eight voxels' rows fall into different banks, whether a lane reads a float or four.
 __host__ __device__ constexpr int local_stride(int K) { return K <= 1 ? 12 : K <= 3 ? 20 : 28; }
@@ -44,9 +43,9 @@ __device__ __forceinline__ int ld_acquire(const int32_t* p) {
   return v;
 }
 
-// dJ/dsigma of a tile (Rician NLL), behind the objective's partials: [kMaxIters][ntiles].
+// dJ/dsigma of a tile (Rician NLL), behind the objective's partials; both [kMaxIters][ntiles].
 __device__ __forceinline__ double* local_dsig(const IterArgs& a, int it, int tile) {
-  return a.tile_red + static_cast<size_t>(kMaxIters) * a.ntiles * kLocalRed + static_cast<size_t>(it) * a.ntiles + tile;
+  return a.tile_red + static_cast<size_t>(kMaxIters + it) * a.ntiles + tile;
 }
 
 // Sum of a volume's dJ/dsigma of one iteration, fixed order: strided over the warp's lanes, then a
@@ -60,35 +59,46 @@ __device__ __forceinline__ double local_dsig_sum(const IterArgs& a, const GroupD
 }
 
 // A volume's objective of every iteration of the launch, by the CTA that finished the volume's last
-// tile: a warp takes kSums iterations at a time, so that their loads and butterflies overlap (one after the
-// other they are chains of about half a microsecond each). With the launch's last CTA doing all volumes' sums
-// one by one, 16 volumes of 10^3 voxels took 13.6 us an iteration instead of 7.0 and the 8^3 patch 48 instead of
-// 43 us a call of 16.
-constexpr int kSums = 4;
-__device__ __forceinline__ void local_objectives(const IterArgs& a, const GroupDev& gr, int group, int step) {
+// tile, from one FP64 value per tile and iteration. A lane adds four strided sums, a butterfly the lanes. A warp
+// takes an iteration; with fewer iterations than warps all of them share each (`part`: 128 doubles), in
+// the same order, so that the bits do not depend on how many iterations a launch holds. (Four values per tile, summed by
+// one warp where the launch holds one iteration: a call of one took 235 us for 32,760 voxels with sixteen lanes, of which the
+// iteration was 40. With the launch's last CTA doing all volumes' sums one by one, 16 volumes of 10^3 voxels
+// took 13.6 us an iteration instead of 7.0.)
+__device__ __forceinline__ void local_objectives(const IterArgs& a, const GroupDev& gr, int group, int step, double* part) {
   constexpr int NW = kFusedThreads / 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = gr.ntiles * kLocalRed;
-  const size_t row = static_cast<size_t>(a.ntiles) * kLocalRed;
-  for (int i0 = warp; i0 < a.n_it; i0 += kSums * NW) {
-    const double* red = a.tile_red + i0 * row + static_cast<size_t>(gr.tile0) * kLocalRed;
-    double J[kSums];
-#pragma unroll
-    for (int u = 0; u < kSums; ++u) J[u] = 0.0;
-    for (int i = lane; i < n; i += 32) {
-#pragma unroll
-      for (int u = 0; u < kSums; ++u)
-        if (i0 + u * NW < a.n_it) J[u] += __ldcg(red + u * NW * row + i);
+  static_assert(NW == 4, "four strided sums");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = gr.ntiles;
+  auto store = [&](int it, double s0, double s1, double s2, double s3) {
+    const double J = warp_sum_d((s0 + s1) + (s2 + s3));
+    if (lane != 0) return;
+    if (!isfinite(J)) atomicOr(a.status, kStNonfinite);
+    if (it == a.n_it - 1) a.gloss[group] = J;
+    a.hist[static_cast<size_t>((step + it) % a.hist_len) * a.G + group] = J;
+  };
+  if (a.n_it < NW) {
+    for (int it = 0; it < a.n_it; ++it) {
+      const double* red = a.tile_red + static_cast<size_t>(it) * a.ntiles + gr.tile0;
+      double s = 0.0;
+#pragma unroll 8
+      for (int i = threadIdx.x; i < n; i += kFusedThreads) s += __ldcg(red + i);
+      part[threadIdx.x] = s;
+      __syncthreads();
+      if (warp == 0) store(it, part[lane], part[lane + 32], part[lane + 64], part[lane + 96]);
+      __syncthreads();
     }
+    return;
+  }
+  for (int it = warp; it < a.n_it; it += NW) {
+    const double* red = a.tile_red + static_cast<size_t>(it) * a.ntiles + gr.tile0;
+    double s[NW] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int i = lane; i < n; i += kFusedThreads) {
 #pragma unroll
-    for (int u = 0; u < kSums; ++u) J[u] = warp_sum_d(J[u]);
-#pragma unroll
-    for (int u = 0; u < kSums; ++u) {
-      const int it = i0 + u * NW;
-      if (lane != 0 || it >= a.n_it) continue;
-      if (!isfinite(J[u])) atomicOr(a.status, kStNonfinite);
-      if (it == a.n_it - 1) a.gloss[group] = J[u];
-      a.hist[static_cast<size_t>((step + it) % a.hist_len) * a.G + group] = J[u];
+      for (int u = 0; u < NW; ++u)
+        if (i + 32 * u < n) s[u] += __ldcg(red + i + 32 * u);
     }
+    store(it, s[0], s[1], s[2], s[3]);
   }
 }
 
@@ -105,6 +115,7 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
   __shared__ uint64_t s_bar;
   __shared__ float s_ac[2 * kMaxIters];
   __shared__ int s_last[2];   // this CTA counted in last: of the tile's volume, of the launch
+  __shared__ double s_J[kMaxIters * NW];   // the warps' parts of the objective by iteration; then local_objectives' sums
   __shared__ double s_ex[NW];   // NLL: the warps' dJ/dsigma, and the volume's sigma_log of the next iteration
   __shared__ float s_sig;
   __shared__ float4 s_bess[(LOSS == kLossNLL) ? kBesselTab : 1];
@@ -186,10 +197,20 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
         const int i0 = (LOSS == kLossMSE) ? gr.nb0p : 0;
         if (i0 > js) step2_b0<K>(DP, yc2 + js * VW, TPV * VW, (i0 - js + TPV - 1) / TPV, AP);
         int p = i0 + ((js - i0) % TPV + TPV) % TPV;
-#pragma unroll (K >= 4 || LOSS == kLossNLL ? 1 : 2)
-        for (; p < N / 2; p += TPV)
-          step2<K, false, LOSS>(DP, reinterpret_cast<const MeasPair&>(s_tab[p * kLocalRow]), yc2[p * VW],
-                                make_float2(1.f, 1.f), AP, inv_s2, s_bess);
+        // (the rows' address runs along with the pair; with more than three fibers the signal's too, and it alone ends the
+        // loop: 5 fibers, N = 600, 12^3: 14.3 -> 13.4 us an iteration, 3 fibers 9.6 -> 9.35)
+        const float4* row = s_tab + p * kLocalRow;
+        if constexpr (K >= 4) {
+          const float2* yp = yc2 + p * VW;
+#pragma unroll 1
+          for (const float4* end = s_tab + N / 2 * kLocalRow; row < end; row += TPV * kLocalRow, yp += TPV * VW, p += TPV)
+            step2<K, false, LOSS>(DP, reinterpret_cast<const MeasPair&>(*row), *yp, make_float2(1.f, 1.f), AP, inv_s2, s_bess);
+        } else {
+#pragma unroll (LOSS == kLossNLL ? 1 : 2)
+          for (; p < N / 2; p += TPV, row += TPV * kLocalRow)
+            step2<K, false, LOSS>(DP, reinterpret_cast<const MeasPair&>(*row), yc2[p * VW], make_float2(1.f, 1.f), AP, inv_s2,
+                                  s_bess);
+        }
         if (p < (N + 1) / 2)   // the last measurement of an odd count
           step2<K, true, LOSS>(DP, reinterpret_cast<const MeasPair&>(s_tab[p * kLocalRow]), yc2[p * VW],
                                make_float2(1.f, 0.f), AP, inv_s2, s_bess);
@@ -253,11 +274,11 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
 #pragma unroll
       for (int q = 0; q < Q; ++q) th[q] = st[q];
       transform<K>(th, P);
-      // the warp's partial of the objective: lanes 0 .. VW - 1 hold its voxels
+      // the warp's part of the objective: lanes 0 .. VW - 1 hold its voxels
       double J = act ? static_cast<double>(dloss) + static_cast<double>(ploss) : 0.0;
 #pragma unroll
       for (int o = 1; o < VW; o <<= 1) J += __shfl_xor_sync(0xffffffffu, J, o);
-      if (lane == 0) a.tile_red[(static_cast<size_t>(it) * a.ntiles + t) * kLocalRed + warp] = J;
+      if (lane == 0) s_J[it * NW + warp] = J;
       if (LOSS == kLossNLL) {
         // the first warp alone waits for the volume's tiles and takes its sum (with every warp doing so, a
         // third of the iteration went into the exchange)
@@ -297,6 +318,11 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
       }
     }
     __syncthreads();
+    if (tid < n_it) {   // the tile's objective of each iteration (n_it <= 32: the first warp)
+      const double* w = s_J + tid * NW;
+      a.tile_red[static_cast<size_t>(tid) * a.ntiles + t] = (w[0] + w[1]) + (w[2] + w[3]);
+    }
+    if (warp == 0) __syncwarp();
     if (tid == 0) {   // both counts in flight at once, under the stores below
       __threadfence();
       const int left = gr.ntiles - 1 - atomicAdd(a.gbar + a.G + tl.group, 1);
@@ -317,7 +343,7 @@ __global__ void __launch_bounds__(kFusedThreads, (K >= 4 ? 3 : 4)) k_iter_local(
     __syncthreads();
     if (s_last[0]) {
       __threadfence();
-      local_objectives(a, gr, tl.group, step);
+      local_objectives(a, gr, tl.group, step, s_J);
       if (tid == 0) a.gbar[a.G + tl.group] = 0;
     }
   }

@@ -22,11 +22,9 @@ def test_partials_are_read_after_a_warp_barrier():
 
 
 def test_timed_out_copy_is_waited_for_and_none_follows():
-    """After a copy's wait has run out the CTA lets the copy land, issues no further one and updates and
-    stores nothing, but counts its tiles in."""
+    """After a copy's wait has run out the CTA lets the copy land, issues no further one and stores no state."""
     k = " ".join(kernel().split())
     assert "if (tid == 0 && !failed) { const uint32_t bytes" in k                    # no further copy
     out = k[k.index("if (!failed && !mbar_wait(&s_bar, phase)) {"):]
     assert "mbar_wait(&s_bar, phase);" in out[out.index("{"):out.index("}")]          # lets it land
-    assert "for (int it = failed ? n_it : 0; it < n_it; ++it)" in k and "&& !failed; e +=" in k
-    assert "if (LOSS == kLossNLL && tid == 0 && failed) atomicAdd(a.gbar + tl.group, n_it);" in k
+    assert "e < Q * TV && !failed; e += kFusedThreads" in k                           # no state stored

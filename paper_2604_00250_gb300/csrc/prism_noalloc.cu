@@ -169,6 +169,13 @@ __global__ void __launch_bounds__(kNaThreads, (K >= 4 ? 3 : 4)) k_grad_noalloc(
       }
     }
   }
+  // a mean whose reciprocal overflows: the voxel's row and mean times 2^64 as each chunk arrives
+  const bool tiny = b0 < 1e-37f;
+  if (tiny) b0 *= 18446744073709551616.f;
+  auto scale_up = [&](int j) {
+    float* r = ring + (j & 1) * (32 * kNaStride) + lane * kNaStride;
+    for (int i = 0; tiny && i < kNaChunk; ++i) r[i] *= 18446744073709551616.f;
+  };
   // y = signal / b0 by the reciprocal and one correction (a division's accuracy in three packed operations;
   // the correction of an infinite signal, a NaN, is dropped by fminf, so that it stays infinite)
   const float ib = 1.f / b0;
@@ -192,6 +199,7 @@ __global__ void __launch_bounds__(kNaThreads, (K >= 4 ? 3 : 4)) k_grad_noalloc(
     for (int j = 0; j < nch; ++j) {
       cp_async_wait<1>();
       __syncwarp();
+      scale_up(j);
       const float* row = ring + (j & 1) * (32 * kNaStride) + lane * kNaStride;
       const int pc0 = j * (kNaChunk / 2), pc1 = min(pc0 + kNaChunk / 2, tb.np);
       int p = pc0;
@@ -239,6 +247,7 @@ __global__ void __launch_bounds__(kNaThreads, (K >= 4 ? 3 : 4)) k_grad_noalloc(
     for (int j = 0; j < nch; ++j) {
       cp_async_wait<1>();
       __syncwarp();
+      scale_up(j);
       const float* row = ring + (j & 1) * (32 * kNaStride) + lane * kNaStride;
       const int pc0 = j * (kNaChunk / 2), pe = min(pc0 + kNaChunk / 2, tb.np), pf = min(pe, N / 2);
       int p = pc0;

@@ -446,10 +446,19 @@ def _make_autograd():
                 f.forward(*ctx.point)
                 ctx.token = f._fwd_token
             gth, gg = f.backward()
-            # Out of place: the factor may be part of a graph (create_graph) or a batch of factors
-            # (is_grads_batched, a vectorised Jacobian). 0-dim, it takes the gradients' type.
-            g_theta = (gth * gout).to(ctx.dtypes[0]) if ctx.needs_input_grad[0] else None
-            g_groups = (gg * gout).to(ctx.dtypes[1]) if ctx.needs_input_grad[1] else None
+            # In place on the fresh gradients where that is possible (two allocations less, 15 of 310 us for a
+            # small patch). Out of place for a factor in a graph (create_graph), and for a batch of factors
+            # (is_grads_batched, a vectorised Jacobian), for which mul_ raises before it writes.
+            # The 0-dim factor takes the gradients' type.
+            inplace = not gout.requires_grad
+            if inplace:
+                try:
+                    gth.mul_(gout)
+                except RuntimeError:
+                    inplace = False
+            gth, gg = (gth, gg.mul_(gout)) if inplace else (gth * gout, gg * gout)
+            g_theta = gth.to(ctx.dtypes[0]) if ctx.needs_input_grad[0] else None
+            g_groups = gg.to(ctx.dtypes[1]) if ctx.needs_input_grad[1] else None
             return g_theta, g_groups, None
 
     return PrismLoss

@@ -1438,6 +1438,10 @@ __global__ void __launch_bounds__(kFusedThreads, (fused_min_blocks<K, TPV, LOSS,
         }
         if (a.nb_priors) {
           for (int c = 0; c < kPgRows<K>; ++c) prefetch_l2(a.pg + static_cast<size_t>(c) * Vp + slot0, rb);
+        } else if (a.nb_priors) {
+          for (int e = 0; e < a.n_nbr; ++e) prefetch_l2(a.nbr + static_cast<size_t>(e) * Vp + slot0, rb);
+          if (a.lam_sp > 0.f)
+            for (int c = 0; c < NF; ++c) prefetch_l2(a.hsp + static_cast<size_t>(c) * Vp + slot0, rb);
         }
       };
       if (t == s_first) rows(tl.slot0);

@@ -56,9 +56,9 @@ FLOPS_PER_B0_PAIR_SHELL = 4
 # scaled brain (traffic grows in proportion to the voxels), valid only for the kernel sources
 # whose SHA-256 (comments and blank lines left out, fused_sources_sha256) is
 # TRAFFIC_SOURCES_SHA256: any other hash reports the traffic as null.
-# 212,900 voxels: 350.2 MB read and 35.2 MB written in one launch (profiles/k_iter_fused_hcp_brain_dram_traffic.md).
-TRAFFIC_BYTES_PER_VOXEL_ITER = 1810.0
-TRAFFIC_SOURCES_SHA256 = "4690d88d01b46a6c1f647a85768af13f5f41b04cc38e3393abcc26d1f90479af"
+# 212,900 voxels: 349.6 MB read and 35.4 MB written in one launch (profiles/k_iter_fused_hcp_brain_dram_traffic.md).
+TRAFFIC_BYTES_PER_VOXEL_ITER = 1808.1
+TRAFFIC_SOURCES_SHA256 = "b5f4be7847b910ed176cbdcea53adf8ad0972a350ff87f05f534bf71c9508761"
 FUSED_SOURCES = ("prism_kernels.cuh", "prism_device.cuh", "prism_kset.cuh", "bessel_fit.h", "prism_k3.cu")
 # FP32 lanes per SM on GB300 (4 sub-partitions x 32); the peak multiplies them by the device's
 # SM count, 2 flops per fused multiply-add and the maximum SM clock seen by nvidia-smi.

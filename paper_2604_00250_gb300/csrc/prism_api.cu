@@ -1142,10 +1142,11 @@ int init_impl(prism_handle* h, const prism_volume* vols, int n_vols, const std::
 int choose_shape(const prism_options& o, const prism_volume* vols, int n, const std::vector<MaskIndex>& idx, int64_t V,
                  bool shell, int* tpv, int* nt) {
   // No neighbour priors and no calibration: the local kernel with four or sixteen lanes. Sixteen below
-  // 1,400 voxels with the MSE (10^3 at N = 96: 2.8 against 3.2 with four, 12^3 4.1 and 3.5; N = 288 3.4 and
-  // 5.5, 4.9 and 5.7) and below 4,200 with the NLL, whose measurements cost more (N = 96: 12^3 6.0 and 8.0,
-  // 16^3 8.1 and 7.5; N = 288 16^3 11.4 and 14.5); one from 32,768 on (28^3 at N = 96: 13.7 with four, 19.6 with
-  // one; 32^3 21.3 and 19.8). The NLL's tiles must fit the chip at once: where those of eight voxels do not
+  // 1,400 voxels with the MSE (10^3 at N = 96: 2.0 against 3.2 with four; N = 288 2.6 and 5.5) and below 4,200 with the
+  // NLL, whose measurements cost more (N = 96: 12^3 5.6 and 7.2, 16^3 8.0 and 6.9; N = 288 16^3 11.7 and 13.9); one
+  // from 32,768 on. (The MSE's two lines were set before a tile wrote one objective per iteration; now sixteen lanes lead up to
+  // about 3,000 voxels, 12^3 2.5 against 3.2 and 3.5 against 5.5, 16^3 3.6 and 3.2, 5.7 and 5.5, and four against one beyond
+  // 31^3, 11.7 and 20.0. The NLL's last: 31^3 at N = 96 37.8 and 26.7, at N = 288 59.5 and 53.0.) The NLL's tiles must fit the chip at once: where those of eight voxels do not
   // (large N, K >= 4, many part-filled tiles), four lanes, whose tiles hold 32 (16^3, K = 5, N = 96: general kernel
   // with sixteen lanes 25.6, local with four 8.3; K = 3, N = 1,000: 68 and 40); where neither does, the general
   // kernel's lines.

@@ -8,15 +8,14 @@
 // arithmetic is under 1 us. Here a voxel's lanes sit in one warp: all of them carry out the voxel's
 // chain rule on the summed accumulators (issue slots that a small fit leaves idle) and share its update,
 // so that an iteration of the MSE has no block barrier. Measured per iteration (GB300, MSE, K = 3, N = 96):
-// 8^3 voxels 2.3 us (general kernel 13.8), 16^3 4.1 and 24^3 8.9 us (general kernel with one thread per
-// voxel 17.5 and 18.1).
+// 8^3 voxels 2.0 us (general kernel 13.8), 16^3 3.2 (17.5) and 28^3 8.5 us (19.6 with one thread per voxel).
 //
 // Rician NLL: dJ/dsigma is a sum over the volume in each iteration. The tiles of a volume
 // write their FP64 partials and count themselves in on a per-volume counter, before the chain rule and the
 // update; after these they wait for the count of the iteration; then every tile takes the same
 // fixed-order sum and updates its own copy of sigma.
 // The launch is cooperative (every CTA resident, one tile each) and every wait has a limit. 16
-// volumes of 10^3 voxels: 75 -> 11.6 us an iteration (N = 96; 12.2 with the partials written after the update).
+// volumes of 10^3 voxels: 75 -> 11.5 us an iteration (N = 96; 12.2 with the partials written after the update).
 #pragma once
 
 #include "prism_kernels.cuh"
